@@ -313,7 +313,7 @@ int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmar
     const double *key = lnw ? lnw : lnL_tmarg;
     CK(launch_reduce(key, lnL_tmarg, n, h->red_partial, h->stats, kScratchSlot, h->pooled_scratch, 1, h->err,
                      h->stream));
-    CK(launch_select(key, n, h->stats, kScratchSlot, kMixedMargin, h->sel_idx, h->sel_count, h->stream));
+    CK(launch_select(key, h->perm, n, h->stats, kScratchSlot, kMixedMargin, h->sel_idx, h->sel_count, h->stream));
     // the tensor-core kernel recomputes the float32 per-bin ln L of the first refine_rows
     // selected samples (a few tiles), so the refinement itself evaluates only the bins
     // within its margin in float64

@@ -147,14 +147,14 @@ cudaError_t launch_prep_tc(const double2 *Q64, int K, int M, int n_q, int groups
                            __half *Qtc, cudaStream_t st);
 
 // Precision mode RIFT_MIXED: indices of the samples with key[i] >= stats[slot].max - margin
-// (idx[*count], ascending), then their float64 re-evaluation in place (lnL_tmarg, and lnw
+// (idx[*count], in the order of perm), then their float64 re-evaluation in place (lnL_tmarg, and lnw
 // when given).  count points to kSelectWords words (the count, then block scratch).
 constexpr int kSelectWords = 1 + 1024;
 // selected samples whose float32 per-bin values the tiled kernel recomputes for the
 // refinement (the rest are recomputed by the refinement itself)
 constexpr int64_t kRefineRows = 16384;
-cudaError_t launch_select(const double *key, int64_t n, const double *stats, int slot, double margin, uint32_t *idx,
-                          uint32_t *count, cudaStream_t st);
+cudaError_t launch_select(const double *key, const uint32_t *perm, int64_t n, const double *stats, int slot,
+                          double margin, uint32_t *idx, uint32_t *count, cudaStream_t st);
 // v32 (optional): float32 per-bin ln L of the selected samples, row w for the w-th selected
 // sample, for w < v32_rows; the others get their float32 bins recomputed.
 cudaError_t launch_refine(const Problem &P, const double *theta, const uint32_t *idx, const uint32_t *count,
