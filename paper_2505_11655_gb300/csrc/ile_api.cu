@@ -29,6 +29,9 @@ struct StateHeader {
     uint32_t reserved;
 };
 
+// Shared memory a block may use on sm_103a (for sizing without a CUDA call).
+constexpr int kSmemOptin = 227 * 1024;
+
 // Q window padding of the float32 planes: one chunk window past the end.
 constexpr int kQPad = 256 + 16;
 
@@ -308,12 +311,48 @@ constexpr double kMixedMargin = 40.0;
 // exceeds this (k_fixup.cu)
 constexpr float kFixThreshold = 600.f;
 
+// Below this many samples the sort costs more than it saves (2 detectors, 2 modes, 401 bins:
+// 512 samples 137 us sorted, 110 us unsorted; with 3 detectors and 21 modes the sort's windows
+// and launches break even there).
+constexpr int64_t kTc64Unsorted = 512;
+
+int lnl_float64(rift_ile_t *h, const double *theta, int64_t n, bool keyed, double *lnL_tmarg, double *lnL_t,
+                const double *lnpw, double *lnw)
+{
+    if (!h->tc64_on) {
+        CK(launch_lnl_fp64(h->prob, theta, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err, h->stream));
+        h->launches += 1;
+        return RIFT_OK;
+    }
+    // a few tiles fill the device by splitting the bins, whatever their windows' width
+    const bool sort = n > kTc64Unsorted;
+    int k = 0;
+    if (sort) {
+        if (!keyed) {
+            RK(grid_for_batch(h, n));
+            CK(launch_keys(h->grid, theta, n, h->key, h->stream));
+        }
+        CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, h->stream, &k));
+        k += keyed ? 0 : 1;
+    }
+    CK(launch_lnl_tc64(h->prob, h->x64, theta, sort ? h->perm : nullptr, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err,
+                       h->stream));
+    h->launches += k + 2;
+    return RIFT_OK;
+}
+
 int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg, const double *lnpw, double *lnw)
 {
     const double *key = lnw ? lnw : lnL_tmarg;
     CK(launch_reduce(key, lnL_tmarg, n, h->red_partial, h->stats, kScratchSlot, h->pooled_scratch, 1, h->err,
                      h->stream));
     CK(launch_select(key, h->perm, n, h->stats, kScratchSlot, kMixedMargin, h->sel_idx, h->sel_count, h->stream));
+    if (h->tc64_on) {
+        CK(launch_lnl_tc64(h->prob, h->x64, theta, h->sel_idx, n, lnL_tmarg, nullptr, lnpw, lnw, h->err,
+                           h->stream, h->sel_count));
+        h->launches += 7;
+        return RIFT_OK;
+    }
     // the tensor-core kernel recomputes the float32 per-bin ln L of the first refine_rows
     // selected samples (a few tiles), so the refinement itself evaluates only the bins
     // within its margin in float64
@@ -372,11 +411,8 @@ cudaError_t mark(rift_ile_t *h, int slot, int stage)
 int eval_device(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg, double *lnL_t, const double *lnpw,
                 double *lnw)
 {
-    if (!use_fp32(h)) {
-        CK(launch_lnl_fp64(h->prob, theta, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err, h->stream));
-        h->launches += 1;
-        return RIFT_OK;
-    }
+    if (!use_fp32(h))
+        return lnl_float64(h, theta, n, false, lnL_tmarg, lnL_t, lnpw, lnw);
     RK(choose_plan(h, n, false));
     RK(grid_for_batch(h, n));
     int sorted = 0;
@@ -402,7 +438,7 @@ int run_iteration(rift_ile_t *h, int64_t n, int slot, bool adapt, bool reset_poo
         CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, h->stream, &sorted));
     CK(mark(h, slot, 1));
     if (!use_fp32(h)) {
-        CK(launch_lnl_fp64(h->prob, h->theta, n, h->lnL, nullptr, h->lnpw, h->lnw, h->err, h->stream));
+        RK(lnl_float64(h, h->theta, n, true, h->lnL, nullptr, h->lnpw, h->lnw));
     } else {
         CK(launch_tiled(h, h->theta, n, h->lnL, nullptr, h->lnpw, h->lnw));
         if (h->cfg.precision == RIFT_MIXED)
@@ -415,7 +451,7 @@ int run_iteration(rift_ile_t *h, int64_t n, int slot, bool adapt, bool reset_poo
     if (adapt)
         CK(launch_adapt(S, h->bins, h->lnw, n, h->stats, slot, h->hist_partial, h->stream, f32_terms));
     CK(mark(h, slot, 3));
-    h->launches += 1 + sorted + 1 + 2 + (adapt ? 2 : 0);
+    h->launches += 1 + sorted + (use_fp32(h) ? 1 : 0) + 2 + (adapt ? 2 : 0);
     return RIFT_OK;
 }
 
@@ -725,7 +761,41 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
         if (const char *env = std::getenv("RIFT_ILE_FIX_T"))
             h->fix_thr = (float)std::atof(env);
     }
-    if (cfg->precision == RIFT_MIXED) {
+    int dev = 0, max_smem = 0, major = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    P.tc_groups = (cfg->n_q + 7) / 8 + 17;
+    {
+        const char *env = std::getenv("RIFT_ILE_TC");
+        h->tc64_on = cfg->precision != RIFT_FP32 && major == 10 && !(env && env[0] == '0') && lnl_tc64_fits(P, max_smem);
+    }
+    if (h->tc64_on) {
+        unsigned char *scratch = nullptr, *records = nullptr;
+        int *unit_counter = nullptr;
+        long long *pos = nullptr;
+        if ((rc = dalloc(h, &h->qmax64, (size_t)2)) || (rc = dalloc(h, &h->q_dig, tc64_q_halves(K, M, P.tc_groups))) ||
+            (rc = dalloc(h, &h->t_dig, tc64_t_halves(K, M))) || (rc = dalloc(h, &h->t_exp64, (size_t)kMaxDet)) ||
+            (rc = dalloc(h, &scratch, tc64_scratch_bytes(K, M, N, sms))) ||
+            (rc = dalloc(h, &records, tc64_record_bytes(N, cfg->n_t))) || (rc = dalloc(h, &pos, (size_t)cfg->n_t + kTc64Table)) ||
+            (rc = dalloc(h, &unit_counter, (size_t)4))) {
+            release(h);
+            return rc;
+        }
+        h->x64 = Tc64{h->qmax64, h->q_dig, h->t_dig, h->t_exp64, scratch, records, unit_counter,
+                      pos, {}};
+        std::vector<long long> host_pos(cfg->n_t + kTc64Table);
+        tc64_positions(h->cfg, host_pos.data(), h->x64.u0);
+        if (cudaMemsetAsync(unit_counter, 0, sizeof(int), h->stream) ||
+            cudaMemcpyAsync(pos, host_pos.data(), sizeof(long long) * host_pos.size(), cudaMemcpyHostToDevice, h->stream) ||
+            cudaStreamSynchronize(h->stream)) {
+            cudaGetLastError();
+            release(h);
+            return RIFT_ECUDA;
+        }
+    }
+    if (cfg->precision == RIFT_MIXED && !h->tc64_on) {
         h->refine_rows = std::min<int64_t>(N, kRefineRows);
         if ((rc = dalloc(h, &h->refine_bins, (size_t)h->refine_rows * cfg->n_t))) {
             release(h);
@@ -756,14 +826,9 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
         release(h);
         return RIFT_ECUDA;
     }
-    P.tc_groups = (cfg->n_q + 7) / 8 + 17;
     P.Qtc = h->Qtc;
     P.qmax_bits = h->qmax_bits;
     {
-        int dev = 0, max_smem = 0, major = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
         h->tc_ok = major == 10 && lnl_tc_fits(P, max_smem);
         const char *env = std::getenv("RIFT_ILE_TC");
         if (env && env[0] == '0')
@@ -772,7 +837,7 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
             h->tc_mode = 1;
         if (prepare_sampler_kernels() != cudaSuccess || prepare_refine_kernels() != cudaSuccess ||
             prepare_tile_kernels() != cudaSuccess || (h->tc_ok && prepare_tc_kernels() != cudaSuccess) ||
-            prepare_fix_kernels() != cudaSuccess) {
+            prepare_fix_kernels() != cudaSuccess || (h->tc64_on && prepare_tc64_kernels() != cudaSuccess)) {
             cudaGetLastError();
             release(h);
             return RIFT_ECUDA;
@@ -813,13 +878,24 @@ int64_t rift_ile_footprint(const rift_ile_config *cfg)
     const int64_t K = cfg->n_det, M = cfg->n_modes, N = cfg->max_samples, B = cfg->n_bins, nt = cfg->n_t;
     const int64_t nq = cfg->n_q, nq_pad = ((nq + 3) & ~3) + kQPad;
     const int64_t groups = (nq + 7) / 8 + 17, kp = (2 * M + 15) / 16 * 16;
+    // digits and scratch of the float64-accurate tensor-core kernel (k_tile_tc64.cu)
+    Problem Pf{};
+    Pf.K = cfg->n_det;
+    Pf.M = cfg->n_modes;
+    Pf.n_q = cfg->n_q;
+    Pf.n_t = cfg->n_t;
+    Pf.dist_marg = cfg->distance_marg;
+    const bool digits = cfg->precision != RIFT_FP32 && lnl_tc64_fits(Pf, kSmemOptin);
     const int64_t sizes[] = {
         K * M * nq * 16, 2 * K * M * M * 16, K * 2 * M * nq_pad * 4, 2 * K * M * M * 8, K * 2 * kp * kp * 2, K * 4,
         2 * nt * 4,
         N * 6 * 8, 3 * N * 8, N * 8, 2 * N * 4, (int64_t)sort_scratch_words(N) * 4, 16, 16,
         K * 2 * groups * kp * 8 * 2, 5 * kRedBlocks * 8, 152 * 12 * B * 8, 8 * (RIFT_MAX_ITER + 1) * 8, 3 * 8 * 8,
         N * 4, 16, 6 * B * 8, 6 * (B + 1) * 8, 6 * B * 8, 16, (int64_t)kSelectWords * 4,
-        cfg->precision == RIFT_MIXED ? std::min<int64_t>(N, kRefineRows) * nt * 8 : 0,
+        cfg->precision == RIFT_MIXED && !digits ? std::min<int64_t>(N, kRefineRows) * nt * 8 : 0,
+        digits ? 2 * (int64_t)(tc64_q_halves(K, M, groups) + tc64_t_halves(K, M)) + 7 * 16 + 8 * (nt + kTc64Table) +
+                     (int64_t)(tc64_scratch_bytes(K, M, N, 152) + tc64_record_bytes(N, cfg->n_t))
+               : 0,
         // large-term correction: per-sample side outputs and list, pair tables, double-float
         // copies of U, V (at most M^2 pairs each) and Q
         cfg->precision != RIFT_FP64 && !cfg->distance_marg ? 4 * N * 4 + 16 + 4 * M * M + 8 * 64 +
@@ -1009,6 +1085,10 @@ int install_overlaps(rift_ile_t *h)
     if (h->tc_ok) {
         CK(launch_prep_tc(h->Q64, K, M, nq, h->prob.tc_groups, h->qmax_bits, h->Qtc, h->stream));
         CK(launch_prep_tt(h->U64, h->V64, K, M, h->Ttc, h->tt_exp, h->stream));
+        h->launches += 3;
+    }
+    if (h->tc64_on) {
+        CK(launch_prep_tc64(h->prob, h->qmax64, h->q_dig, h->t_dig, h->t_exp64, h->stream));
         h->launches += 3;
     }
     if (h->fix_on) {
@@ -1234,7 +1314,9 @@ int rift_ile_fair_draws(rift_ile_t *h, int64_t n_draws, uint64_t seed, int mem, 
     if (n == 0)
         return RIFT_ESTATE;
     const int nt = h->prob.n_t;
-    const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_draws, (int64_t)(16 << 20) / nt));
+    int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_draws, (int64_t)(16 << 20) / nt));
+    if (h->tc64_on)
+        chunk = std::min(chunk, h->cap);   // the sort's buffers hold cap samples
     std::vector<void *> tmp;
     auto grab = [&](size_t bytes) -> void * {
         void *q = nullptr;
@@ -1269,9 +1351,9 @@ int rift_ile_fair_draws(rift_ile_t *h, int64_t n_draws, uint64_t seed, int mem, 
         // time bins from each drawn sample's per-bin ln L, in float64 (the draws are few)
         for (int64_t c0 = 0; c0 < n_draws; c0 += chunk) {
             const int64_t m = std::min(chunk, n_draws - c0);
-            CK(launch_lnl_fp64(h->prob, th + 6 * c0, m, lt, bins, nullptr, nullptr, h->err, h->stream));
+            RK(lnl_float64(h, th + 6 * c0, m, false, lt, bins, nullptr, nullptr));
             CK(launch_fair_time(bins, m, nt, Ut + c0, h->prob.t_lo, h->prob.t_step, jj + c0, tt + c0, h->stream));
-            h->launches += 2;
+            h->launches += 1;
         }
         if (theta)
             CK(cudaMemcpyAsync(theta, th, sizeof(double) * 6 * n_draws, kind, h->stream));

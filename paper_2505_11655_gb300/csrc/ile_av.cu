@@ -301,7 +301,7 @@ int av_iteration(rift_ile_t *h, int64_t n, int slot, bool reset_pooled, double p
     CK(mark(h, slot, 1));
     // 2. likelihood
     if (!use_fp32(h)) {
-        CK(launch_lnl_fp64(h->prob, h->theta, n, h->lnL, nullptr, h->lnpw, h->lnw, h->err, st));
+        RK(lnl_float64(h, h->theta, n, false, h->lnL, nullptr, h->lnpw, h->lnw));
     } else {
         CK(launch_tiled(h, h->theta, n, h->lnL, nullptr, h->lnpw, h->lnw));
         if (h->cfg.precision == RIFT_MIXED)
@@ -311,7 +311,7 @@ int av_iteration(rift_ile_t *h, int64_t n, int slot, bool reset_pooled, double p
     CK(launch_reduce(h->lnw, h->lnL, n, h->red_partial, h->stats, slot, h->pooled, reset_pooled ? 1 : 0, h->err,
                      st, h->cfg.precision == RIFT_FP32));
     CK(mark(h, slot, 3));
-    h->launches += 1 + sorted + 1 + 2;
+    h->launches += 1 + sorted + (use_fp32(h) ? 1 : 0) + 2;
     return av_update(h, a.v_fresh, h->lnL, n, p_thr, n_min_star);
 }
 

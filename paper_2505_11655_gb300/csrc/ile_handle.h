@@ -69,6 +69,12 @@ struct rift_ile {
     rift::FixTables fix{};
     bool fix_on = false;
     float fix_thr = 0.f;
+    // float64-accurate tensor-core likelihood (RIFT_FP64 batches, RIFT_MIXED re-evaluation)
+    bool tc64_on = false;
+    rift::Tc64 x64{};
+    unsigned long long *qmax64 = nullptr;
+    __half *q_dig = nullptr, *t_dig = nullptr;
+    int *t_exp64 = nullptr;
     double *P = nullptr, *C = nullptr, *Lg = nullptr;
     int *err = nullptr;
     uint32_t *iter_dev = nullptr;   // sampler iteration counter read by the draw kernel
@@ -179,6 +185,11 @@ cudaError_t launch_tiled(rift_ile_t *h, const double *theta, int64_t n, double *
 void drop_graph(rift_ile_t *h);
 int install_overlaps(rift_ile_t *h);
 cudaError_t mark(rift_ile_t *h, int slot, int stage);
+// Float64 ln L of n device-resident samples (RIFT_FP64): the tensor-core kernel on large
+// batches (sorted by h->key when `keyed`, else by keys computed here), the plain kernel on
+// the others.  Uses h->key and h->perm.
+int lnl_float64(rift_ile_t *h, const double *theta, int64_t n, bool keyed, double *lnL_tmarg, double *lnL_t,
+                const double *lnpw, double *lnw);
 int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg, const double *lnpw, double *lnw);
 int sync_and_err(rift_ile_t *h, int *flags_out = nullptr);
 // Device buffer from the stream-ordered pool on the handle's stream, freed at destroy.

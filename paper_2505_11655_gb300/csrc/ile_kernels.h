@@ -146,6 +146,36 @@ cudaError_t launch_lnl_tc(const Problem &P, BinTable bt, const double *theta, co
 cudaError_t launch_prep_tc(const double2 *Q64, int K, int M, int n_q, int groups, unsigned int *qmax_bits,
                            __half *Qtc, cudaStream_t st);
 
+// Float64-accurate likelihood on the tensor cores (k_tile_tc64.cu): digits of Q and of the
+// template matrices, and the kernel's scratch.
+struct Tc64 {
+    const unsigned long long *qmax;   // bits of max|Q|
+    const __half *q_dig, *t_dig;
+    const int *t_exp;
+    unsigned char *scratch;           // coefficient digits of the resident tiles
+    unsigned char *records;           // the chunks' sums of a batch whose time bins are split
+    int *unit_counter;                // 0 between launches
+    const long long *pos;             // [n_t] Q positions of the bins relative to the first (2^-48),
+                                      // then the exponential's table
+    long long u0[kMaxDet];            // Q position of the first bin without delay (2^-48)
+};
+bool lnl_tc64_fits(const Problem &P, int max_smem);
+size_t tc64_q_halves(int K, int M, int groups);
+size_t tc64_t_halves(int K, int M);
+size_t tc64_record_bytes(int64_t n_max, int n_t);
+// Fills pos [n_t + kTc64Table] and u0 [n_det] (host).
+constexpr int kTc64Table = 128;
+void tc64_positions(const rift_ile_config &cfg, long long *pos, long long *u0);
+size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms);
+cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half *q_dig, __half *t_dig, int *t_exp,
+                             cudaStream_t st);
+// perm lists the samples (min(n, *n_dev) of them when a device count is given; null: in
+// order); outputs at the sample's index.
+cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta, const uint32_t *perm, int64_t n,
+                            double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
+                            cudaStream_t st, const uint32_t *n_dev = nullptr);
+cudaError_t prepare_tc64_kernels();
+
 // Precision mode RIFT_MIXED: indices of the samples with key[i] >= stats[slot].max - margin
 // (idx[*count], in the order of perm), then their float64 re-evaluation in place (lnL_tmarg, and lnw
 // when given).  count points to kSelectWords words (the count, then block scratch).

@@ -668,7 +668,7 @@ int portfolio_iteration(rift_ile_t *h, int64_t n, int slot, bool reset_pooled, c
     CK(mark(h, slot, 1));
     // 2. likelihood and the iteration's record
     if (!use_fp32(h)) {
-        CK(launch_lnl_fp64(h->prob, h->theta, n, h->lnL, nullptr, h->lnpw, h->lnw, h->err, st));
+        RK(lnl_float64(h, h->theta, n, true, h->lnL, nullptr, h->lnpw, h->lnw));
     } else {
         CK(launch_tiled(h, h->theta, n, h->lnL, nullptr, h->lnpw, h->lnw));
         if (h->cfg.precision == RIFT_MIXED)
@@ -682,7 +682,7 @@ int portfolio_iteration(rift_ile_t *h, int64_t n, int slot, bool reset_pooled, c
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(kPfSumBlocks, (n + kPfThreads - 1) / kPfThreads));
     member_sums_kernel<<<nb, kPfThreads, 0, st>>>(h->lnw, p.member, n, p.part);
     member_sums_final_kernel<<<1, 32 * kNMembers, 0, st>>>(p.part, nb, p.sums);
-    h->launches += 1 + sorted + 1 + 2 + 2;
+    h->launches += 1 + sorted + (use_fp32(h) ? 1 : 0) + 2 + 2;
     const int n_em = act[2] ? kEmStride * p.gmm_C : 0;
     if (act[2]) {
         const size_t em_smem = sizeof(double) * (kGmmTab + 6 * kPfThreads + (size_t)kPfThreads * p.gmm_C);

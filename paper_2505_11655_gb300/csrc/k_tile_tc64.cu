@@ -1,0 +1,1020 @@
+// Float64-accurate likelihood on the tensor cores (arXiv:2505.11655 Sec. II A,
+// Eq. (def:lnL:Decomposed), time-marginalised).
+//
+// The float64 pipe of this part does about two operations a clock and SM, so the plain
+// float64 kernel (k_lnl.cu) is bound by it: 6 operations a mode, bin and detector.  Here
+// the mode sum, the interpolation and the log-sum-exp over the time bins run in fixed point
+// instead, exactly or to at least float64's resolution, and the float64 pipe is left with
+// the per-sample geometry:
+//   * the coefficients c_k,lm of a sample (one power-of-two scale over its detectors and
+//     modes) and Q (one scale) are rounded to 55-bit integers, each cut into kDig = 7
+//     balanced base-256 digits d_0..d_6 (|d| <= 128, exact in float16);
+//   * R[s, c] = Re sum_lm conj(c_lm) Q_lm on the Q grid is contracted digit by digit with
+//     tcgen05 kind::f16 MMAs into one float32 accumulator per order o = i + j <= 6 of digit
+//     products: an order holds at most 7 x 42 products below 2^14, so every partial sum is
+//     an integer below 2^22 (order 6: 2^23) and exact.  Digit i of the coefficients meets
+//     digits 0..6-i of Q in one MMA (N = 32 (7 - i) columns: the digits of 32 Q columns side by
+//     side), so the accumulators of all orders are filled by 7 MMAs per 16 components.  The
+//     orders beyond 6 are left out: below 2^-53 of max|c| max|Q|, as is the rounding of the
+//     55-bit integers;
+//   * the seven accumulators are drained from tensor memory and joined to one 64-bit integer
+//     X = sum_o a_o 2^(40 - 8 o) (float additions of 1.5 2^23 turn them into integers);
+//   * interpolation between neighbouring columns by a 64-bit high multiplication with the
+//     node fraction (48 bits), sums over detectors in 64-bit integers;
+//   * the log-sum-exp takes differences to the running maximum as integers and 2^-t from a
+//     128-entry table and a short polynomial in 64-bit fixed point; sums with 2^-52
+//     resolution.  A chunk's bins are summed by four threads, their sums and the chunks'
+//     merged in a fixed order.
+// The template term is contracted the same way, W_k = Z_k T_k (the real quadratic form of
+// k_tile_tc.cu) and summed against the float64 components.
+//
+// Tiles are 128 samples in the order of the sky sort.  A tile's window on the Q grid is as
+// wide as its samples' delays need (no sub-groups: a chunk of 64 time bins walks the
+// detector's window in blocks of 64 columns and every sample takes the bins whose nodes lie
+// in the block).  The coefficients' digits (86 KB a detector at 21 modes) are written once per
+// tile to a scratch in global memory (L2) and loaded into shared memory by bulk copies
+// whenever the detector changes.  When a batch has few tiles its time bins are split over
+// several blocks (units), and a second kernel merges the chunks' sums.  Every step of a
+// sample's value is exact or done in a fixed order on the sample's own numbers, so it does
+// not depend on the batch, the tile or the split.
+//
+// Measured (3 detectors, 21 modes, 16384 Hz, 1001 bins, 20011 prior samples): 20.3 ms for the
+// plain float64 kernel (70% of the float64 issue rate), 1.35 ms here; 100,000 samples 98.5 ->
+// 4.3 ms; 64 samples of the smallest problem (2 detectors, 2 modes) 109 -> 107 us.  Against
+// 80-bit arithmetic its per-bin values are closer than the plain kernel's (rms 2.7e-13
+// against 4.1e-13 here).  What bounds it now is instruction issue (46% of the slots: the
+// joins of the accumulators, the gathers' 64-bit arithmetic) and the tail of uneven tiles; the
+// tensor pipe is 26% busy, the float64 pipe 11%.
+//
+// All waits are bounded (1 s by the global timer), as in k_tile_tc.cu.
+#include <algorithm>
+#include <climits>
+#include <cmath>
+#include <cuda_fp16.h>
+
+#include "ile_kernels.h"
+#include "tc_ptx.cuh"
+
+namespace rift {
+
+namespace {
+
+constexpr int kDig = 7;             // base-256 digits of a 55-bit integer
+constexpr int kS = 128;             // samples per tile (MMA M)
+constexpr int kSub = 32;            // Q columns per MMA batch
+constexpr int kBlk = 64;            // Q columns per gathered block (two batches)
+constexpr int kConsumers = 512;
+constexpr int kThreads = kConsumers + 64;
+constexpr int kIssuer = kConsumers / 32, kStager = kIssuer + 1;
+constexpr int kQ = kConsumers / kS;      // threads per sample
+constexpr int kBpt = 16;                 // time bins per thread and chunk
+constexpr int kChunk = kQ * kBpt;
+constexpr int kAccCols = kDig * kSub;    // tensor-memory columns of one set of accumulators
+constexpr int kTable = kTc64Table;       // entries 2^-(i/128) of the exponential
+constexpr int kFrac = 48;                // fraction bits of a Q position
+constexpr int kPows = kMaxPow + 1;
+constexpr uint64_t kWait = 1000000000ull;
+constexpr int kRecords = 4096;           // (tile, chunk) pairs of a batch whose time bins are split
+constexpr int kSumBits = 52;             // resolution of the log-sum-exp (at most 4000 terms <= 1)
+constexpr size_t kMinSmem = 120 * 1024;  // one block per SM
+static_assert(2 * kAccCols <= 512, "two sets of accumulators in tensor memory");
+static_assert(kS * kMaxDet <= kConsumers, "one (sample, detector) item per consumer thread");
+
+struct Layout64 {
+    size_t a, b, r, pos, u0, quad, sc, gid, bad, tbl, m2, lo, bar, tptr, end;
+    size_t nv, e5, ps, pw, pe, F, Y, pend;   // prologue tables, aliased on a, b, r
+    int kp;
+};
+
+__host__ __device__ inline size_t al64(size_t o, size_t a = 128) { return (o + a - 1) / a * a; }
+
+__host__ __device__ inline Layout64 layout64(int K, int M, int n_t)
+{
+    Layout64 L;
+    L.kp = (2 * M + 15) / 16 * 16;
+    size_t o = 0;
+    L.a = o;   o = al64(o + (size_t)kDig * kS * L.kp * 2);
+    L.b = o;   o = al64(o + (size_t)2 * kDig * kSub * L.kp * 2);
+    L.r = o;   o = al64(o + (size_t)(kBlk + 1) * kS * 8);
+    size_t p = 0;   // sample-minor tables of the prologue
+    L.nv = p;  p += (size_t)3 * kS * 8;
+    L.e5 = p;  p += (size_t)5 * kS * 8;
+    L.ps = p;  p += (size_t)3 * kS * 8;
+    L.pw = p;  p += (size_t)2 * kPows * kS * 8;
+    L.pe = p;  p += (size_t)(kMaxL + 1) * kS * 16;
+    L.F = p;   p += (size_t)K * kS * 16;
+    L.Y = p;   p += (size_t)M * kS * 16;
+    L.pend = p;
+    o = p > o ? al64(p) : o;
+    L.pos = o;  o = al64(o + (size_t)n_t * 8, 16);
+    L.u0 = o;   o = al64(o + (size_t)K * kS * 8, 16);
+    L.quad = o; o = al64(o + (size_t)kQ * kS * 8, 16);
+    L.sc = o;   o = al64(o + (size_t)kS * 4, 16);
+    L.gid = o;  o = al64(o + (size_t)kS * 4, 16);
+    L.bad = o;  o = al64(o + (size_t)kS * 4, 16);
+    L.tbl = o;  o = al64(o + (size_t)kTable * 8, 16);
+    L.m2 = o;   o = al64(o + (size_t)2 * kS * 8, 16);
+    L.lo = o;   o = al64(o + (size_t)2 * kMaxDet * 8, 16);
+    L.bar = o;  o = al64(o + (size_t)8 * 8, 16);
+    L.tptr = o; o = al64(o + 16, 16);
+    L.end = o;
+    return L;
+}
+
+// bytes of one detector's coefficient digits, and of a block's scratch
+__host__ __device__ inline size_t a_bytes(int kp) { return (size_t)kDig * kS * kp * 2; }
+
+// Units (tile x part of the time bins) of a batch: parts chosen so that the units fill the
+// blocks evenly, where the split's records fit.  A unit costs its prologue (about a fifth of
+// a whole tile's work) plus its share of the bins.
+__host__ __device__ inline int parts64(int64_t tiles, int grid, int n_chunks)
+{
+    int best = 1;
+    float cost = 1e30f;
+    for (int p = 1; p <= 16 && p <= n_chunks; ++p) {
+        if (p > 1 && tiles * n_chunks > (int64_t)kRecords)
+            break;
+        const float c = (float)((tiles * p + grid - 1) / grid) * (0.2f + 1.0f / p);
+        if (c < cost) {
+            cost = c;
+            best = p;
+        }
+    }
+    return best;
+}
+
+// ---------------------------------------------------------------- digits
+
+// Position of the leading bit: |x| < 2^e for every x with |x| <= m (0 for m = 0).
+__device__ __forceinline__ int exp_above(double m)
+{
+    int e = 0;
+    if (m > 0.0)
+        frexp(m, &e);
+    return e;
+}
+
+// x 2^e by a multiplication (float64 is slow on this part, and ldexp is several operations)
+__device__ __forceinline__ double mul_pow2(double x, int e)
+{
+    if (e > 1000 || e < -1000)
+        return ldexp(x, e);
+    return x * __hiloint2double((1023 + e) << 20, 0);
+}
+
+// The seven digits of a 55-bit integer as float16 bit patterns: the integer plus a bias of
+// 128 in each of its six low bytes has the biased digits as bytes (the top one in bits
+// 48..56), and float16 1024 + b is the pattern 0x6400 | b.
+__device__ __forceinline__ uint64_t digit_bytes(long long I) { return (uint64_t)I + 0x0080808080808080ull; }
+
+__device__ __forceinline__ uint32_t digit_pair(uint64_t x, uint64_t y, int part)
+{
+    // bytes of x and y biased by 128 -> two float16 digits
+    const int sh = 8 * (kDig - 1 - part);
+    const uint32_t mask = part == 0 ? 0x1ffu : 0xffu;
+    const uint32_t a = (uint32_t)(x >> sh) & mask, b = (uint32_t)(y >> sh) & mask;
+    const uint32_t v = 0x64006400u | a | (b << 16);
+    __half2 h;
+    memcpy(&h, &v, 4);
+    h = __hsub2(h, __floats2half2_rn(1152.f, 1152.f));
+    uint32_t r;
+    memcpy(&r, &h, 4);
+    return r;
+}
+
+__global__ void max64_kernel(const double2 *__restrict__ Q, int64_t count, unsigned long long *__restrict__ out)
+{
+    unsigned long long m = 0ull;   // non-negative doubles order as integers
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x) {
+        const double2 q = Q[e];
+        m = max(m, (unsigned long long)__double_as_longlong(fabs(q.x)));
+        m = max(m, (unsigned long long)__double_as_longlong(fabs(q.y)));
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0 && m)
+        atomicMax(out, m);
+}
+
+// Q digits: [K][kDig][groups][kp/8][8 columns][8 components]
+__global__ void digits_q_kernel(const double2 *__restrict__ Q, int K, int M, int n_q, int groups, int kp,
+                                const unsigned long long *__restrict__ qmax, __half *__restrict__ out)
+{
+    const int sq = 55 - exp_above(__longlong_as_double((long long)*qmax));
+    const int64_t per_part = (int64_t)groups * kp * 8, total = (int64_t)K * per_part / 2;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t f = 2 * e;   // an even component and the odd one behind it: one mode
+        const int k = (int)(f / per_part);
+        const int64_t w = f - (int64_t)k * per_part;
+        const int g = (int)(w / (kp * 8)), rem = (int)(w - (int64_t)g * kp * 8);
+        const int kc = rem / 64, row = (rem / 8) % 8, m = (8 * kc + rem % 8) / 2, c = 8 * g + row;
+        uint64_t x = digit_bytes(0), y = x;
+        if (c < n_q && m < M) {
+            const double2 q = Q[((int64_t)k * M + m) * n_q + c];
+            x = digit_bytes(__double2ll_rn(ldexp(q.x, sq)));
+            y = digit_bytes(__double2ll_rn(ldexp(q.y, sq)));
+        }
+        for (int p = 0; p < kDig; ++p)
+            reinterpret_cast<uint32_t *>(out + ((int64_t)k * kDig + p) * per_part)[w / 2] = digit_pair(x, y, p);
+    }
+}
+
+// Entry (r, c) of the real template matrix: z^T T z = c^H U c + Re(c^T V c) (see k_tile_tc.cu)
+__device__ __forceinline__ double template_entry(const double2 *U, const double2 *V, int M, int r, int c)
+{
+    const double2 u = U[(size_t)(r >> 1) * M + (c >> 1)], v = V[(size_t)(r >> 1) * M + (c >> 1)];
+    if (!(r & 1))
+        return (c & 1) ? -u.y - v.y : u.x + v.x;
+    return (c & 1) ? u.x - v.x : u.y - v.y;
+}
+
+// Template digits: [K][kDig][kBlk/8 groups][kp/8][8 columns of T][8 components]; exps[k]
+// such that |T_k| < 2^exps[k].  One block per detector.
+__global__ void digits_t_kernel(const double2 *__restrict__ U64, const double2 *__restrict__ V64, int M, int kp,
+                                __half *__restrict__ out, int *__restrict__ exps)
+{
+    __shared__ unsigned long long mx;
+    const int k = blockIdx.x, R2 = 2 * M;
+    const double2 *U = U64 + (size_t)k * M * M, *V = V64 + (size_t)k * M * M;
+    if (threadIdx.x == 0)
+        mx = 0ull;
+    __syncthreads();
+    for (int e = threadIdx.x; e < R2 * R2; e += blockDim.x)
+        atomicMax(&mx, (unsigned long long)__double_as_longlong(fabs(template_entry(U, V, M, e / R2, e % R2))));
+    __syncthreads();
+    const int et = exp_above(__longlong_as_double((long long)mx));
+    if (threadIdx.x == 0)
+        exps[k] = et;
+    const int per_part = kBlk * kp;
+    for (int f = 2 * threadIdx.x; f < per_part; f += 2 * blockDim.x) {
+        const int g = f / (kp * 8), rem = f - g * kp * 8;
+        const int kc = rem / 64, row = (rem / 8) % 8, c = 8 * kc + rem % 8, n = 8 * g + row;
+        uint64_t x = digit_bytes(0), y = x;
+        if (n < R2 && c < R2) {
+            x = digit_bytes(__double2ll_rn(ldexp(template_entry(U, V, M, c, n), 55 - et)));
+            y = digit_bytes(__double2ll_rn(ldexp(template_entry(U, V, M, c + 1, n), 55 - et)));
+        }
+        for (int p = 0; p < kDig; ++p)
+            reinterpret_cast<uint32_t *>(out + ((size_t)k * kDig + p) * per_part)[f / 2] = digit_pair(x, y, p);
+    }
+}
+
+// ---------------------------------------------------------------- fixed point
+
+// 2^-t of t = T 2^-57 (0 <= t < 64) as E 2^-63 times 2^-n: table of 2^-(i/128), and with
+// g = r ln 2 of the rest r < 2^-7 the nested series 1 - g (1 - g/2 (1 - g/3 (1 - g/4 + g^2/20 -
+// g^3/120))) in 64-bit fixed point (the innermost factor needs 32 bits only).
+__device__ __forceinline__ uint64_t exp2_neg(uint64_t T, const uint64_t *__restrict__ tbl, int &n)
+{
+    n = (int)(T >> 57);
+    const uint64_t f = T & ((1ull << 57) - 1ull);
+    const uint64_t G = __umul64hi((f & ((1ull << 50) - 1ull)) << 14, 0xB17217F7D1CF79ACull);   // g 2^71
+    const uint32_t g32 = (uint32_t)(G >> 39), gh = (uint32_t)(G >> 32);
+    const uint32_t gg = __umulhi(g32, g32);
+    // (1 - g/4 + g^2/20 - g^3/120) / 3 in units 2^-32
+    const uint32_t c3 = 0x55555555u - __umulhi(gh, 2796202u) + __umulhi(gg, 71582788u - __umulhi(g32, 11930465u));
+    const uint64_t a3 = ~(((uint64_t)gh * c3) >> 7);        // 1 - g/3 (...), units 2^-64
+    const uint64_t a2 = ~(__umul64hi(G, a3) >> 8);          // 1 - g/2 (...)
+    const uint64_t p = ~(__umul64hi(G, a2) >> 7);           // 1 - g (...)
+    return __umul64hi(tbl[f >> 50], p);
+}
+
+// Scaled differences of a sample: lin = X 2^L.
+struct DiffScale {
+    int sh;          // T = (D << sh) log2(e) 2^-1 with sh = L + 58 (D >> -sh when negative)
+    uint64_t dmax;   // larger differences are e^-44 and below
+    __device__ void set(int L)
+    {
+        sh = max(-63, min(63, L + 58));
+        const int s = -L;
+        dmax = s >= 58 ? ~0ull : s >= 0 ? 44ull << s : s > -6 ? 44ull >> -s : 0ull;
+    }
+    __device__ uint64_t exponent(uint64_t D) const
+    {
+        return __umul64hi(sh >= 0 ? D << sh : D >> -sh, 0xB8AA3B295C17F0BCull);
+    }
+};
+
+// Log-sum-exp over bins: sum of exp(lin - max) in units 2^-kSumBits, max as an integer.
+struct Lse {
+    long long m;
+    uint64_t s;
+};
+
+// exp(-D 2^L) in units 2^-kSumBits
+__device__ __forceinline__ uint64_t term64(const DiffScale &ds, uint64_t D, const uint64_t *tbl)
+{
+    if (D > ds.dmax)
+        return 0ull;
+    int n;
+    const uint64_t e = exp2_neg(ds.exponent(D), tbl, n);
+    return ((e >> (62 - kSumBits + min(n, kSumBits + 1))) + 1ull) >> 1;
+}
+
+__device__ __forceinline__ Lse merge64(const DiffScale &ds, Lse a, Lse b, const uint64_t *tbl)
+{
+    if (a.m < b.m) {
+        const Lse t = a;
+        a = b;
+        b = t;
+    }
+    const uint64_t D = (uint64_t)a.m - (uint64_t)b.m;
+    if (b.s != 0ull && D <= ds.dmax) {
+        int n;
+        const uint64_t e = exp2_neg(ds.exponent(D), tbl, n);
+        a.s += ((__umul64hi(b.s, e) << 1) | ((b.s * e) >> 63)) >> n;
+    }
+    return a;
+}
+
+__device__ __forceinline__ double lse_value(Lse v, int lexp, double quad, int n_t)
+{
+    const double sum = (double)v.s * (1.0 / (double)(1ull << kSumBits));
+    return __dsub_rn(mul_pow2((double)v.m, lexp), quad) + __dsub_rn(log(sum), log((double)n_t));
+}
+
+// one accumulator set joined to X (see the head of the file)
+__device__ __forceinline__ long long join_orders(const uint32_t (&v)[kDig][4], int i)
+{
+    constexpr float kMagic = 12582912.f;   // 1.5 2^23: float bits 0x4B400000 + integer
+    constexpr uint64_t kB = 0x4B400000ull;
+    constexpr uint64_t kBias = (kB << 40) + (kB << 32) + (kB << 24) + (kB << 16) + (kB << 8) + kB + kB;
+    const uint32_t b0 = __float_as_uint(__uint_as_float(v[0][i]) + kMagic);
+    const uint32_t b1 = __float_as_uint(__uint_as_float(v[1][i]) + kMagic);
+    const uint32_t b2 = __float_as_uint(__uint_as_float(v[2][i]) + kMagic);
+    const uint32_t b3 = __float_as_uint(__uint_as_float(v[3][i]) + kMagic);
+    const uint32_t b4 = __float_as_uint(__uint_as_float(v[4][i]) + kMagic);
+    const uint32_t b5 = __float_as_uint(__uint_as_float(v[5][i]) + kMagic);
+    const uint32_t b6 = __float_as_uint(fmaf(__uint_as_float(v[6][i]), 0x1p-8f, kMagic));
+    uint64_t x = (uint64_t)b5 + b6 - kBias;
+    x += (uint64_t)b4 * 256u;
+    x += (uint64_t)b3 * 65536u;
+    x += (uint64_t)b2 * 16777216u;
+    x += (uint64_t)((b0 << 8) + b1) << 32;
+    return (long long)x;
+}
+
+}  // namespace
+
+bool lnl_tc64_fits(const Problem &P, int max_smem)
+{
+    // at most 42 components (order 5: 6 x 42 products of 2^14 stay below 2^22)
+    return !P.dist_marg && 2 * P.M <= 42 && P.n_q < (1 << 14) && P.n_t <= 4000 &&
+           layout64(P.K, P.M, P.n_t).end + 2048 <= (size_t)max_smem;
+}
+
+size_t tc64_q_halves(int K, int M, int groups)
+{
+    return (size_t)K * kDig * groups * ((2 * M + 15) / 16 * 16) * 8;
+}
+
+size_t tc64_t_halves(int K, int M) { return (size_t)K * kDig * kBlk * ((2 * M + 15) / 16 * 16); }
+
+// records of the split: per (chunk, sample) the chunk's Lse, and per sample its template term
+// and scale
+static int64_t split_tiles(int64_t n_max, int n_t)
+{
+    const int64_t n_chunks = (n_t + kChunk - 1) / kChunk;
+    return std::min<int64_t>((n_max + kS - 1) / kS, kRecords / n_chunks);
+}
+
+size_t tc64_record_bytes(int64_t n_max, int n_t)
+{
+    return (size_t)split_tiles(n_max, n_t) * kS * 16 * ((n_t + kChunk - 1) / kChunk + 1);
+}
+
+size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms)
+{
+    const int64_t tiles = (n_max + kS - 1) / kS, blocks = std::min<int64_t>(sms, 16 * tiles);
+    return (size_t)blocks * K * a_bytes((2 * M + 15) / 16 * 16);
+}
+
+void tc64_positions(const rift_ile_config &cfg, long long *pos, long long *u0)
+{
+    for (int j = 0; j < cfg.n_t; ++j) {
+        const long double t =
+            cfg.n_t > 1 ? j * ((long double)cfg.t_hi_s - (long double)cfg.t_lo_s) / (cfg.n_t - 1) : 0.0L;
+        pos[j] = std::llround(std::ldexp(t * (long double)cfg.fs_hz, kFrac));
+    }
+    for (int i = 0; i < kTable; ++i)
+        pos[cfg.n_t + i] = (long long)(uint64_t)std::ldexp(std::exp2(-(long double)i / kTable), 63);
+    for (int k = 0; k < cfg.n_det; ++k)
+        u0[k] = std::llround(
+            std::ldexp(((long double)cfg.t_lo_s - (long double)cfg.q_t0_s[k]) * (long double)cfg.fs_hz, kFrac));
+}
+
+cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half *q_dig, __half *t_dig, int *t_exp,
+                             cudaStream_t st)
+{
+    const int kp = (2 * P.M + 15) / 16 * 16;
+    cudaError_t e = cudaMemsetAsync(qmax, 0, sizeof(unsigned long long), st);
+    if (e != cudaSuccess)
+        return e;
+    const int64_t cnt = (int64_t)P.K * P.M * P.n_q;
+    max64_kernel<<<(int)std::min<int64_t>((cnt + 255) / 256, 512), 256, 0, st>>>(P.Q64, cnt, qmax);
+    const int64_t tot = (int64_t)P.K * P.tc_groups * kp * 4;
+    digits_q_kernel<<<(int)std::min<int64_t>((tot + 255) / 256, 2048), 256, 0, st>>>(P.Q64, P.K, P.M, P.n_q,
+                                                                                    P.tc_groups, kp, qmax, q_dig);
+    digits_t_kernel<<<P.K, 512, 0, st>>>(P.U64, P.V64, P.M, kp, t_dig, t_exp);
+    return cudaGetLastError();
+}
+
+namespace {
+
+__global__ void __launch_bounds__(kThreads, 1)
+lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
+                double *__restrict__ lnL_tmarg, double *__restrict__ lnL_t, const double *__restrict__ lnpw,
+                double *__restrict__ lnw, int *err, int *unit_counter, const uint32_t *__restrict__ n_dev)
+{
+    extern __shared__ __align__(128) unsigned char sm[];
+    const int K = P.K, M = P.M, NT = P.n_t;
+    const Layout64 L = layout64(K, M, NT);
+    const int kp = L.kp, kcs = kp / 8;
+    __half *As = reinterpret_cast<__half *>(sm + L.a);              // [kDig][kS x kp]
+    __half *Bs = reinterpret_cast<__half *>(sm + L.b);              // [2][kDig][kSub x kp]
+    long long *Rs = reinterpret_cast<long long *>(sm + L.r);        // [1 + kBlk][kS]; row 0 the previous block's last
+    long long *pos = reinterpret_cast<long long *>(sm + L.pos);     // [NT] bin offset in Q samples, kFrac fraction bits
+    long long *U0 = reinterpret_cast<long long *>(sm + L.u0);       // [K][kS] Q position of the first bin
+    double *quads = reinterpret_cast<double *>(sm + L.quad);        // [kQ][kS] template term partials
+    int *scs = reinterpret_cast<int *>(sm + L.sc);                  // [kS] c = I 2^-sc
+    uint32_t *gid = reinterpret_cast<uint32_t *>(sm + L.gid);
+    int *bad = reinterpret_cast<int *>(sm + L.bad);                 // [kS] error flags of the sample
+    uint64_t *tbl = reinterpret_cast<uint64_t *>(sm + L.tbl);       // 2^-(i/128) 2^63
+    unsigned long long *mF2 = reinterpret_cast<unsigned long long *>(sm + L.m2), *mY2 = mF2 + kS;
+    long long *ulo = reinterpret_cast<long long *>(sm + L.lo), *uhi = ulo + kMaxDet;
+    uint64_t *full = reinterpret_cast<uint64_t *>(sm + L.bar);      // [0,1] Q digits staged
+    uint64_t *done = full + 2;                                      // [0,1] MMAs of a batch complete
+    uint64_t *empty = full + 4;                                     // [0,1] accumulators drained
+    uint64_t *fullA = full + 6;                                     // coefficient digits staged
+    uint32_t *tptr = reinterpret_cast<uint32_t *>(sm + L.tptr);
+    double *nv = reinterpret_cast<double *>(sm + L.nv), *e5 = reinterpret_cast<double *>(sm + L.e5);
+    double *ps = reinterpret_cast<double *>(sm + L.ps), *pw = reinterpret_cast<double *>(sm + L.pw);
+    double2 *pe = reinterpret_cast<double2 *>(sm + L.pe), *Fs = reinterpret_cast<double2 *>(sm + L.F);
+    double2 *Ys = reinterpret_cast<double2 *>(sm + L.Y);
+    __shared__ int unit_s, abort_s;
+
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const bool producer = warp >= kIssuer;
+    const int64_t n_use = n_dev ? min(n, (int64_t)*n_dev) : n;
+    const int64_t n_tiles = (n_use + kS - 1) / kS;
+    const int n_chunks = (NT + kChunk - 1) / kChunk, jnom = (NT + n_chunks - 1) / n_chunks;
+    const int parts = parts64(n_tiles, (int)gridDim.x, n_chunks);
+    const int sq = 55 - exp_above(__longlong_as_double((long long)*X.qmax));
+    const uint32_t sub_bytes = (uint32_t)(kSub * kp * 2);           // one digit of a batch's columns
+    const size_t ab = a_bytes(kp);
+    __half *scratch = reinterpret_cast<__half *>(X.scratch + (size_t)blockIdx.x * K * ab);
+    Lse *records = reinterpret_cast<Lse *>(X.records);
+    const uint32_t sbo = (uint32_t)kcs * 128u;
+    auto desc = [&](const void *p, uint32_t off) {
+        return ((uint64_t)(((sbo >> 4) & 0x3FFFu) | (1u << 14)) << 32) |
+               (((tc::smem_u32(p) + off) & 0x3FFFFu) >> 4) | ((uint64_t)(128u >> 4) << 16);
+    };
+
+    for (int j = tid; j < NT; j += kThreads)
+        pos[j] = X.pos[j];
+    for (int i = tid; i < kTable; i += kThreads)
+        tbl[i] = (uint64_t)X.pos[NT + i];
+    if (warp == 0)
+        tc::tmem_alloc(tptr, 512);
+    if (tid == 0) {
+        for (int i = 0; i < 4; ++i)
+            tc::mbar_init(full + i, 1);
+        for (int i = 4; i < 6; ++i)
+            tc::mbar_init(full + i, kConsumers / 32);
+        tc::mbar_init(fullA, 1);
+        tc::fence_mbar_init();
+        abort_s = 0;
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    tc::tc_fence_after();
+    const uint32_t tmem = *tptr;
+    // every role walks the same sequence of batches: g counts them (buffer g & 1, its
+    // (g >> 1)-th use), ga the loads of coefficient digits
+    uint32_t g = 0, ga = 0;
+    bool first = true;
+
+    for (;;) {
+        // the shared memory that the next unit's copies overwrite was last touched by generic
+        // accesses of this thread
+        tc::fence_proxy_async_smem();
+        if (tid == 0) {
+            // the first unit by the block's index, the others from the counter
+            unit_s = abort_s ? INT_MAX : first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(unit_counter, 1);
+            first = false;
+        }
+        if (tid < K) {
+            ulo[tid] = LLONG_MAX;
+            uhi[tid] = LLONG_MIN;
+        }
+        if (tid < kS) {
+            mF2[tid] = 0ull;
+            mY2[tid] = 0ull;
+            bad[tid] = 0;
+        }
+        __syncthreads();
+        const int64_t unit = unit_s;
+        if (unit >= n_tiles * parts)
+            break;
+        const int64_t tile = unit / parts;
+        const int part = (int)(unit - tile * parts);
+        const int s_of = tid & (kS - 1), grp = tid >> 7;
+
+        // ---------------- prologue A: trigonometry in float64, a quarter of it per thread
+        if (!producer) {
+            const int64_t si = tile * kS + s_of;
+            const uint32_t gi = si >= n_use ? 0xffffffffu : perm ? perm[si] : (uint32_t)si;
+            const double *th = theta + 6 * (int64_t)gi;
+            const bool valid = gi != 0xffffffffu;
+            if (grp == 0) {
+                gid[s_of] = gi;
+                const Sky sk = sky_of(valid ? th[0] : 0.0, valid ? th[1] : 0.0, P.gmst);
+                nv[s_of] = sk.cd * sk.ch;
+                nv[kS + s_of] = sk.cd * sk.sh;
+                nv[2 * kS + s_of] = sk.sd;
+                e5[s_of] = sk.cd;
+                e5[kS + s_of] = sk.sd;
+                e5[2 * kS + s_of] = sk.ch;
+                e5[3 * kS + s_of] = sk.sh;
+            } else if (grp == 1) {
+                double s2, c2;
+                sincos(2.0 * (valid ? th[2] : 0.0), &s2, &c2);
+                ps[s_of] = c2;
+                ps[kS + s_of] = s2;
+                ps[2 * kS + s_of] = valid ? P.d_ref / th[5] : 0.0;
+            } else if (grp == 2) {
+                double sh, ch;
+                sincos(0.5 * (valid ? th[4] : 0.0), &sh, &ch);
+                double pc = 1.0, pp = 1.0;
+                for (int q = 0; q < kPows; ++q) {
+                    pw[q * kS + s_of] = pc;
+                    pw[(kPows + q) * kS + s_of] = pp;
+                    pc *= ch;
+                    pp *= sh;
+                }
+            } else {
+                double sp, cp;
+                sincos(valid ? th[3] : 0.0, &sp, &cp);
+                double er = 1.0, ei = 0.0;   // exp(-i j phi)
+                for (int j = 0; j <= kMaxL; ++j) {
+                    pe[j * kS + s_of] = make_double2(er, ei);
+                    const double t = er * cp + ei * sp;
+                    ei = ei * cp - er * sp;
+                    er = t;
+                }
+            }
+        }
+        __syncthreads();
+        // ---------------- B: delays, x F_k, harmonics, and the largest |F|^2 and |Y|^2
+        if (!producer) {
+            if (tid < kS * K) {
+                const int k = grp;
+                const double n0 = nv[s_of], n1 = nv[kS + s_of], n2 = nv[2 * kS + s_of];
+                const Sky sk{e5[s_of], e5[kS + s_of], e5[2 * kS + s_of], e5[3 * kS + s_of]};
+                // the delay in Q samples; the first bin's position is added in fixed point, so that
+                // its rounding, which every bin shares, is that of the delay alone
+                const double u0 = fma(P.xfs[k][0], n0, fma(P.xfs[k][1], n1, P.xfs[k][2] * n2));
+                const bool valid = gid[s_of] != 0xffffffffu, ok = isfinite(u0);
+                if (valid && !ok)
+                    atomicOr(bad + s_of, kErrRange | kErrNonFinite);
+                const long long u = ok ? X.u0[k] + __double2ll_rn(u0 * (double)(1ll << kFrac)) : 0;
+                U0[k * kS + s_of] = u;
+                long long ulow = valid && ok ? u : LLONG_MAX, uhigh = valid && ok ? u : LLONG_MIN;
+#pragma unroll
+                for (int o = 16; o; o >>= 1) {
+                    ulow = min(ulow, __shfl_xor_sync(0xffffffffu, ulow, o));
+                    uhigh = max(uhigh, __shfl_xor_sync(0xffffffffu, uhigh, o));
+                }
+                if (lane == 0 && ulow != LLONG_MAX) {
+                    atomicMin(ulo + k, ulow);
+                    atomicMax(uhi + k, uhigh);
+                }
+                Cx<double> F = response<double>(P, k, sk, ps[s_of], ps[kS + s_of]);
+                const double x = ps[2 * kS + s_of];
+                F.re *= x;
+                F.im *= x;
+                Fs[k * kS + s_of] = make_double2(F.re, F.im);
+                atomicMax(mF2 + s_of, (unsigned long long)__double_as_longlong(fma(F.re, F.re, F.im * F.im)));
+            }
+            for (int m = grp; m < M; m += kQ) {
+                double d = 0.0;
+                for (int t = 0; t < P.wn[m]; ++t)
+                    d += P.wcoef[m][t] * pw[P.wpc[m][t] * kS + s_of] * pw[(kPows + P.wps[m][t]) * kS + s_of];
+                const int mm = P.mode_m[m];
+                const double2 e = pe[(mm < 0 ? -mm : mm) * kS + s_of];
+                const double2 y = make_double2(d * e.x, d * (mm < 0 ? -e.y : e.y));
+                Ys[m * kS + s_of] = y;
+                atomicMax(mY2 + s_of, (unsigned long long)__double_as_longlong(d * d * fma(e.x, e.x, e.y * e.y)));
+            }
+        }
+        __syncthreads();
+        // ---------------- C: the sample's scale and the digits of its coefficients
+        if (!producer) {
+            const double f2 = __longlong_as_double((long long)mF2[s_of]), y2 = __longlong_as_double((long long)mY2[s_of]);
+            int ef = 0, ey = 0;
+            const bool zero = !(f2 > 0.0) || !(y2 > 0.0) || !isfinite(f2) || !isfinite(y2);
+            if (!zero) {
+                frexp(f2, &ef);
+                frexp(y2, &ey);
+            }
+            // |c|^2 <= f2 y2 < 2^(ef + ey): |c| < 2^ceil((ef + ey) / 2)
+            const int sc = zero ? 0 : 55 - ((ef + ey + 1) >> 1);
+            if (grp == 0) {
+                scs[s_of] = sc;
+                if (gid[s_of] != 0xffffffffu && (!isfinite(f2) || !isfinite(y2)))
+                    atomicOr(bad + s_of, kErrNonFinite);
+            }
+            for (int it = grp; it < K * kcs; it += kQ) {
+                const int k = it / kcs, kc = it - k * kcs;
+                double2 f = zero ? make_double2(0.0, 0.0) : Fs[k * kS + s_of];
+                f.x = mul_pow2(f.x, sc);
+                f.y = mul_pow2(f.y, sc);
+                uint64_t d[8];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int m = 4 * kc + j;
+                    long long cr = 0, ci = 0;
+                    if (m < M && !zero) {
+                        const double2 y = Ys[m * kS + s_of];
+                        cr = __double2ll_rn(f.x * y.x - f.y * y.y);
+                        ci = __double2ll_rn(f.x * y.y + f.y * y.x);
+                    }
+                    d[2 * j] = digit_bytes(cr);
+                    d[2 * j + 1] = digit_bytes(ci);
+                }
+                __half *o = scratch + ((size_t)k * kDig * kS + (size_t)(s_of >> 3) * 8) * kp + kc * 64 + (s_of & 7) * 8;
+#pragma unroll
+                for (int p = 0; p < kDig; ++p)
+                    *reinterpret_cast<uint4 *>(o + (size_t)p * kS * kp) =
+                        make_uint4(digit_pair(d[0], d[1], p), digit_pair(d[2], d[3], p), digit_pair(d[4], d[5], p),
+                                   digit_pair(d[6], d[7], p));
+            }
+            __threadfence();
+        }
+        // the tables (generic accesses) share their bytes with the targets of bulk copies, and
+        // the scratch is read by them
+        tc::fence_proxy_async();
+        __syncthreads();
+
+        const int ch0 = (int)((int64_t)part * n_chunks / parts), ch1 = (int)((int64_t)(part + 1) * n_chunks / parts);
+        const bool any = ulo[0] != LLONG_MAX;   // a sample with finite delays
+        // first column (a multiple of 8) and batches of detector k's window for the bins [j0, j1)
+        auto window = [&](int k, int j0, int j1, int &w0, int &nsub) {
+            const int c0 = (int)((ulo[k] + pos[j0]) >> kFrac), c1 = (int)((uhi[k] + pos[j1 - 1]) >> kFrac) + 1;
+            w0 = max(c0, 0) & ~7;
+            nsub = (min(c1, P.n_q - 1) - w0) / kSub + 1;
+        };
+        int failed = 0;
+        if (warp == kIssuer) {
+            if (lane == 0 && any) {
+                auto batch = [&]() {
+                    const uint32_t b = g & 1u, u = g >> 1;
+                    if (!tc::mbar_wait(full + b, u & 1u, kWait) ||
+                        (u > 0 && !tc::mbar_wait(empty + b, (u - 1u) & 1u, kWait)))
+                        return false;
+                    tc::tc_fence_after();
+                    const __half *B = Bs + (size_t)b * kDig * kSub * kp;
+                    for (int kk = 0; kk < kp / 16; ++kk) {
+                        const uint64_t bd = desc(B, 256u * (uint32_t)kk);
+#pragma unroll
+                        for (int i = 0; i < kDig; ++i)
+                            tc::mma_f16_ss(tmem + b * kAccCols + (uint32_t)(i * kSub),
+                                           desc(As + (size_t)i * kS * kp, 256u * (uint32_t)kk), bd,
+                                           tc::idesc_f16_f32(kS, (uint32_t)((kDig - i) * kSub)), (kk | i) != 0);
+                    }
+                    tc::mma_commit(done + b);
+                    ++g;
+                    return true;
+                };
+                auto digits = [&]() { return tc::mbar_wait(fullA, (ga++) & 1u, kWait); };
+                for (int k = 0; k < K && !failed; ++k)
+                    failed = !digits() || !batch() || !batch();
+                for (int ch = ch0; ch < ch1 && !failed; ++ch)
+                    for (int k = 0; k < K && !failed; ++k) {
+                        int w0, nsub;
+                        window(k, ch * jnom, min(NT, (ch + 1) * jnom), w0, nsub);
+                        if (K > 1)
+                            failed = !digits();
+                        for (int t = 0; t < nsub && !failed; ++t)
+                            failed = !batch();
+                    }
+            }
+            __syncwarp();
+        } else if (warp == kStager) {
+            if (lane == 0 && any) {
+                auto stage = [&](const __half *src, size_t stride) {
+                    const uint32_t b = g & 1u, u = g >> 1;
+                    if (u > 0 && !tc::mbar_wait(done + b, (u - 1u) & 1u, kWait))
+                        return false;
+                    __half *dst = Bs + (size_t)b * kDig * kSub * kp;
+                    tc::mbar_expect_tx(full + b, kDig * sub_bytes);
+                    for (int p = 0; p < kDig; ++p)
+                        tc::bulk_g2s(dst + (size_t)p * kSub * kp, src + (size_t)p * stride, sub_bytes, full + b);
+                    ++g;
+                    return true;
+                };
+                auto digits = [&](int k) {
+                    // every batch so far is complete: nothing reads the old digits any more
+                    if (g > 0 && !tc::mbar_wait(done + ((g - 1u) & 1u), ((g - 1u) >> 1) & 1u, kWait))
+                        return false;
+                    tc::mbar_expect_tx(fullA, (uint32_t)ab);
+                    tc::bulk_g2s(As, scratch + (size_t)k * kDig * kS * kp, (uint32_t)ab, fullA);
+                    ++ga;
+                    return true;
+                };
+                for (int k = 0; k < K && !failed; ++k) {
+                    const __half *T = X.t_dig + (size_t)k * kDig * kBlk * kp;
+                    failed = !digits(k) || !stage(T, (size_t)kBlk * kp) ||
+                             !stage(T + (size_t)kSub * kp, (size_t)kBlk * kp);
+                }
+                for (int ch = ch0; ch < ch1 && !failed; ++ch)
+                    for (int k = 0; k < K && !failed; ++k) {
+                        int w0, nsub;
+                        window(k, ch * jnom, min(NT, (ch + 1) * jnom), w0, nsub);
+                        if (K > 1)
+                            failed = !digits(k);
+                        const size_t part_h = (size_t)P.tc_groups * kp * 8;
+                        const __half *src = X.q_dig + (size_t)k * kDig * part_h + (size_t)(w0 >> 3) * kp * 8;
+                        for (int t = 0; t < nsub && !failed; ++t)
+                            failed = !stage(src + (size_t)t * kSub * kp, part_h);
+                    }
+            }
+            __syncwarp();
+        } else if (any) {
+            const int q = warp & 3, cb = warp >> 2, s = 32 * q + lane;   // drain: quarter, 8 columns of 32
+            const int gs = s_of, gh = grp;                               // gather: sample, quarter of the bins
+            const bool mine = gid[gs] != 0xffffffffu && !bad[gs];
+            // drain one batch into rows 1 + 32 sub.. of R
+            auto drain = [&](int sub) {
+                const uint32_t b = g & 1u;
+                const int ok = tc::mbar_wait(done + b, (g >> 1) & 1u, kWait) ? 1 : 0;
+                ++g;
+                tc::tc_fence_after();
+                long long *out = Rs + (size_t)(1 + kSub * sub + 8 * cb) * kS + s;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    uint32_t v[kDig][4];
+#pragma unroll
+                    for (int o = 0; o < kDig; ++o)
+                        tc::tmem_ld4(tmem + ((uint32_t)(32 * q) << 16) + b * kAccCols +
+                                         (uint32_t)(o * kSub + 8 * cb + 4 * h),
+                                     v[o]);
+                    tc::tmem_ld_wait();
+#pragma unroll
+                    for (int i = 0; i < 4; ++i)
+                        out[(4 * h + i) * kS] = join_orders(v, i);
+                }
+                tc::tc_fence_before();
+                __syncwarp();
+                tc::mbar_arrive_if(empty + b, lane == 0);
+                return ok;
+            };
+            const int qbar = 2 + q;
+            const int sc = scs[gs];
+
+            // ---- template term: W = Z T, quad = kappa sum_k sum_n z_n W_n
+            double qacc = 0.0;
+            for (int k = 0; k < K && !failed; ++k) {
+                tc::named_bar_or(qbar, kConsumers / 4, 0);   // R free
+                const int ok0 = drain(0), ok1 = drain(1);
+                failed = tc::named_bar_or(qbar, kConsumers / 4, !ok0 || !ok1 || abort_s);
+                if (failed)
+                    break;
+                double acc = 0.0;
+                const __half *zs = scratch + ((size_t)k * kDig * kS + (size_t)(gs >> 3) * 8) * kp + (gs & 7) * 8;
+                for (int kc = gh; kc < kcs; kc += kQ) {
+                    uint32_t w[kDig][4];
+#pragma unroll
+                    for (int p = 0; p < kDig; ++p) {
+                        const uint4 v = *reinterpret_cast<const uint4 *>(zs + (size_t)p * kS * kp + kc * 64);
+                        w[p][0] = v.x;
+                        w[p][1] = v.y;
+                        w[p][2] = v.z;
+                        w[p][3] = v.w;
+                    }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        const int nn = 8 * kc + j;
+                        if (nn >= 2 * M)
+                            break;
+                        long long I = 0;
+#pragma unroll
+                        for (int p = 0; p < kDig; ++p) {
+                            const uint32_t hb = w[p][j >> 1] >> (16 * (j & 1));
+                            I = I * 256 + (long long)__half2int_rn(__ushort_as_half((unsigned short)hb));
+                        }
+                        acc = fma((double)I, (double)Rs[(size_t)(1 + nn) * kS + gs], acc);
+                    }
+                }
+                qacc += mul_pow2(acc, 56 - 2 * sc - (55 - X.t_exp[k]));
+            }
+            quads[gh * kS + gs] = qacc;
+            // the four partials of a sample belong to the warps of its quarter (q == gs / 32)
+            failed = tc::named_bar_or(qbar, kConsumers / 4, failed);
+            const double quad = P.kappa * ((quads[gs] + quads[kS + gs]) + (quads[2 * kS + gs] + quads[3 * kS + gs]));
+
+            const int lexp = 56 - sc - sq;   // lin = X 2^lexp
+            DiffScale ds;
+            ds.set(lexp);
+            Lse run{LLONG_MIN, 0ull};
+            for (int ch = ch0; ch < ch1 && !failed; ++ch) {
+                const int j0 = ch * jnom, J = min(jnom, NT - j0);
+                const int jq = (J + kQ - 1) / kQ, jb = j0 + gh * jq;
+                const int jn = mine ? max(0, min(jq, j0 + J - jb)) : 0;   // this thread's bins
+                long long lin[kBpt];
+#pragma unroll
+                for (int i = 0; i < kBpt; ++i)
+                    lin[i] = 0;
+                for (int k = 0; k < K && !failed; ++k) {
+                    int w0, nsub;
+                    window(k, j0, j0 + J, w0, nsub);
+                    const long long uk = U0[k * kS + gs];
+                    for (int t = 0; t < nsub; t += 2) {
+                        tc::named_bar_or(qbar, kConsumers / 4, 0);   // the previous block's gathers are done
+                        if (cb == 3 && t > 0)
+                            Rs[s] = Rs[(size_t)kBlk * kS + s];
+                        int ok = drain(0);
+                        if (t + 1 < nsub)
+                            ok &= drain(1);
+                        if ((failed = tc::named_bar_or(qbar, kConsumers / 4, !ok || abort_s)))
+                            break;
+                        const int rel = w0 + kSub * t - 1;
+                        const unsigned cols = (unsigned)(kSub * min(2, nsub - t));
+#pragma unroll
+                        for (int i = 0; i < kBpt; ++i) {
+                            const long long u = uk + pos[min(jb + i, NT - 1)];
+                            const int c = (int)(u >> kFrac) - rel;
+                            if (i < jn && (unsigned)c < cols) {
+                                const long long *r = Rs + (size_t)c * kS + gs;
+                                const long long r0 = r[0], dr = (r[kS] - r0) * 2;
+                                const long long f63 = (u << (63 - kFrac)) & 0x7fffffffffffffffLL;
+                                lin[i] += r0 + __mul64hi(dr, f63);
+                            }
+                        }
+                    }
+                }
+                if (failed)
+                    break;
+                long long cm = LLONG_MIN;
+#pragma unroll
+                for (int i = 0; i < kBpt; ++i)
+                    if (i < jn)
+                        cm = max(cm, lin[i]);
+                if (lnL_t) {
+                    const int64_t row = (int64_t)gid[gs] * NT + jb;
+#pragma unroll
+                    for (int i = 0; i < kBpt; ++i)
+                        if (i < jn)
+                            lnL_t[row + i] = __dsub_rn(mul_pow2((double)lin[i], lexp), quad);
+                }
+                Lse part_l{cm, 0ull};
+#pragma unroll
+                for (int i = 0; i < kBpt; ++i)
+                    if (i < jn)
+                        part_l.s += term64(ds, (uint64_t)cm - (uint64_t)lin[i], tbl);
+                // the chunk's four parts, where R was; merged by the sample's first thread
+                tc::named_bar_or(qbar, kConsumers / 4, 0);
+                Rs[gh * kS + gs] = part_l.m;
+                Rs[(kQ + gh) * kS + gs] = (long long)part_l.s;
+                tc::named_bar_or(qbar, kConsumers / 4, 0);
+                if (gh == 0) {
+                    Lse c{Rs[gs], (uint64_t)Rs[kQ * kS + gs]};
+                    for (int h = 1; h < kQ; ++h)
+                        c = merge64(ds, c, Lse{Rs[h * kS + gs], (uint64_t)Rs[(kQ + h) * kS + gs]}, tbl);
+                    if (parts == 1)
+                        run = ch == 0 ? c : merge64(ds, run, c, tbl);
+                    else
+                        records[((int64_t)ch * n_tiles + tile) * kS + gs] = c;
+                }
+            }
+            // the sample's value (or what the combination needs), by its first thread
+            if (!failed && gh == 0 && gid[gs] != 0xffffffffu) {
+                const uint32_t gi = gid[gs];
+                int flags = bad[gs];
+                if (parts == 1) {
+                    const double r = flags ? __longlong_as_double(0x7ff8000000000000LL)
+                                           : lse_value(run, lexp, quad, NT);
+                    if (!isfinite(r))
+                        flags |= kErrNonFinite;
+                    lnL_tmarg[gi] = r;
+                    if (lnw && lnpw)
+                        lnw[gi] = r + lnpw[gi];
+                } else if (part == 0) {
+                    records[((int64_t)n_chunks * n_tiles + tile) * kS + gs] =
+                        Lse{__double_as_longlong(quad), (uint64_t)(uint32_t)lexp | ((uint64_t)(uint32_t)flags << 32)};
+                }
+                if (flags)
+                    atomicOr(err, flags);
+            }
+        } else if (!producer && grp == 0 && gid[s_of] != 0xffffffffu) {
+            // no sample of the tile has finite delays
+            const uint32_t gi = gid[s_of];
+            const double r = __longlong_as_double(0x7ff8000000000000LL);
+            atomicOr(err, bad[s_of] | kErrNonFinite);
+            if (parts == 1) {
+                lnL_tmarg[gi] = r;
+                if (lnw && lnpw)
+                    lnw[gi] = r;
+            } else if (part == 0) {
+                records[((int64_t)n_chunks * n_tiles + tile) * kS + s_of] = Lse{0, (uint64_t)kErrNonFinite << 32};
+            }
+        }
+        failed = __syncthreads_or(failed || abort_s);
+        if (failed) {
+            if (tid == 0) {
+                atomicOr(err, kErrTimeout);
+                abort_s = 1;
+            }
+            __syncthreads();
+            continue;
+        }
+    }
+    // leave: no copy of this block still landing (after a failure the issuer may not have
+    // consumed the last ones; bounded waits), then free the tensor memory
+    if (warp == kStager && lane == 0) {
+        for (uint32_t b = 0; b < 2; ++b) {
+            const uint32_t uses = (g + 1u - b) >> 1;
+            if (uses > 0)
+                tc::mbar_wait(full + b, (uses - 1u) & 1u, kWait);
+        }
+        if (ga > 0)
+            tc::mbar_wait(fullA, (ga - 1u) & 1u, kWait);
+    }
+    tc::tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc::tc_fence_after();
+        tc::tmem_dealloc(tmem, 512);
+    }
+}
+
+// Merges the chunks' sums of every sample (nothing to do when the bins were not split) and
+// resets the unit counter.
+__global__ void combine64_kernel(const Lse *__restrict__ records, const long long *__restrict__ pos, const uint32_t *__restrict__ perm, int64_t n,
+                                 const uint32_t *__restrict__ n_dev, int grid, int n_t, double *__restrict__ lnL_tmarg,
+                                 const double *__restrict__ lnpw, double *__restrict__ lnw, int *err,
+                                 int *unit_counter)
+{
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        *unit_counter = 0;   // for the next launch
+    const int64_t n_use = n_dev ? min(n, (int64_t)*n_dev) : n;
+    const int64_t n_tiles = (n_use + kS - 1) / kS;
+    const int n_chunks = (n_t + kChunk - 1) / kChunk;
+    if (parts64(n_tiles, grid, n_chunks) == 1)
+        return;
+    __shared__ uint64_t tbl[kTable];
+    for (int i = threadIdx.x; i < kTable; i += blockDim.x)
+        tbl[i] = (uint64_t)pos[n_t + i];
+    __syncthreads();
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_use; i += (int64_t)gridDim.x * blockDim.x) {
+        const Lse info = records[(int64_t)n_chunks * n_tiles * kS + i];
+        const int lexp = (int)(uint32_t)info.s;
+        const uint32_t g = perm ? perm[i] : (uint32_t)i;
+        double r = __longlong_as_double(0x7ff8000000000000LL);
+        if ((info.s >> 32) == 0) {
+            DiffScale ds;
+            ds.set(lexp);
+            Lse run = records[i];
+            for (int c = 1; c < n_chunks; ++c)
+                run = merge64(ds, run, records[(int64_t)c * n_tiles * kS + i], tbl);
+            r = lse_value(run, lexp, __longlong_as_double(info.m), n_t);
+        }
+        if (!isfinite(r))
+            atomicOr(err, kErrNonFinite);
+        lnL_tmarg[g] = r;
+        if (lnw && lnpw)
+            lnw[g] = r + lnpw[g];
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta, const uint32_t *perm, int64_t n,
+                            double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
+                            cudaStream_t st, const uint32_t *n_dev)
+{
+    if (n <= 0)
+        return cudaSuccess;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaError_t e = allow_max_dynamic_smem(lnl_tc64_kernel);
+    if (e != cudaSuccess)
+        return e;
+    const size_t smem = std::max(kMinSmem, layout64(P.K, P.M, P.n_t).end);
+    const int64_t tiles = (n + kS - 1) / kS;
+    const int grid = (int)std::min<int64_t>(sms, 16 * tiles);
+    lnl_tc64_kernel<<<grid, kThreads, smem, st>>>(P, X, theta, perm, n, lnL_tmarg, lnL_t, lnpw, lnw, err,
+                                                  X.unit_counter, n_dev);
+    // the split depends on the device count; it never has more tiles than there are records for
+    const int64_t most = std::min<int64_t>(tiles, split_tiles(n, P.n_t));
+    combine64_kernel<<<(int)std::max<int64_t>(1, most), 128, 0, st>>>(reinterpret_cast<const Lse *>(X.records), X.pos, perm, n,
+                                                                    n_dev, grid, P.n_t, lnL_tmarg, lnpw, lnw, err,
+                                                                    X.unit_counter);
+    return cudaGetLastError();
+}
+
+cudaError_t prepare_tc64_kernels() { return allow_max_dynamic_smem(lnl_tc64_kernel); }
+
+}  // namespace rift
