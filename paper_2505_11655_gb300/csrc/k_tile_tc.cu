@@ -36,6 +36,7 @@ constexpr int kTcStagerWarp = kTcIssuerWarp + 1;
 constexpr int kTcQ = kTcConsumers / kTcS;  // threads per sample in the gather (bin quarters)
 constexpr int kTcBPT = 16;         // bins per thread per chunk
 constexpr int kTcMaxBins = kTcQ * kTcBPT;
+constexpr int kTcFrac = 24;        // fraction bits of a node position in the R tile
 // phases B and E give every (sample, detector) item its own consumer thread, whole warps
 // per detector
 static_assert(kTcS * kMaxDet <= kTcConsumers && kTcS % 32 == 0, "one item per consumer thread");
@@ -265,9 +266,9 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
     __half *Bs = reinterpret_cast<__half *>(sm + L.b);          // [2 buf][2 part][kTcW x kp]
     float *Rs = reinterpret_cast<float *>(sm + L.r);            // Rt [kTcW][kTcS] (prologue: Y [M][kTcS])
     float *Rs2 = reinterpret_cast<float *>(sm + L.r2);          // Rt of the odd steps
-    int2 *bins = reinterpret_cast<int2 *>(sm + L.bins);          // (bin_i, bits of bin_f) per bin
+    int2 *bins = reinterpret_cast<int2 *>(sm + L.bins);          // per bin: bin_i, (bin_i + bin_f) 2^24 mod 2^32
     int *i0s = reinterpret_cast<int *>(sm + L.i0);              // [K][kTcS]
-    float *f0s = reinterpret_cast<float *>(sm + L.f0);
+    uint32_t *f0s = reinterpret_cast<uint32_t *>(sm + L.f0);    // [K][kTcS] fraction of the first node, 2^-24
     float *invs = reinterpret_cast<float *>(sm + L.inv);        // [K][kTcS] 2^-(row exponent + Q exponent)
     float *qsc = reinterpret_cast<float *>(sm + L.qsc);         // [K][kTcS] 2^-(2 row exponent)
     uint32_t *gid = reinterpret_cast<uint32_t *>(sm + L.gid);
@@ -318,7 +319,8 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
     auto a_col = [&](int k, int part) { return 256u + (uint32_t)((2 * k + part) * (kp / 2)); };
 
     for (int j = tid; j < NT; j += blockDim.x) {
-        bins[j] = make_int2(bt.bin_i[j], __float_as_int(bt.bin_f[j]));
+        const int bi = bt.bin_i[j];
+        bins[j] = make_int2(bi, (int)(((uint32_t)bi << kTcFrac) + __float2uint_rn(bt.bin_f[j] * 0x1p24f)));
     }
     // the nodes read for the bins j0 .. j0 + jmax - 1 lie within (jmax - 1) beta + 3 columns of
     // a sample's first node; with the spread of the sub-group's offsets and up to 7 columns of
@@ -432,7 +434,7 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
             double fl = floor(u0);
             int i0 = (int)fl;
             i0s[k * kTcS + s] = i0;
-            f0s[k * kTcS + s] = (float)(u0 - fl);
+            f0s[k * kTcS + s] = __float2uint_rn((float)(u0 - fl) * 0x1p24f);
             // offset range of the tile at detector k: a warp holds 32 samples of one detector
             // (one item per thread), so reduce over the warp, then one atomic per warp
             const bool valid = gid[s] != 0xffffffffu;
@@ -724,13 +726,12 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                 __syncwarp();
             } else {
                 // ============ consumer warps: drain, gather, fold
-                float lin[kTcBPT], bfj[kTcBPT];
-                int bj[kTcBPT];
+                float lin[kTcBPT];
+                uint32_t bj[kTcBPT];
 #pragma unroll
                 for (int i = 0; i < kTcBPT; ++i) {
                     lin[i] = 0.f;
-                    bfj[i] = 0.f;
-                    bj[i] = 0;
+                    bj[i] = 0u;
                 }
                 for (int t = 0, k = 0, j0 = 0; t < n_steps; ++t) {
                     const int b = t & 1, J = min(jnom, NT - j0);
@@ -754,8 +755,10 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                     // in the row; their sums are discarded.
                     const int iw0 = win0(k, j0);
                     const bool mine = gok && in_grp;
-                    const float *Rcol = Rt + ((mine ? i0s[k * kTcS + gs] : glo[grp][k]) - iw0) * kTcS + gs;
-                    const float ff = mine ? f0s[k * kTcS + gs] : 0.f;
+                    // position of the sample's first node: column (plus 128 in the upper half of the
+                    // tile's samples) in the top byte, fraction below (modulo 2^32)
+                    const uint32_t ub = ((uint32_t)((mine ? i0s[k * kTcS + gs] : glo[grp][k]) - iw0 + 2 * (gs & 64)) << kTcFrac) +
+                                        (mine ? f0s[k * kTcS + gs] : 0u);
                     const float sc = invs[k * kTcS + gs];
                     if (k == 0) {
                         // this thread's bins of the chunk, shared by every detector (idle slots
@@ -764,16 +767,13 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                         const int jl = jn > 0 ? jb + jn - 1 : min(jb, NT - 1);
 #pragma unroll
                         for (int i = 0; i < kTcBPT; ++i) {
-                            const int j = min(jb + i, jl);
-                            const int2 bv = bins[j];
-                            bj[i] = bv.x;
-                            bfj[i] = __int_as_float(bv.y);
+                            bj[i] = (uint32_t)bins[min(jb + i, jl)].y;
                         }
                     }
                     {
                         // drain accumulator b: warp quarter q = rows 32q.., column block w / 4 of 32
                         const int q = warp & 3, cb = warp >> 2;
-                        float *Rcol = Rt + (32 * cb) * kTcS + 32 * q + lane;
+                        float *Rcol = Rt + (q >> 1) * (kTcW * 64) + (32 * cb) * 64 + 32 * (q & 1) + lane;
                         // two loads of 16 columns (fewer live registers than one of 32)
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
@@ -782,7 +782,7 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                             tc::tmem_ld_wait();
 #pragma unroll
                             for (int i = 0; i < 16; ++i)
-                                Rcol[(16 * h + i) * kTcS] = __uint_as_float(v[i]);
+                                Rcol[(16 * h + i) * 64] = __uint_as_float(v[i]);
                         }
                     }
                     tc::tc_fence_before();
@@ -794,18 +794,33 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                         break;
                     }
                     // two bins per packed float32 operation (the same roundings as one at a time)
-#pragma unroll
-                    for (int i = 0; i < kTcBPT; i += 2) {
-                        const float2 sf = __fadd2_rn(make_float2(ff, ff), make_float2(bfj[i], bfj[i + 1]));
-                        const int c0 = sf.x >= 1.f, c1 = sf.y >= 1.f;
-                        const float2 fr = __fadd2_rn(sf, make_float2(-(float)c0, -(float)c1));
-                        const float *ra = Rcol + (bj[i] + c0) * kTcS, *rb = Rcol + (bj[i + 1] + c1) * kTcS;
-                        const float2 r0 = make_float2(ra[0], rb[0]), r1 = make_float2(ra[kTcS], rb[kTcS]);
-                        const float2 v = __ffma2_rn(fr, __fadd2_rn(r1, make_float2(-r0.x, -r0.y)), r0);
+                    const uint32_t lane4 = (uint32_t)(gs & 63) * 4u;
+                    const unsigned char *Rb = reinterpret_cast<const unsigned char *>(Rt);
+                    auto pair = [&](int i) {
+                        const uint32_t u = ub + bj[i], w = ub + bj[i + 1];
+                        // byte offset of the node: column << 8 | (sample of the half tile) * 4
+                        const float *ra = reinterpret_cast<const float *>(Rb + __byte_perm(u, lane4, 0x7734));
+                        const float *rb = reinterpret_cast<const float *>(Rb + __byte_perm(w, lane4, 0x7734));
+                        const float2 r0 = make_float2(ra[0], rb[0]), r1 = make_float2(ra[64], rb[64]);
+                        const float2 fr = __fmul2_rn(make_float2((float)(u & 0xffffffu), (float)(w & 0xffffffu)),
+                                                     make_float2(0x1p-24f, 0x1p-24f));
+                        const float2 v = __ffma2_rn(fr, __ffma2_rn(r0, make_float2(-1.f, -1.f), r1), r0);
                         const float2 l = __ffma2_rn(make_float2(sc, sc), v, make_float2(lin[i], lin[i + 1]));
                         lin[i] = l.x;
                         lin[i + 1] = l.y;
+                    };
+                    pair(0);
+                    pair(2);
+                    pair(4);
+                    pair(6);
+                    if (jq > 8) {
+                        pair(8);
+                        pair(10);
                     }
+                    if (jq > 12)
+                        pair(12);
+                    if (jq > 14)
+                        pair(14);
                     if (k == K - 1) {
                         // fold this thread's bins of the chunk into its running log-sum-exp
                         float cmx = -INFINITY;
@@ -842,14 +857,13 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                             // operations, so that the block holding it is known).  Idle slots
                             // repeat the last bin's value: the maximum is that of the valid
                             // bins, and the lowest block attaining it holds a valid bin.
-                            float qm[kTcBPT / kPeakBlockTc];
-#pragma unroll
-                            for (int a = 0; a < kTcBPT / kPeakBlockTc; ++a) {
-                                qm[a] = lin[kPeakBlockTc * a];
-#pragma unroll
-                                for (int i = kPeakBlockTc * a + 1; i < kPeakBlockTc * (a + 1); ++i)
-                                    qm[a] = fmaxf(qm[a], lin[i]);
-                            }
+                            float qm[4];
+                            qm[0] = fmaxf(fmaxf(lin[0], lin[1]), fmaxf(lin[2], lin[3]));
+                            qm[1] = fmaxf(fmaxf(lin[4], lin[5]), fmaxf(lin[6], lin[7]));
+                            qm[2] = jq > 8 ? fmaxf(fmaxf(lin[8], lin[9]), fmaxf(lin[10], lin[11])) : -INFINITY;
+                            qm[3] = jq > 12 ? fmaxf(lin[12], lin[13]) : -INFINITY;
+                            if (jq > 14)
+                                qm[3] = fmaxf(qm[3], fmaxf(lin[14], lin[15]));
                             const float m01 = fmaxf(qm[0], qm[1]), m23 = fmaxf(qm[2], qm[3]);
                             cmx = fmaxf(m01, m23);
                             if (jn > 0 && in_grp) {
@@ -881,14 +895,25 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                                 // operation
                                 const float off = nm * kLog2e;
                                 float2 cs2 = make_float2(0.f, 0.f);
-#pragma unroll
-                                for (int i = 0; i < kTcBPT; i += 2) {
+                                auto terms = [&](int i) {
                                     const float2 x = __ffma2_rn(make_float2(lin[i], lin[i + 1]), make_float2(kLog2e, kLog2e),
                                                                 make_float2(-off, -off));
                                     const float2 ev = make_float2(i < jn ? ex2_approx(x.x) : 0.f,
                                                                   i + 1 < jn ? ex2_approx(x.y) : 0.f);
                                     cs2 = __fadd2_rn(cs2, ev);
+                                };
+                                terms(0);
+                                terms(2);
+                                terms(4);
+                                terms(6);
+                                if (jq > 8) {
+                                    terms(8);
+                                    terms(10);
                                 }
+                                if (jq > 12)
+                                    terms(12);
+                                if (jq > 14)
+                                    terms(14);
                                 cs = cs2.x + cs2.y;
                             }
                             run_sum = (run_mx == -INFINITY ? 0.f : run_sum * __expf(run_mx - nm)) + cs;
