@@ -289,8 +289,11 @@ cudaError_t launch_tiled(rift_ile_t *h, const double *theta, int64_t n, double *
         po.j = h->aux_j;
     }
     const bool tc = use_tc(h, n);
+    if (tc)
+        h->launches += 1;   // the work units
     cudaError_t e = tc ? launch_lnl_tc(h->prob, bt, theta, h->perm, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err,
-                                       h->tile_counter, h->stream, nullptr, 0, 0, po)
+                                       TcUnits{h->tc_unit_list, h->tc_unit_cap, h->tile_counter}, h->stream,
+                                       nullptr, 0, 0, po)
                        : launch_lnl_fp32(h->prob, bt, theta, h->perm, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err,
                                          h->tile_counter, h->stream, po);
     if (e != cudaSuccess || !h->fix_on)
@@ -361,8 +364,8 @@ int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmar
         const BinTable bt{h->bin_i, h->bin_f, std::log((double)h->prob.n_t)};
         rows = std::min<int64_t>(h->refine_rows, n);
         CK(launch_lnl_tc(h->prob, bt, theta, h->sel_idx, rows, lnL_tmarg, h->refine_bins, lnpw, lnw, h->err,
-                         h->tile_counter, h->stream, h->sel_count, 1, n));
-        h->launches += 1;
+                         TcUnits{h->tc_unit_list, h->tc_unit_cap, h->tile_counter}, h->stream, h->sel_count, 1, n));
+        h->launches += 2;
     }
     CK(launch_refine(h->prob, theta, h->sel_idx, h->sel_count, n, lnL_tmarg, lnpw, lnw, h->err, h->stream,
                      h->refine_bins, rows));
@@ -683,6 +686,7 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
     int rc = RIFT_OK;
     const int64_t N = h->cap;
     const int B = cfg->n_bins;
+    h->tc_unit_cap = tc_units_cap(N);
     if ((rc = dalloc(h, &h->Q64, (size_t)K * M * cfg->n_q)) || (rc = dalloc(h, &h->U64, (size_t)K * M * M)) ||
         (rc = dalloc(h, &h->V64, (size_t)K * M * M)) || (rc = dalloc(h, &h->Qr32, (size_t)K * 2 * M * P.n_q_pad)) ||
         (rc = dalloc(h, &h->U32, (size_t)K * M * M)) || (rc = dalloc(h, &h->V32, (size_t)K * M * M)) ||
@@ -693,7 +697,8 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
         (rc = dalloc(h, &h->lnL, (size_t)N)) || (rc = dalloc(h, &h->lnw, (size_t)N)) ||
         (rc = dalloc(h, &h->bins, (size_t)N)) || (rc = dalloc(h, &h->key, (size_t)N)) ||
         (rc = dalloc(h, &h->perm, (size_t)N)) || (rc = dalloc(h, &h->sort_scratch, sort_scratch_words(N))) ||
-        (rc = dalloc(h, &h->tile_counter, (size_t)4)) ||
+        (rc = dalloc(h, &h->tile_counter, (size_t)8)) ||
+        (rc = dalloc(h, &h->tc_unit_list, (size_t)2 * tc_units_cap(N))) ||
         (rc = dalloc(h, &h->qmax_bits, (size_t)4)) ||
         (rc = dalloc(h, &h->Qtc, (size_t)K * 2 * ((cfg->n_q + 7) / 8 + 17) * ((2 * M + 15) / 16 * 16) * 8)) ||
         (rc = dalloc(h, &h->red_partial, (size_t)5 * kRedBlocks)) ||
@@ -889,7 +894,7 @@ int64_t rift_ile_footprint(const rift_ile_config *cfg)
     const int64_t sizes[] = {
         K * M * nq * 16, 2 * K * M * M * 16, K * 2 * M * nq_pad * 4, 2 * K * M * M * 8, K * 2 * kp * kp * 2, K * 4,
         2 * nt * 4,
-        N * 6 * 8, 3 * N * 8, N * 8, 2 * N * 4, (int64_t)sort_scratch_words(N) * 4, 16, 16,
+        N * 6 * 8, 3 * N * 8, N * 8, 2 * N * 4, (int64_t)sort_scratch_words(N) * 4, 32, 16, 16 * tc_units_cap(N),
         K * 2 * groups * kp * 8 * 2, 5 * kRedBlocks * 8, 152 * 12 * B * 8, 8 * (RIFT_MAX_ITER + 1) * 8, 3 * 8 * 8,
         N * 4, 16, 6 * B * 8, 6 * (B + 1) * 8, 6 * B * 8, 16, (int64_t)kSelectWords * 4,
         cfg->precision == RIFT_MIXED && !digits ? std::min<int64_t>(N, kRefineRows) * nt * 8 : 0,

@@ -44,6 +44,8 @@ struct rift_ile {
     uint32_t *key = nullptr, *perm = nullptr;
     uint32_t *sort_scratch = nullptr;   // radix-sort digit counts, scan totals, ping-pong buffers
     int *tile_counter = nullptr;
+    unsigned long long *tc_unit_list = nullptr;   // work units of the tensor-core likelihood
+    int64_t tc_unit_cap = 0;
     __half *Qtc = nullptr;
     unsigned int *qmax_bits = nullptr;
     int tc_mode = 2;              // 0 never, 1 whenever it fits, 2 autotuned

@@ -138,9 +138,16 @@ cudaError_t launch_prep_tt(const double2 *U64, const double2 *V64, int K, int M,
 // n_theta: theta's sample count when perm indexes a larger batch (default n);
 // lnl_t_compact: the per-bin output of the sample at position i of perm is row i of lnL_t
 // (instead of its sample index's row).
+struct TcUnits {
+    unsigned long long *list = nullptr;   // [2][cap]: classes 0, 1 from the fronts, 3, 2 from the backs
+    int64_t cap = 0;
+    int *counters = nullptr;              // [1 + 4]: units taken, units per class
+};
+constexpr int kTcCounters = 5;
+int64_t tc_units_cap(int64_t n_max);      // words of each half of TcUnits::list
 cudaError_t launch_lnl_tc(const Problem &P, BinTable bt, const double *theta, const uint32_t *perm, int64_t n,
                           double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
-                          int *tile_counter, cudaStream_t st, const uint32_t *n_dev = nullptr,
+                          TcUnits units, cudaStream_t st, const uint32_t *n_dev = nullptr,
                           int lnl_t_compact = 0, int64_t n_theta = 0, PeakOut po = PeakOut());
 // Builds the float16 hi/lo copy of Q for the tensor-core path.
 cudaError_t launch_prep_tc(const double2 *Q64, int K, int M, int n_q, int groups, unsigned int *qmax_bits,
@@ -213,7 +220,7 @@ cudaError_t launch_draw(const SamplerDev &S, const SkyGrid &G, const uint32_t *i
                         double *theta, double *lnpw, uint64_t *bins, uint32_t *key, cudaStream_t st);
 cudaError_t launch_keys(const SkyGrid &G, const double *theta, int64_t n, uint32_t *key, cudaStream_t st);
 // Stable sort of sample indices by sky-cell key (< G.n_cells <= 2^20) into perm: LSD
-// radix, 10-bit digits; ties keep index order.  scratch holds sort_scratch_words(n)
+// radix, digits of up to 10 bits (one block up to 4096 keys); ties keep index order.  scratch holds sort_scratch_words(n)
 // words; *launched (optional) receives the number of kernels enqueued.
 constexpr int kRadixBits = 10;
 constexpr int kRadixBuckets = 1 << kRadixBits;

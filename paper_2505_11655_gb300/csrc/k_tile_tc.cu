@@ -248,14 +248,150 @@ cudaError_t launch_prep_tt(const double2 *U64, const double2 *V64, int K, int M,
 
 // ---------------------------------------------------------------- the kernel
 
+// ---- work units.  A tile whose samples fit one window costs K ceil(n_t / bins per chunk)
+// steps, a tile from a thinly sampled part of the sky that many per sub-group: with whole tiles
+// as the units of work, 200,000 samples of an adapted sampler (3 detectors, 16384 Hz, 1001 bins)
+// have a mean of 72 steps a tile and a largest tile of 2000, and the SMs were idle half of the
+// kernel.  This kernel (one warp per tile, delays in float32: the likelihood kernel cuts its
+// sub-groups itself, from float64 delays) cuts the costly tiles at sub-group boundaries into
+// units of about twice the cheapest tile, at most kTcUnitsPerTile a tile, and files them in
+// four classes by cost, taken in order: the costly ones first, the last ones are small.  A unit
+// is (tile, first, last sample of the tile).
+constexpr int kTcUnitsPerTile = 16;
+constexpr int kTcPlanWarps = 8;
+
+int64_t tc_units_cap(int64_t n_max) { return (n_max + kTcS - 1) / kTcS * kTcUnitsPerTile; }
+
+__global__ void __launch_bounds__(32 * kTcPlanWarps)
+tc_units_kernel(Problem P, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
+                const uint32_t *__restrict__ n_dev, int64_t n_theta, unsigned long long *__restrict__ list, int64_t cap,
+                int *__restrict__ counters)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t tile = (int64_t)blockIdx.x * kTcPlanWarps + (threadIdx.x >> 5);
+    const int64_t n_use = n_dev ? min(n, (int64_t)*n_dev) : n;
+    if (tile >= (n_use + kTcS - 1) / kTcS)
+        return;
+    const int K = P.K;
+    const float beta = (float)(P.t_step * P.fs);
+    // steps of a group whose offsets span `sp` columns (see jmax_s in the likelihood kernel)
+    auto steps = [&](int sp) {
+        int jm = beta > 0.f ? (int)((float)(kTcW - 11 - min(sp, kTcSpreadLimit)) / beta) + 1 : kTcMaxBins;
+        jm = max(1, min(jm, kTcMaxBins));
+        return (float)(K * ((P.n_t + jm - 1) / jm));
+    };
+    // quarters of the tile without a sample of the group skip its drains and gathers, which
+    // take about two thirds of a step
+    auto cost = [&](int a, int b, int sp) {
+        return steps(sp) * (0.35f + 0.65f * 0.25f * (float)((b - 1) / 32 - a / 32 + 1));
+    };
+    int i0[kTcS / 32][kMaxDet];
+    unsigned valid[kTcS / 32];
+    int lo[kMaxDet], hi[kMaxDet];
+#pragma unroll
+    for (int k = 0; k < kMaxDet; ++k) {
+        lo[k] = INT_MAX;
+        hi[k] = INT_MIN;
+    }
+#pragma unroll
+    for (int q = 0; q < kTcS / 32; ++q) {
+        const int64_t si = tile * kTcS + 32 * q + lane;
+        const uint32_t g = si < n_use ? perm[si] : 0xffffffffu;
+        const bool ok = (int64_t)g < n_theta;
+        float sa = 0.f, ca = 1.f, sd = 0.f, cd = 1.f;
+        if (ok) {
+            const double *th = theta + 6 * (int64_t)g;
+            sincosf((float)(th[0] - P.gmst), &sa, &ca);
+            sincosf((float)th[1], &sd, &cd);
+        }
+        valid[q] = __ballot_sync(0xffffffffu, ok);
+#pragma unroll
+        for (int k = 0; k < kMaxDet; ++k) {
+            i0[q][k] = 0;
+            if (k < K && ok) {
+                const float u = fmaf((float)P.xfs[k][0], cd * ca, fmaf((float)P.xfs[k][1], cd * sa,
+                                     fmaf((float)P.xfs[k][2], sd, (float)P.ufs0[k])));
+                i0[q][k] = (int)floorf(u);
+                lo[k] = min(lo[k], i0[q][k]);
+                hi[k] = max(hi[k], i0[q][k]);
+            }
+        }
+    }
+    int spread = 0;
+#pragma unroll
+    for (int k = 0; k < kMaxDet; ++k)
+        if (k < K)
+            spread = max(spread, __reduce_max_sync(0xffffffffu, hi[k]) - __reduce_min_sync(0xffffffffu, lo[k]));
+    const float base = steps(0);
+    auto file = [&](int a, int b, float c) {
+        if (lane != 0)
+            return;
+        const int cls = c > 1.75f * base ? 0 : c > 1.35f * base ? 1 : c > 0.7f * base ? 2 : 3;
+        const int64_t at = atomicAdd(counters + 1 + cls, 1);
+        list[((cls == 1 || cls == 2) ? cap : 0) + (cls < 2 ? at : cap - 1 - at)] =
+            ((unsigned long long)tile << 16) | (unsigned)(a << 8) | (unsigned)(b - 1);
+    };
+    if (spread <= kTcSpreadLimit) {
+        file(0, kTcS, cost(0, kTcS, spread));
+        return;
+    }
+    int units = 0, ua = 0, ga = 0;   // units filed, first sample of the open unit and of the open group
+    float uc = 0.f;                  // cost of the open unit's closed groups
+    bool open = false;
+    auto close = [&](int e) {        // close the open group at sample e; close the unit before it when full
+        int sp = 0;
+#pragma unroll
+        for (int k = 0; k < kMaxDet; ++k)
+            if (k < K)
+                sp = max(sp, hi[k] - lo[k]);
+        const float c = cost(ga, e, sp);
+        if (uc > 0.f && uc + c > 2.f * base && units < kTcUnitsPerTile - 1) {
+            file(ua, ga, uc);
+            ++units;
+            ua = ga;
+            uc = 0.f;
+        }
+        uc += c;
+    };
+#pragma unroll
+    for (int q = 0; q < kTcS / 32; ++q)
+        for (int e = 0; e < 32; ++e) {
+            if (!((valid[q] >> e) & 1u))
+                continue;
+            int v[kMaxDet];
+            bool fits = open;
+#pragma unroll
+            for (int k = 0; k < kMaxDet; ++k)
+                if (k < K) {
+                    v[k] = __shfl_sync(0xffffffffu, i0[q][k], e);
+                    fits = fits && max(hi[k], v[k]) - min(lo[k], v[k]) <= kTcSpreadLimit;
+                }
+            if (!fits) {
+                if (open) {
+                    close(32 * q + e);
+                    ga = 32 * q + e;
+                }
+                open = true;
+            }
+#pragma unroll
+            for (int k = 0; k < kMaxDet; ++k)
+                if (k < K) {
+                    lo[k] = fits ? min(lo[k], v[k]) : v[k];
+                    hi[k] = fits ? max(hi[k], v[k]) : v[k];
+                }
+        }
+    close(kTcS);
+    file(ua, kTcS, uc);
+}
+
 // kDM: distance marginalisation (a separate instantiation, so that the plain path keeps
 // its registers)
 template <bool kDM>
 __global__ void __launch_bounds__(kTcThreads, 1)
 lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
               double *__restrict__ lnL_tmarg, double *__restrict__ lnL_t, const double *__restrict__ lnpw,
-              double *__restrict__ lnw, int *err, int *tile_counter, const uint32_t *__restrict__ n_dev,
-              int64_t n_theta, int lnl_t_compact, PeakOut po)
+              double *__restrict__ lnw, int *err, TcUnits units, const uint32_t *__restrict__ n_dev, int64_t n_theta,
+              int lnl_t_compact, PeakOut po)
 {
     // n entries of perm (fewer when a device count is given, read where needed so that no
     // register holds it); every sample index in perm is below n_theta
@@ -293,14 +429,13 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
     float2 *Ys = reinterpret_cast<float2 *>(Rs);               // [M][kTcS] -2Y_lm(iota, -phi)
     __shared__ int lo_s[kMaxDet], hi_s[kMaxDet];        // current sub-group's offset range
     __shared__ int glo[kTcS][kMaxDet], ghi[kTcS][kMaxDet], gstart[kTcS + 1];
-    __shared__ int tile_s, abort_s, ngroups_s;
+    __shared__ int tile_s, range_s, abort_s, ngroups_s;
     // bins per chunk for each sub-group offset spread (the float64 division once per block:
     // float64 is slow on this part)
     __shared__ int jmax_s[kTcSpreadLimit + 1];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const double beta = P.t_step * P.fs;
-    const int64_t n_tiles = ((n_dev ? min(n, (int64_t)*n_dev) : n) + kTcS - 1) / kTcS;
     const uint32_t idesc = tc::idesc_f16_f32(kTcS, kTcW);
     const uint32_t sbo = (uint32_t)kcores * 128u;
     const size_t part_halves = (size_t)kTcW * kp;                 // one B part
@@ -359,15 +494,26 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
         // the R tile, written by this thread's drains, is the target of the next tile's bulk
         // copy of the template matrices
         tc::fence_proxy_async_smem();
-        if (tid == 0)
-            tile_s = abort_s ? INT_MAX : atomicAdd(tile_counter, 1);
+        if (tid == 0) {
+            // the next unit: classes in order (see tc_units_kernel)
+            int u = abort_s ? INT_MAX : atomicAdd(units.counters, 1), cls = 0;
+            for (; cls < 4 && u >= units.counters[1 + cls]; ++cls)
+                u -= units.counters[1 + cls];
+            tile_s = INT_MAX;
+            if (cls < 4) {
+                const unsigned long long w =
+                    units.list[((cls == 1 || cls == 2) ? units.cap : 0) + (cls < 2 ? u : units.cap - 1 - u)];
+                tile_s = (int)(w >> 16);
+                range_s = (int)(w & 0xffffu);
+            }
+        }
         if (tid < kMaxDet) {
             lo_s[tid] = INT_MAX;
             hi_s[tid] = INT_MIN;
         }
         __syncthreads();
         const int64_t tile = tile_s;
-        if (tile >= n_tiles)
+        if (tile == INT_MAX)
             break;
         if (warp == kTcStagerWarp && lane == 0) {
             // template matrices into the tail of the R tile (free: the previous tile's last
@@ -381,7 +527,9 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
         if (tid < kTcS) {
             const int64_t si = tile * kTcS + tid;
             const int64_t n_use = n_dev ? min(n, (int64_t)*n_dev) : n;
-            uint32_t g = si < n_use ? perm[si] : 0xffffffffu;
+            // samples of the tile outside the unit count as padding
+            const bool in_unit = tid >= (range_s >> 8) && tid <= (range_s & 255);
+            uint32_t g = in_unit && si < n_use ? perm[si] : 0xffffffffu;
             const bool valid = (int64_t)g < n_theta;
             gid[tid] = valid ? g : 0xffffffffu;
             peak[tid] = 0ull;
@@ -733,7 +881,20 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                     lin[i] = 0.f;
                     bj[i] = 0u;
                 }
-                for (int t = 0, k = 0, j0 = 0; t < n_steps; ++t) {
+                // a lane quarter without a sample of the group (its four warps agree) leaves its
+                // rows in tensor memory
+                const bool idle = !__any_sync(0xffffffffu, gok && in_grp);
+                for (int t = 0; idle && t < n_steps; ++t) {
+                    const int b = t & 1;
+                    if (!tc::mbar_wait(fullb + b, phbit(kPhFull, b), kWaitNs))
+                        failed = 1;
+                    ph ^= 1u << (kPhFull + b);
+                    __syncwarp();
+                    tc::mbar_arrive_if(emptyb + b, lane == 0);
+                    if (failed)
+                        break;
+                }
+                for (int t = idle ? n_steps : 0, k = 0, j0 = 0; t < n_steps; ++t) {
                     const int b = t & 1, J = min(jnom, NT - j0);
                     const int jq = (J + kTcQ - 1) / kTcQ;                 // bins per quarter
                     const int jb = j0 + gh * jq, jn = max(0, min(jq, j0 + J - jb));   // this thread's bins
@@ -991,7 +1152,7 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
 
 cudaError_t launch_lnl_tc(const Problem &P, BinTable bt, const double *theta, const uint32_t *perm, int64_t n,
                           double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
-                          int *tile_counter, cudaStream_t st, const uint32_t *n_dev, int lnl_t_compact,
+                          TcUnits units, cudaStream_t st, const uint32_t *n_dev, int lnl_t_compact,
                           int64_t n_theta, PeakOut po)
 {
     if (n_theta <= 0)
@@ -1009,13 +1170,17 @@ cudaError_t launch_lnl_tc(const Problem &P, BinTable bt, const double *theta, co
     cudaError_t e = allow_max_dynamic_smem(kern);
     if (e != cudaSuccess)
         return e;
-    e = cudaMemsetAsync(tile_counter, 0, sizeof(int), st);
+    if (tc_units_cap(n) > units.cap)
+        return cudaErrorInvalidValue;
+    e = cudaMemsetAsync(units.counters, 0, kTcCounters * sizeof(int), st);
     if (e != cudaSuccess)
         return e;
     const int64_t tiles = (n + kTcS - 1) / kTcS;
-    const int grid = (int)(tiles < sms ? tiles : sms);
-    kern<<<grid, kTcThreads, smem, st>>>(P, bt, theta, perm, n, lnL_tmarg, lnL_t, lnpw, lnw, err, tile_counter,
-                                          n_dev, n_theta, lnl_t_compact, po);
+    tc_units_kernel<<<(unsigned)((tiles + kTcPlanWarps - 1) / kTcPlanWarps), 32 * kTcPlanWarps, 0, st>>>(
+        P, theta, perm, n, n_dev, n_theta, units.list, units.cap, units.counters);
+    const int grid = (int)std::min<int64_t>(kTcUnitsPerTile * tiles, sms);
+    kern<<<grid, kTcThreads, smem, st>>>(P, bt, theta, perm, n, lnL_tmarg, lnL_t, lnpw, lnw, err, units, n_dev,
+                                          n_theta, lnl_t_compact, po);
     return cudaGetLastError();
 }
 
