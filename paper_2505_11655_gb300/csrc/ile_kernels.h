@@ -224,6 +224,7 @@ cudaError_t launch_keys(const SkyGrid &G, const double *theta, int64_t n, uint32
 // words; *launched (optional) receives the number of kernels enqueued.
 constexpr int kRadixBits = 10;
 constexpr int kRadixBuckets = 1 << kRadixBits;
+constexpr int kRadixPasses = 7;   // 64-bit keys
 size_t sort_scratch_words(int64_t n_max);
 // Stable ascending sort of 64-bit keys in place (the low `bits` bits; tmp holds n keys,
 // scratch sort64_scratch_words(n) words).

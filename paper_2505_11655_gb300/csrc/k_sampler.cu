@@ -105,61 +105,149 @@ SkyGrid sky_grid_for(int64_t n, int per_cell)
 
 // ======================================================================== stable sort by sky cell
 //
-// Least-significant-digit radix sort of the cell keys (10-bit digits: one pass for
-// grids of up to 1024 cells, two for up to 2^20), stable in the sample index: samples
-// of one cell keep their draw order, so the tiles the likelihood kernels form, and
-// with them every float32 result, are the same from run to run.  Each pass: per-tile
-// digit counts (8192 samples per tile), an exclusive scan of the counts in
-// digit-major order, and a scatter in which each warp walks its contiguous quarter of
-// the tile in order and ranks equal digits with a warp match.
+// Least-significant-digit radix sort of the keys (digits of up to 10 bits, as wide as the keys
+// need for the fewest passes), stable in the sample index: samples of one cell keep their draw
+// order, so the tiles the likelihood kernels form, and with them every float32 result, are the
+// same from run to run.  Each pass:
+//   hist     digit counts of every tile of 2048 keys, and their totals per digit;
+//   rows     exclusive sums of each digit's counts over the tiles;
+//   scatter  each warp ranks its contiguous 256 keys of the tile digit by digit with a warp
+//            match (ranks in registers), then writes every key at digit base + tile row + rank.
+// The work of a pass is a few microseconds; what bounds it is the latency of one block's chain
+// of rounds, so the tiles are small enough to spread 50,000 keys over 25 SMs (with 8192-key
+// tiles and a three-kernel scan of the counts a sort of 250,000 20-bit keys took 180 us).
+// Up to 4096 keys are sorted by one block instead: (key, index) words by a bitonic network.
 
 constexpr int kRadixThreads = 256;
 constexpr int kRadixWarps = kRadixThreads / 32;
-constexpr int kRadixPerWarp = 1024;
+constexpr int kRadixRounds = 8;
+constexpr int kRadixPerWarp = 32 * kRadixRounds;
 constexpr int kRadixTile = kRadixWarps * kRadixPerWarp;
+constexpr int kSmallSort = 4096;      // keys of a one-block sort (12 index bits beside 20 key bits)
+constexpr int kSmallThreads = 1024;
 
 template <typename K>
-__global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const K *__restrict__ keys, int64_t n,
-                                                                   int shift, int nblk, uint32_t *__restrict__ hist)
+__global__ void __launch_bounds__(kRadixThreads) radix_hist_kernel(const K *__restrict__ keys, int64_t n, int shift,
+                                                                   int buckets, uint32_t *__restrict__ hist,
+                                                                   uint32_t *__restrict__ totals)
 {
     __shared__ uint32_t h[kRadixBuckets];
-    for (int d = threadIdx.x; d < kRadixBuckets; d += kRadixThreads)
+    for (int d = threadIdx.x; d < buckets; d += kRadixThreads)
         h[d] = 0u;
-    __syncthreads();
     const int64_t base = (int64_t)blockIdx.x * kRadixTile;
-    for (int j = threadIdx.x; j < kRadixTile; j += kRadixThreads) {
-        const int64_t i = base + j;
-        if (i < n)
-            atomicAdd(&h[(uint32_t)(keys[i] >> shift) & (kRadixBuckets - 1)], 1u);
+    K k[kRadixRounds];
+#pragma unroll
+    for (int r = 0; r < kRadixRounds; ++r) {
+        const int64_t i = base + r * kRadixThreads + threadIdx.x;
+        k[r] = i < n ? keys[i] : (K)0;
     }
     __syncthreads();
-    for (int d = threadIdx.x; d < kRadixBuckets; d += kRadixThreads)
-        hist[(size_t)d * nblk + blockIdx.x] = h[d];
+#pragma unroll
+    for (int r = 0; r < kRadixRounds; ++r)
+        if (base + r * kRadixThreads + threadIdx.x < n)
+            atomicAdd(&h[(uint32_t)(k[r] >> shift) & (uint32_t)(buckets - 1)], 1u);
+    __syncthreads();
+    for (int d = threadIdx.x; d < buckets; d += kRadixThreads) {
+        const uint32_t c = h[d];
+        hist[(size_t)blockIdx.x * buckets + d] = c;
+        if (c)
+            atomicAdd(totals + d, c);
+    }
+}
+
+// One block per 32 digits (a lane each); warp w owns a contiguous range of tiles.
+__global__ void __launch_bounds__(1024) radix_rows_kernel(uint32_t *__restrict__ hist, int nblk, int buckets)
+{
+    __shared__ uint32_t tot[32][33];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    uint32_t *col = hist + blockIdx.x * 32 + lane;
+    const int per = (nblk + 31) / 32, b0 = min(nblk, w * per), b1 = min(nblk, b0 + per);
+    uint32_t sum = 0;
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b)
+        sum += col[(size_t)b * buckets];
+    tot[w][lane] = sum;
+    __syncthreads();
+    uint32_t run = 0;
+    for (int v = 0; v < w; ++v)
+        run += tot[v][lane];
+#pragma unroll 8
+    for (int b = b0; b < b1; ++b) {
+        const uint32_t c = col[(size_t)b * buckets];
+        col[(size_t)b * buckets] = run;
+        run += c;
+    }
 }
 
 template <typename K>
 __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const K *__restrict__ keys_in,
                                                                       const uint32_t *__restrict__ vals_in, int64_t n,
-                                                                      int shift, int nblk,
-                                                                      const uint32_t *__restrict__ offsets,
+                                                                      int shift, int buckets,
+                                                                      const uint32_t *__restrict__ hist,
+                                                                      const uint32_t *__restrict__ totals,
                                                                       K *__restrict__ keys_out,
                                                                       uint32_t *__restrict__ vals_out)
 {
     __shared__ uint32_t wpos[kRadixWarps][kRadixBuckets];   // per-warp digit counts, then positions
+    __shared__ uint32_t wtot[kRadixWarps];
+    constexpr int kPer = kRadixBuckets / kRadixThreads;     // digits per thread in the scan of the totals
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int e = threadIdx.x; e < kRadixWarps * kRadixBuckets; e += kRadixThreads)
-        (&wpos[0][0])[e] = 0u;
-    __syncthreads();
+    for (int d = threadIdx.x; d < buckets; d += kRadixThreads)
+#pragma unroll
+        for (int v = 0; v < kRadixWarps; ++v)
+            wpos[v][d] = 0u;
     const int64_t base = (int64_t)blockIdx.x * kRadixTile + (int64_t)w * kRadixPerWarp;
-    for (int j = lane; j < kRadixPerWarp; j += 32) {
-        const int64_t i = base + j;
-        if (i < n)
-            atomicAdd(&wpos[w][(uint32_t)(keys_in[i] >> shift) & (kRadixBuckets - 1)], 1u);
+    K k[kRadixRounds];
+    uint32_t rank[kRadixRounds];
+#pragma unroll
+    for (int r = 0; r < kRadixRounds; ++r) {
+        const int64_t i = base + 32 * r + lane;
+        k[r] = i < n ? keys_in[i] : (K)0;
+    }
+    // exclusive sums of the digit totals: kPer consecutive digits per thread
+    uint32_t t[kPer], mine = 0;
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int d = threadIdx.x * kPer + q;
+        t[q] = mine;
+        mine += d < buckets ? totals[d] : 0u;
+    }
+    uint32_t x = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o)
+            x += y;
+    }
+    if (lane == 31)
+        wtot[w] = x;
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kRadixRounds; ++r) {
+        const bool ok = base + 32 * r + lane < n;
+        const uint32_t d = ok ? (uint32_t)(k[r] >> shift) & (uint32_t)(buckets - 1) : 0xffffffffu;
+        const unsigned peers = __match_any_sync(0xffffffffu, d);
+        uint32_t before = 0;
+        if (ok)
+            before = wpos[w][d];
+        __syncwarp();
+        rank[r] = before + __popc(peers & ((1u << lane) - 1u));
+        if (ok && lane == __ffs(peers) - 1)
+            wpos[w][d] = before + (uint32_t)__popc(peers);
+        __syncwarp();
     }
     __syncthreads();
-    // first position of each digit for each warp: the tile's offset, then warps in order
-    for (int d = threadIdx.x; d < kRadixBuckets; d += kRadixThreads) {
-        uint32_t run = offsets[(size_t)d * nblk + blockIdx.x];
+    // first position of each digit for each warp: the digit's base, the tile's row, then the
+    // warps in order
+    uint32_t off = x - mine;
+    for (int v = 0; v < w; ++v)
+        off += wtot[v];
+#pragma unroll
+    for (int q = 0; q < kPer; ++q) {
+        const int d = threadIdx.x * kPer + q;
+        if (d >= buckets)
+            break;
+        uint32_t run = off + t[q] + hist[(size_t)blockIdx.x * buckets + d];
 #pragma unroll
         for (int v = 0; v < kRadixWarps; ++v) {
             const uint32_t c = wpos[v][d];
@@ -168,24 +256,42 @@ __global__ void __launch_bounds__(kRadixThreads) radix_scatter_kernel(const K *_
         }
     }
     __syncthreads();
-    for (int j0 = 0; j0 < kRadixPerWarp && base + j0 < n; j0 += 32) {
-        const int64_t i = base + j0 + lane;
-        const bool ok = i < n;
-        const K k = ok ? keys_in[i] : (K)0;
-        const uint32_t d = ok ? (uint32_t)(k >> shift) & (kRadixBuckets - 1) : 0xffffffffu;
-        const unsigned peers = __match_any_sync(0xffffffffu, d);
-        if (ok) {
-            const uint32_t pos = wpos[w][d] + __popc(peers & ((1u << lane) - 1u));
+#pragma unroll
+    for (int r = 0; r < kRadixRounds; ++r) {
+        const int64_t i = base + 32 * r + lane;
+        if (i < n) {
+            const uint32_t pos = wpos[w][(uint32_t)(k[r] >> shift) & (uint32_t)(buckets - 1)] + rank[r];
             if (vals_out)
                 vals_out[pos] = vals_in ? vals_in[i] : (uint32_t)i;
             if (keys_out)
-                keys_out[pos] = k;
+                keys_out[pos] = k[r];
         }
-        __syncwarp();
-        if (ok && lane == __ffs(peers) - 1)
-            wpos[w][d] += (uint32_t)__popc(peers);
-        __syncwarp();
     }
+}
+
+// At most kSmallSort keys of at most 20 bits, one block: words (key, index) are distinct, so
+// any sort of them is the stable one; the network runs over `size` words, a power of two.
+__global__ void __launch_bounds__(kSmallThreads) small_sort_kernel(const uint32_t *__restrict__ keys, int n, int size,
+                                                                   uint32_t *__restrict__ perm)
+{
+    __shared__ uint32_t a[kSmallSort];
+    for (int i = threadIdx.x; i < size; i += (int)blockDim.x)
+        a[i] = i < n ? (keys[i] << 12) | (uint32_t)i : 0xffffffffu;
+    for (int len = 2; len <= size; len <<= 1)
+        for (int step = len >> 1; step > 0; step >>= 1) {
+            __syncthreads();
+            for (int e = threadIdx.x; e < size / 2; e += (int)blockDim.x) {
+                const int i = 2 * e - (e & (step - 1)), j = i + step;
+                const uint32_t u = a[i], v = a[j];
+                if ((u > v) == ((i & len) == 0)) {
+                    a[i] = v;
+                    a[j] = u;
+                }
+            }
+        }
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += (int)blockDim.x)
+        perm[i] = a[i] & 4095u;
 }
 
 // Exclusive scan of L counts in place: per-tile totals of 4096 counts, a scan of the
@@ -321,15 +427,35 @@ cudaError_t launch_scan_u64(uint64_t *data, int64_t L, uint64_t *scratch, cudaSt
     return cudaGetLastError();
 }
 
-size_t sort_scratch_words(int64_t n_max)
+// digit counts of every tile and pass totals
+static size_t radix_words(int64_t n_max)
 {
     const int64_t nblk = (n_max + kRadixTile - 1) / kRadixTile;
-    int64_t L = (int64_t)kRadixBuckets * (nblk > 0 ? nblk : 1), words = L;
-    while (L > 1) {   // totals of every scan level
-        L = (L + kScanTile - 1) / kScanTile;
-        words += L;
-    }
-    return (size_t)(words + 2 * n_max + 64);
+    return (size_t)kRadixBuckets * (size_t)((nblk > 0 ? nblk : 1) + kRadixPasses);
+}
+
+size_t sort_scratch_words(int64_t n_max) { return radix_words(n_max) + (size_t)(2 * n_max + 64); }
+
+size_t sort64_scratch_words(int64_t n_max) { return radix_words(n_max) + 64; }
+
+// One pass over the digit of `bits` bits at `shift`; totals zeroed by the caller.
+template <typename K>
+static void radix_pass(const K *in, const uint32_t *vin, int64_t n, int shift, int bits, uint32_t *hist,
+                       uint32_t *totals, K *out, uint32_t *vout, cudaStream_t st)
+{
+    const int nblk = (int)((n + kRadixTile - 1) / kRadixTile), buckets = 1 << bits;
+    radix_hist_kernel<K><<<nblk, kRadixThreads, 0, st>>>(in, n, shift, buckets, hist, totals);
+    radix_rows_kernel<<<buckets / 32, 1024, 0, st>>>(hist, nblk, buckets);
+    radix_scatter_kernel<K><<<nblk, kRadixThreads, 0, st>>>(in, vin, n, shift, buckets, hist, totals, out, vout);
+}
+
+// passes of a sort of `bits`-bit keys, and the digit width (5 bits at least: whole warps of
+// digits)
+static int radix_plan(int bits, int *digit)
+{
+    const int passes = bits <= 0 ? 0 : (bits + kRadixBits - 1) / kRadixBits;
+    *digit = passes ? std::max(5, (bits + passes - 1) / passes) : 0;
+    return passes;
 }
 
 cudaError_t launch_sort(const SkyGrid &G, const uint32_t *key, int64_t n, uint32_t *scratch, uint32_t *perm,
@@ -339,38 +465,32 @@ cudaError_t launch_sort(const SkyGrid &G, const uint32_t *key, int64_t n, uint32
         *launched = 0;
     if (n <= 0)
         return cudaSuccess;
-    const int nblk = (int)((n + kRadixTile - 1) / kRadixTile);
-    const int L = kRadixBuckets * nblk;
-    uint32_t *hist = scratch;
-    uint32_t *key_tmp = hist + L, *val_tmp = key_tmp + n;
-    uint32_t *scan_scratch = val_tmp + n;
-    const int passes = G.n_cells <= kRadixBuckets ? 1 : 2;
-    int count = 0;
+    int bits = 0, digit = 0;
+    while ((1ll << bits) < (int64_t)G.n_cells)
+        ++bits;
+    if (n <= kSmallSort && bits <= 20) {
+        int size = 2;
+        while (size < n)
+            size <<= 1;
+        small_sort_kernel<<<1, std::min(kSmallThreads, std::max(32, size / 2)), 0, st>>>(key, (int)n, size, perm);
+        if (launched)
+            *launched = 1;
+        return cudaGetLastError();
+    }
+    const int passes = radix_plan(std::max(bits, 1), &digit);
+    uint32_t *totals = scratch, *hist = totals + kRadixPasses * kRadixBuckets;
+    uint32_t *key_tmp = scratch + radix_words(n), *val_tmp = key_tmp + n;
+    cudaError_t e = cudaMemsetAsync(totals, 0, sizeof(uint32_t) * kRadixBuckets * passes, st);
+    if (e != cudaSuccess)
+        return e;
     for (int pass = 0; pass < passes; ++pass) {
-        const int shift = pass * kRadixBits;
         const bool last = pass == passes - 1;
-        const uint32_t *kin = pass == 0 ? key : key_tmp;
-        const uint32_t *vin = pass == 0 ? nullptr : val_tmp;
-        radix_hist_kernel<uint32_t><<<nblk, kRadixThreads, 0, st>>>(kin, n, shift, nblk, hist);
-        count += 1 + launch_scan<uint32_t>(hist, L, scan_scratch, st);
-        radix_scatter_kernel<uint32_t><<<nblk, kRadixThreads, 0, st>>>(kin, vin, n, shift, nblk, hist,
-                                                                       last ? nullptr : key_tmp, last ? perm : val_tmp);
-        count += 1;
+        radix_pass<uint32_t>(pass == 0 ? key : key_tmp, pass == 0 ? nullptr : val_tmp, n, pass * digit, digit, hist,
+                             totals + pass * kRadixBuckets, last ? nullptr : key_tmp, last ? perm : val_tmp, st);
     }
     if (launched)
-        *launched = count;
+        *launched = 3 * passes;
     return cudaGetLastError();
-}
-
-size_t sort64_scratch_words(int64_t n_max)
-{
-    const int64_t nblk = (n_max + kRadixTile - 1) / kRadixTile;
-    int64_t L = (int64_t)kRadixBuckets * (nblk > 0 ? nblk : 1), words = L;
-    while (L > 1) {
-        L = (L + kScanTile - 1) / kScanTile;
-        words += L;
-    }
-    return (size_t)(words + 64);
 }
 
 cudaError_t launch_sort64(uint64_t *keys, uint64_t *tmp, int64_t n, int bits, uint32_t *scratch, cudaStream_t st,
@@ -380,22 +500,20 @@ cudaError_t launch_sort64(uint64_t *keys, uint64_t *tmp, int64_t n, int bits, ui
         *launched = 0;
     if (n <= 0)
         return cudaSuccess;
-    const int nblk = (int)((n + kRadixTile - 1) / kRadixTile);
-    const int L = kRadixBuckets * nblk;
-    uint32_t *hist = scratch, *scan_scratch = scratch + L;
-    const int passes = bits <= 0 ? 0 : (bits + kRadixBits - 1) / kRadixBits;
-    int count = 0;
+    int digit = 0;
+    const int passes = radix_plan(bits, &digit);
+    if (passes > kRadixPasses)
+        return cudaErrorInvalidValue;
+    uint32_t *totals = scratch, *hist = totals + kRadixPasses * kRadixBuckets;
+    if (passes) {
+        cudaError_t e = cudaMemsetAsync(totals, 0, sizeof(uint32_t) * kRadixBuckets * passes, st);
+        if (e != cudaSuccess)
+            return e;
+    }
     uint64_t *in = keys, *out = tmp;
     for (int pass = 0; pass < passes; ++pass) {
-        const int shift = pass * kRadixBits;
-        radix_hist_kernel<uint64_t><<<nblk, kRadixThreads, 0, st>>>(in, n, shift, nblk, hist);
-        count += 1 + launch_scan<uint32_t>(hist, L, scan_scratch, st);
-        radix_scatter_kernel<uint64_t><<<nblk, kRadixThreads, 0, st>>>(in, nullptr, n, shift, nblk, hist, out,
-                                                                       nullptr);
-        count += 1;
-        uint64_t *t = in;
-        in = out;
-        out = t;
+        radix_pass<uint64_t>(in, nullptr, n, pass * digit, digit, hist, totals + pass * kRadixBuckets, out, nullptr, st);
+        std::swap(in, out);
     }
     if (in != keys) {   // odd number of passes: the sorted keys are in tmp
         cudaError_t e = cudaMemcpyAsync(keys, in, sizeof(uint64_t) * n, cudaMemcpyDeviceToDevice, st);
@@ -403,7 +521,7 @@ cudaError_t launch_sort64(uint64_t *keys, uint64_t *tmp, int64_t n, int bits, ui
             return e;
     }
     if (launched)
-        *launched = count;
+        *launched = 3 * passes;
     return cudaGetLastError();
 }
 
