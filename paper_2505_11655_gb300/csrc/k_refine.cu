@@ -57,18 +57,29 @@ __global__ void __launch_bounds__(kSelThreads) select_count_kernel(const double 
     }
 }
 
-// exclusive scan of the nb block counts in place; the total goes to *count
-__global__ void select_scan_kernel(uint32_t *__restrict__ blk, int nb, uint32_t *__restrict__ count)
+// exclusive scan of the nb <= kSelMaxBlocks block counts in place; the total goes to *count
+__global__ void __launch_bounds__(kSelMaxBlocks) select_scan_kernel(uint32_t *__restrict__ blk, int nb,
+                                                                    uint32_t *__restrict__ count)
 {
-    if (threadIdx.x == 0) {
-        uint32_t run = 0;
-        for (int b = 0; b < nb; ++b) {
-            const uint32_t c = blk[b];
-            blk[b] = run;
-            run += c;
-        }
-        *count = run;
+    __shared__ uint32_t ws[kSelMaxBlocks / 32];
+    const int t = threadIdx.x, lane = t & 31;
+    const uint32_t c = t < nb ? blk[t] : 0u;
+    uint32_t x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o)
+            x += y;
     }
+    if (lane == 31)
+        ws[t >> 5] = x;
+    __syncthreads();
+    for (int v = 0; v < (t >> 5); ++v)
+        x += ws[v];
+    if (t < nb)
+        blk[t] = x - c;
+    if (t == (int)blockDim.x - 1)
+        *count = x;
 }
 
 __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const double *__restrict__ key,
@@ -264,7 +275,7 @@ cudaError_t launch_select(const double *key, const uint32_t *perm, int64_t n, co
     const int64_t want = (n + 4 * kSelThreads - 1) / (4 * kSelThreads);
     const int grid = (int)(want < kSelMaxBlocks ? (want > 0 ? want : 1) : kSelMaxBlocks);
     select_count_kernel<<<grid, kSelThreads, 0, st>>>(key, perm, n, stats, slot, margin, blk);
-    select_scan_kernel<<<1, 32, 0, st>>>(blk, grid, count);
+    select_scan_kernel<<<1, (grid + 31) / 32 * 32, 0, st>>>(blk, grid, count);
     select_write_kernel<<<grid, kSelThreads, 0, st>>>(key, perm, n, stats, slot, margin, blk, idx);
     return cudaGetLastError();
 }

@@ -555,45 +555,54 @@ __device__ __forceinline__ Acc acc_merge(Acc a, Acc b)
     return r;
 }
 
-__device__ Acc block_merge(Acc a)
+// Block-wide maximum of (mx, lmx, bad), then sum of (s1, s2).  The maximum comes first and the
+// sums are taken relative to it, so that no merge step needs an exponential: a float64
+// exponential is a chain of some forty operations on this part's slow float64 pipe, and the
+// former merge of (maximum, sums) records had two of them at each of its ten levels (250,000
+// samples: 52 + 35 us for the partial sums and the final merge).
+__device__ void block_max(Acc &a)
 {
-    __shared__ double smx[32], ss1[32], ss2[32], slm[32];
+    __shared__ double smx[32], slm[32];
     __shared__ int sbad[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
 #pragma unroll
     for (int o = 16; o; o >>= 1) {
-        Acc b;
-        b.mx = __shfl_xor_sync(0xffffffffu, a.mx, o);
-        b.s1 = __shfl_xor_sync(0xffffffffu, a.s1, o);
-        b.s2 = __shfl_xor_sync(0xffffffffu, a.s2, o);
-        b.lmx = __shfl_xor_sync(0xffffffffu, a.lmx, o);
-        b.bad = __shfl_xor_sync(0xffffffffu, a.bad, o);
-        a = acc_merge(a, b);
+        a.mx = fmax(a.mx, __shfl_xor_sync(0xffffffffu, a.mx, o));
+        a.lmx = fmax(a.lmx, __shfl_xor_sync(0xffffffffu, a.lmx, o));
+        a.bad |= __shfl_xor_sync(0xffffffffu, a.bad, o);
     }
     if (lane == 0) {
         smx[w] = a.mx;
-        ss1[w] = a.s1;
-        ss2[w] = a.s2;
         slm[w] = a.lmx;
         sbad[w] = a.bad;
     }
     __syncthreads();
-    if (w == 0) {
-        Acc b = lane < nw ? Acc{smx[lane], ss1[lane], ss2[lane], slm[lane], sbad[lane]}
-                          : Acc{-INFINITY, 0.0, 0.0, -INFINITY, 0};
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            Acc c;
-            c.mx = __shfl_xor_sync(0xffffffffu, b.mx, o);
-            c.s1 = __shfl_xor_sync(0xffffffffu, b.s1, o);
-            c.s2 = __shfl_xor_sync(0xffffffffu, b.s2, o);
-            c.lmx = __shfl_xor_sync(0xffffffffu, b.lmx, o);
-            c.bad = __shfl_xor_sync(0xffffffffu, b.bad, o);
-            b = acc_merge(b, c);
-        }
-        a = b;
+    for (int v = 0; v < nw; ++v) {
+        a.mx = fmax(a.mx, smx[v]);
+        a.lmx = fmax(a.lmx, slm[v]);
+        a.bad |= sbad[v];
     }
-    return a;   // valid in warp 0
+}
+
+__device__ void block_sum(Acc &a)   // valid in thread 0
+{
+    __shared__ double ss1[32], ss2[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        a.s1 += __shfl_xor_sync(0xffffffffu, a.s1, o);
+        a.s2 += __shfl_xor_sync(0xffffffffu, a.s2, o);
+    }
+    if (lane == 0) {
+        ss1[w] = a.s1;
+        ss2[w] = a.s2;
+    }
+    __syncthreads();
+    a.s1 = a.s2 = 0.0;
+    for (int v = 0; v < nw; ++v) {
+        a.s1 += ss1[v];
+        a.s2 += ss2[v];
+    }
 }
 
 // exp(t) for t <= 0: float64, or float32 for terms that carry float32 errors already
@@ -611,27 +620,27 @@ __global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(const doubl
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = (int64_t)blockIdx.x * per;
     const int64_t b1 = min(n, b0 + per);
-    // local max first, then sums relative to it
+    // the stripe's maximum first, then sums relative to it
     Acc a{-INFINITY, 0.0, 0.0, -INFINITY, 0};
     for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
-        double x = lnw[i];
+        const double x = lnw[i];
         if (!isfinite(x)) {
             a.bad = 1;
             continue;
         }
-        if (x > a.mx) {
-            double f = (a.mx == -INFINITY) ? 0.0 : term_exp(a.mx - x, f32);
-            a.s1 = a.s1 * f + 1.0;
-            a.s2 = a.s2 * f * f + 1.0;
-            a.mx = x;
-        } else {
-            double e = term_exp(x - a.mx, f32);
-            a.s1 += e;
-            a.s2 += e * e;
-        }
+        a.mx = fmax(a.mx, x);
         a.lmx = fmax(a.lmx, lnL[i]);
     }
-    a = block_merge(a);
+    block_max(a);
+    for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
+        const double x = lnw[i];
+        if (!isfinite(x))
+            continue;
+        const double e = term_exp(x - a.mx, f32);
+        a.s1 += e;
+        a.s2 += e * e;
+    }
+    block_sum(a);
     if (threadIdx.x == 0) {
         double *o = partial + 5 * blockIdx.x;
         o[0] = a.mx;
@@ -651,9 +660,20 @@ __global__ void __launch_bounds__(kRedThreads) reduce_final_kernel(const double 
     Acc a{-INFINITY, 0.0, 0.0, -INFINITY, 0};
     for (int b = threadIdx.x; b < nb; b += blockDim.x) {
         const double *o = partial + 5 * b;
-        a = acc_merge(a, Acc{o[0], o[1], o[2], o[3], o[4] != 0.0});
+        a.mx = fmax(a.mx, o[0]);
+        a.lmx = fmax(a.lmx, o[3]);
+        a.bad |= o[4] != 0.0;
     }
-    a = block_merge(a);
+    block_max(a);
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+        const double *o = partial + 5 * b;
+        if (o[0] == -INFINITY)
+            continue;
+        const double f = exp(o[0] - a.mx);
+        a.s1 += o[1] * f;
+        a.s2 += o[2] * f * f;
+    }
+    block_sum(a);
     if (threadIdx.x == 0) {
         double N = (double)n;
         double *s = stats + 8 * slot;
@@ -791,6 +811,19 @@ __global__ void __launch_bounds__(256) hist_partial_kernel(SamplerDev S, const u
         partial[(size_t)blockIdx.x * 12 * B + e] = sF[e];
 }
 
+// Masses P of dimension d and their running sums C (shared memory) to the sampler's tables.
+__device__ __forceinline__ void write_cdf(const SamplerDev &S, int d, const double *P, const double *C)
+{
+    const int B = S.B;
+    if (threadIdx.x == 0)
+        S.C[d * (B + 1)] = 0.0;
+    for (int b = threadIdx.x; b < B; b += blockDim.x) {
+        S.P[d * B + b] = P[b];
+        S.C[d * (B + 1) + b + 1] = C[b];
+        S.L[d * B + b] = log(B * P[b] / C[B - 1]);
+    }
+}
+
 // Sum the partial histograms exactly (128-bit); P <- (1-eps) H / sum H + eps / B; rebuild C.
 // One block per dimension: the bins' sums over the block partials are split across the
 // block's threads (integer sums, so the same H in any split), then one warp finishes.
@@ -801,6 +834,9 @@ __global__ void __launch_bounds__(kAdaptFinalThreads) adapt_final_kernel(Sampler
     const int B = S.B, d = blockIdx.x;
     if (d >= 6 || (S.marg && d == 5))   // a marginalised distance keeps its masses
         return;
+    // (the masses and their running sums in shared memory: a serial loop over global memory
+    // was most of this kernel's time)
+    __shared__ double H[RIFT_MAX_BINS], C[RIFT_MAX_BINS];
     __shared__ unsigned long long acc[3][kAdaptFinalThreads];
     const int tpb = B < kAdaptFinalThreads ? kAdaptFinalThreads / B : 1;   // threads per bin
     const int t = threadIdx.x, j = t % tpb, b0 = t / tpb, bstride = kAdaptFinalThreads / tpb;
@@ -832,37 +868,29 @@ __global__ void __launch_bounds__(kAdaptFinalThreads) adapt_final_kernel(Sampler
             }
             const uint64_t a = l0 + (l1 << 32);
             hi += (l1 >> 32) + (a < l0 ? 1u : 0u);
-            S.C[d * (B + 1) + b + 1] = ldexp((double)hi, 64 - kFixShift) + ldexp((double)a, -kFixShift);   // H
+            H[b] = ldexp((double)hi, 64 - kFixShift) + ldexp((double)a, -kFixShift);
         }
         __syncthreads();
     }
-    if (t >= 32)
-        return;
-    const int lane = t;
-    double tot = 0.0;
-    for (int b = lane; b < B; b += 32)
-        tot += S.C[d * (B + 1) + b + 1];   // H stashed in the C slots while reducing
+    if (t < 32) {
+        double tot = 0.0;
+        for (int b = t; b < B; b += 32)
+            tot += H[b];
 #pragma unroll
-    for (int o = 16; o; o >>= 1)
-        tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    __syncwarp();
-    if (tot > 0.0 && isfinite(tot)) {
-        for (int b = lane; b < B; b += 32)
-            S.P[d * B + b] = (1.0 - S.floor_eps) * S.C[d * (B + 1) + b + 1] / tot + S.floor_eps / B;
-    }
-    __syncwarp();
-    if (lane == 0) {
-        double run = 0.0;
-        S.C[d * (B + 1)] = 0.0;
-        for (int b = 0; b < B; ++b) {
-            run += S.P[d * B + b];
-            S.C[d * (B + 1) + b + 1] = run;
+        for (int o = 16; o; o >>= 1)
+            tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        const bool adapt = tot > 0.0 && isfinite(tot);
+        for (int b = t; b < B; b += 32)
+            H[b] = adapt ? (1.0 - S.floor_eps) * H[b] / tot + S.floor_eps / B : S.P[d * B + b];
+        __syncwarp();
+        if (t == 0) {
+            double run = 0.0;
+            for (int b = 0; b < B; ++b)
+                C[b] = run += H[b];
         }
     }
-    __syncwarp();
-    const double ctot = S.C[d * (B + 1) + B];
-    for (int b = lane; b < B; b += 32)
-        S.L[d * B + b] = log(B * S.P[d * B + b] / ctot);
+    __syncthreads();
+    write_cdf(S, d, H, C);
 }
 
 cudaError_t launch_adapt(const SamplerDev &S, const uint64_t *bins, const double *lnw, int64_t n, const double *stats,
@@ -884,24 +912,27 @@ cudaError_t launch_adapt(const SamplerDev &S, const uint64_t *bins, const double
     return cudaGetLastError();
 }
 
-__global__ void build_cdf_kernel(SamplerDev S)
+// One block per dimension (one thread a dimension, with a logarithm per bin in turn, took 93 us
+// for 64 bins).
+__global__ void __launch_bounds__(128) build_cdf_kernel(SamplerDev S)
 {
-    const int d = threadIdx.x;
-    if (d >= 6)
-        return;
-    double run = 0.0;
-    S.C[d * (S.B + 1)] = 0.0;
-    for (int b = 0; b < S.B; ++b) {
-        run += S.P[d * S.B + b];
-        S.C[d * (S.B + 1) + b + 1] = run;
+    __shared__ double P[RIFT_MAX_BINS], C[RIFT_MAX_BINS];
+    const int d = blockIdx.x;
+    for (int b = threadIdx.x; b < S.B; b += blockDim.x)
+        P[b] = S.P[d * S.B + b];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double run = 0.0;
+        for (int b = 0; b < S.B; ++b)
+            C[b] = run += P[b];
     }
-    for (int b = 0; b < S.B; ++b)
-        S.L[d * S.B + b] = log(S.B * S.P[d * S.B + b] / run);
+    __syncthreads();
+    write_cdf(S, d, P, C);
 }
 
 cudaError_t launch_build_cdf(const SamplerDev &S, cudaStream_t st)
 {
-    build_cdf_kernel<<<1, 32, 0, st>>>(S);
+    build_cdf_kernel<<<6, 128, 0, st>>>(S);
     return cudaGetLastError();
 }
 
