@@ -962,23 +962,6 @@ int rift_ile_set_waveforms(rift_ile_t *h, int32_t n_freq, const double *freqs, c
     const int K = h->prob.K, M = h->prob.M, F = n_freq;
     const size_t fb = sizeof(double) * F, hb = sizeof(double2) * (size_t)M * F, db = sizeof(double2) * (size_t)K * F,
                  wb = sizeof(double) * (size_t)K * F;
-    // host checks: mirror-symmetric grid, weights finite, non-negative and symmetric in f
-    std::vector<double> hf(F), hw((size_t)K * F);
-    const cudaMemcpyKind to_host = mem == RIFT_MEM_HOST ? cudaMemcpyHostToHost : cudaMemcpyDeviceToHost;
-    CK(cudaMemcpyAsync(hf.data(), freqs, fb, to_host, h->stream));
-    CK(cudaMemcpyAsync(hw.data(), weights, wb, to_host, h->stream));
-    CK(cudaStreamSynchronize(h->stream));
-    for (int j = 0; j < F; ++j) {
-        if (!std::isfinite(hf[j]) || hf[F - 1 - j] != -hf[j])
-            return RIFT_EINVAL;
-        for (int k = 0; k < K; ++k) {
-            const double a = hw[(size_t)k * F + j];
-            if (!std::isfinite(a))
-                return RIFT_ENONFINITE;
-            if (a < 0.0 || a != hw[(size_t)k * F + (F - 1 - j)])
-                return RIFT_EINVAL;
-        }
-    }
     std::vector<void *> tmp;
     auto grab = [&](size_t bytes) -> void * {
         void *q = nullptr;
@@ -991,52 +974,13 @@ int rift_ile_set_waveforms(rift_ile_t *h, int32_t n_freq, const double *freqs, c
     };
     auto A = static_cast<double2 *>(grab(sizeof(double2) * (size_t)K * M * F));
     auto t0 = static_cast<double *>(grab(sizeof(double) * K));
-    // Q by FFT when the grid lies on a lattice f_j = f_0 + n_j df (ascending, integer n_j
-    // within 1e-9 relative) and L = f_s / df is a power of two spanning every n_j; else the
-    // direct sum.  RIFT_ILE_DFT=1 forces the direct sum.
-    FftPlan plan{};
-    bool use_fft = !(std::getenv("RIFT_ILE_DFT") && std::getenv("RIFT_ILE_DFT")[0] == '1');
-    std::vector<int> nidx(F);
-    {
-        double df = 0.0, fmax = 0.0;
-        for (int j = 0; j < F; ++j)
-            fmax = std::max(fmax, std::fabs(hf[j]));
-        for (int j = 1; j < F && use_fft; ++j) {
-            const double gap = hf[j] - hf[j - 1];
-            if (!(gap > 0.0))
-                use_fft = false;
-            else if (df == 0.0 || gap < df)
-                df = gap;
-        }
-        const double Lr = use_fft && df > 0.0 ? h->prob.fs / df : 0.0;
-        const int64_t L = (int64_t)std::llround(Lr);
-        use_fft = use_fft && L >= 2 && L <= ((int64_t)1 << 26) && (L & (L - 1)) == 0 &&
-                  std::fabs(Lr - (double)L) <= 1e-9 * (double)L;
-        for (int j = 0; j < F && use_fft; ++j) {
-            const double nr = (hf[j] - hf[0]) / df;
-            const int64_t nj = std::llround(nr);
-            if (std::fabs(hf[j] - hf[0] - (double)nj * df) > 1e-9 * std::max(1.0, fmax) || nj < 0 || nj >= L)
-                use_fft = false;
-            else
-                nidx[j] = (int)nj;
-        }
-        if (use_fft) {
-            plan.L = (int)L;
-            plan.f0 = hf[0];
-            auto ni = static_cast<int *>(grab(sizeof(int) * F));
-            plan.X = static_cast<double2 *>(grab(sizeof(double2) * (size_t)K * M * L));
-            plan.Y = static_cast<double2 *>(grab(sizeof(double2) * (size_t)K * M * L));
-            plan.T = static_cast<double2 *>(grab(sizeof(double2) * (size_t)std::max<int64_t>(1, L / 2)));
-            if (!ni || !plan.X || !plan.Y || !plan.T ||
-                cudaMemcpyAsync(ni, nidx.data(), sizeof(int) * F, cudaMemcpyHostToDevice, h->stream) != cudaSuccess)
-                use_fft = false;   // the direct sum needs no scratch of this size
-            plan.nidx = ni;
-        }
-    }
+    auto uvp = static_cast<double *>(grab(sizeof(double) * uv_scratch_doubles(K, M, F)));
+    auto nidx = static_cast<int *>(grab(sizeof(int) * F));
+    auto info_dev = static_cast<WaveformInfo *>(grab(sizeof(WaveformInfo)));
     int launched = 0;
     const double *df = freqs, *dw = weights;
     const double2 *dh = static_cast<const double2 *>(hlm), *dd = static_cast<const double2 *>(data);
-    int rc = (A && t0) ? RIFT_OK : RIFT_ENOMEM;
+    int rc = (A && t0 && uvp && nidx && info_dev) ? RIFT_OK : RIFT_ENOMEM;
     if (rc == RIFT_OK && mem == RIFT_MEM_HOST) {
         auto f2 = static_cast<double *>(grab(fb));
         auto h2 = static_cast<double2 *>(grab(hb));
@@ -1054,14 +998,43 @@ int rift_ile_set_waveforms(rift_ile_t *h, int32_t n_freq, const double *freqs, c
         dd = d2;
         dw = w2;
     }
+    // mirror-symmetric grid, weights finite, non-negative and symmetric in f: checked on the
+    // device (of device inputs, a copy of the grid and the weights to the host and the loops over
+    // them took a fifth of the call).  Q by FFT when the grid lies on a lattice, else the direct
+    // sum.  RIFT_ILE_DFT=1 forces the direct sum.
+    WaveformInfo info{};
+    if (rc == RIFT_OK &&
+        (launch_waveform_check(df, dw, K, F, h->prob.fs, nidx, info_dev, h->stream) ||
+         cudaMemcpyAsync(&info, info_dev, sizeof(info), cudaMemcpyDeviceToHost, h->stream) ||
+         cudaStreamSynchronize(h->stream)))
+        rc = RIFT_ECUDA;
+    if (rc == RIFT_OK && info.bad != ~0ull)
+        rc = (info.bad & 3ull) == (unsigned)kWaveformNonFinite ? RIFT_ENONFINITE : RIFT_EINVAL;
+    FftPlan plan{};
+    bool use_fft = rc == RIFT_OK && info.L > 0 &&
+                   !(std::getenv("RIFT_ILE_DFT") && std::getenv("RIFT_ILE_DFT")[0] == '1');
+    if (use_fft) {
+        plan.L = info.L;
+        plan.f0 = info.f0;
+        plan.nidx = nidx;
+        const bool pruned = fft_pruned(plan.L, h->prob.n_q);
+        plan.X = static_cast<double2 *>(grab(sizeof(double2) * (size_t)K * M * plan.L));
+        plan.T = static_cast<double2 *>(grab(sizeof(double2) * (size_t)(plan.L / 2)));
+        if (pruned)
+            plan.jidx = static_cast<int *>(grab(sizeof(int) * (size_t)plan.L));
+        else
+            plan.Y = static_cast<double2 *>(grab(sizeof(double2) * (size_t)K * M * plan.L));
+        if (!plan.X || !plan.T || (pruned ? !plan.jidx : !plan.Y))
+            use_fft = false;   // the direct sum needs no scratch of this size
+    }
     if (rc == RIFT_OK &&
         (cudaMemcpyAsync(t0, h->q_t0.data(), sizeof(double) * K, cudaMemcpyHostToDevice, h->stream) ||
          cudaMemsetAsync(h->err, 0, sizeof(int), h->stream) ||
-         launch_precompute(dh, dd, dw, df, K, M, F, t0, h->prob.fs, h->prob.n_q, A, h->Q64, h->U64, h->V64,
+         launch_precompute(dh, dd, dw, df, K, M, F, t0, h->prob.fs, h->prob.n_q, A, uvp, h->Q64, h->U64, h->V64,
                            h->stream, use_fft ? &plan : nullptr, &launched)))
         rc = RIFT_ECUDA;
     if (rc == RIFT_OK)
-        h->launches += launched;
+        h->launches += launched + 2;
     for (void *q : tmp)
         cudaFreeAsync(q, h->stream);
     if (rc != RIFT_OK) {

@@ -49,11 +49,26 @@ struct FftPlan {
     int L;
     double f0;
     const int *nidx;
-    double2 *X, *Y, *T;
+    double2 *X, *Y, *T;   // (Y: the radix-2 transform only)
+    int *jidx;            // [L] (the pruned transform only)
 };
+// Whether a length-L transform of which n_q outputs are needed runs pruned, as R = L / P
+// transforms of length P.
+bool fft_pruned(int L, int n_q, int *P = nullptr, int *R = nullptr);
+// Checks of the frequency-domain inputs, on the device.
+constexpr int kWaveformInvalid = 1, kWaveformNonFinite = 2;
+struct WaveformInfo {
+    unsigned long long bad;   // first violation (see waveform_check_kernel), ~0: none
+    double f0;
+    int L;                    // lattice length, 0: not on a lattice
+    int unused;
+};
+cudaError_t launch_waveform_check(const double *f, const double *w, int K, int F, double fs, int *nidx,
+                                  WaveformInfo *info, cudaStream_t st);
+size_t uv_scratch_doubles(int K, int M, int F);
 cudaError_t launch_precompute(const double2 *h, const double2 *d, const double *w, const double *f, int K, int M,
-                              int F, const double *q_t0_dev, double fs, int n_q, double2 *A_scratch, double2 *Q,
-                              double2 *U, double2 *V, cudaStream_t st, const FftPlan *fft = nullptr,
+                              int F, const double *q_t0_dev, double fs, int n_q, double2 *A_scratch, double *uv_scratch,
+                              double2 *Q, double2 *U, double2 *V, cudaStream_t st, const FftPlan *fft = nullptr,
                               int *launched = nullptr);
 
 // Fair draws (k_fair.cu): fixed-point weights of lnw (max from stats[slot]), their

@@ -14,9 +14,15 @@
 //   exp(2 pi i f_j t_s) = exp(2 pi i f_j q_t0) exp(2 pi i f_0 s / f_s) exp(2 pi i n_j s / L),
 // so Q_k,lm(t_s) = exp(2 pi i f_0 s / f_s) Y[s mod L], Y the length-L transform (sign +)
 // of X[n_j] = A_j exp(2 pi i f_j q_t0): O(L log L) per (detector, mode) instead of
-// O(n_q F).  The transform is a radix-2 Stockham (self-sorting) FFT, one kernel per
-// stage over every (detector, mode) sequence at once, twiddles exp(2 pi i e / L) from a
-// table.  Grids off a lattice (or with L not a power of two) take the direct sum.
+// O(n_q F).  Only the outputs s < n_q are needed: with P the power of two >= n_q (at most L)
+// and R = L / P,
+//   Y[s] = sum_r exp(2 pi i r s / L) Z_r[s mod P],  Z_r the length-P transform of X[R m + r],
+// so one block per (detector, mode, r) runs a radix-4 Stockham (self-sorting) FFT in shared
+// memory, reading h and the data products directly, and a second kernel sums the R terms of
+// each output.  The float64 pipe bounds both (a 4 s segment at 4096 Hz, 3 detectors, 21 modes:
+// ~50e6 operations of two a clock and SM).  Longer outputs or larger R take a radix-2 transform,
+// one kernel per stage over every sequence at once; grids off a lattice (or with L not a power
+// of two) the direct sum.
 #include <algorithm>
 #include <cmath>
 
@@ -87,49 +93,121 @@ __global__ void __launch_bounds__(kPcThreads) q_series_kernel(const double2 *__r
     }
 }
 
-// One warp per (detector, pair a <= b): U and V, mirrored.
-__global__ void uv_kernel(const double2 *__restrict__ h, const double *__restrict__ w, int K, int M, int F,
-                          double2 *__restrict__ U, double2 *__restrict__ V)
+// U and V of every pair a <= b, mirrored.  Eight float64 multiply-adds a pair and frequency: the
+// float64 pipe (two a clock and SM) bounds it, so the frequencies are split over two blocks per
+// SM, a block stages tiles of 32 frequencies of h(f), h(-f) and 2 w h(f) in shared memory, and a
+// thread owns one pair (several when there are more pairs than threads; a share of the tile's
+// frequencies when there are few).  Partial sums of the blocks are added in their order.  One
+// warp per pair with all loads from L2, a few warps per SM, took 461 us for 3 detectors, 21 modes
+// and 16384 frequencies.
+constexpr int kUvThreads = 256;
+constexpr int kUvTile = 32;
+constexpr int kUvPer = (kMaxModes * (kMaxModes + 1) / 2 + kUvThreads - 1) / kUvThreads;   // pairs per thread
+
+__device__ __forceinline__ void uv_pair(int p, int M, int &a, int &b)
 {
-    const int lane = threadIdx.x & 31;
-    const int pairs = M * (M + 1) / 2;
-    const int64_t total = (int64_t)K * pairs;
-    const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-    for (int64_t e = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); e < total; e += warps) {
-        const int k = (int)(e / pairs);
-        int p = (int)(e % pairs), a = 0;
-        while (p >= M - a) {   // pair index -> (a, b), a <= b
-            p -= M - a;
-            ++a;
-        }
-        const int b = a + p;
-        double ur = 0, ui = 0, vr = 0, vi = 0;
-        for (int j = lane; j < F; j += 32) {
-            const double wj = 2.0 * w[(size_t)k * F + j];
-            const double2 ha = h[(size_t)a * F + j], hb = h[(size_t)b * F + j];
-            const double2 hm = h[(size_t)a * F + (F - 1 - j)];   // h_a(-f_j)
-            ur += wj * (ha.x * hb.x + ha.y * hb.y);
-            ui += wj * (ha.x * hb.y - ha.y * hb.x);
-            vr += wj * (hm.x * hb.x - hm.y * hb.y);
-            vi += wj * (hm.x * hb.y + hm.y * hb.x);
-        }
-#pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            ur += __shfl_xor_sync(0xffffffffu, ur, o);
-            ui += __shfl_xor_sync(0xffffffffu, ui, o);
-            vr += __shfl_xor_sync(0xffffffffu, vr, o);
-            vi += __shfl_xor_sync(0xffffffffu, vi, o);
-        }
-        if (a == b)
-            ui = 0.0;   // w |h|^2 is real (the fused products leave a rounding residual)
-        if (lane == 0) {
-            const size_t ab = ((size_t)k * M + a) * M + b, ba = ((size_t)k * M + b) * M + a;
-            U[ab] = make_double2(ur, ui);
-            U[ba] = make_double2(ur, -ui);
-            V[ab] = make_double2(vr, vi);
-            V[ba] = make_double2(vr, vi);
-        }
+    a = 0;
+    while (p >= M - a) {   // pair index -> (a, b), a <= b
+        p -= M - a;
+        ++a;
     }
+    b = a + p;
+}
+
+__global__ void __launch_bounds__(kUvThreads) uv_partial_kernel(const double2 *__restrict__ h,
+                                                                const double *__restrict__ w, int M, int F,
+                                                                double *__restrict__ part)
+{
+    extern __shared__ double2 uvs[];
+    double2 *hp = uvs, *hm = hp + kUvTile * M, *hw = hm + kUvTile * M;   // [kUvTile][M]
+    const int k = blockIdx.y, pairs = M * (M + 1) / 2;
+    const int groups = pairs < kUvThreads ? kUvThreads / pairs : 1;      // threads per pair
+    const int g = pairs < kUvThreads ? threadIdx.x / pairs : 0;
+    const int p0 = pairs < kUvThreads ? threadIdx.x - g * pairs : threadIdx.x;
+    const int per = (F + gridDim.x - 1) / gridDim.x;
+    const int j0 = blockIdx.x * per, j1 = min(F, j0 + per);
+    double acc[kUvPer][4];
+    int pa[kUvPer], pb[kUvPer];
+#pragma unroll
+    for (int q = 0; q < kUvPer; ++q) {
+        acc[q][0] = acc[q][1] = acc[q][2] = acc[q][3] = 0.0;
+        const int p = p0 + q * kUvThreads;
+        pa[q] = pb[q] = 0;
+        if (p < pairs && g < groups)
+            uv_pair(p, M, pa[q], pb[q]);
+    }
+    for (int t0 = j0; t0 < j1; t0 += kUvTile) {
+        const int nj = min(kUvTile, j1 - t0);
+        __syncthreads();
+        for (int e = threadIdx.x; e < M * kUvTile; e += kUvThreads) {
+            const int m = e / kUvTile, j = e % kUvTile;
+            if (j < nj) {
+                const double2 v = h[(size_t)m * F + t0 + j];
+                const double s = 2.0 * w[(size_t)k * F + t0 + j];
+                hp[j * M + m] = v;
+                hw[j * M + m] = make_double2(s * v.x, s * v.y);
+                hm[j * M + m] = h[(size_t)m * F + (F - 1 - t0 - j)];   // h(-f)
+            }
+        }
+        __syncthreads();
+        if (g < groups)
+            for (int j = g; j < nj; j += groups)
+#pragma unroll
+                for (int q = 0; q < kUvPer; ++q)
+                    if (p0 + q * kUvThreads < pairs) {
+                        const double2 a = hp[j * M + pa[q]], c = hm[j * M + pa[q]], b = hw[j * M + pb[q]];
+                        acc[q][0] = fma(a.x, b.x, fma(a.y, b.y, acc[q][0]));
+                        acc[q][1] = fma(a.x, b.y, fma(-a.y, b.x, acc[q][1]));
+                        acc[q][2] = fma(c.x, b.x, fma(-c.y, b.y, acc[q][2]));
+                        acc[q][3] = fma(c.x, b.y, fma(c.y, b.x, acc[q][3]));
+                    }
+    }
+    double *out = part + (size_t)(k * gridDim.x + blockIdx.x) * 4 * pairs;   // [4][pairs]
+    if (groups == 1) {
+#pragma unroll
+        for (int q = 0; q < kUvPer; ++q)
+            if (g == 0 && p0 + q * kUvThreads < pairs)
+                for (int c = 0; c < 4; ++c)
+                    out[c * pairs + p0 + q * kUvThreads] = acc[q][c];
+        return;
+    }
+    // the threads of a pair in order
+    __shared__ double red[4][kUvThreads];
+    for (int c = 0; c < 4; ++c)
+        red[c][threadIdx.x] = acc[0][c];
+    __syncthreads();
+    for (int e = threadIdx.x; e < 4 * pairs; e += kUvThreads) {
+        const int c = e / pairs, p = e - c * pairs;
+        double v = 0.0;
+        for (int u = 0; u < groups; ++u)
+            v += red[c][u * pairs + p];
+        out[e] = v;
+    }
+}
+
+__global__ void uv_final_kernel(const double *__restrict__ part, int nch, int M, double2 *__restrict__ U,
+                                double2 *__restrict__ V)
+{
+    const int k = blockIdx.y, pairs = M * (M + 1) / 2;
+    const int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p >= pairs)
+        return;
+    int a, b;
+    uv_pair(p, M, a, b);
+    double v[4] = {0.0, 0.0, 0.0, 0.0};
+    const double *q = part + (size_t)k * nch * 4 * pairs + p;
+#pragma unroll 8
+    for (int c = 0; c < nch; ++c)
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            v[e] += q[(size_t)(4 * c + e) * pairs];
+    if (a == b)
+        v[1] = 0.0;   // w |h|^2 is real (the fused products leave a rounding residual)
+    const size_t ab = ((size_t)k * M + a) * M + b, ba = ((size_t)k * M + b) * M + a;
+    U[ab] = make_double2(v[0], v[1]);
+    U[ba] = make_double2(v[0], -v[1]);
+    V[ab] = make_double2(v[2], v[3]);
+    V[ba] = make_double2(v[2], v[3]);
 }
 
 // ---------------------------------------------------------------- FFT path for Q
@@ -198,21 +276,282 @@ __global__ void fft_extract_kernel(const double2 *__restrict__ Y, int64_t n_seq,
     }
 }
 
-cudaError_t launch_precompute(const double2 *h, const double2 *d, const double *w, const double *f, int K, int M,
-                              int F, const double *q_t0_dev, double fs, int n_q, double2 *A_scratch, double2 *Q,
-                              double2 *U, double2 *V, cudaStream_t st, const FftPlan *fft, int *launched)
+// ---------------------------------------------------------------- pruned transform
+
+constexpr int kFftMaxP = 8192;      // 128 KB of shared memory
+constexpr int kFftMaxR = 64;
+constexpr int kFftMaxThreads = 512;
+constexpr int kFftItems = kFftMaxP / 4 / kFftMaxThreads;   // radix-4 butterflies per thread
+
+bool fft_pruned(int L, int n_q, int *P, int *R)
 {
-    const int64_t nA = (int64_t)K * M * F;
-    int k = 0;
-    qfreq_kernel<<<(int)std::min<int64_t>((nA + 255) / 256, 152 * 8), 256, 0, st>>>(h, d, w, K, M, F, A_scratch);
-    ++k;
-    if (fft) {
-        const int L = fft->L;
-        const int64_t nseq = (int64_t)K * M;
-        cudaError_t e = cudaMemsetAsync(fft->X, 0, sizeof(double2) * (size_t)nseq * L, st);
-        if (e != cudaSuccess)
+    int p = 2;
+    while (p < n_q && p < L)
+        p <<= 1;
+    if (P) {
+        *P = p;
+        *R = L / p;
+    }
+    return p <= kFftMaxP && L / p <= kFftMaxR;
+}
+
+// D[k][j] = 2 w_k(f_j) d_k(f_j) exp(2 pi i f_j q_t0_k), and jidx[n_j] = j (-1 elsewhere)
+__global__ void fft_data_kernel(const double2 *__restrict__ d, const double *__restrict__ w,
+                                const double *__restrict__ f, const int *__restrict__ nidx, int K, int F,
+                                const double *__restrict__ q_t0, double2 *__restrict__ D, int *__restrict__ jidx)
+{
+    const int64_t total = (int64_t)K * F;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int k = (int)(e / F), j = (int)(e - (int64_t)k * F);
+        double sn, cs;
+        sincospi(2.0 * f[j] * q_t0[k], &sn, &cs);
+        const double s = 2.0 * w[e];
+        const double2 v = d[e];
+        D[e] = make_double2(s * (v.x * cs - v.y * sn), s * (v.x * sn + v.y * cs));
+        if (k == 0)
+            jidx[nidx[j]] = j;
+    }
+}
+
+// Z[km][r][.] = length-P transform (sign +) of X[R m + r] = conj(h_m(f_j)) D_k(f_j), j = jidx[R m + r]
+__global__ void __launch_bounds__(kFftMaxThreads) fft_block_kernel(const double2 *__restrict__ h,
+                                                                   const double2 *__restrict__ D,
+                                                                   const int *__restrict__ jidx, int M, int F, int P,
+                                                                   int R, const double2 *__restrict__ T,
+                                                                   double2 *__restrict__ Z)
+{
+    extern __shared__ double2 fx[];
+    const int r = blockIdx.x, km = blockIdx.y, k = km / M, m = km - k * M;
+    const int half = (P * R) >> 1;   // entries of T
+    for (int i = threadIdx.x; i < P; i += blockDim.x) {
+        const int j = jidx[R * i + r];
+        double2 x = make_double2(0.0, 0.0);
+        if (j >= 0) {
+            const double2 a = h[(size_t)m * F + j], b = D[(size_t)k * F + j];
+            x = make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
+        }
+        fx[i] = x;
+    }
+    // exp(2 pi i e / (P R)), e < P R
+    auto tw = [&](int e) {
+        const double2 t = T[e < half ? e : e - half];
+        return e < half ? t : make_double2(-t.x, -t.y);
+    };
+    auto mul = [](double2 a, double2 b) { return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x); };
+    int Ns = 1;
+    double2 v[kFftItems][4];
+    if ((__ffs(P) - 1) & 1) {   // an odd number of factors 2: one radix-2 stage (no twiddles) first
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2 * kFftItems; ++q) {
+            const int j = threadIdx.x + q * blockDim.x;
+            if (j < P / 2) {
+                v[q >> 1][2 * (q & 1)] = fx[j];
+                v[q >> 1][2 * (q & 1) + 1] = fx[j + P / 2];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 2 * kFftItems; ++q) {
+            const int j = threadIdx.x + q * blockDim.x;
+            if (j < P / 2) {
+                const double2 a = v[q >> 1][2 * (q & 1)], b = v[q >> 1][2 * (q & 1) + 1];
+                fx[2 * j] = make_double2(a.x + b.x, a.y + b.y);
+                fx[2 * j + 1] = make_double2(a.x - b.x, a.y - b.y);
+            }
+        }
+        Ns = 2;
+    }
+    const int quarter = P >> 2;
+    for (; Ns < P; Ns <<= 2) {
+        const int step = quarter / Ns * R;   // T index of one unit of kk
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kFftItems; ++q) {
+            const int j = threadIdx.x + q * blockDim.x;
+            if (j < quarter) {
+                const int kk = j & (Ns - 1);
+                v[q][0] = fx[j];
+                v[q][1] = mul(fx[j + quarter], tw(kk * step));
+                v[q][2] = mul(fx[j + 2 * quarter], tw(2 * kk * step));
+                v[q][3] = mul(fx[j + 3 * quarter], tw(3 * kk * step));
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kFftItems; ++q) {
+            const int j = threadIdx.x + q * blockDim.x;
+            if (j < quarter) {
+                const int o = (j & ~(Ns - 1)) * 4 + (j & (Ns - 1));
+                const double2 s02 = make_double2(v[q][0].x + v[q][2].x, v[q][0].y + v[q][2].y);
+                const double2 d02 = make_double2(v[q][0].x - v[q][2].x, v[q][0].y - v[q][2].y);
+                const double2 s13 = make_double2(v[q][1].x + v[q][3].x, v[q][1].y + v[q][3].y);
+                const double2 d13 = make_double2(v[q][1].x - v[q][3].x, v[q][1].y - v[q][3].y);
+                fx[o] = make_double2(s02.x + s13.x, s02.y + s13.y);
+                fx[o + Ns] = make_double2(d02.x - d13.y, d02.y + d13.x);       // + i d13
+                fx[o + 2 * Ns] = make_double2(s02.x - s13.x, s02.y - s13.y);
+                fx[o + 3 * Ns] = make_double2(d02.x + d13.y, d02.y - d13.x);   // - i d13
+            }
+        }
+    }
+    __syncthreads();
+    double2 *out = Z + ((size_t)km * R + r) * P;
+    for (int i = threadIdx.x; i < P; i += blockDim.x)
+        out[i] = fx[i];
+}
+
+// Q[km][s] = exp(2 pi i f_0 s / f_s) sum_r exp(2 pi i r s / L) Z[km][r][s mod P]
+__global__ void fft_combine_kernel(const double2 *__restrict__ Z, int KM, int P, int R, const double2 *__restrict__ T,
+                                   double f0, double fs, int n_q, double2 *__restrict__ Q)
+{
+    const int L = P * R, half = L >> 1;
+    for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n_q; s += gridDim.x * blockDim.x) {
+        const int km = blockIdx.y, sl = s & (L - 1);
+        const double2 *z = Z + (size_t)km * R * P + (sl & (P - 1));
+        double re = z[0].x, im = z[0].y;
+#pragma unroll 4
+        for (int r = 1; r < R; ++r) {
+            const int e = (int)(((int64_t)r * sl) & (L - 1));
+            double2 t = T[e < half ? e : e - half];
+            if (e >= half)
+                t = make_double2(-t.x, -t.y);
+            const double2 v = z[(size_t)r * P];
+            re += v.x * t.x - v.y * t.y;
+            im += v.x * t.y + v.y * t.x;
+        }
+        double sn, cs;
+        sincospi(2.0 * f0 * ((double)s / fs), &sn, &cs);
+        Q[(size_t)km * n_q + s] = make_double2(re * cs - im * sn, re * sn + im * cs);
+    }
+}
+
+// ---------------------------------------------------------------- input checks
+
+// Weights finite, non-negative and symmetric in f, frequencies finite and mirror-symmetric:
+// the first violation in the order of a loop over j, then the frequency, then the detectors, as
+// 4 (j (K + 1) + [0 frequency, 1 + k weights]) + code.
+__global__ void waveform_check_kernel(const double *__restrict__ f, const double *__restrict__ w, int K, int F,
+                                      WaveformInfo *__restrict__ info)
+{
+    unsigned long long bad = ~0ull;
+    const int64_t total = (int64_t)(K + 1) * F;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+        const int c = (int)(e / F), j = (int)(e - (int64_t)c * F);
+        const double *row = c == 0 ? f : w + (size_t)(c - 1) * F;
+        const double a = row[j], b = row[F - 1 - j];
+        int code = 0;
+        if (c == 0)
+            code = !isfinite(a) || b != -a ? kWaveformInvalid : 0;
+        else
+            code = !isfinite(a) ? kWaveformNonFinite : a < 0.0 || a != b ? kWaveformInvalid : 0;
+        if (code)
+            bad = min(bad, 4ull * ((unsigned long long)j * (K + 1) + c) + code);
+    }
+    if (bad != ~0ull)
+        atomicMin(&info->bad, bad);
+}
+
+// One block: the lattice f_j = f_0 + n_j df (df the smallest step; ascending frequencies, integers
+// n_j to 1e-9 relative, L = f_s / df a power of two above every n_j); n_j to nidx, L to info (0:
+// not on a lattice).
+__global__ void __launch_bounds__(1024) waveform_lattice_kernel(const double *__restrict__ f, int F, double fs,
+                                                                int *__restrict__ nidx, WaveformInfo *__restrict__ info)
+{
+    __shared__ unsigned long long gap_s, fmax_s;   // non-negative doubles order like their bits
+    __shared__ int off_s;
+    if (threadIdx.x == 0) {
+        gap_s = ~0ull;
+        fmax_s = 0ull;
+        off_s = 0;
+    }
+    __syncthreads();
+    unsigned long long gap = ~0ull, fm = 0ull;
+    bool off = false;
+    for (int j = threadIdx.x; j < F; j += blockDim.x) {
+        fm = max(fm, (unsigned long long)__double_as_longlong(fabs(f[j])));
+        if (j > 0) {
+            const double g = f[j] - f[j - 1];
+            if (g > 0.0)
+                gap = min(gap, (unsigned long long)__double_as_longlong(g));
+            else
+                off = true;
+        }
+    }
+    atomicMin(&gap_s, gap);
+    atomicMax(&fmax_s, fm);
+    if (off)
+        off_s = 1;
+    __syncthreads();
+    const double df = __longlong_as_double((long long)gap_s), fmax = __longlong_as_double((long long)fmax_s);
+    const double Lr = off_s ? 0.0 : fs / df;
+    const long long L = Lr < 1e9 ? llround(Lr) : 0;   // (a NaN ratio: 0)
+    if (off_s || L < 2 || L > (1ll << 26) || (L & (L - 1)) != 0 || !(fabs(Lr - (double)L) <= 1e-9 * (double)L))
+        return;
+    off = false;
+    for (int j = threadIdx.x; j < F; j += blockDim.x) {
+        const long long n = llround((f[j] - f[0]) / df);
+        if (fabs(f[j] - f[0] - (double)n * df) > 1e-9 * (fmax > 1.0 ? fmax : 1.0) || n < 0 || n >= L)
+            off = true;
+        else
+            nidx[j] = (int)n;
+    }
+    if (off)
+        off_s = 1;
+    __syncthreads();
+    if (threadIdx.x == 0 && !off_s) {
+        info->L = (int)L;
+        info->f0 = f[0];
+    }
+}
+
+cudaError_t launch_waveform_check(const double *f, const double *w, int K, int F, double fs, int *nidx,
+                                  WaveformInfo *info, cudaStream_t st)
+{
+    cudaError_t e = cudaMemsetAsync(info, 0, sizeof(WaveformInfo), st);
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(&info->bad, 0xff, sizeof(info->bad), st);
+    if (e != cudaSuccess)
+        return e;
+    const int64_t total = (int64_t)(K + 1) * F;
+    waveform_check_kernel<<<(int)std::min<int64_t>((total + 255) / 256, 152 * 8), 256, 0, st>>>(f, w, K, F, info);
+    waveform_lattice_kernel<<<1, 1024, 0, st>>>(f, F, fs, nidx, info);
+    return cudaGetLastError();
+}
+
+static int uv_chunks(int K, int F) { return std::max(1, std::min((F + kUvTile - 1) / kUvTile, 2 * 152 / K)); }
+
+size_t uv_scratch_doubles(int K, int M, int F) { return (size_t)K * uv_chunks(K, F) * 4 * (M * (M + 1) / 2); }
+
+cudaError_t launch_precompute(const double2 *h, const double2 *d, const double *w, const double *f, int K, int M,
+                              int F, const double *q_t0_dev, double fs, int n_q, double2 *A_scratch, double *uv_scratch,
+                              double2 *Q, double2 *U, double2 *V, cudaStream_t st, const FftPlan *fft, int *launched)
+{
+    const int64_t nA = (int64_t)K * M * F, nseq = (int64_t)K * M;
+    int k = 0, P = 0, R = 0;
+    cudaError_t e = cudaSuccess;
+    if (fft)
+        fft_twiddle_kernel<<<std::max(1, std::min(fft->L / 2 / 256, 152 * 8)), 256, 0, st>>>(fft->L, fft->T);
+    if (fft && fft_pruned(fft->L, n_q, &P, &R)) {
+        if ((e = cudaMemsetAsync(fft->jidx, 0xff, sizeof(int) * (size_t)fft->L, st)) != cudaSuccess)
             return e;
-        fft_twiddle_kernel<<<std::max(1, std::min(L / 2 / 256, 152 * 8)), 256, 0, st>>>(L, fft->T);
+        const int64_t nd = (int64_t)K * F;
+        fft_data_kernel<<<(int)std::min<int64_t>((nd + 255) / 256, 152 * 8), 256, 0, st>>>(d, w, f, fft->nidx, K, F,
+                                                                                          q_t0_dev, A_scratch, fft->jidx);
+        const size_t smem = sizeof(double2) * (size_t)P;
+        if (smem > 48 * 1024 && (e = allow_max_dynamic_smem(fft_block_kernel)) != cudaSuccess)
+            return e;
+        // butterflies of a stage spread over up to 512 threads
+        const int threads = std::min(kFftMaxThreads, std::max(32, P / 4));
+        fft_block_kernel<<<dim3(R, (unsigned)nseq), threads, smem, st>>>(h, A_scratch, fft->jidx, M, F, P, R, fft->T,
+                                                                        fft->X);
+        fft_combine_kernel<<<dim3((n_q + 127) / 128, (unsigned)nseq), 128, 0, st>>>(fft->X, (int)nseq, P, R, fft->T,
+                                                                                    fft->f0, fs, n_q, Q);
+        k += 4;
+    } else if (fft) {
+        const int L = fft->L;
+        qfreq_kernel<<<(int)std::min<int64_t>((nA + 255) / 256, 152 * 8), 256, 0, st>>>(h, d, w, K, M, F, A_scratch);
+        if ((e = cudaMemsetAsync(fft->X, 0, sizeof(double2) * (size_t)nseq * L, st)) != cudaSuccess)
+            return e;
         fft_scatter_kernel<<<(int)std::min<int64_t>((nA + 255) / 256, 152 * 8), 256, 0, st>>>(
             A_scratch, f, fft->nidx, K, M, F, q_t0_dev, L, fft->X);
         double2 *a = fft->X, *b = fft->Y;
@@ -226,16 +565,21 @@ cudaError_t launch_precompute(const double2 *h, const double2 *d, const double *
         const int64_t nqt = nseq * n_q;
         fft_extract_kernel<<<(int)std::min<int64_t>((nqt + 255) / 256, 152 * 8), 256, 0, st>>>(a, nseq, L, fft->f0,
                                                                                               fs, n_q, Q);
-        k += 3;
+        k += 4;
     } else {
+        qfreq_kernel<<<(int)std::min<int64_t>((nA + 255) / 256, 152 * 8), 256, 0, st>>>(h, d, w, K, M, F, A_scratch);
         dim3 grid((n_q + kPcThreads - 1) / kPcThreads, K);
         q_series_kernel<<<grid, kPcThreads, 0, st>>>(A_scratch, f, K, M, F, q_t0_dev, fs, n_q, Q);
-        ++k;
+        k += 2;
     }
-    const int64_t pairs = (int64_t)K * M * (M + 1) / 2;
-    uv_kernel<<<(int)std::min<int64_t>((pairs + 7) / 8, 152 * 8), 256, 0, st>>>(h, w, K, M, F, U, V);
+    const int nch = uv_chunks(K, F), pairs = M * (M + 1) / 2;
+    const size_t uv_smem = sizeof(double2) * 3 * kUvTile * M;
+    if (uv_smem > 40 * 1024 && (e = allow_max_dynamic_smem(uv_partial_kernel)) != cudaSuccess)
+        return e;   // (beside the static array of the pairs' threads)
+    uv_partial_kernel<<<dim3(nch, K), kUvThreads, uv_smem, st>>>(h, w, M, F, uv_scratch);
+    uv_final_kernel<<<dim3((pairs + 63) / 64, K), 64, 0, st>>>(uv_scratch, nch, M, U, V);
     if (launched)
-        *launched = k + 1;
+        *launched = k + 2;
     return cudaGetLastError();
 }
 
