@@ -265,9 +265,28 @@ int sync_and_err(rift_ile_t *h, int *flags_out)
 
 bool use_fp32(const rift_ile_t *h) { return h->cfg.precision != RIFT_FP64; }
 
-// Without a tuned plan: tensor-core tiles pay off once a batch fills the sky densely
-// enough that 128 samples share a 128-column Q window.
-constexpr int64_t kTcMinBatch = 100000;
+// Without a tuned plan: tensor-core tiles pay off from the batch size at which they overtake the
+// CUDA-core kernel (which takes any spread of delays at the same cost): 10,000 samples with one
+// detector, 16,000 with more, and with three detectors, whose sort key is the sky position, once
+// a tile of the sorted batch spans about one window of 64 columns (256 samples per patch of that
+// size on the delays' surface).  Measured (us, CUDA cores | tensor cores): 2 detectors, 9 modes,
+// 16384 Hz, 10,000 samples 272 | 347, 30,000 457 | 333; 3 detectors, 21 modes, 16384 Hz, 20,000
+// samples 639 | 761, 30,000 847 | 793; 3 detectors, 9 modes, 4096 Hz, 10,000 samples 256 | 330,
+// 20,000 331 | 303; 1 detector, 2 modes, 10,000 samples 182 | 181.
+int64_t tc_min_batch(const rift_ile_t *h)
+{
+    const Problem &P = h->prob;
+    if (P.K == 1)
+        return 10000;
+    double span = 0.0;
+    for (int k = 0; P.K >= 3 && k < P.K; ++k) {
+        double r2 = 0.0;
+        for (int i = 0; i < 3; ++i)
+            r2 += P.xpos[k][i] * P.xpos[k][i];
+        span = std::max(span, 2.0 * std::sqrt(r2) * P.fs / 64.0);
+    }
+    return (int64_t)std::min(1e6, std::max(16000.0, 256.0 * span * span));
+}
 
 bool use_tc(const rift_ile_t *h, int64_t n)
 {
@@ -275,7 +294,19 @@ bool use_tc(const rift_ile_t *h, int64_t n)
         return false;
     if (h->tc_mode == 1)
         return true;
-    return h->plan.tc >= 0 ? h->plan.tc == 1 : n >= kTcMinBatch;
+    return h->plan.tc >= 0 ? h->plan.tc == 1 : n >= tc_min_batch(h);
+}
+
+// Below this many samples the CUDA-core kernel takes them in index order: their windows'
+// union costs less than the sort.
+constexpr int64_t kCoreUnsorted = 1024;
+
+bool sorts_batch(const rift_ile_t *h, int64_t n) { return use_tc(h, n) || n > kCoreUnsorted; }
+
+cudaError_t sort_batch(rift_ile_t *h, int64_t n, int *launched)
+{
+    *launched = 0;
+    return sorts_batch(h, n) ? launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, h->stream, launched) : cudaSuccess;
 }
 
 cudaError_t launch_tiled(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg, double *lnL_t,
@@ -294,8 +325,8 @@ cudaError_t launch_tiled(rift_ile_t *h, const double *theta, int64_t n, double *
     cudaError_t e = tc ? launch_lnl_tc(h->prob, bt, theta, h->perm, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err,
                                        TcUnits{h->tc_unit_list, h->tc_unit_cap, h->tile_counter}, h->stream,
                                        nullptr, 0, 0, po)
-                       : launch_lnl_fp32(h->prob, bt, theta, h->perm, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err,
-                                         h->tile_counter, h->stream, po);
+                       : launch_lnl_fp32(h->prob, bt, theta, sorts_batch(h, n) ? h->perm : nullptr, n, lnL_tmarg,
+                                         lnL_t, lnpw, lnw, h->err, h->stream, po);
     if (e != cudaSuccess || !h->fix_on)
         return e;
     // the samples whose float32 terms are large enough for their rounding to reach the
@@ -349,7 +380,7 @@ int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmar
     const double *key = lnw ? lnw : lnL_tmarg;
     CK(launch_reduce(key, lnL_tmarg, n, h->red_partial, h->stats, kScratchSlot, h->pooled_scratch, 1, h->err,
                      h->stream));
-    CK(launch_select(key, h->perm, n, h->stats, kScratchSlot, kMixedMargin, h->sel_idx, h->sel_count, h->stream));
+    CK(launch_select(key, sorts_batch(h, n) ? h->perm : nullptr, n, h->stats, kScratchSlot, kMixedMargin, h->sel_idx, h->sel_count, h->stream));
     if (h->tc64_on) {
         CK(launch_lnl_tc64(h->prob, h->x64, theta, h->sel_idx, n, lnL_tmarg, nullptr, lnpw, lnw, h->err,
                            h->stream, h->sel_count));
@@ -419,9 +450,12 @@ int eval_device(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg
     RK(choose_plan(h, n, false));
     RK(grid_for_batch(h, n));
     int sorted = 0;
-    CK(launch_keys(h->grid, theta, n, h->key, h->stream));
-    CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, h->stream, &sorted));
-    h->launches += 2 + sorted;   // keys, sort, tiled likelihood
+    if (sorts_batch(h, n)) {
+        CK(launch_keys(h->grid, theta, n, h->key, h->stream));
+        CK(sort_batch(h, n, &sorted));
+        ++sorted;
+    }
+    h->launches += 1 + sorted;   // keys, sort, likelihood
     CK(launch_tiled(h, theta, n, lnL_tmarg, lnL_t, lnpw, lnw));
     if (h->cfg.precision == RIFT_MIXED)
         RK(refine_batch(h, theta, n, lnL_tmarg, lnpw, lnw));
@@ -438,7 +472,7 @@ int run_iteration(rift_ile_t *h, int64_t n, int slot, bool adapt, bool reset_poo
     CK(launch_draw(S, h->grid, h->iter_dev, (uint32_t)slot, n, h->theta, h->lnpw, h->bins, h->key, h->stream));
     int sorted = 0;
     if (use_fp32(h))
-        CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, h->stream, &sorted));
+        CK(sort_batch(h, n, &sorted));
     CK(mark(h, slot, 1));
     if (!use_fp32(h)) {
         RK(lnl_float64(h, h->theta, n, true, h->lnL, nullptr, h->lnpw, h->lnw));

@@ -294,9 +294,11 @@ int av_iteration(rift_ile_t *h, int64_t n, int slot, bool reset_pooled, double p
     int sorted = 0;
     if (use_fp32(h)) {
         RK(grid_for_batch(h, n));
-        CK(launch_keys(h->grid, h->theta, n, h->key, st));
-        CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, st, &sorted));
-        sorted += 1;
+        if (sorts_batch(h, n)) {
+            CK(launch_keys(h->grid, h->theta, n, h->key, st));
+            CK(sort_batch(h, n, &sorted));
+            sorted += 1;
+        }
     }
     CK(mark(h, slot, 1));
     // 2. likelihood

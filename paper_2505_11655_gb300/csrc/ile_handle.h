@@ -182,6 +182,9 @@ int collect_result(rift_ile_t *h, int n_iter, rift_ile_result *out);
 int choose_plan(rift_ile_t *h, int64_t n, bool measure = true);
 bool use_tc(const rift_ile_t *h, int64_t n);
 int grid_for_batch(rift_ile_t *h, int64_t n);
+// whether a batch of the float32 modes is sorted, and the sort of h->key into h->perm if so
+bool sorts_batch(const rift_ile_t *h, int64_t n);
+cudaError_t sort_batch(rift_ile_t *h, int64_t n, int *launched);
 cudaError_t launch_tiled(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg, double *lnL_t,
                          const double *lnpw, double *lnw);
 void drop_graph(rift_ile_t *h);

@@ -137,12 +137,11 @@ cudaError_t launch_fix(const Problem &P, BinTable bt, FixTables T, const double 
                        int blen, float thr, uint32_t *idx, uint32_t *count, double *lnL_tmarg, double *lnL_t,
                        const double *lnpw, double *lnw, int *err, cudaStream_t st, int *launched);
 
-// Float32 tiled path.  perm[n] lists sample indices in sky-cell order; outputs are
-// written at the original index.  tile_counter: one device int (reset by the launcher).
+// Float32 path on the CUDA cores.  perm[n] lists sample indices in sky-cell order (null: index
+// order); outputs are written at the original index.
 cudaError_t launch_lnl_fp32(const Problem &P, BinTable bt, const double *theta, const uint32_t *perm, int64_t n,
                             double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
-                            int *tile_counter, cudaStream_t st, PeakOut po = PeakOut());
-size_t lnl_fp32_smem_bytes(const Problem &P);
+                            cudaStream_t st, PeakOut po = PeakOut());
 
 // Tensor-core variant of the float32 tiled path (tiles of 128 samples, tcgen05 MMA).
 bool lnl_tc_fits(const Problem &P, int max_smem);

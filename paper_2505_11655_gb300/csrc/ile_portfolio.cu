@@ -664,7 +664,7 @@ int portfolio_iteration(rift_ile_t *h, int64_t n, int slot, bool reset_pooled, c
     CK(cudaGetLastError());
     int sorted = 0;
     if (use_fp32(h))
-        CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, st, &sorted));
+        CK(sort_batch(h, n, &sorted));
     CK(mark(h, slot, 1));
     // 2. likelihood and the iteration's record
     if (!use_fp32(h)) {

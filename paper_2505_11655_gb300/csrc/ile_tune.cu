@@ -101,8 +101,9 @@ int time_plan(rift_ile_t *h, int64_t n, const LaunchPlan &p, cudaEvent_t e0, cud
     float best = INFINITY;
     for (int rep = 0; rep < 2; ++rep) {
         CK(cudaEventRecord(e0, h->stream));
+        int sorted = 0;
         CK(launch_keys(h->grid, h->theta, n, h->key, h->stream));
-        CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, h->stream));
+        CK(sort_batch(h, n, &sorted));
         CK(launch_tiled(h, h->theta, n, h->lnL, nullptr, nullptr, nullptr));
         CK(cudaEventRecord(e1, h->stream));
         CK(cudaEventSynchronize(e1));

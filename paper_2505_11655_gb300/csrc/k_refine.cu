@@ -22,8 +22,8 @@ namespace rift {
 constexpr int kRefThreads = 128;   // 4 warps, one sample each
 constexpr double kRefineBins = 40.0;
 
-// Selection of the samples with key[perm[i]] >= max - margin, in the order of perm (the
-// sky sort, which is stable, so the list, and everything computed from it, is the same from
+// Selection of the samples with key[perm[i]] >= max - margin, in the order of perm (index
+// order when null; the sky sort, which is stable, so the list, and everything computed from it, is the same from
 // run to run): block b of the grid owns the contiguous range [b per, (b + 1) per) of perm;
 // pass 1 counts per block, a single block scans the counts, pass 2 writes each block's
 // matches at its offset in order.  In the sort's order neighbours of the list keep close
@@ -43,7 +43,7 @@ __global__ void __launch_bounds__(kSelThreads) select_count_kernel(const double 
     const int64_t b0 = (int64_t)blockIdx.x * per, b1 = min(n, b0 + per);
     uint32_t c = 0;
     for (int64_t i = b0 + threadIdx.x; i < b1; i += kSelThreads)
-        c += key[perm[i]] >= cut ? 1u : 0u;
+        c += key[perm ? perm[i] : i] >= cut ? 1u : 0u;
     c = __reduce_add_sync(0xffffffffu, c);
     __shared__ uint32_t ws[kSelThreads / 32];
     if ((threadIdx.x & 31) == 0)
@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(kSelThreads) select_write_kernel(const double 
     uint32_t base = blk[blockIdx.x];
     for (int64_t c0 = b0; c0 < b1; c0 += kSelThreads) {
         const int64_t i = c0 + threadIdx.x;
-        const uint32_t g = i < b1 ? perm[i] : 0u;
+        const uint32_t g = i < b1 ? (perm ? perm[i] : (uint32_t)i) : 0u;
         const bool take = i < b1 && key[g] >= cut;
         const unsigned mask = __ballot_sync(0xffffffffu, take);
         if (lane == 0)
