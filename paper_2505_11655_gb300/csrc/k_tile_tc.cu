@@ -13,9 +13,14 @@
 //     one TMA bulk copy per part into a double buffer;
 //   * one thread issues 3 (Kp/16) tcgen05.mma.kind::f16 (M=128, N=128, K=16) into one
 //     of two TMEM accumulators (128 columns each) and commits to an mbarrier;
-//   * the block drains the accumulator with tcgen05.ld (warp quarter = 32 rows),
-//     rescales, stores R to shared memory and gathers the two interpolation nodes of
-//     every bin, while the next step's MMAs run.
+//   * the consumer warps drain the accumulator with tcgen05.ld (warp quarter = 32 rows) to
+//     shared memory and gather the two interpolation nodes of every bin.  The four warps of a
+//     lane quarter (they share an SM sub-partition) form two pairs; each pair owns one
+//     accumulator, one window buffer and one R tile and takes every other chunk of time bins, so
+//     that one pair drains while the other gathers and the MMAs of a third step run.  With all
+//     four warps on the same step the sub-partition's warps were in the same phase, and the
+//     scheduler issued in half of its cycles (250,000 samples, 3 detectors, 21 modes, 1001 bins
+//     at 16384 Hz: 1.43 ms, now 1.26 ms; the shared-memory pipe is 60% busy).
 // All waits are bounded (1 s by the global timer); a timeout raises kErrTimeout, the
 // block abandons its tiles, frees its tensor memory and returns.
 #include <cfloat>
@@ -33,9 +38,10 @@ constexpr int kTcConsumers = 512;  // 16 consumer warps: drain, gather, log-sum-
 constexpr int kTcThreads = kTcConsumers + 64;   // plus an MMA-issue warp and a TMA-staging warp
 constexpr int kTcIssuerWarp = kTcConsumers / 32;
 constexpr int kTcStagerWarp = kTcIssuerWarp + 1;
-constexpr int kTcQ = kTcConsumers / kTcS;  // threads per sample in the gather (bin quarters)
-constexpr int kTcBPT = 16;         // bins per thread per chunk
-constexpr int kTcMaxBins = kTcQ * kTcBPT;
+constexpr int kTcQ = kTcConsumers / kTcS;  // threads per sample: (pair, half of a chunk's bins)
+constexpr int kTcBPT = 32;         // bins per thread per chunk
+constexpr int kTcMaxBins = 2 * kTcBPT;
+constexpr int kTcPairThreads = 64;
 constexpr int kTcFrac = 24;        // fraction bits of a node position in the R tile
 // phases B and E give every (sample, detector) item its own consumer thread, whole warps
 // per detector
@@ -59,7 +65,7 @@ __device__ __forceinline__ float ex2_approx(float x)
 constexpr int kTcSpreadLimit = 64;
 
 struct TcLayout {
-    size_t b, r, r2, tt, bins, i0, f0, inv, qsc, gid, lse, bar, tptr, end;
+    size_t b, r, r2, tt, bins, bini, i0, f0, inv, qsc, gid, lse, bar, tptr, end;
     size_t sky, e5, par, pw, pe, fx;   // prologue scratch, aliased on the B buffers
     int kp;
 };
@@ -89,15 +95,17 @@ __host__ __device__ inline TcLayout tc_layout(int K, int M, int n_t)
     L.tt = tc_al(L.r + (size_t)M * kTcS * 8);
     const size_t rbytes = (size_t)kTcW * kTcS * 4, pbytes = L.tt - L.r + (size_t)K * 2 * L.kp * L.kp * 2;
     o = tc_al(o + (rbytes > pbytes ? rbytes : pbytes));
-    L.r2 = o;   // second R tile: steps alternate between the two
+    L.r2 = o;   // second R tile: one per pair of warps
     o = tc_al(o + rbytes, 16);
-    L.bins = o; o = tc_al(o + (size_t)n_t * 8, 16);   // (integer offset, fraction) per bin
+    L.bins = o; o = tc_al(o + (size_t)n_t * 4, 16);                   // node position per bin
+    o = tc_al(o + (size_t)kTcBPT * 4, 16);
+    L.bini = o; o = tc_al(o + (size_t)n_t * 4, 16);                   // its integer part
     L.i0 = o;   o = tc_al(o + (size_t)K * kTcS * 4, 16);
     L.f0 = o;   o = tc_al(o + (size_t)K * kTcS * 4, 16);
     L.inv = o;  o = tc_al(o + (size_t)K * kTcS * 4, 16);
     L.qsc = o;  o = tc_al(o + (size_t)K * kTcS * 4, 16);
     L.gid = o;  o = tc_al(o + (size_t)kTcS * 4, 16);
-    L.lse = o;  o = tc_al(o + (size_t)(2 * kTcQ + 2) * kTcS * 4, 16);
+    L.lse = o;  o = tc_al(o + (size_t)3 * kTcQ * kTcS * 4, 16);
     L.bar = o;  o = tc_al(o + 8 * 8, 16);
     L.tptr = o; o = tc_al(o + 16, 16);
     L.end = o;
@@ -401,8 +409,10 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
     const int kp = L.kp, kcores = kp / 8;
     __half *Bs = reinterpret_cast<__half *>(sm + L.b);          // [2 buf][2 part][kTcW x kp]
     float *Rs = reinterpret_cast<float *>(sm + L.r);            // Rt [kTcW][kTcS] (prologue: Y [M][kTcS])
-    float *Rs2 = reinterpret_cast<float *>(sm + L.r2);          // Rt of the odd steps
-    int2 *bins = reinterpret_cast<int2 *>(sm + L.bins);          // per bin: bin_i, (bin_i + bin_f) 2^24 mod 2^32
+    float *Rs2 = reinterpret_cast<float *>(sm + L.r2);          // Rt of the odd pair
+    // [NT + kTcBPT] (bin_i + bin_f) 2^24 mod 2^32 (zero behind the last bin), [NT] bin_i
+    uint32_t *bins = reinterpret_cast<uint32_t *>(sm + L.bins);
+    int *bini = reinterpret_cast<int *>(sm + L.bini);
     int *i0s = reinterpret_cast<int *>(sm + L.i0);              // [K][kTcS]
     uint32_t *f0s = reinterpret_cast<uint32_t *>(sm + L.f0);    // [K][kTcS] fraction of the first node, 2^-24
     float *invs = reinterpret_cast<float *>(sm + L.inv);        // [K][kTcS] 2^-(row exponent + Q exponent)
@@ -410,7 +420,7 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
     uint32_t *gid = reinterpret_cast<uint32_t *>(sm + L.gid);
     uint64_t *bbar = reinterpret_cast<uint64_t *>(sm + L.bar);  // [0,1] windows staged
     uint64_t *fullb = bbar + 2;   // [0,1] MMAs of an accumulator complete (tcgen05.commit)
-    uint64_t *emptyb = bbar + 4;  // [0,1] accumulator drained by the 16 consumer warps
+    uint64_t *emptyb = bbar + 4;  // [0,1] accumulator drained by its pair's 8 warps
     uint64_t *tbar = bbar + 6;    // template matrices staged (once per tile)
     uint64_t *wbar = bbar + 7;    // template products W = Z T complete (once per tile)
     uint32_t *tptr = reinterpret_cast<uint32_t *>(sm + L.tptr);
@@ -420,11 +430,8 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
     float *pw = reinterpret_cast<float *>(sm + L.pw);          // [2 kTcPow][kTcS] cos^q, sin^q (iota/2)
     float2 *pe = reinterpret_cast<float2 *>(sm + L.pe);        // [kMaxL + 1][kTcS] exp(-i j phi)
     float2 *fx = reinterpret_cast<float2 *>(sm + L.fx);        // [K][kTcS] (D_ref/D) F_k
-    float *lse = reinterpret_cast<float *>(sm + L.lse);         // [2][kTcQ][kTcS] running max, sum
-    // [kTcS] per sample: the largest data term over its bins (order-preserving bits, high
-    // word) and the first bin of the block of bins holding it (NT - bin, low word, so that
-    // the lowest bin wins among equals), by one 64-bit shared atomic max per chunk and thread
-    unsigned long long *peak = reinterpret_cast<unsigned long long *>(lse + 2 * kTcQ * kTcS);
+    float *lse = reinterpret_cast<float *>(sm + L.lse);         // [2][kTcQ][kTcS] running max, sum; then peak
+    int *peak = reinterpret_cast<int *>(lse + 2 * kTcQ * kTcS); // [kTcQ][kTcS] block of bins holding the running max
     float *qsum = lse;                                          // [kTcQ][kTcS] template term partials
     float2 *Ys = reinterpret_cast<float2 *>(Rs);               // [M][kTcS] -2Y_lm(iota, -phi)
     __shared__ int lo_s[kMaxDet], hi_s[kMaxDet];        // current sub-group's offset range
@@ -453,9 +460,11 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
     // components per column) of detector k, part p at 256 + (2 k + p) kp / 2
     auto a_col = [&](int k, int part) { return 256u + (uint32_t)((2 * k + part) * (kp / 2)); };
 
-    for (int j = tid; j < NT; j += blockDim.x) {
-        const int bi = bt.bin_i[j];
-        bins[j] = make_int2(bi, (int)(((uint32_t)bi << kTcFrac) + __float2uint_rn(bt.bin_f[j] * 0x1p24f)));
+    for (int j = tid; j < NT + kTcBPT; j += blockDim.x) {
+        const int bi = j < NT ? bt.bin_i[j] : 0;
+        bins[j] = j < NT ? ((uint32_t)bi << kTcFrac) + __float2uint_rn(bt.bin_f[j] * 0x1p24f) : 0u;
+        if (j < NT)
+            bini[j] = bi;
     }
     // the nodes read for the bins j0 .. j0 + jmax - 1 lie within (jmax - 1) beta + 3 columns of
     // a sample's first node; with the spread of the sub-group's offsets and up to 7 columns of
@@ -470,7 +479,7 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
         for (int i = 0; i < 4; ++i)
             tc::mbar_init(bbar + i, 1);
         for (int i = 4; i < 6; ++i)
-            tc::mbar_init(bbar + i, kTcConsumers / 32);
+            tc::mbar_init(bbar + i, kTcConsumers / 64);
         tc::mbar_init(tbar, 1);
         tc::mbar_init(wbar, 1);
         tc::fence_mbar_init();
@@ -532,7 +541,6 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
             uint32_t g = in_unit && si < n_use ? perm[si] : 0xffffffffu;
             const bool valid = (int64_t)g < n_theta;
             gid[tid] = valid ? g : 0xffffffffu;
-            peak[tid] = 0ull;
             double th[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 1.0};
             if (valid)
                 for (int d = 0; d < 6; ++d)
@@ -713,8 +721,9 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
         tc::fence_proxy_async_smem();
         __syncthreads();
 
-        // gather / fold ownership: thread -> sample s, bin quarter h of every chunk
-        const int gs = tid & (kTcS - 1), gh = (tid >> 7) & (kTcQ - 1);
+        // gather / fold ownership: thread -> sample gs, pair pb (chunks pb, pb + 2, ...), half hh
+        // of a chunk's bins
+        const int gs = tid & (kTcS - 1), gh = (tid >> 7) & (kTcQ - 1), pb = gh & 1, hh = gh >> 1;
         const bool gok = !producer && gid[gs] != 0xffffffffu;
 
         // ---------------- D: template term on the tensor cores.  W_k = Z_k T_k (Z_k: the A
@@ -786,6 +795,7 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
         const float gqd =
             (float)P.kappa * ((qsum[gs] + qsum[kTcS + gs]) + (qsum[2 * kTcS + gs] + qsum[3 * kTcS + gs]));
         float run_mx = -INFINITY, run_sum = 0.f;
+        int run_j = 0;
         const int ngroups = ngroups_s;
         for (int grp = 0; grp < ngroups && !failed; ++grp) {
             int spread = 0;
@@ -797,28 +807,31 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
             int jmax = spread <= kTcSpreadLimit ? jmax_s[spread]
                                                 : (!(beta > 0.0) ? kTcMaxBins : (int)floor((double)(kTcW - 11 - spread) / beta) + 1);
             jmax = max(1, min(jmax, kTcMaxBins));
-            const int n_chunks = (NT + jmax - 1) / jmax;
-            const int jnom = (NT + n_chunks - 1) / n_chunks;
-            const int n_steps = n_chunks * K;
-            // Step t covers detector t % K and the bins of chunk t / K (both tracked as
-            // counters).  First Q column of the window of detector k for the chunk starting at
-            // bin j0, clamped so that a window never leaves the allocation of the Q copy.
+            // as many chunks for one pair as for the other, of a multiple of 8 bins (the halves'
+            // bins are then read four at a time)
+            int n_chunks = (NT + jmax - 1) / jmax;
+            n_chunks += n_chunks > 1 ? n_chunks & 1 : 0;
+            int jnom = (NT + n_chunks - 1) / n_chunks;
+            if (((jnom + 7) & ~7) <= jmax)
+                jnom = (jnom + 7) & ~7;
+            n_chunks = (NT + jnom - 1) / jnom;
+            // Steps: (chunk, detector), the two chunks of the pairs in turn; chunk ch uses
+            // buffers ch & 1.  First Q column of the window of detector k for the chunk starting
+            // at bin j0, clamped so that a window never leaves the allocation of the Q copy.
             auto win0 = [&](int k, int j0) {
-                return min(max(glo[grp][k] + bins[j0].x, 0), 8 * (P.tc_groups - 16)) & ~7;
+                return min(max(glo[grp][k] + bini[j0], 0), 8 * (P.tc_groups - 16)) & ~7;
             };
 
             if (warp == kTcIssuerWarp) {
                 // ============ issuer warp, lane 0: one MMA batch per staged window
                 if (lane == 0) {
                     const uint32_t b_lo0 = desc_lo(Bs), b_part = part_bytes >> 4;
-                    int k = 0;
-                    for (int t = 0; t < n_steps && !failed; ++t, k = k + 1 == K ? 0 : k + 1) {
-                        const int b = t & 1;
-                        // window t staged; accumulator b drained by the consumers
+                    auto step = [&](int k, int b) {
+                        // window staged; accumulator b drained by its pair
                         if (!tc::mbar_wait(bbar + b, phbit(kPhCons, b), kWaitNs) ||
                             (phbit(kPhPend, b) && !tc::mbar_wait(emptyb + b, phbit(kPhDrn, b), kWaitNs))) {
                             failed = 1;
-                            break;
+                            return;
                         }
                         ph ^= 1u << (kPhCons + b);
                         if (phbit(kPhPend, b))
@@ -836,7 +849,13 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                         }
                         tc::mma_commit(fullb + b);
                         ph |= 1u << (kPhPend + b);
-                    }
+                    };
+                    for (int ch = 0; ch < n_chunks && !failed; ch += 2)
+                        for (int k = 0; k < K && !failed; ++k) {
+                            step(k, 0);
+                            if (ch + 1 < n_chunks && !failed)
+                                step(k, 1);
+                        }
                     if (failed)
                         abort_s = 1;
                 }
@@ -848,12 +867,11 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                 // (j - 1)-th completion of fullb[b] (that of the previous group or tile when
                 // this is a group's first window into b).
                 if (lane == 0) {
-                    int sk = 0, sch = 0;   // detector and chunk of the next window
-                    for (int t = 0; t < n_steps && !failed; ++t) {
-                        const int b = t & 1;
+                    auto stage = [&](int sk, int sch) {
+                        const int b = sch & 1;
                         if (phbit(kPhUsed, b) && !tc::mbar_wait(fullb + b, phbit(kPhStg, b) ^ 1u, kWaitNs)) {
                             failed = 1;
-                            break;
+                            return;
                         }
                         const int g0 = win0(sk, sch * jnom) >> 3;
                         const __half *src = P.Qtc + ((size_t)sk * 2 * P.tc_groups + g0) * (size_t)kp * 8;
@@ -863,231 +881,255 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                         tc::bulk_g2s(dst + part_halves, src + (size_t)P.tc_groups * kp * 8, part_bytes, bbar + b);
                         ph ^= 1u << (kPhStg + b);
                         ph |= 1u << (kPhUsed + b);
-                        if (++sk == K) {
-                            sk = 0;
-                            ++sch;
+                    };
+                    for (int ch = 0; ch < n_chunks && !failed; ch += 2)
+                        for (int k = 0; k < K && !failed; ++k) {
+                            stage(k, ch);
+                            if (ch + 1 < n_chunks && !failed)
+                                stage(k, ch + 1);
                         }
-                    }
                     if (failed)
                         abort_s = 1;
                 }
                 __syncwarp();
             } else {
                 // ============ consumer warps: drain, gather, fold
-                float lin[kTcBPT];
-                uint32_t bj[kTcBPT];
-#pragma unroll
-                for (int i = 0; i < kTcBPT; ++i) {
-                    lin[i] = 0.f;
-                    bj[i] = 0u;
-                }
                 // a lane quarter without a sample of the group (its four warps agree) leaves its
                 // rows in tensor memory
                 const bool idle = !__any_sync(0xffffffffu, gok && in_grp);
-                for (int t = 0; idle && t < n_steps; ++t) {
-                    const int b = t & 1;
-                    if (!tc::mbar_wait(fullb + b, phbit(kPhFull, b), kWaitNs))
-                        failed = 1;
-                    ph ^= 1u << (kPhFull + b);
-                    __syncwarp();
-                    tc::mbar_arrive_if(emptyb + b, lane == 0);
-                    if (failed)
-                        break;
-                }
-                for (int t = idle ? n_steps : 0, k = 0, j0 = 0; t < n_steps; ++t) {
-                    const int b = t & 1, J = min(jnom, NT - j0);
-                    const int jq = (J + kTcQ - 1) / kTcQ;                 // bins per quarter
-                    const int jb = j0 + gh * jq, jn = max(0, min(jq, j0 + J - jb));   // this thread's bins
-                    // every lane waits for the MMAs of step t (the same barrier word: no
-                    // divergent branch, no broadcast of the result)
-                    const int ok = tc::mbar_wait(fullb + b, phbit(kPhFull, b), kWaitNs) ? 1 : 0;
-                    ph ^= 1u << (kPhFull + b);
-                    tc::tc_fence_after();
-                    // The rows of sample quarter q (TMEM lanes 32q..) are drained and gathered by
-                    // the same four warps (warp & 3 == q), which synchronise on their own barrier
-                    // once per step, after the drain.  Steps alternate between two R tiles: the
-                    // tile step t drains into was last read by the gathers of step t - 2, which
-                    // every warp of the quarter finished before the barrier of step t - 1.
-                    const int qbar = 2 + (warp & 3);
-                    float *Rt = (t & 1) ? Rs2 : Rs;
-                    // The gather's own loads do not depend on the drain: issued before it, their
-                    // shared-memory latency overlaps the drain.  Padding samples and samples of
-                    // other sub-groups read at the group's lowest offset, which keeps every read
-                    // in the row; their sums are discarded.
-                    const int iw0 = win0(k, j0);
-                    const bool mine = gok && in_grp;
-                    // position of the sample's first node: column (plus 128 in the upper half of the
-                    // tile's samples) in the top byte, fraction below (modulo 2^32)
-                    const uint32_t ub = ((uint32_t)((mine ? i0s[k * kTcS + gs] : glo[grp][k]) - iw0 + 2 * (gs & 64)) << kTcFrac) +
-                                        (mine ? f0s[k * kTcS + gs] : 0u);
-                    const float sc = invs[k * kTcS + gs];
-                    if (k == 0) {
-                        // this thread's bins of the chunk, shared by every detector (idle slots
-                        // re-read the quarter's last bin, so that they repeat its value, or a
-                        // valid bin when the quarter has none; one 8-byte broadcast load each)
-                        const int jl = jn > 0 ? jb + jn - 1 : min(jb, NT - 1);
+                const int q = warp & 3, pbar = 1 + 2 * q + pb;   // the pair's named barrier
+                float *Rt = pb ? Rs2 : Rs;
+                const unsigned char *Rb = reinterpret_cast<const unsigned char *>(Rt);
+                float *Rd = Rt + (q >> 1) * (kTcW * 64) + (64 * hh) * 64 + 32 * (q & 1) + lane;   // drained columns
+                const uint32_t taddr = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(pb * kTcW + 64 * hh);
+                const uint32_t lane4 = (uint32_t)(gs & 63) * 4u;
+                const bool mine = gok && in_grp;
+                float lin[kTcBPT];
 #pragma unroll
-                        for (int i = 0; i < kTcBPT; ++i) {
-                            bj[i] = (uint32_t)bins[min(jb + i, jl)].y;
+                for (int i = 0; i < kTcBPT; ++i)
+                    lin[i] = 0.f;
+                for (int ch = pb; ch < n_chunks && !failed; ch += 2) {
+                    const int j0 = ch * jnom, J = min(jnom, NT - j0), jq = (J + 1) >> 1;
+                    const int jb = j0 + hh * jq, jn = max(0, min(jq, j0 + J - jb));   // this thread's bins
+                    // groups of four bins that are gathered (every slot of them: those behind the
+                    // last bin hold something in the window's neighbourhood and are masked)
+                    const int ng = jq <= 16 ? 4 : jq <= 24 ? 6 : (jq + 3) >> 2;
+                    for (int k = 0; k < K; ++k) {
+                        // every lane waits for the MMAs of the step (the same barrier word: no
+                        // divergent branch, no broadcast of the result)
+                        const int ok = tc::mbar_wait(fullb + pb, phbit(kPhFull, pb), kWaitNs) ? 1 : 0;
+                        ph ^= 1u << (kPhFull + pb);
+                        if (idle) {
+                            __syncwarp();
+                            tc::mbar_arrive_if(emptyb + pb, lane == 0);
+                            if (!ok) {
+                                failed = 1;
+                                break;
+                            }
+                            continue;
                         }
-                    }
-                    {
-                        // drain accumulator b: warp quarter q = rows 32q.., column block w / 4 of 32
-                        const int q = warp & 3, cb = warp >> 2;
-                        float *Rcol = Rt + (q >> 1) * (kTcW * 64) + (32 * cb) * 64 + 32 * (q & 1) + lane;
-                        // two loads of 16 columns (fewer live registers than one of 32)
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
+                        tc::tc_fence_after();
+                        // drain this warp's 64 columns of the 32 rows, 16 at a time
+                        {
                             uint32_t v[16];
-                            tc::tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(b * kTcW + 32 * cb + 16 * h), v);
+                            tc::tmem_ld16(taddr, v);
+                            tc::tmem_ld_wait();
+                            // the pair's gathers of the previous step are done with the R tile
+                            tc::named_bar_or(pbar, kTcPairThreads, 0);
+#pragma unroll
+                            for (int i = 0; i < 16; ++i)
+                                Rd[i * 64] = __uint_as_float(v[i]);
+                        }
+#pragma unroll
+                        for (int h = 1; h < 4; ++h) {
+                            uint32_t v[16];
+                            tc::tmem_ld16(taddr + 16u * (uint32_t)h, v);
                             tc::tmem_ld_wait();
 #pragma unroll
                             for (int i = 0; i < 16; ++i)
-                                Rcol[(16 * h + i) * 64] = __uint_as_float(v[i]);
+                                Rd[(16 * h + i) * 64] = __uint_as_float(v[i]);
                         }
-                    }
-                    tc::tc_fence_before();
-                    __syncwarp();
-                    tc::mbar_arrive_if(emptyb + b, lane == 0);
-                    // this quarter's rows of R complete; agree on failure
-                    if (tc::named_bar_or(qbar, kTcConsumers / 4, !ok || abort_s)) {
-                        failed = 1;
-                        break;
-                    }
-                    // two bins per packed float32 operation (the same roundings as one at a time)
-                    const uint32_t lane4 = (uint32_t)(gs & 63) * 4u;
-                    const unsigned char *Rb = reinterpret_cast<const unsigned char *>(Rt);
-                    auto pair = [&](int i) {
-                        const uint32_t u = ub + bj[i], w = ub + bj[i + 1];
-                        // byte offset of the node: column << 8 | (sample of the half tile) * 4
-                        const float *ra = reinterpret_cast<const float *>(Rb + __byte_perm(u, lane4, 0x7734));
-                        const float *rb = reinterpret_cast<const float *>(Rb + __byte_perm(w, lane4, 0x7734));
-                        const float2 r0 = make_float2(ra[0], rb[0]), r1 = make_float2(ra[64], rb[64]);
-                        const float2 fr = __fmul2_rn(make_float2((float)(u & 0xffffffu), (float)(w & 0xffffffu)),
-                                                     make_float2(0x1p-24f, 0x1p-24f));
-                        const float2 v = __ffma2_rn(fr, __ffma2_rn(r0, make_float2(-1.f, -1.f), r1), r0);
-                        const float2 l = __ffma2_rn(make_float2(sc, sc), v, make_float2(lin[i], lin[i + 1]));
-                        lin[i] = l.x;
-                        lin[i + 1] = l.y;
-                    };
-                    pair(0);
-                    pair(2);
-                    pair(4);
-                    pair(6);
-                    if (jq > 8) {
-                        pair(8);
-                        pair(10);
-                    }
-                    if (jq > 12)
-                        pair(12);
-                    if (jq > 14)
-                        pair(14);
-                    if (k == K - 1) {
-                        // fold this thread's bins of the chunk into its running log-sum-exp
-                        float cmx = -INFINITY;
-                        if (kDM) {
-                            // distance marginal per bin: a cheap upper bound first; the bin
-                            // with the highest bound is evaluated, and a bin whose bound lies
-                            // more than 40 below the larger of that value and the running
-                            // maximum cannot move the marginal (< e^-40): left out
-                            // (the bound is recomputed in the second loop rather than kept: it is
-                            // a handful of operations, a register array of it is not)
-                            float bmax = -INFINITY, abest = 0.f;
-#pragma unroll
-                            for (int i = 0; i < kTcBPT; ++i) {
-                                const float bd = i < jn ? dm_bound32(P, lin[i], gqd) : -INFINITY;
-                                if (bd > bmax) {
-                                    bmax = bd;
-                                    abest = lin[i];
-                                }
-                            }
-                            const float vbest = jn > 0 ? ln_dist_marg32(P, abest, gqd) : -INFINITY;
-                            // (every bin exact when the per-bin values are written out)
-                            const float thr = lnL_t ? -INFINITY : fmaxf(run_mx, vbest) - 40.f;
-#pragma unroll
-                            for (int i = 0; i < kTcBPT; ++i) {
-                                lin[i] = (i < jn && dm_bound32(P, lin[i], gqd) >= thr) ? ln_dist_marg32(P, lin[i], gqd)
-                                                                                      : -INFINITY;
-                                if (i < jn)
-                                    cmx = fmaxf(cmx, lin[i]);
-                            }
-                        } else {
-                            // lin holds the data term; ln L = lin - gqd, the template term
-                            // subtracted once per sample in the epilogue (in float64)
-                            // (the maximum by blocks of kPeakBlockTc bins, the same number of
-                            // operations, so that the block holding it is known).  Idle slots
-                            // repeat the last bin's value: the maximum is that of the valid
-                            // bins, and the lowest block attaining it holds a valid bin.
-                            float qm[4];
-                            qm[0] = fmaxf(fmaxf(lin[0], lin[1]), fmaxf(lin[2], lin[3]));
-                            qm[1] = fmaxf(fmaxf(lin[4], lin[5]), fmaxf(lin[6], lin[7]));
-                            qm[2] = jq > 8 ? fmaxf(fmaxf(lin[8], lin[9]), fmaxf(lin[10], lin[11])) : -INFINITY;
-                            qm[3] = jq > 12 ? fmaxf(lin[12], lin[13]) : -INFINITY;
-                            if (jq > 14)
-                                qm[3] = fmaxf(qm[3], fmaxf(lin[14], lin[15]));
-                            const float m01 = fmaxf(qm[0], qm[1]), m23 = fmaxf(qm[2], qm[3]);
-                            cmx = fmaxf(m01, m23);
-                            if (jn > 0 && in_grp) {
-                                const int a = m01 >= m23 ? (qm[0] >= qm[1] ? 0 : 1) : (qm[2] >= qm[3] ? 2 : 3);
-                                const uint32_t ob = __float_as_uint(cmx) ^
-                                                    ((uint32_t)((int)__float_as_uint(cmx) >> 31) | 0x80000000u);
-                                atomicMax(peak + gs,
-                                          ((unsigned long long)ob << 32) | (unsigned)(NT - jb - kPeakBlockTc * a));
-                            }
+                        tc::tc_fence_before();
+                        __syncwarp();
+                        tc::mbar_arrive_if(emptyb + pb, lane == 0);
+                        // position of the sample's first node: column (plus 128 in the upper half of
+                        // the tile's samples) in the top byte, fraction below (modulo 2^32).  Padding
+                        // samples and samples of other sub-groups read at the group's lowest offset;
+                        // their sums are discarded.
+                        const uint32_t ub =
+                            ((uint32_t)((mine ? i0s[k * kTcS + gs] : glo[grp][k]) - win0(k, j0) + 2 * (gs & 64)) << kTcFrac) +
+                            (mine ? f0s[k * kTcS + gs] : 0u);
+                        const float sc = invs[k * kTcS + gs];
+                        // the pair's columns of R complete; agree on failure
+                        if (tc::named_bar_or(pbar, kTcPairThreads, !ok || abort_s)) {
+                            failed = 1;
+                            break;
                         }
-                        if (lnL_t && gok && in_grp) {
-                            for (int i = 0; i < jn; ++i)
-#pragma unroll
-                                for (int u = 0; u < kTcBPT; ++u)
-                                    if (u == i)
-                                        lnL_t[(lnl_t_compact ? (int64_t)tile_s * kTcS + gs : (int64_t)gid[gs]) * NT + jb + i] =
-                                            kDM ? (double)lin[u] : (double)lin[u] - (double)gqd;
-                        }
-                        if (jn > 0 && in_grp) {
-                            const float nm = fmaxf(run_mx, cmx);
-                            float cs = 0.f;
-                            if (kDM) {
-#pragma unroll
-                                for (int i = 0; i < kTcBPT; ++i)
-                                    if (i < jn)
-                                        cs += __expf(lin[i] - nm);
+                        // four bins (two packed pairs, the same roundings as one at a time)
+                        auto four = [&](int i) {
+                            uint32_t u[4];
+                            if ((jb & 3) == 0) {
+                                const uint4 w = *reinterpret_cast<const uint4 *>(bins + jb + i);
+                                u[0] = w.x;
+                                u[1] = w.y;
+                                u[2] = w.z;
+                                u[3] = w.w;
                             } else {
-                                // exp(lin - nm) = 2^(lin log2(e) - nm log2(e)), two bins per packed
-                                // operation
-                                const float off = nm * kLog2e;
-                                float2 cs2 = make_float2(0.f, 0.f);
-                                auto terms = [&](int i) {
-                                    const float2 x = __ffma2_rn(make_float2(lin[i], lin[i + 1]), make_float2(kLog2e, kLog2e),
-                                                                make_float2(-off, -off));
-                                    const float2 ev = make_float2(i < jn ? ex2_approx(x.x) : 0.f,
-                                                                  i + 1 < jn ? ex2_approx(x.y) : 0.f);
-                                    cs2 = __fadd2_rn(cs2, ev);
-                                };
-                                terms(0);
-                                terms(2);
-                                terms(4);
-                                terms(6);
-                                if (jq > 8) {
-                                    terms(8);
-                                    terms(10);
-                                }
-                                if (jq > 12)
-                                    terms(12);
-                                if (jq > 14)
-                                    terms(14);
-                                cs = cs2.x + cs2.y;
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    u[e] = bins[jb + i + e];
                             }
-                            run_sum = (run_mx == -INFINITY ? 0.f : run_sum * __expf(run_mx - nm)) + cs;
-                            run_mx = nm;
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                u[e] += ub;
+#pragma unroll
+                            for (int e = 0; e < 4; e += 2) {
+                                // byte offset of the node: column << 8 | (sample of the half tile) * 4
+                                const float *ra = reinterpret_cast<const float *>(Rb + __byte_perm(u[e], lane4, 0x7734));
+                                const float *rb = reinterpret_cast<const float *>(Rb + __byte_perm(u[e + 1], lane4, 0x7734));
+                                const float2 r0 = make_float2(ra[0], rb[0]), r1 = make_float2(ra[64], rb[64]);
+                                const float2 fr =
+                                    __fmul2_rn(make_float2((float)(u[e] & 0xffffffu), (float)(u[e + 1] & 0xffffffu)),
+                                               make_float2(0x1p-24f, 0x1p-24f));
+                                const float2 v = __ffma2_rn(fr, __ffma2_rn(r0, make_float2(-1.f, -1.f), r1), r0);
+                                const float2 l = __ffma2_rn(make_float2(sc, sc), v, make_float2(lin[i + e], lin[i + e + 1]));
+                                lin[i + e] = l.x;
+                                lin[i + e + 1] = l.y;
+                            }
+                        };
+                        four(0);
+                        four(4);
+                        four(8);
+                        four(12);
+                        if (ng > 4) {
+                            four(16);
+                            four(20);
                         }
+                        if (ng > 6)
+                            four(24);
+                        if (ng > 7)
+                            four(28);
+                    }
+                    if (failed || idle)
+                        continue;
+                    // fold this thread's bins of the chunk into its running log-sum-exp
+                    if (jn < 4 * ng) {
 #pragma unroll
                         for (int i = 0; i < kTcBPT; ++i)
-                            lin[i] = 0.f;
+                            lin[i] = i < jn ? lin[i] : -INFINITY;
                     }
-                    if (++k == K) {
-                        k = 0;
-                        j0 += jnom;
+                    float cmx = -INFINITY;
+                    if (kDM) {
+                        // distance marginal per bin: a cheap upper bound first; the bin with the
+                        // highest bound is evaluated, and a bin whose bound lies more than 40
+                        // below the larger of that value and the running maximum cannot move the
+                        // marginal (< e^-40): left out.  The bins wait in this thread's slots of
+                        // the R tile (its warp's drained columns), so that the quadrature is not
+                        // unrolled over registers.
+                        tc::named_bar_or(pbar, kTcPairThreads, 0);
+                        float bmax = -INFINITY, abest = 0.f;
+#pragma unroll
+                        for (int i = 0; i < kTcBPT; ++i) {
+                            const float bd = i < jn ? dm_bound32(P, lin[i], gqd) : -INFINITY;
+                            if (bd > bmax) {
+                                bmax = bd;
+                                abest = lin[i];
+                            }
+                            Rd[i * 64] = lin[i];
+                        }
+                        const float vbest = jn > 0 ? ln_dist_marg32(P, abest, gqd) : -INFINITY;
+                        // (every bin exact when the per-bin values are written out)
+                        const float thr = lnL_t ? -INFINITY : fmaxf(run_mx, vbest) - 40.f;
+#pragma unroll 1
+                        for (int i = 0; i < jn; ++i) {
+                            const float x = Rd[i * 64];
+                            const float v = dm_bound32(P, x, gqd) >= thr ? ln_dist_marg32(P, x, gqd) : -INFINITY;
+                            Rd[i * 64] = v;
+                            cmx = fmaxf(cmx, v);
+                        }
+                        if (mine && jn > 0) {
+                            const float nm = fmaxf(run_mx, cmx);
+                            float cs = 0.f;
+                            for (int i = 0; i < jn; ++i)
+                                cs += __expf(Rd[i * 64] - nm);
+                            run_sum = (run_mx == -INFINITY ? 0.f : run_sum * __expf(run_mx - nm)) + cs;
+                            run_mx = nm;
+                            if (lnL_t)
+                                for (int i = 0; i < jn; ++i)
+                                    lnL_t[(lnl_t_compact ? (int64_t)tile_s * kTcS + gs : (int64_t)gid[gs]) * NT + jb + i] =
+                                        (double)Rd[i * 64];
+                        }
+                    } else {
+                        // lin holds the data term; ln L = lin - gqd, the template term subtracted
+                        // once per sample in the epilogue (in float64).  The maximum by blocks of
+                        // kPeakBlockTc bins, so that the block holding it is known.
+                        static_assert(kPeakBlockTc == 4, "a group of the gather");
+                        float qm[kTcBPT / 4];
+                        auto top = [&](int a) {
+                            qm[a] = fmaxf(fmaxf(lin[4 * a], lin[4 * a + 1]), fmaxf(lin[4 * a + 2], lin[4 * a + 3]));
+                            cmx = fmaxf(cmx, qm[a]);
+                        };
+#pragma unroll
+                        for (int a = 4; a < kTcBPT / 4; ++a)
+                            qm[a] = -INFINITY;
+                        top(0);
+                        top(1);
+                        top(2);
+                        top(3);
+                        if (ng > 4) {
+                            top(4);
+                            top(5);
+                        }
+                        if (ng > 6)
+                            top(6);
+                        if (ng > 7)
+                            top(7);
+                        if (mine && lnL_t)
+#pragma unroll
+                            for (int i = 0; i < kTcBPT; ++i)
+                                if (i < jn)
+                                    lnL_t[(lnl_t_compact ? (int64_t)tile_s * kTcS + gs : (int64_t)gid[gs]) * NT + jb + i] =
+                                        (double)lin[i] - (double)gqd;
+                        if (mine && jn > 0) {
+                            if (cmx > run_mx) {   // the lowest block of the thread's bins holding the maximum
+                                int a = 0;
+#pragma unroll
+                                for (int e = kTcBPT / 4 - 1; e >= 0; --e)
+                                    a = qm[e] == cmx ? e : a;
+                                run_j = jb + 4 * a;
+                            }
+                            const float nm = fmaxf(run_mx, cmx);
+                            // exp(lin - nm) = 2^(lin log2(e) - nm log2(e)), two bins per packed
+                            // operation
+                            const float off = nm * kLog2e;
+                            float2 cs2 = make_float2(0.f, 0.f);
+                            auto terms = [&](int i0) {
+#pragma unroll
+                                for (int i = i0; i < i0 + 4; i += 2) {
+                                    const float2 x = __ffma2_rn(make_float2(lin[i], lin[i + 1]), make_float2(kLog2e, kLog2e),
+                                                                make_float2(-off, -off));
+                                    cs2 = __fadd2_rn(cs2, make_float2(ex2_approx(x.x), ex2_approx(x.y)));
+                                }
+                            };
+                            terms(0);
+                            terms(4);
+                            terms(8);
+                            terms(12);
+                            if (ng > 4) {
+                                terms(16);
+                                terms(20);
+                            }
+                            if (ng > 6)
+                                terms(24);
+                            if (ng > 7)
+                                terms(28);
+                            run_sum = (run_mx == -INFINITY ? 0.f : run_sum * __expf(run_mx - nm)) + (cs2.x + cs2.y);
+                            run_mx = nm;
+                        }
                     }
+#pragma unroll
+                    for (int i = 0; i < kTcBPT; ++i)
+                        lin[i] = 0.f;
                 }
             }
             // producer and consumers meet between sub-groups (and learn of a failure)
@@ -1105,6 +1147,7 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
         if (!producer) {
             lse[gh * kTcS + gs] = run_mx;
             lse[(kTcQ + gh) * kTcS + gs] = run_sum;
+            peak[gh * kTcS + gs] = run_j;
         }
         __syncthreads();
         if (tid < kTcS && gid[tid] != 0xffffffffu) {
@@ -1126,7 +1169,11 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
             if (!kDM && po.q) {
                 po.q[g] = gqd;
                 po.m[g] = mx;
-                po.j[g] = NT - (int)(uint32_t)peak[tid];
+                int j = INT_MAX;   // the lowest block among the partials holding the maximum
+                for (int h = 0; h < kTcQ; ++h)
+                    if (lse[h * kTcS + tid] == mx)
+                        j = min(j, peak[h * kTcS + tid]);
+                po.j[g] = j;
             }
             if (!isfinite(r))
                 atomicOr(err, kErrNonFinite);
