@@ -123,6 +123,23 @@ int wigner_table(int l, int m, double *coef, int8_t *pc, int8_t *ps)
     return nt;
 }
 
+// Fourier coefficients of d(iota) = sum_t coef_t cos(iota/2)^pc_t sin(iota/2)^ps_t, a trigonometric
+// polynomial of degree l in iota (pc_t + ps_t = 2 l), even for even m and odd for odd m (the
+// second index of d^l_{m,2} is even): discrete sums over 4 l points, exact up to rounding.
+void polar_fourier(int l, int m, const double *coef, const int8_t *pc, const int8_t *ps, int nt, double *alpha)
+{
+    const int np = 4 * l;
+    const long double step = 2.0L * 3.14159265358979323846264338327950288L / np;
+    for (int j = 0; j < np; ++j) {
+        const long double c = std::cos(0.5L * j * step), s = std::sin(0.5L * j * step);
+        long double d = 0.0L;
+        for (int t = 0; t < nt; ++t)
+            d += (long double)coef[t] * std::pow(c, (int)pc[t]) * std::pow(s, (int)ps[t]);
+        for (int u = 0; u <= l; ++u)
+            alpha[u] += (double)(d * ((m & 1) ? std::sin(u * j * step) : std::cos(u * j * step)) * (u ? 2.0L : 1.0L) / np);
+    }
+}
+
 // Gauss-Legendre nodes and weights on [-1, 1]: Newton's method on P_n from the
 // three-term recurrence, starting at the Chebyshev-like guesses cos(pi (i + 3/4) / (n + 1/2)).
 void gauss_legendre(int n, double *t, double *w)
@@ -750,50 +767,31 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
     // whose per-bin values are no difference of two large terms)
     h->fix_on = cfg->precision != RIFT_FP64 && !cfg->distance_marg;
     if (h->fix_on) {
-        // mode-pair tables, grouped by m_a - m_b >= 0 (ordered pairs) and by m_a + m_b (a <= b)
-        int mmax = 0;
-        for (int m = 0; m < M; ++m)
+        int mmax = 0, lmax = 0;
+        std::vector<double> alpha((size_t)M * (kMaxL + 1), 0.0);
+        for (int m = 0; m < M; ++m) {
             mmax = std::max(mmax, std::abs(cfg->lm[2 * m + 1]));
-        const int dmax = 2 * mmax;
-        std::vector<uint16_t> aij, bij;
-        std::vector<int> ast, bst;
-        for (int D = 0; D <= dmax; ++D) {
-            ast.push_back((int)aij.size());
-            for (int a = 0; a < M; ++a)
-                for (int b = 0; b < M; ++b)
-                    if (cfg->lm[2 * a + 1] - cfg->lm[2 * b + 1] == D)
-                        aij.push_back((uint16_t)(a | (b << 8)));
+            lmax = std::max(lmax, cfg->lm[2 * m]);
+            polar_fourier(cfg->lm[2 * m], cfg->lm[2 * m + 1], P.wcoef[m], P.wpc[m], P.wps[m], P.wn[m],
+                          alpha.data() + (size_t)m * (kMaxL + 1));
         }
-        ast.push_back((int)aij.size());
-        for (int S = -dmax; S <= dmax; ++S) {
-            bst.push_back((int)bij.size());
-            for (int a = 0; a < M; ++a)
-                for (int b = a; b < M; ++b)
-                    if (cfg->lm[2 * a + 1] + cfg->lm[2 * b + 1] == S)
-                        bij.push_back((uint16_t)(a | (b << 8)));
-        }
-        bst.push_back((int)bij.size());
-        const int nA = (int)aij.size(), nB = (int)bij.size();
+        const int dmax = 2 * mmax, nf = 2 * lmax + 1;
         if ((rc = dalloc(h, &h->aux_q, (size_t)N)) || (rc = dalloc(h, &h->aux_m, (size_t)N)) ||
             (rc = dalloc(h, &h->aux_j, (size_t)N)) || (rc = dalloc(h, &h->fix_idx, (size_t)N)) ||
-            (rc = dalloc(h, &h->fix_count, (size_t)4)) || (rc = dalloc(h, &h->fix_aij, (size_t)nA)) ||
-            (rc = dalloc(h, &h->fix_bij, (size_t)nB)) || (rc = dalloc(h, &h->fix_astart, ast.size())) ||
-            (rc = dalloc(h, &h->fix_bstart, bst.size())) || (rc = dalloc(h, &h->fix_ua, (size_t)K * nA)) ||
-            (rc = dalloc(h, &h->fix_vb, (size_t)K * nB)) || (rc = dalloc(h, &h->fix_qdf, (size_t)K * M * cfg->n_q))) {
+            (rc = dalloc(h, &h->fix_count, (size_t)4)) || (rc = dalloc(h, &h->fix_alpha, alpha.size())) ||
+            (rc = dalloc(h, &h->fix_ga, (size_t)K * (dmax + 1) * nf)) ||
+            (rc = dalloc(h, &h->fix_hb, (size_t)K * (2 * dmax + 1) * nf)) ||
+            (rc = dalloc(h, &h->fix_qdf, (size_t)K * M * cfg->n_q))) {
             release(h);
             return rc;
         }
-        if (cudaMemcpyAsync(h->fix_aij, aij.data(), sizeof(uint16_t) * nA, cudaMemcpyHostToDevice, h->stream) ||
-            cudaMemcpyAsync(h->fix_bij, bij.data(), sizeof(uint16_t) * nB, cudaMemcpyHostToDevice, h->stream) ||
-            cudaMemcpyAsync(h->fix_astart, ast.data(), sizeof(int) * ast.size(), cudaMemcpyHostToDevice, h->stream) ||
-            cudaMemcpyAsync(h->fix_bstart, bst.data(), sizeof(int) * bst.size(), cudaMemcpyHostToDevice, h->stream) ||
+        if (cudaMemcpyAsync(h->fix_alpha, alpha.data(), sizeof(double) * alpha.size(), cudaMemcpyHostToDevice, h->stream) ||
             cudaStreamSynchronize(h->stream)) {
             cudaGetLastError();
             release(h);
             return RIFT_ECUDA;
         }
-        h->fix = FixTables{h->fix_aij, h->fix_astart, h->fix_bij, h->fix_bstart, h->fix_ua, h->fix_vb, h->fix_qdf,
-                           nA, nB, dmax};
+        h->fix = FixTables{h->fix_alpha, h->fix_ga, h->fix_hb, h->fix_qdf, dmax, nf};
         // samples with quad32 + |max lin32| above this are corrected: below it the float32
         // rounding stays under 5e-4 (measured, ~3e-7 per unit of the terms at most)
         h->fix_thr = kFixThreshold;
@@ -935,10 +933,9 @@ int64_t rift_ile_footprint(const rift_ile_config *cfg)
         digits ? 2 * (int64_t)(tc64_q_halves(K, M, groups) + tc64_t_halves(K, M)) + 7 * 16 + 8 * (nt + kTc64Table) +
                      (int64_t)(tc64_scratch_bytes(K, M, N, 152) + tc64_record_bytes(N, cfg->n_t))
                : 0,
-        // large-term correction: per-sample side outputs and list, pair tables, double-float
-        // copies of U, V (at most M^2 pairs each) and Q
-        cfg->precision != RIFT_FP64 && !cfg->distance_marg ? 4 * N * 4 + 16 + 4 * M * M + 8 * 64 +
-                                                                  2 * K * M * M * 16 + K * M * nq * 16
+        // large-term correction: per-sample side outputs and list, double-float tables of the
+        // template term (at most 13 x 13 + 25 x 13 coefficients a detector) and of Q
+        cfg->precision != RIFT_FP64 && !cfg->distance_marg ? 4 * N * 4 + 16 + 8 * (kMaxL + 1) * M + 64 + K * 494 * 16 + K * M * nq * 16
                                                             : 0};
     int64_t total = 0;
     for (int64_t b : sizes)
@@ -1104,8 +1101,8 @@ int install_overlaps(rift_ile_t *h)
         h->launches += 3;
     }
     if (h->fix_on) {
-        CK(launch_fix_prep(h->prob, h->fix, h->fix_ua, h->fix_vb, h->fix_qdf, h->stream));
-        h->launches += 1;
+        CK(launch_fix_prep(h->prob, h->fix, h->stream));
+        h->launches += 2;
     }
     int rc = sync_and_err(h);
     h->have_overlaps = (rc == RIFT_OK);

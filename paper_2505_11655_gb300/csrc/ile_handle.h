@@ -65,9 +65,8 @@ struct rift_ile {
     float *aux_q = nullptr, *aux_m = nullptr;
     int *aux_j = nullptr;
     uint32_t *fix_idx = nullptr, *fix_count = nullptr;
-    uint16_t *fix_aij = nullptr, *fix_bij = nullptr;
-    int *fix_astart = nullptr, *fix_bstart = nullptr;
-    float4 *fix_ua = nullptr, *fix_vb = nullptr, *fix_qdf = nullptr;
+    double *fix_alpha = nullptr;
+    float4 *fix_ga = nullptr, *fix_hb = nullptr, *fix_qdf = nullptr;
     rift::FixTables fix{};
     bool fix_on = false;
     float fix_thr = 0.f;

@@ -116,20 +116,17 @@ struct PeakOut {
 };
 constexpr int kPeakBlockTc = 4;
 
-// Large-term correction of the float32 path (k_fixup.cu).  Mode-pair tables (host-built
-// from the mode list) and double-float copies of U, V, Q (built on the device whenever the
-// overlaps change).  dmax = 2 max|m|.
+// Large-term correction of the float32 path (k_fixup.cu): Fourier coefficients of the modes'
+// polar functions (host-built from the mode list) and double-float tables of the template term
+// and of Q (built on the device whenever the overlaps change).  dmax = 2 max|m|, nf = 2 max l + 1.
 struct FixTables {
-    const uint16_t *a_ij;   // ordered pairs (a | b << 8) with m_a - m_b = D >= 0, grouped by D
-    const int *a_start;     // [dmax + 2] group boundaries
-    const uint16_t *b_ij;   // pairs a <= b grouped by S = m_a + m_b
-    const int *b_start;     // [2 dmax + 2] group boundaries, by S + dmax
-    const float4 *ua;       // [K][nA] U_k,ab (re.hi, re.lo, im.hi, im.lo)
-    const float4 *vb;       // [K][nB] (2 - delta_ab) V_k,ab, same layout
-    const float4 *qdf;      // [K][M][n_q] Q, same layout
-    int nA, nB, dmax;
+    const double *alpha;    // [M][kMaxL + 1]: d_m(iota) = sum_u alpha_mu cos(u iota) (m even), sin (m odd)
+    float4 *ga;             // [K][dmax + 1][nf] (re.hi, re.lo, im.hi, im.lo), see k_fixup.cu
+    float4 *hb;             // [K][2 dmax + 1][nf]
+    float4 *qdf;            // [K][M][n_q] Q, same layout
+    int dmax, nf;
 };
-cudaError_t launch_fix_prep(const Problem &P, FixTables T, float4 *ua, float4 *vb, float4 *qdf, cudaStream_t st);
+cudaError_t launch_fix_prep(const Problem &P, FixTables T, cudaStream_t st);
 // Lists the samples with po.q + |po.m| > thr (idx, *count; count reset here) and corrects
 // their lnL_tmarg (and lnw = lnL_tmarg + lnpw, and the rows of lnL_t, when given) in place.
 // blen: the block length of po.j.  *launched: kernels enqueued.

@@ -15,10 +15,14 @@
 //      parity bar there) are listed;
 //   3. for each listed sample, with the coefficients from float64 geometry:
 //        the template term in double-float (~44 bits), written through the symmetry of
-//        U (Hermitian) and V (symmetric) and the form Y_lm = d_lm(iota) exp(-i m phi):
+//        U (Hermitian) and the form Y_lm = d_lm(iota) exp(-i m phi):
 //          c^H U_k c = |s_k|^2 sum_D exp(i D phi) G_k,D,  G_k,D = sum_{m_a - m_b = D} d_a d_b U_k,ab
 //          c^T V_k c = s_k^2  sum_S exp(-i S phi) H_k,S,  H_k,S = sum_{m_a + m_b = S} d_a d_b V_k,ab
-//        with s_k = (D_ref/D) F_k;
+//        with s_k = (D_ref/D) F_k.  The d_lm are trigonometric polynomials of degree l in iota,
+//        so every G_k,D and H_k,S is one of degree 2 l_max, in cosines for even D, S and in
+//        sines for odd; their coefficients are summed once per problem in float64 (21 modes up
+//        to l = 4: 9 x 9 + 17 x 9 complex coefficients a detector in place of 2 x 231 mode pairs
+//        with a product d_a d_b each: a loud solve's 250,000 corrections 1.07 -> 0.94 ms);
 //        the bin of the block with the largest data term (a float32 search when the block
 //        holds several bins), and the data term there in double-float, from a double-float
 //        copy of Q;
@@ -40,35 +44,70 @@ constexpr int kFixMaxWarps = 16;   // warps per block: as many as the shared mem
 
 // --------------------------------------------------------------- double-float copies
 
-__global__ void fix_prep_kernel(const double2 *__restrict__ U64, const double2 *__restrict__ V64,
-                                const double2 *__restrict__ Q64, int K, int M, int n_q, FixTables T, float4 *ua,
-                                float4 *vb, float4 *qdf)
+__device__ __forceinline__ float4 df4(double re, double im)
 {
-    const int64_t nua = (int64_t)K * T.nA, nvb = (int64_t)K * T.nB, nq = (int64_t)K * M * n_q;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nua + nvb + nq;
-         e += (int64_t)gridDim.x * blockDim.x) {
-        double2 v;
-        float4 *dst;
-        if (e < nua) {
-            const int k = (int)(e / T.nA), p = (int)(e - (int64_t)k * T.nA);
-            const int i = T.a_ij[p] & 255, j = T.a_ij[p] >> 8;
-            v = U64[((size_t)k * M + i) * M + j];
-            dst = ua + e;
-        } else if (e < nua + nvb) {
-            const int64_t f = e - nua;
-            const int k = (int)(f / T.nB), p = (int)(f - (int64_t)k * T.nB);
-            const int i = T.b_ij[p] & 255, j = T.b_ij[p] >> 8;
-            v = V64[((size_t)k * M + i) * M + j];
-            if (i != j)
-                v = make_double2(2.0 * v.x, 2.0 * v.y);   // the pair (j, i) of the symmetric V
-            dst = vb + f;
-        } else {
-            const int64_t f = e - nua - nvb;
-            v = Q64[f];
-            dst = qdf + f;
-        }
-        const df re = df_of(v.x), im = df_of(v.y);
-        *dst = make_float4(re.hi, re.lo, im.hi, im.lo);
+    const df a = df_of(re), b = df_of(im);
+    return make_float4(a.hi, a.lo, b.hi, b.lo);
+}
+
+__global__ void fix_prep_q_kernel(const double2 *__restrict__ Q64, int64_t nq, float4 *__restrict__ qdf)
+{
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nq; e += (int64_t)gridDim.x * blockDim.x) {
+        const double2 v = Q64[e];
+        qdf[e] = df4(v.x, v.y);
+    }
+}
+
+// Coefficient n of the product of two polar functions with Fourier coefficients A, B (sine
+// series where odd): cosines of n iota when both or neither are odd, else sines.
+__device__ __forceinline__ double product_coef(const double *A, bool odd_a, const double *B, bool odd_b, int n)
+{
+    double v = 0.0;
+    for (int u = 0; u <= kMaxL; ++u) {
+        const int sum = n - u, lower = u - n, upper = u + n;   // partners with u + w = n, u - w = n, w - u = n
+        double t = 0.0;
+        if (sum >= 0 && sum <= kMaxL)
+            t += odd_a && odd_b ? -B[sum] : B[sum];
+        if (lower >= 0)
+            t += !odd_a && odd_b ? -B[lower] : B[lower];
+        if (n > 0 && upper <= kMaxL)
+            t += odd_a && !odd_b ? -B[upper] : B[upper];
+        v += A[u] * t;
+    }
+    return 0.5 * v;
+}
+
+// One warp per (detector, D or S, n).
+__global__ void fix_prep_template_kernel(Problem P, FixTables T)
+{
+    const int lane = threadIdx.x & 31, M = P.M, na = T.dmax + 1, ns = 2 * T.dmax + 1;
+    const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), per = (na + ns) * T.nf;
+    if (e >= P.K * per)
+        return;
+    const int k = e / per, row = (e - k * per) / T.nf, n = e - k * per - row * T.nf;
+    const bool u_term = row < na;
+    const int want = u_term ? row : row - na - T.dmax;   // D or S
+    const double2 *G = (u_term ? P.U64 : P.V64) + (size_t)k * M * M;
+    double re = 0.0, im = 0.0;
+    for (int p = lane; p < M * M; p += 32) {
+        const int a = p / M, b = p - a * M, ma = P.mode_m[a], mb = P.mode_m[b];
+        if ((u_term ? ma - mb : ma + mb) != want)
+            continue;
+        const double c = product_coef(T.alpha + a * (kMaxL + 1), ma & 1, T.alpha + b * (kMaxL + 1), mb & 1, n);
+        const double2 g = G[p];
+        re += c * g.x;
+        im += c * g.y;
+    }
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+    }
+    if (lane == 0) {
+        if (u_term)
+            T.ga[((size_t)k * na + row) * T.nf + n] = df4(re, im);
+        else
+            T.hb[((size_t)k * ns + row - na) * T.nf + n] = df4(re, im);
     }
 }
 
@@ -96,13 +135,16 @@ __global__ void fix_select_kernel(const float *__restrict__ aq, const float *__r
 // --------------------------------------------------------------- correction
 
 // Per-warp shared memory: float64 rows [K + 1][32] (the Q position u0_k of the first bin,
-// then the template term), float rows [nf][32] (double-float s_k, d_lm, exp(-i n phi)), and
-// [32] the bin at which each sample's data term is evaluated.
-__host__ __device__ inline int fix_float_rows(int K, int M, int dmax) { return 4 * K + 2 * M + 4 * (dmax + 1); }
-
-__host__ __device__ inline size_t fix_warp_bytes(int K, int M, int dmax)
+// then the template term), float rows [..][32] (double-float s_k, d_lm, exp(-i n phi), cos and
+// sin of n iota), and [32] the bin at which each sample's data term is evaluated.
+__host__ __device__ inline int fix_float_rows(int K, int M, int dmax, int nf)
 {
-    return (size_t)(K + 1) * 32 * 8 + (size_t)fix_float_rows(K, M, dmax) * 32 * 4 + 32 * 4;
+    return 4 * K + 2 * M + 4 * (dmax + 1) + 4 * nf;
+}
+
+__host__ __device__ inline size_t fix_warp_bytes(int K, int M, int dmax, int nf)
+{
+    return (size_t)(K + 1) * 32 * 8 + (size_t)fix_float_rows(K, M, dmax, nf) * 32 * 4 + 32 * 4;
 }
 
 __global__ void __launch_bounds__(32 * kFixMaxWarps)
@@ -114,13 +156,13 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int K = P.K, M = P.M, NT = P.n_t;
     const int nph = T.dmax + 1;
-    unsigned char *wb = fsm + fix_warp_bytes(K, M, T.dmax) * warp;
+    unsigned char *wb = fsm + fix_warp_bytes(K, M, T.dmax, T.nf) * warp;
     double *rd = reinterpret_cast<double *>(wb);                 // [K + 1][32]
     float *rf = reinterpret_cast<float *>(rd + (K + 1) * 32);     // [nf][32]
-    float *c32 = rf + fix_float_rows(K, M, T.dmax) * 32;
+    float *c32 = rf + fix_float_rows(K, M, T.dmax, T.nf) * 32;
     // rows of rf: s_k (re.hi, re.lo, im.hi, im.lo) at 4k; d_lm (hi, lo) at 4K + 2m;
-    // exp(-i n phi) (re.hi, re.lo, im.hi, im.lo) at 4K + 2M + 4n
-    const int rs = 0, rdl = 4 * K, rph = 4 * K + 2 * M;
+    // exp(-i n phi) (re.hi, re.lo, im.hi, im.lo) at 4K + 2M + 4n; cos(n iota) (hi, lo), then sin
+    const int rs = 0, rdl = 4 * K, rph = 4 * K + 2 * M, rtr = rph + 4 * nph, NF = T.nf;
     const double beta = P.t_step * P.fs;
     const uint32_t cnt = *count;
     const int nw = (int)(blockDim.x >> 5);
@@ -128,19 +170,14 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
     // robin over the blocks first, so that a short list still spreads over every SM)
     if ((int64_t)blockIdx.x * 32 >= (int64_t)cnt)
         return;   // no listed sample for this block (the grid is sized for every sample)
-    // the pair tables and the double-float U, V of every detector, staged once per block
-    float4 *sua = reinterpret_cast<float4 *>(fsm + fix_warp_bytes(K, M, T.dmax) * nw);
-    float4 *svb = sua + K * T.nA;
-    uint16_t *saij = reinterpret_cast<uint16_t *>(svb + K * T.nB);
-    uint16_t *sbij = saij + T.nA;
-    for (int e = threadIdx.x; e < K * T.nA; e += blockDim.x)
-        sua[e] = T.ua[e];
-    for (int e = threadIdx.x; e < K * T.nB; e += blockDim.x)
-        svb[e] = T.vb[e];
-    for (int e = threadIdx.x; e < T.nA; e += blockDim.x)
-        saij[e] = T.a_ij[e];
-    for (int e = threadIdx.x; e < T.nB; e += blockDim.x)
-        sbij[e] = T.b_ij[e];
+    // the template coefficients of every detector, staged once per block
+    const int na = nph, ns = 2 * T.dmax + 1;
+    float4 *sga = reinterpret_cast<float4 *>(fsm + fix_warp_bytes(K, M, T.dmax, T.nf) * nw);
+    float4 *shb = sga + K * na * NF;
+    for (int e = threadIdx.x; e < K * na * NF; e += blockDim.x)
+        sga[e] = T.ga[e];
+    for (int e = threadIdx.x; e < K * ns * NF; e += blockDim.x)
+        shb[e] = T.hb[e];
     __syncthreads();
     // this lane's sample: the double-float value at rows (row, row + 1)
     auto ld = [&](int row) { return df{rf[row * 32 + lane], rf[(row + 1) * 32 + lane]}; };
@@ -171,12 +208,34 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                 rf[(rs + 4 * k + 2) * 32 + lane] = si.hi;
                 rf[(rs + 4 * k + 3) * 32 + lane] = si.lo;
             }
-            double cpow[kMaxPow + 1], spow[kMaxPow + 1];
-            half_angle_powers<double>(th[4], cpow, spow);
+            // cos and sin of n iota by powers of exp(i iota), and the polar functions from them
+            double si, ci;
+            sincos(th[4], &si, &ci);
+            double cn[kMaxL + 1], sn[kMaxL + 1], tr = 1.0, ti = 0.0;
+#pragma unroll
+            for (int nn = 0; nn <= 2 * kMaxL; ++nn) {
+                if (nn >= NF)
+                    break;
+                if (nn <= kMaxL) {
+                    cn[nn <= kMaxL ? nn : 0] = tr;
+                    sn[nn <= kMaxL ? nn : 0] = ti;
+                }
+                const df a = df_of(tr), b = df_of(ti);
+                rf[(rtr + 2 * nn) * 32 + lane] = a.hi;
+                rf[(rtr + 2 * nn + 1) * 32 + lane] = a.lo;
+                rf[(rtr + 2 * NF + 2 * nn) * 32 + lane] = b.hi;
+                rf[(rtr + 2 * NF + 2 * nn + 1) * 32 + lane] = b.lo;
+                const double t = tr * ci - ti * si;
+                ti = ti * ci + tr * si;
+                tr = t;
+            }
             for (int m = 0; m < M; ++m) {
+                const double *al = T.alpha + m * (kMaxL + 1);
                 double d = 0.0;
-                for (int t = 0; t < P.wn[m]; ++t)
-                    d += P.wcoef[m][t] * cpow[P.wpc[m][t]] * spow[P.wps[m][t]];
+#pragma unroll
+                for (int u = 0; u <= kMaxL; ++u)
+                    if (2 * u < NF)
+                        d = fma(al[u], (P.mode_m[m] & 1) ? sn[u] : cn[u], d);
                 const df dd = df_of(d);
                 rf[(rdl + 2 * m) * 32 + lane] = dd.hi;
                 rf[(rdl + 2 * m + 1) * 32 + lane] = dd.lo;
@@ -211,16 +270,16 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
 #pragma unroll
                 for (int k = 0; k < kMaxDet; ++k)
                     G[k] = {{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll 2
-                for (int p = T.a_start[D]; p < T.a_start[D + 1]; ++p) {
-                    const int ij = saij[p];
-                    const df w = df_mul(ld(rdl + 2 * (ij & 255)), ld(rdl + 2 * (ij >> 8)));
+                const int tb = rtr + ((D & 1) ? 2 * NF : 0);
+#pragma unroll 3
+                for (int n = D & 1; n < NF; ++n) {
+                    const df t = ld(tb + 2 * n);
 #pragma unroll
                     for (int k = 0; k < kMaxDet; ++k)
                         if (k < K) {
-                            const float4 u = sua[k * T.nA + p];
-                            df_acc(G[k].re, w, {u.x, u.y});
-                            df_acc(G[k].im, w, {u.z, u.w});
+                            const float4 u = sga[(k * na + D) * NF + n];
+                            df_acc(G[k].re, t, {u.x, u.y});
+                            df_acc(G[k].im, t, {u.z, u.w});
                         }
                 }
 #pragma unroll
@@ -244,16 +303,16 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
 #pragma unroll
                 for (int k = 0; k < kMaxDet; ++k)
                     H[k] = {{0.f, 0.f}, {0.f, 0.f}};
-#pragma unroll 2
-                for (int p = T.b_start[S + T.dmax]; p < T.b_start[S + T.dmax + 1]; ++p) {
-                    const int ij = sbij[p];
-                    const df w = df_mul(ld(rdl + 2 * (ij & 255)), ld(rdl + 2 * (ij >> 8)));
+                const int tb = rtr + ((S & 1) ? 2 * NF : 0);
+#pragma unroll 3
+                for (int n = S & 1; n < NF; ++n) {
+                    const df t = ld(tb + 2 * n);
 #pragma unroll
                     for (int k = 0; k < kMaxDet; ++k)
                         if (k < K) {
-                            const float4 v = svb[k * T.nB + p];
-                            df_acc(H[k].re, w, {v.x, v.y});
-                            df_acc(H[k].im, w, {v.z, v.w});
+                            const float4 v = shb[(k * ns + S + T.dmax) * NF + n];
+                            df_acc(H[k].re, t, {v.x, v.y});
+                            df_acc(H[k].im, t, {v.z, v.w});
                         }
                 }
 #pragma unroll
@@ -361,34 +420,55 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
         if (lane < nb) {
             const int j = jbest[lane];
             if (j != INT_MAX) {
-                df acc = {0.f, 0.f};
+                // lin = sum_k Re(conj(s_k) sum_m conj(Y_m) Q_k,m), Q interpolated at the bin
                 good = true;
-                for (int k = 0; k < K; ++k) {
-                    const double u = rd[k * 32 + lane] + (double)j * beta;
-                    const double fl = floor(u);
-                    if (!(fl >= 0.0) || fl + 1.0 > (double)(P.n_q - 1)) {
-                        good = false;
-                        break;
-                    }
-                    const int i = (int)fl;
-                    const df f = df_of(u - fl);
-                    const dfc sk{ld(rs + 4 * k), ld(rs + 4 * k + 2)};
-                    const float4 *qk = T.qdf + (size_t)k * M * P.n_q + i;
-                    for (int m = 0; m < M; ++m) {
-                        const float4 q0 = qk[(size_t)m * P.n_q], q1 = qk[(size_t)m * P.n_q + 1];
-                        const df r0{q0.x, q0.y}, r1{q1.x, q1.y}, i0{q0.z, q0.w}, i1{q1.z, q1.w};
-                        const df qre = df_add(r0, df_mul(f, df_sub(r1, r0)));
-                        const df qim = df_add(i0, df_mul(f, df_sub(i1, i0)));
-                        // Y_lm = d_lm exp(-i m phi): the table entry for m >= 0, its conjugate for m < 0
-                        const int mm = P.mode_m[m], a = mm < 0 ? -mm : mm;
-                        const df d = ld(rdl + 2 * m);
-                        df er = ld(rph + 4 * a), ei = ld(rph + 4 * a + 2);
-                        if (mm < 0)
-                            ei = {-ei.hi, -ei.lo};
-                        const dfc c = dfc_mul(sk, dfc{df_mul(d, er), df_mul(d, ei)});
-                        acc = df_add(acc, df_add(df_mul(c.re, qre), df_mul(c.im, qim)));
+                df f[kMaxDet];
+                int i[kMaxDet];
+                dfc w[kMaxDet];
+#pragma unroll
+                for (int k = 0; k < kMaxDet; ++k) {
+                    w[k] = {{0.f, 0.f}, {0.f, 0.f}};
+                    f[k] = {0.f, 0.f};
+                    i[k] = 0;
+                    if (k < K) {
+                        const double u = rd[k * 32 + lane] + (double)j * beta;
+                        const double fl = floor(u);
+                        if (!(fl >= 0.0) || fl + 1.0 > (double)(P.n_q - 1)) {
+                            good = false;
+                        } else {
+                            i[k] = (int)fl;
+                            f[k] = df_of(u - fl);
+                        }
                     }
                 }
+                for (int m = 0; m < M && good; ++m) {
+                    // Y_lm = d_lm exp(-i m phi): the table entry for m >= 0, its conjugate for m < 0
+                    const int mm = P.mode_m[m], a = mm < 0 ? -mm : mm;
+                    const df d = ld(rdl + 2 * m);
+                    df yi = df_mul(d, ld(rph + 4 * a + 2));
+                    const df yr = df_mul(d, ld(rph + 4 * a));
+                    if (mm < 0)
+                        yi = {-yi.hi, -yi.lo};
+#pragma unroll
+                    for (int k = 0; k < kMaxDet; ++k)
+                        if (k < K) {
+                            const float4 *qk = T.qdf + ((size_t)k * M + m) * P.n_q + i[k];
+                            const float4 q0 = qk[0], q1 = qk[1];
+                            const df r0{q0.x, q0.y}, r1{q1.x, q1.y}, i0{q0.z, q0.w}, i1{q1.z, q1.w};
+                            const df qre = df_add(r0, df_mul(f[k], df_sub(r1, r0)));
+                            const df qim = df_add(i0, df_mul(f[k], df_sub(i1, i0)));
+                            df_acc(w[k].re, yr, qre);
+                            df_acc(w[k].re, yi, qim);
+                            df_acc(w[k].im, yr, qim);
+                            df_acc(w[k].im, {-yi.hi, -yi.lo}, qre);
+                        }
+                }
+                df acc = {0.f, 0.f};
+#pragma unroll
+                for (int k = 0; k < kMaxDet; ++k)
+                    if (k < K)
+                        acc = df_add(acc, df_add(df_mul(ld(rs + 4 * k), df_norm(w[k].re)),
+                                                 df_mul(ld(rs + 4 * k + 2), df_norm(w[k].im))));
                 if (good)
                     corr = ((double)po.q[g] - rd[K * 32 + lane]) + (df_to_double(acc) - (double)po.m[g]);
             }
@@ -417,11 +497,12 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
     }
 }
 
-cudaError_t launch_fix_prep(const Problem &P, FixTables T, float4 *ua, float4 *vb, float4 *qdf, cudaStream_t st)
+cudaError_t launch_fix_prep(const Problem &P, FixTables T, cudaStream_t st)
 {
-    const int64_t total = (int64_t)P.K * (T.nA + T.nB) + (int64_t)P.K * P.M * P.n_q;
-    const int grid = (int)std::min<int64_t>((total + 255) / 256, 4096);
-    fix_prep_kernel<<<grid, 256, 0, st>>>(P.U64, P.V64, P.Q64, P.K, P.M, P.n_q, T, ua, vb, qdf);
+    const int64_t nq = (int64_t)P.K * P.M * P.n_q;
+    fix_prep_q_kernel<<<(int)std::min<int64_t>((nq + 255) / 256, 4096), 256, 0, st>>>(P.Q64, nq, T.qdf);
+    const int rows = P.K * (3 * T.dmax + 2) * T.nf;
+    fix_prep_template_kernel<<<(rows + 7) / 8, 256, 0, st>>>(P, T);
     return cudaGetLastError();
 }
 
@@ -438,13 +519,13 @@ cudaError_t launch_fix(const Problem &P, BinTable bt, FixTables T, const double 
     int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    // one block per SM with as many warps as its shared memory holds (the pair tables are
+    // one block per SM with as many warps as its shared memory holds (the coefficients are
     // staged once per block, the per-warp scratch grows with the warps): latency-bound
     // double-float chains want the warps
     int max_smem = 0;
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const size_t wbytes = fix_warp_bytes(P.K, P.M, T.dmax);
-    const size_t tbytes = (size_t)P.K * (T.nA + T.nB) * 16 + (size_t)(T.nA + T.nB) * 2;
+    const size_t wbytes = fix_warp_bytes(P.K, P.M, T.dmax, T.nf);
+    const size_t tbytes = (size_t)P.K * (3 * T.dmax + 2) * T.nf * 16;
     int nw = kFixMaxWarps;
     while (nw > 1 && wbytes * nw + tbytes > (size_t)max_smem)
         --nw;
