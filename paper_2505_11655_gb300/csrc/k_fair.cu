@@ -19,7 +19,9 @@ namespace rift {
 
 __device__ __forceinline__ uint64_t fix_weight(double x, double mx, int S)
 {
-    if (!isfinite(x))
+    // (below 2^-(S + 1) the weight is 0: no exponential, which is some forty operations on this
+    // part's slow float64 pipe)
+    if (!isfinite(x) || x - mx < -0.693147180559945 * (S + 1))
         return 0ull;
     return (uint64_t)ldexp(exp(x - mx), S);
 }
@@ -75,12 +77,19 @@ __global__ void fair_select_kernel(const uint64_t *__restrict__ W, const uint64_
     }
 }
 
-// One warp per draw: the time bin from the draw's per-bin ln L (row of n_t values).
-__global__ void fair_time_kernel(const double *__restrict__ lnL_t, int64_t m, int n_t, int S2,
+// One warp per draw: the time bin from the draw's per-bin ln L (row of n_t values); the bins'
+// weights wait in shared memory for the second walk (4000 draws of 401 bins 150 us with every
+// weight computed twice).
+constexpr int kFairWarps = 4;
+constexpr int kFairCached = 2048;   // time bins
+__global__ void __launch_bounds__(32 * kFairWarps) fair_time_kernel(const double *__restrict__ lnL_t, int64_t m, int n_t, int S2,
                                  const uint64_t *__restrict__ U_time, double t_lo, double t_step,
                                  int32_t *__restrict__ j_out, double *__restrict__ t_out)
 {
+    extern __shared__ uint64_t fws[];
     const int lane = threadIdx.x & 31;
+    const bool cached = n_t <= kFairCached;
+    uint64_t *ws = fws + (cached ? (size_t)(threadIdx.x >> 5) * n_t : 0);
     const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
     for (int64_t d = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); d < m; d += warps) {
         const double *row = lnL_t + (size_t)d * n_t;
@@ -92,8 +101,12 @@ __global__ void fair_time_kernel(const double *__restrict__ lnL_t, int64_t m, in
         for (int o = 16; o; o >>= 1)
             mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, o));
         uint64_t tot = 0;
-        for (int j = lane; j < n_t; j += 32)
-            tot += fix_weight(row[j], mx, S2);
+        for (int j = lane; j < n_t; j += 32) {
+            const uint64_t w = fix_weight(row[j], mx, S2);
+            if (cached)
+                ws[j] = w;
+            tot += w;
+        }
 #pragma unroll
         for (int o = 16; o; o >>= 1)
             tot += __shfl_xor_sync(0xffffffffu, tot, o);
@@ -103,7 +116,7 @@ __global__ void fair_time_kernel(const double *__restrict__ lnL_t, int64_t m, in
             uint64_t base = 0;
             for (int j0 = 0; j0 < n_t; j0 += 32) {
                 const int j = j0 + lane;
-                const uint64_t w = j < n_t ? fix_weight(row[j], mx, S2) : 0ull;
+                const uint64_t w = j >= n_t ? 0ull : cached ? ws[j] : fix_weight(row[j], mx, S2);   // (this lane wrote it)
                 uint64_t inc = w;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -166,7 +179,13 @@ cudaError_t launch_fair_time(const double *lnL_t, int64_t m, int n_t, const uint
 {
     if (m <= 0)
         return cudaSuccess;
-    fair_time_kernel<<<blocks_for(m * 32, 256), 256, 0, st>>>(lnL_t, m, n_t, fix_shift(n_t), U_time, t_lo, t_step,
+    const size_t smem = n_t <= kFairCached ? sizeof(uint64_t) * kFairWarps * n_t : 0;
+    if (smem > 48 * 1024) {
+        cudaError_t e = allow_max_dynamic_smem(fair_time_kernel);
+        if (e != cudaSuccess)
+            return e;
+    }
+    fair_time_kernel<<<blocks_for(m * 32, 32 * kFairWarps), 32 * kFairWarps, smem, st>>>(lnL_t, m, n_t, fix_shift(n_t), U_time, t_lo, t_step,
                                                               j_out, t_out);
     return cudaGetLastError();
 }
