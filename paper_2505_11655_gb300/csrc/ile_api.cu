@@ -1042,10 +1042,11 @@ int rift_ile_set_waveforms(rift_ile_t *h, int32_t n_freq, const double *freqs, c
     if (rc == RIFT_OK && info.bad != ~0ull)
         rc = (info.bad & 3ull) == (unsigned)kWaveformNonFinite ? RIFT_ENONFINITE : RIFT_EINVAL;
     FftPlan plan{};
-    bool use_fft = rc == RIFT_OK && info.L > 0 &&
+    const int lattice = info.off ? 0 : waveform_lattice(h->prob.fs, info.gap);
+    bool use_fft = rc == RIFT_OK && lattice > 0 &&
                    !(std::getenv("RIFT_ILE_DFT") && std::getenv("RIFT_ILE_DFT")[0] == '1');
     if (use_fft) {
-        plan.L = info.L;
+        plan.L = lattice;
         plan.f0 = info.f0;
         plan.nidx = nidx;
         const bool pruned = fft_pruned(plan.L, h->prob.n_q);

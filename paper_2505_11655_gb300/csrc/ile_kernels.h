@@ -58,11 +58,14 @@ bool fft_pruned(int L, int n_q, int *P = nullptr, int *R = nullptr);
 // Checks of the frequency-domain inputs, on the device.
 constexpr int kWaveformInvalid = 1, kWaveformNonFinite = 2;
 struct WaveformInfo {
-    unsigned long long bad;   // first violation (see waveform_check_kernel), ~0: none
+    unsigned long long bad;    // first violation (see waveform_check_kernel), ~0: none
+    unsigned long long gap;    // bits of the smallest step (0: not ascending)
+    unsigned long long fmax;   // bits of the largest |f|
     double f0;
-    int L;                    // lattice length, 0: not on a lattice
+    int off;                   // a frequency lies off the lattice of that step
     int unused;
 };
+int waveform_lattice(double fs, unsigned long long gap);   // L = f_s / step (0: no power of two)
 cudaError_t launch_waveform_check(const double *f, const double *w, int K, int F, double fs, int *nidx,
                                   WaveformInfo *info, cudaStream_t st);
 size_t uv_scratch_doubles(int K, int M, int F);

@@ -25,6 +25,7 @@
 // of two) the direct sum.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "ile_kernels.h"
 
@@ -185,22 +186,30 @@ __global__ void __launch_bounds__(kUvThreads) uv_partial_kernel(const double2 *_
     }
 }
 
-__global__ void uv_final_kernel(const double *__restrict__ part, int nch, int M, double2 *__restrict__ U,
+// One warp per (detector, pair): the blocks' sums in a fixed order.
+__global__ void uv_final_kernel(const double *__restrict__ part, int nch, int K, int M, double2 *__restrict__ U,
                                 double2 *__restrict__ V)
 {
-    const int k = blockIdx.y, pairs = M * (M + 1) / 2;
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= pairs)
+    const int lane = threadIdx.x & 31, pairs = M * (M + 1) / 2;
+    const int e = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (e >= K * pairs)
         return;
+    const int k = e / pairs, p = e - k * pairs;
     int a, b;
     uv_pair(p, M, a, b);
     double v[4] = {0.0, 0.0, 0.0, 0.0};
     const double *q = part + (size_t)k * nch * 4 * pairs + p;
-#pragma unroll 8
-    for (int c = 0; c < nch; ++c)
+    for (int c = lane; c < nch; c += 32)
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            v[e] += q[(size_t)(4 * c + e) * pairs];
+        for (int i = 0; i < 4; ++i)
+            v[i] += q[(size_t)(4 * c + i) * pairs];
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
+    if (lane)
+        return;
     if (a == b)
         v[1] = 0.0;   // w |h|^2 is real (the fused products leave a rounding residual)
     const size_t ab = ((size_t)k * M + a) * M + b, ba = ((size_t)k * M + b) * M + a;
@@ -429,79 +438,76 @@ __global__ void fft_combine_kernel(const double2 *__restrict__ Z, int KM, int P,
 
 // Weights finite, non-negative and symmetric in f, frequencies finite and mirror-symmetric:
 // the first violation in the order of a loop over j, then the frequency, then the detectors, as
-// 4 (j (K + 1) + [0 frequency, 1 + k weights]) + code.
+// 4 (j (K + 1) + [0 frequency, 1 + k weights]) + code; and the smallest step and largest modulus of
+// the frequencies (non-negative doubles order like their bits).
 __global__ void waveform_check_kernel(const double *__restrict__ f, const double *__restrict__ w, int K, int F,
                                       WaveformInfo *__restrict__ info)
 {
-    unsigned long long bad = ~0ull;
+    unsigned long long bad = ~0ull, gap = ~0ull, fm = 0ull;
     const int64_t total = (int64_t)(K + 1) * F;
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
         const int c = (int)(e / F), j = (int)(e - (int64_t)c * F);
         const double *row = c == 0 ? f : w + (size_t)(c - 1) * F;
         const double a = row[j], b = row[F - 1 - j];
         int code = 0;
-        if (c == 0)
+        if (c == 0) {
             code = !isfinite(a) || b != -a ? kWaveformInvalid : 0;
-        else
+            fm = max(fm, (unsigned long long)__double_as_longlong(fabs(a)));
+            if (j > 0) {
+                const double g = a - row[j - 1];
+                gap = min(gap, g > 0.0 ? (unsigned long long)__double_as_longlong(g) : 0ull);
+            }
+        } else
             code = !isfinite(a) ? kWaveformNonFinite : a < 0.0 || a != b ? kWaveformInvalid : 0;
         if (code)
             bad = min(bad, 4ull * ((unsigned long long)j * (K + 1) + c) + code);
     }
     if (bad != ~0ull)
         atomicMin(&info->bad, bad);
+#pragma unroll
+    for (int o = 16; o; o >>= 1) {
+        gap = min(gap, __shfl_xor_sync(0xffffffffu, gap, o));
+        fm = max(fm, __shfl_xor_sync(0xffffffffu, fm, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        if (gap != ~0ull)
+            atomicMin(&info->gap, gap);
+        if (fm)
+            atomicMax(&info->fmax, fm);
+    }
 }
 
-// One block: the lattice f_j = f_0 + n_j df (df the smallest step; ascending frequencies, integers
-// n_j to 1e-9 relative, L = f_s / df a power of two above every n_j); n_j to nidx, L to info (0:
-// not on a lattice).
-__global__ void __launch_bounds__(1024) waveform_lattice_kernel(const double *__restrict__ f, int F, double fs,
-                                                                int *__restrict__ nidx, WaveformInfo *__restrict__ info)
+int waveform_lattice(double fs, unsigned long long gap)
 {
-    __shared__ unsigned long long gap_s, fmax_s;   // non-negative doubles order like their bits
-    __shared__ int off_s;
-    if (threadIdx.x == 0) {
-        gap_s = ~0ull;
-        fmax_s = 0ull;
-        off_s = 0;
-    }
-    __syncthreads();
-    unsigned long long gap = ~0ull, fm = 0ull;
-    bool off = false;
-    for (int j = threadIdx.x; j < F; j += blockDim.x) {
-        fm = max(fm, (unsigned long long)__double_as_longlong(fabs(f[j])));
-        if (j > 0) {
-            const double g = f[j] - f[j - 1];
-            if (g > 0.0)
-                gap = min(gap, (unsigned long long)__double_as_longlong(g));
-            else
-                off = true;
-        }
-    }
-    atomicMin(&gap_s, gap);
-    atomicMax(&fmax_s, fm);
-    if (off)
-        off_s = 1;
-    __syncthreads();
-    const double df = __longlong_as_double((long long)gap_s), fmax = __longlong_as_double((long long)fmax_s);
-    const double Lr = off_s ? 0.0 : fs / df;
-    const long long L = Lr < 1e9 ? llround(Lr) : 0;   // (a NaN ratio: 0)
-    if (off_s || L < 2 || L > (1ll << 26) || (L & (L - 1)) != 0 || !(fabs(Lr - (double)L) <= 1e-9 * (double)L))
-        return;
-    off = false;
-    for (int j = threadIdx.x; j < F; j += blockDim.x) {
-        const long long n = llround((f[j] - f[0]) / df);
-        if (fabs(f[j] - f[0] - (double)n * df) > 1e-9 * (fmax > 1.0 ? fmax : 1.0) || n < 0 || n >= L)
+    double df;
+    memcpy(&df, &gap, 8);
+    if (!(df > 0.0) || !(fs / df < 1e9))
+        return 0;
+    const double Lr = fs / df;
+    const long long L = std::llround(Lr);
+    return L >= 2 && L <= (1ll << 26) && (L & (L - 1)) == 0 && std::fabs(Lr - (double)L) <= 1e-9 * (double)L ? (int)L : 0;
+}
+
+// The lattice f_j = f_0 + n_j df (df the smallest step; ascending frequencies, integers n_j to
+// 1e-9 relative, below L = f_s / df): n_j to nidx, info->off set when a frequency lies off it.
+__global__ void waveform_lattice_kernel(const double *__restrict__ f, int F, double fs, int *__restrict__ nidx,
+                                        WaveformInfo *__restrict__ info)
+{
+    const double df = __longlong_as_double((long long)info->gap), fmax = __longlong_as_double((long long)info->fmax);
+    const double f0 = f[0];
+    bool off = !(df > 0.0) || !(fs / df < 1e9);
+    const long long L = off ? 0 : llround(fs / df);
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < F; j += gridDim.x * blockDim.x) {
+        const long long n = off ? -1 : llround((f[j] - f0) / df);
+        if (n < 0 || n >= L || fabs(f[j] - f0 - (double)n * df) > 1e-9 * (fmax > 1.0 ? fmax : 1.0))
             off = true;
         else
             nidx[j] = (int)n;
     }
     if (off)
-        off_s = 1;
-    __syncthreads();
-    if (threadIdx.x == 0 && !off_s) {
-        info->L = (int)L;
-        info->f0 = f[0];
-    }
+        info->off = 1;
+    if (blockIdx.x == 0 && threadIdx.x == 0)
+        info->f0 = f0;
 }
 
 cudaError_t launch_waveform_check(const double *f, const double *w, int K, int F, double fs, int *nidx,
@@ -509,12 +515,12 @@ cudaError_t launch_waveform_check(const double *f, const double *w, int K, int F
 {
     cudaError_t e = cudaMemsetAsync(info, 0, sizeof(WaveformInfo), st);
     if (e == cudaSuccess)
-        e = cudaMemsetAsync(&info->bad, 0xff, sizeof(info->bad), st);
+        e = cudaMemsetAsync(&info->bad, 0xff, 2 * sizeof(info->bad), st);   // bad and gap
     if (e != cudaSuccess)
         return e;
     const int64_t total = (int64_t)(K + 1) * F;
     waveform_check_kernel<<<(int)std::min<int64_t>((total + 255) / 256, 152 * 8), 256, 0, st>>>(f, w, K, F, info);
-    waveform_lattice_kernel<<<1, 1024, 0, st>>>(f, F, fs, nidx, info);
+    waveform_lattice_kernel<<<std::min((F + 255) / 256, 152 * 8), 256, 0, st>>>(f, F, fs, nidx, info);
     return cudaGetLastError();
 }
 
@@ -577,7 +583,7 @@ cudaError_t launch_precompute(const double2 *h, const double2 *d, const double *
     if (uv_smem > 40 * 1024 && (e = allow_max_dynamic_smem(uv_partial_kernel)) != cudaSuccess)
         return e;   // (beside the static array of the pairs' threads)
     uv_partial_kernel<<<dim3(nch, K), kUvThreads, uv_smem, st>>>(h, w, M, F, uv_scratch);
-    uv_final_kernel<<<dim3((pairs + 63) / 64, K), 64, 0, st>>>(uv_scratch, nch, M, U, V);
+    uv_final_kernel<<<(K * pairs + 7) / 8, 256, 0, st>>>(uv_scratch, nch, K, M, U, V);
     if (launched)
         *launched = k + 2;
     return cudaGetLastError();
