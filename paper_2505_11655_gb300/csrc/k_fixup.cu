@@ -166,9 +166,14 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
     const double beta = P.t_step * P.fs;
     const uint32_t cnt = *count;
     const int nw = (int)(blockDim.x >> 5);
-    // batch b of 32 listed samples goes to block b % gridDim.x, warp b / gridDim.x (round
+    // A lane corrects a sample of its own, or eight lanes share one when the list fits the grid
+    // that way: they split the angles, detectors, modes and azimuthal orders, and a short list
+    // takes the latency of a few of these instead of all.
+    const int gsh = (int64_t)cnt <= (int64_t)gridDim.x * nw * 4 ? 3 : 0, G = 1 << gsh, spw = 32 >> gsh;
+    const int col = lane >> gsh, sub = lane & (G - 1);
+    // batch b of spw listed samples goes to block b % gridDim.x, warp b / gridDim.x (round
     // robin over the blocks first, so that a short list still spreads over every SM)
-    if ((int64_t)blockIdx.x * 32 >= (int64_t)cnt)
+    if ((int64_t)blockIdx.x * spw >= (int64_t)cnt)
         return;   // no listed sample for this block (the grid is sized for every sample)
     // the template coefficients of every detector, staged once per block
     const int na = nph, ns = 2 * T.dmax + 1;
@@ -180,37 +185,62 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
         shb[e] = T.hb[e];
     __syncthreads();
     // this lane's sample: the double-float value at rows (row, row + 1)
-    auto ld = [&](int row) { return df{rf[row * 32 + lane], rf[(row + 1) * 32 + lane]}; };
+    auto ld = [&](int row) { return df{rf[row * 32 + col], rf[(row + 1) * 32 + col]}; };
+    auto st = [&](int row, double v) {
+        const df d = df_of(v);
+        rf[row * 32 + col] = d.hi;
+        rf[(row + 1) * 32 + col] = d.lo;
+    };
+    // sums over the lanes of a sample
+    auto join = [&](df v) {
+        for (int o = 1; o < G; o <<= 1)
+            v = df_add(v, df_shfl_xor(v, o));
+        return v;
+    };
 
-    for (int64_t base = ((int64_t)warp * gridDim.x + blockIdx.x) * 32; base < (int64_t)cnt;
-         base += (int64_t)gridDim.x * nw * 32) {
-        const int64_t e = base + lane;
+    for (int64_t base = ((int64_t)warp * gridDim.x + blockIdx.x) * spw; base < (int64_t)cnt;
+         base += (int64_t)gridDim.x * nw * spw) {
+        const int64_t e = base + col;
         const bool active = e < (int64_t)cnt;
         const uint32_t g = active ? idx[e] : 0u;
 
-        // ---- phase A, one sample per lane: geometry in float64, rounded to double-float
+        // ---- phase A: geometry in float64, rounded to double-float
         {
             double th[6] = {0.0, 0.0, 0.0, 0.0, 0.0, P.d_ref};   // inert values on idle lanes
             if (active)
                 for (int d = 0; d < 6; ++d)
                     th[d] = theta[6 * (int64_t)g + d];
-            const Sky sky = sky_of(th[0], th[1], P.gmst);
+            Sky sky;
+            double s2p, c2p, si, ci, sp, cp;
+            if (G == 1) {
+                sky = sky_of(th[0], th[1], P.gmst);
+                sincos(2.0 * th[2], &s2p, &c2p);
+                sincos(th[4], &si, &ci);
+                sincos(th[3], &sp, &cp);
+            } else {   // an angle per lane
+                double sn, cs;
+                sincos(sub == 0 ? th[1] : sub == 1 ? th[0] - P.gmst : sub == 2 ? 2.0 * th[2] : sub == 3 ? th[4] : th[3], &sn, &cs);
+                const int l0 = lane & ~7;
+                sky.sd = __shfl_sync(0xffffffffu, sn, l0);
+                sky.cd = __shfl_sync(0xffffffffu, cs, l0);
+                sky.sh = __shfl_sync(0xffffffffu, sn, l0 + 1);
+                sky.ch = __shfl_sync(0xffffffffu, cs, l0 + 1);
+                s2p = __shfl_sync(0xffffffffu, sn, l0 + 2);
+                c2p = __shfl_sync(0xffffffffu, cs, l0 + 2);
+                si = __shfl_sync(0xffffffffu, sn, l0 + 3);
+                ci = __shfl_sync(0xffffffffu, cs, l0 + 3);
+                sp = __shfl_sync(0xffffffffu, sn, l0 + 4);
+                cp = __shfl_sync(0xffffffffu, cs, l0 + 4);
+            }
             const double n0 = sky.cd * sky.ch, n1 = sky.cd * sky.sh, n2 = sky.sd;
-            double s2p, c2p;
-            sincos(2.0 * th[2], &s2p, &c2p);
             const double x = P.d_ref / th[5];
-            for (int k = 0; k < K; ++k) {
-                rd[k * 32 + lane] = fma(P.xfs[k][0], n0, fma(P.xfs[k][1], n1, fma(P.xfs[k][2], n2, P.ufs0[k])));
+            for (int k = sub; k < K; k += G) {
+                rd[k * 32 + col] = fma(P.xfs[k][0], n0, fma(P.xfs[k][1], n1, fma(P.xfs[k][2], n2, P.ufs0[k])));
                 const Cx<double> F = response<double>(P, k, sky, c2p, s2p);
-                const df sr = df_of(x * F.re), si = df_of(x * F.im);
-                rf[(rs + 4 * k) * 32 + lane] = sr.hi;
-                rf[(rs + 4 * k + 1) * 32 + lane] = sr.lo;
-                rf[(rs + 4 * k + 2) * 32 + lane] = si.hi;
-                rf[(rs + 4 * k + 3) * 32 + lane] = si.lo;
+                st(rs + 4 * k, x * F.re);
+                st(rs + 4 * k + 2, x * F.im);
             }
             // cos and sin of n iota by powers of exp(i iota), and the polar functions from them
-            double si, ci;
-            sincos(th[4], &si, &ci);
             double cn[kMaxL + 1], sn[kMaxL + 1], tr = 1.0, ti = 0.0;
 #pragma unroll
             for (int nn = 0; nn <= 2 * kMaxL; ++nn) {
@@ -220,35 +250,30 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                     cn[nn <= kMaxL ? nn : 0] = tr;
                     sn[nn <= kMaxL ? nn : 0] = ti;
                 }
-                const df a = df_of(tr), b = df_of(ti);
-                rf[(rtr + 2 * nn) * 32 + lane] = a.hi;
-                rf[(rtr + 2 * nn + 1) * 32 + lane] = a.lo;
-                rf[(rtr + 2 * NF + 2 * nn) * 32 + lane] = b.hi;
-                rf[(rtr + 2 * NF + 2 * nn + 1) * 32 + lane] = b.lo;
+                if (sub == 0) {
+                    st(rtr + 2 * nn, tr);
+                    st(rtr + 2 * NF + 2 * nn, ti);
+                }
                 const double t = tr * ci - ti * si;
                 ti = ti * ci + tr * si;
                 tr = t;
             }
-            for (int m = 0; m < M; ++m) {
+            for (int m = sub; m < M; m += G) {
                 const double *al = T.alpha + m * (kMaxL + 1);
+                const bool odd = P.mode_m[m] & 1;
                 double d = 0.0;
 #pragma unroll
                 for (int u = 0; u <= kMaxL; ++u)
                     if (2 * u < NF)
-                        d = fma(al[u], (P.mode_m[m] & 1) ? sn[u] : cn[u], d);
-                const df dd = df_of(d);
-                rf[(rdl + 2 * m) * 32 + lane] = dd.hi;
-                rf[(rdl + 2 * m + 1) * 32 + lane] = dd.lo;
+                        d = fma(al[u], odd ? sn[u] : cn[u], d);
+                st(rdl + 2 * m, d);
             }
-            double sp, cp;
-            sincos(th[3], &sp, &cp);
             double er = 1.0, ei = 0.0;   // exp(-i n phi), n = 0, 1, ...
             for (int nn = 0; nn < nph; ++nn) {
-                const df a = df_of(er), b = df_of(ei);
-                rf[(rph + 4 * nn) * 32 + lane] = a.hi;
-                rf[(rph + 4 * nn + 1) * 32 + lane] = a.lo;
-                rf[(rph + 4 * nn + 2) * 32 + lane] = b.hi;
-                rf[(rph + 4 * nn + 3) * 32 + lane] = b.lo;
+                if (sub == 0) {
+                    st(rph + 4 * nn, er);
+                    st(rph + 4 * nn + 2, ei);
+                }
                 const double t = er * cp + ei * sp;
                 ei = ei * cp - er * sp;
                 er = t;
@@ -256,7 +281,7 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
         }
         __syncwarp();
 
-        // ---- the template term in double-float, one sample per lane
+        // ---- the template term in double-float
         {
             df A[kMaxDet];
             dfc B[kMaxDet];
@@ -265,7 +290,7 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                 A[k] = {0.f, 0.f};
                 B[k] = {{0.f, 0.f}, {0.f, 0.f}};
             }
-            for (int D = 0; D <= T.dmax; ++D) {
+            for (int D = sub; D <= T.dmax; D += G) {
                 dfc G[kMaxDet];
 #pragma unroll
                 for (int k = 0; k < kMaxDet; ++k)
@@ -298,7 +323,7 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                         }
                     }
             }
-            for (int S = -T.dmax; S <= T.dmax; ++S) {
+            for (int S = sub - T.dmax; S <= T.dmax; S += G) {
                 dfc H[kMaxDet];
 #pragma unroll
                 for (int k = 0; k < kMaxDet; ++k)
@@ -331,6 +356,13 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                         B[k].im = df_add(B[k].im, t.im);
                     }
             }
+            __syncwarp();
+#pragma unroll
+            for (int k = 0; k < kMaxDet; ++k)
+                if (k < K) {
+                    A[k] = join(A[k]);
+                    B[k] = {join(B[k].re), join(B[k].im)};
+                }
             // quad = kappa sum_k |s_k|^2 A_k + Re(s_k^2 B_k)
             df q = {0.f, 0.f};
 #pragma unroll
@@ -342,18 +374,18 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                     q = df_add(q, df_mul(abs2, A[k]));
                     q = df_add(q, df_sub(df_mul(s2r, B[k].re), df_mul(s2i, B[k].im)));
                 }
-            rd[K * 32 + lane] = P.kappa * df_to_double(q);
+            rd[K * 32 + col] = P.kappa * df_to_double(q);
         }
         __syncwarp();
 
         // ---- phase B: the bin of the largest data term in the kernel's block (float32
         // search; lanes = (sample, bin of the block) pairs), then the data term there in
         // double-float, one sample per lane
-        const int nb = (int)((int64_t)cnt - base < 32 ? (int64_t)cnt - base : 32);
+        const int nb = (int)((int64_t)cnt - base < spw ? (int64_t)cnt - base : spw);
         int *jbest = reinterpret_cast<int *>(c32);   // [32] the bin each sample is evaluated at
         if (blen <= 1) {
-            if (lane < nb)
-                jbest[lane] = po.j[g];
+            if (col < nb && sub == 0)
+                jbest[col] = po.j[g];
         } else {
             int lps = 1;   // lanes per sample: the block length rounded up to a power of two
             while (lps < blen)
@@ -361,7 +393,7 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
             const int spr = 32 / lps;   // samples per round
             for (int r0 = 0; r0 < nb; r0 += spr) {
                 const int t = r0 + lane / lps, b = lane % lps;
-                const uint32_t gt = __shfl_sync(0xffffffffu, g, t & 31);
+                const uint32_t gt = __shfl_sync(0xffffffffu, g, (t << gsh) & 31);
                 float best = -INFINITY;
                 int bj = INT_MAX;
                 if (t < nb && b < blen) {
@@ -417,21 +449,23 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
         __syncwarp();
         double corr = 0.0;
         bool good = false;
-        if (lane < nb) {
-            const int j = jbest[lane];
+        {
+            const int j = col < nb ? jbest[col] : INT_MAX;
+            dfc w[kMaxDet];
+#pragma unroll
+            for (int k = 0; k < kMaxDet; ++k)
+                w[k] = {{0.f, 0.f}, {0.f, 0.f}};
             if (j != INT_MAX) {
                 // lin = sum_k Re(conj(s_k) sum_m conj(Y_m) Q_k,m), Q interpolated at the bin
                 good = true;
                 df f[kMaxDet];
                 int i[kMaxDet];
-                dfc w[kMaxDet];
 #pragma unroll
                 for (int k = 0; k < kMaxDet; ++k) {
-                    w[k] = {{0.f, 0.f}, {0.f, 0.f}};
                     f[k] = {0.f, 0.f};
                     i[k] = 0;
                     if (k < K) {
-                        const double u = rd[k * 32 + lane] + (double)j * beta;
+                        const double u = rd[k * 32 + col] + (double)j * beta;
                         const double fl = floor(u);
                         if (!(fl >= 0.0) || fl + 1.0 > (double)(P.n_q - 1)) {
                             good = false;
@@ -441,7 +475,7 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                         }
                     }
                 }
-                for (int m = 0; m < M && good; ++m) {
+                for (int m = sub; m < M && good; m += G) {
                     // Y_lm = d_lm exp(-i m phi): the table entry for m >= 0, its conjugate for m < 0
                     const int mm = P.mode_m[m], a = mm < 0 ? -mm : mm;
                     const df d = ld(rdl + 2 * m);
@@ -463,18 +497,19 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
                             df_acc(w[k].im, {-yi.hi, -yi.lo}, qre);
                         }
                 }
-                df acc = {0.f, 0.f};
-#pragma unroll
-                for (int k = 0; k < kMaxDet; ++k)
-                    if (k < K)
-                        acc = df_add(acc, df_add(df_mul(ld(rs + 4 * k), df_norm(w[k].re)),
-                                                 df_mul(ld(rs + 4 * k + 2), df_norm(w[k].im))));
-                if (good)
-                    corr = ((double)po.q[g] - rd[K * 32 + lane]) + (df_to_double(acc) - (double)po.m[g]);
             }
-            if (!good) {
+            __syncwarp();
+            df acc = {0.f, 0.f};
+#pragma unroll
+            for (int k = 0; k < kMaxDet; ++k)
+                if (k < K)
+                    acc = df_add(acc, df_add(df_mul(ld(rs + 4 * k), join(df_norm(w[k].re))),
+                                             df_mul(ld(rs + 4 * k + 2), join(df_norm(w[k].im)))));
+            if (good)
+                corr = ((double)po.q[g] - rd[K * 32 + col]) + (df_to_double(acc) - (double)po.m[g]);
+            if (col < nb && !good) {
                 atomicOr(err, kErrRange);
-            } else {
+            } else if (col < nb && sub == 0) {
                 const double r = lnL_tmarg[g] + corr;
                 if (!isfinite(r))
                     atomicOr(err, kErrNonFinite);
@@ -486,9 +521,9 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
         if (lnL_t) {
             // the per-bin values of the warp's samples move by the same amount
             for (int t = 0; t < nb; ++t) {
-                const uint32_t gt = __shfl_sync(0xffffffffu, g, t);
-                const double ct = __shfl_sync(0xffffffffu, corr, t);
-                if (__shfl_sync(0xffffffffu, good ? 1 : 0, t))
+                const uint32_t gt = __shfl_sync(0xffffffffu, g, t << gsh);
+                const double ct = __shfl_sync(0xffffffffu, corr, t << gsh);
+                if (__shfl_sync(0xffffffffu, good ? 1 : 0, t << gsh))
                     for (int j = lane; j < NT; j += 32)
                         lnL_t[(int64_t)gt * NT + j] += ct;
             }
@@ -529,8 +564,7 @@ cudaError_t launch_fix(const Problem &P, BinTable bt, FixTables T, const double 
     int nw = kFixMaxWarps;
     while (nw > 1 && wbytes * nw + tbytes > (size_t)max_smem)
         --nw;
-    const int64_t per_block = 32 * nw;
-    const int grid = (int)std::min<int64_t>((n + per_block - 1) / per_block, (int64_t)sms);
+    const int grid = (int)std::min<int64_t>((n + 3) / 4, (int64_t)sms);
     const size_t smem = wbytes * nw + tbytes;
     fix_kernel<<<grid, 32 * nw, smem, st>>>(P, bt, T, theta, idx, count, po, blen, lnL_tmarg, lnL_t, lnpw,
                                                     lnw, err);
