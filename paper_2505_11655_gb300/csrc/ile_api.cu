@@ -776,6 +776,13 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
                           alpha.data() + (size_t)m * (kMaxL + 1));
         }
         const int dmax = 2 * mmax, nf = 2 * lmax + 1;
+        // behind them, their double-float parts (hi, lo)
+        const size_t na = alpha.size();
+        alpha.resize(2 * na);
+        for (size_t i = 0; i < na; ++i) {
+            const float pair[2] = {(float)alpha[i], (float)(alpha[i] - (double)(float)alpha[i])};
+            std::memcpy(&alpha[na + i], pair, sizeof(double));
+        }
         if ((rc = dalloc(h, &h->aux_q, (size_t)N)) || (rc = dalloc(h, &h->aux_m, (size_t)N)) ||
             (rc = dalloc(h, &h->aux_j, (size_t)N)) || (rc = dalloc(h, &h->fix_idx, (size_t)N)) ||
             (rc = dalloc(h, &h->fix_count, (size_t)4)) || (rc = dalloc(h, &h->fix_alpha, alpha.size())) ||
@@ -791,7 +798,7 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
             release(h);
             return RIFT_ECUDA;
         }
-        h->fix = FixTables{h->fix_alpha, h->fix_ga, h->fix_hb, h->fix_qdf, dmax, nf};
+        h->fix = FixTables{h->fix_alpha, reinterpret_cast<const float2 *>(h->fix_alpha + na), h->fix_ga, h->fix_hb, h->fix_qdf, dmax, nf};
         // samples with quad32 + |max lin32| above this are corrected: below it the float32
         // rounding stays under 5e-4 (measured, ~3e-7 per unit of the terms at most)
         h->fix_thr = kFixThreshold;
@@ -935,7 +942,7 @@ int64_t rift_ile_footprint(const rift_ile_config *cfg)
                : 0,
         // large-term correction: per-sample side outputs and list, double-float tables of the
         // template term (at most 13 x 13 + 25 x 13 coefficients a detector) and of Q
-        cfg->precision != RIFT_FP64 && !cfg->distance_marg ? 4 * N * 4 + 16 + 8 * (kMaxL + 1) * M + 64 + K * 494 * 16 + K * M * nq * 16
+        cfg->precision != RIFT_FP64 && !cfg->distance_marg ? 4 * N * 4 + 16 + 16 * (kMaxL + 1) * M + 64 + K * 494 * 16 + K * M * nq * 16
                                                             : 0};
     int64_t total = 0;
     for (int64_t b : sizes)

@@ -124,6 +124,7 @@ constexpr int kPeakBlockTc = 4;
 // and of Q (built on the device whenever the overlaps change).  dmax = 2 max|m|, nf = 2 max l + 1.
 struct FixTables {
     const double *alpha;    // [M][kMaxL + 1]: d_m(iota) = sum_u alpha_mu cos(u iota) (m even), sin (m odd)
+    const float2 *alpha32;  // the same in double-float
     float4 *ga;             // [K][dmax + 1][nf] (re.hi, re.lo, im.hi, im.lo), see k_fixup.cu
     float4 *hb;             // [K][2 dmax + 1][nf]
     float4 *qdf;            // [K][M][n_q] Q, same layout

@@ -22,7 +22,7 @@
 //        so every G_k,D and H_k,S is one of degree 2 l_max, in cosines for even D, S and in
 //        sines for odd; their coefficients are summed once per problem in float64 (21 modes up
 //        to l = 4: 9 x 9 + 17 x 9 complex coefficients a detector in place of 2 x 231 mode pairs
-//        with a product d_a d_b each: a loud solve's 250,000 corrections 1.07 -> 0.94 ms);
+//        with a product d_a d_b each: a loud solve's 250,000 corrections 1.07 -> 0.79 ms);
 //        the bin of the block with the largest data term (a float32 search when the block
 //        holds several bins), and the data term there in double-float, from a double-float
 //        copy of Q;
@@ -168,7 +168,8 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
     const int nw = (int)(blockDim.x >> 5);
     // A lane corrects a sample of its own, or eight lanes share one when the list fits the grid
     // that way: they split the angles, detectors, modes and azimuthal orders, and a short list
-    // takes the latency of a few of these instead of all.
+    // takes the latency of a few of these instead of all (256 samples of the plain problem 45 us,
+    // now 28).
     const int gsh = (int64_t)cnt <= (int64_t)gridDim.x * nw * 4 ? 3 : 0, G = 1 << gsh, spw = 32 >> gsh;
     const int col = lane >> gsh, sub = lane & (G - 1);
     // batch b of spw listed samples goes to block b % gridDim.x, warp b / gridDim.x (round
@@ -186,8 +187,8 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
     __syncthreads();
     // this lane's sample: the double-float value at rows (row, row + 1)
     auto ld = [&](int row) { return df{rf[row * 32 + col], rf[(row + 1) * 32 + col]}; };
-    auto st = [&](int row, double v) {
-        const df d = df_of(v);
+    // (the lanes of a sample write the same value, or each its own row)
+    auto put = [&](int row, df d) {
         rf[row * 32 + col] = d.hi;
         rf[(row + 1) * 32 + col] = d.lo;
     };
@@ -237,46 +238,36 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
             for (int k = sub; k < K; k += G) {
                 rd[k * 32 + col] = fma(P.xfs[k][0], n0, fma(P.xfs[k][1], n1, fma(P.xfs[k][2], n2, P.ufs0[k])));
                 const Cx<double> F = response<double>(P, k, sky, c2p, s2p);
-                st(rs + 4 * k, x * F.re);
-                st(rs + 4 * k + 2, x * F.im);
+                put(rs + 4 * k, df_of(x * F.re));
+                put(rs + 4 * k + 2, df_of(x * F.im));
             }
-            // cos and sin of n iota by powers of exp(i iota), and the polar functions from them
-            double cn[kMaxL + 1], sn[kMaxL + 1], tr = 1.0, ti = 0.0;
-#pragma unroll
-            for (int nn = 0; nn <= 2 * kMaxL; ++nn) {
-                if (nn >= NF)
-                    break;
-                if (nn <= kMaxL) {
-                    cn[nn <= kMaxL ? nn : 0] = tr;
-                    sn[nn <= kMaxL ? nn : 0] = ti;
-                }
-                if (sub == 0) {
-                    st(rtr + 2 * nn, tr);
-                    st(rtr + 2 * NF + 2 * nn, ti);
-                }
-                const double t = tr * ci - ti * si;
-                ti = ti * ci + tr * si;
-                tr = t;
+            // cos and sin of n iota by powers of exp(i iota), exp(-i n phi), and the polar functions
+            // from their Fourier coefficients, in double-float (in float64, with a conversion per
+            // value, they were half of the kernel's float64 operations)
+            dfc r{{1.f, 0.f}, {0.f, 0.f}};
+            const dfc r1{df_of(ci), df_of(si)};
+            for (int nn = 0; nn < NF; ++nn) {
+                put(rtr + 2 * nn, r.re);
+                put(rtr + 2 * NF + 2 * nn, r.im);
+                r = dfc_mul(r, r1);
             }
+            r = {{1.f, 0.f}, {0.f, 0.f}};
+            const dfc e1{df_of(cp), df_of(-sp)};
+            for (int nn = 0; nn < nph; ++nn) {
+                put(rph + 4 * nn, r.re);
+                put(rph + 4 * nn + 2, r.im);
+                r = dfc_mul(r, e1);
+            }
+            __syncwarp();
             for (int m = sub; m < M; m += G) {
-                const double *al = T.alpha + m * (kMaxL + 1);
-                const bool odd = P.mode_m[m] & 1;
-                double d = 0.0;
+                const float2 *al = T.alpha32 + m * (kMaxL + 1);
+                const int tb = rtr + ((P.mode_m[m] & 1) ? 2 * NF : 0);
+                df d{0.f, 0.f};
 #pragma unroll
                 for (int u = 0; u <= kMaxL; ++u)
                     if (2 * u < NF)
-                        d = fma(al[u], odd ? sn[u] : cn[u], d);
-                st(rdl + 2 * m, d);
-            }
-            double er = 1.0, ei = 0.0;   // exp(-i n phi), n = 0, 1, ...
-            for (int nn = 0; nn < nph; ++nn) {
-                if (sub == 0) {
-                    st(rph + 4 * nn, er);
-                    st(rph + 4 * nn + 2, ei);
-                }
-                const double t = er * cp + ei * sp;
-                ei = ei * cp - er * sp;
-                er = t;
+                        df_acc(d, ld(tb + 2 * u), {al[u].x, al[u].y});
+                put(rdl + 2 * m, df_norm(d));
             }
         }
         __syncwarp();

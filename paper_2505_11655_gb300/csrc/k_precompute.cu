@@ -381,9 +381,14 @@ __global__ void __launch_bounds__(kFftMaxThreads) fft_block_kernel(const double2
             if (j < quarter) {
                 const int kk = j & (Ns - 1);
                 v[q][0] = fx[j];
-                v[q][1] = mul(fx[j + quarter], tw(kk * step));
-                v[q][2] = mul(fx[j + 2 * quarter], tw(2 * kk * step));
-                v[q][3] = mul(fx[j + 3 * quarter], tw(3 * kk * step));
+                v[q][1] = fx[j + quarter];
+                v[q][2] = fx[j + 2 * quarter];
+                v[q][3] = fx[j + 3 * quarter];
+                if (Ns > 1) {
+                    v[q][1] = mul(v[q][1], tw(kk * step));
+                    v[q][2] = mul(v[q][2], tw(2 * kk * step));
+                    v[q][3] = mul(v[q][3], tw(3 * kk * step));
+                }
             }
         }
         __syncthreads();
