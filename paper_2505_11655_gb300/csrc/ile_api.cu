@@ -946,8 +946,11 @@ int64_t rift_ile_footprint(const rift_ile_config *cfg)
                                                             : 0};
     int64_t total = 0;
     for (int64_t b : sizes)
-        total += b + 16;
-    return total + 64 * 1024;   // event and stream bookkeeping slack
+        total += b + 16 + 255;
+    // the unused ends of the slabs (at most a quarter each, 17 of them hold fifty buffers of the
+    // largest size that shares one) and the rest of the last, event and stream
+    // bookkeeping
+    return total + 17 * (int64_t)(kSlab / 4) + (int64_t)kSlab + 64 * 1024;
 }
 
 int rift_ile_set_overlaps(rift_ile_t *h, const void *Q, const void *U, const void *V, int mem)
