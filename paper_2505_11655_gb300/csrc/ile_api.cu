@@ -421,12 +421,21 @@ int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmar
     return RIFT_OK;
 }
 
+// Cells per side of a face, at most 2^kMaxFaceOrder (19-bit keys: two digits of the sort).
+constexpr int kMaxFaceOrder = 8;
+
 // Sky grid sized for a batch of n samples.
 int grid_for_batch(rift_ile_t *h, int64_t n)
 {
     SkyGrid g = sky_grid_for(n, h->plan.per_cell);
     const Problem &P = h->prob;
     const bool delay3 = P.K >= 3 && h->plan.delay3;
+    if (P.K >= 3 && !delay3) {   // the six faces of a cube
+        g.order = 3;
+        while (g.order < kMaxFaceOrder && ((6 * (int64_t)h->plan.per_cell) << (2 * g.order)) < n)
+            ++g.order;
+        g.n_cells = 6 << (2 * g.order);
+    }
     if (P.K <= 2 || delay3) {
         g.mode = P.K == 1 ? kSortDelay1 : P.K == 2 ? kSortDelay2 : kSortDelay3;
         if (delay3) {   // as many cells as the sky grid, 8 per level of three delays
