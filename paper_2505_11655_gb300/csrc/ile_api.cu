@@ -392,6 +392,11 @@ int lnl_float64(rift_ile_t *h, const double *theta, int64_t n, bool keyed, doubl
     return RIFT_OK;
 }
 
+// Up to this many selected samples are re-evaluated by a block each in plain float64, longer lists
+// on the tensor cores (the count is on the device: each of the two kernels looks at it and leaves
+// when it is not its own).
+constexpr uint32_t kRefineFew = 512;
+
 int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg, const double *lnpw, double *lnw)
 {
     const double *key = lnw ? lnw : lnL_tmarg;
@@ -399,9 +404,11 @@ int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmar
                      h->stream));
     CK(launch_select(key, sorts_batch(h, n) ? h->perm : nullptr, n, h->stats, kScratchSlot, kMixedMargin, h->sel_idx, h->sel_count, h->stream));
     if (h->tc64_on) {
+        CK(launch_refine_few(h->prob, theta, h->sel_idx, h->sel_count, kRefineFew, lnL_tmarg, lnpw, lnw, h->err,
+                             h->stream));
         CK(launch_lnl_tc64(h->prob, h->x64, theta, h->sel_idx, n, lnL_tmarg, nullptr, lnpw, lnw, h->err,
-                           h->stream, h->sel_count));
-        h->launches += 7;
+                           h->stream, h->sel_count, kRefineFew));
+        h->launches += 8;
         return RIFT_OK;
     }
     // the tensor-core kernel recomputes the float32 per-bin ln L of the first refine_rows

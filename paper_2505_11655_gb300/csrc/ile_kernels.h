@@ -191,11 +191,11 @@ void tc64_positions(const rift_ile_config &cfg, long long *pos, long long *u0);
 size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms);
 cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half *q_dig, __half *t_dig, int *t_exp,
                              cudaStream_t st);
-// perm lists the samples (min(n, *n_dev) of them when a device count is given; null: in
-// order); outputs at the sample's index.
+// perm lists the samples (min(n, *n_dev) of them when a device count is given, none when that is
+// at most `skip`; null: in order); outputs at the sample's index.
 cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta, const uint32_t *perm, int64_t n,
                             double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
-                            cudaStream_t st, const uint32_t *n_dev = nullptr);
+                            cudaStream_t st, const uint32_t *n_dev = nullptr, uint32_t skip = 0);
 cudaError_t prepare_tc64_kernels();
 
 // Precision mode RIFT_MIXED: indices of the samples with key[i] >= stats[slot].max - margin
@@ -212,6 +212,11 @@ cudaError_t launch_select(const double *key, const uint32_t *perm, int64_t n, co
 cudaError_t launch_refine(const Problem &P, const double *theta, const uint32_t *idx, const uint32_t *count,
                           int64_t max_count, double *lnL_tmarg, const double *lnpw, double *lnw, int *err,
                           cudaStream_t st, const double *v32 = nullptr, int64_t v32_rows = 0);
+// The same for a list of at most `most` samples (else nothing), a block per sample; not with the
+// distance marginalised.
+cudaError_t launch_refine_few(const Problem &P, const double *theta, const uint32_t *idx, const uint32_t *count,
+                              uint32_t most, double *lnL_tmarg, const double *lnpw, double *lnw, int *err,
+                              cudaStream_t st);
 
 // Per-sample coefficients: c[n][K][M] (complex), dt[n][K], quad[n]; any may be null.
 cudaError_t launch_coeffs(const Problem &P, bool fp64, const double *theta, int64_t n, double2 *c, double *dt,

@@ -422,10 +422,21 @@ cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half 
 
 namespace {
 
+// Samples of the launch: n, or the device's count, of which counts up to `skip` are left to the
+// caller's other kernel.
+__device__ __forceinline__ int64_t device_count(int64_t n, const uint32_t *n_dev, uint32_t skip)
+{
+    if (!n_dev)
+        return n;
+    const uint32_t c = *n_dev;
+    return c <= skip ? 0 : min(n, (int64_t)c);
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
 lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
                 double *__restrict__ lnL_tmarg, double *__restrict__ lnL_t, const double *__restrict__ lnpw,
-                double *__restrict__ lnw, int *err, int *unit_counter, const uint32_t *__restrict__ n_dev)
+                double *__restrict__ lnw, int *err, int *unit_counter, const uint32_t *__restrict__ n_dev,
+                uint32_t skip)
 {
     extern __shared__ __align__(128) unsigned char sm[];
     const int K = P.K, M = P.M, NT = P.n_t;
@@ -456,7 +467,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool producer = warp >= kIssuer;
-    const int64_t n_use = n_dev ? min(n, (int64_t)*n_dev) : n;
+    const int64_t n_use = device_count(n, n_dev, skip);
     const int64_t n_tiles = (n_use + kS - 1) / kS;
     const int n_chunks = (NT + kChunk - 1) / kChunk, jnom = (NT + n_chunks - 1) / n_chunks;
     const int parts = parts64(n_tiles, (int)gridDim.x, n_chunks);
@@ -952,13 +963,13 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
 // Merges the chunks' sums of every sample (nothing to do when the bins were not split) and
 // resets the unit counter.
 __global__ void combine64_kernel(const Lse *__restrict__ records, const long long *__restrict__ pos, const uint32_t *__restrict__ perm, int64_t n,
-                                 const uint32_t *__restrict__ n_dev, int grid, int n_t, double *__restrict__ lnL_tmarg,
+                                 const uint32_t *__restrict__ n_dev, uint32_t skip, int grid, int n_t, double *__restrict__ lnL_tmarg,
                                  const double *__restrict__ lnpw, double *__restrict__ lnw, int *err,
                                  int *unit_counter)
 {
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *unit_counter = 0;   // for the next launch
-    const int64_t n_use = n_dev ? min(n, (int64_t)*n_dev) : n;
+    const int64_t n_use = device_count(n, n_dev, skip);
     const int64_t n_tiles = (n_use + kS - 1) / kS;
     const int n_chunks = (n_t + kChunk - 1) / kChunk;
     if (parts64(n_tiles, grid, n_chunks) == 1)
@@ -992,7 +1003,7 @@ __global__ void combine64_kernel(const Lse *__restrict__ records, const long lon
 
 cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta, const uint32_t *perm, int64_t n,
                             double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
-                            cudaStream_t st, const uint32_t *n_dev)
+                            cudaStream_t st, const uint32_t *n_dev, uint32_t skip)
 {
     if (n <= 0)
         return cudaSuccess;
@@ -1006,11 +1017,11 @@ cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta
     const int64_t tiles = (n + kS - 1) / kS;
     const int grid = (int)std::min<int64_t>(sms, 16 * tiles);
     lnl_tc64_kernel<<<grid, kThreads, smem, st>>>(P, X, theta, perm, n, lnL_tmarg, lnL_t, lnpw, lnw, err,
-                                                  X.unit_counter, n_dev);
+                                                  X.unit_counter, n_dev, skip);
     // the split depends on the device count; it never has more tiles than there are records for
     const int64_t most = std::min<int64_t>(tiles, split_tiles(n, P.n_t));
     combine64_kernel<<<(int)std::max<int64_t>(1, most), 128, 0, st>>>(reinterpret_cast<const Lse *>(X.records), X.pos, perm, n,
-                                                                    n_dev, grid, P.n_t, lnL_tmarg, lnpw, lnw, err,
+                                                                    n_dev, skip, grid, P.n_t, lnL_tmarg, lnpw, lnw, err,
                                                                     X.unit_counter);
     return cudaGetLastError();
 }
