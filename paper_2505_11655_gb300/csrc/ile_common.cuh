@@ -425,6 +425,57 @@ __device__ __forceinline__ float ln_dist_marg32(const Problem &P, float a, float
     return ln_dist_marg<float, 10, 2>(P.gl10_tf, P.gl10_wf, P.dm_xlo_f, P.dm_xhi_f, P.dm_lnC_f, a, b, 18.f);
 }
 
+// Two bins of one sample (the same b): the same rule as ln_dist_marg32 in packed float32, node by
+// node over both panels, so that a node's two ex2 per bin and the exponent's multiply-adds of the
+// two bins are one instruction stream.  One bin at a time left the unit waiting on the chain from
+// the support's logarithms to the nodes.
+__device__ __forceinline__ float2 ln_dist_marg32x2(const Problem &P, float2 a, float b)
+{
+    const float xlo = P.dm_xlo_f, xhi = P.dm_xhi_f, thr = 18.f, ks = 1.4426950408889634f;
+    float xm[2], slope[2], phim[2], L[2], ul[2], h[2];
+    const float av[2] = {a.x, a.y};
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+        xm[e] = b > 0.f ? __fdividef(av[e], 2.f * b) : (av[e] > 0.f ? xhi : xlo);
+        xm[e] = xm[e] < xlo ? xlo : (xm[e] > xhi ? xhi : xm[e]);
+        slope[e] = av[e] - 2.f * b * xm[e];
+        phim[e] = xm[e] * (av[e] - b * xm[e]);
+        const float g = fabsf(slope[e]), den = g + sqrtf(g * g + 4.f * b * thr);
+        float R = xhi;
+        L[e] = xlo;
+        if (den > 0.f) {
+            const float d = __fdividef(2.f * thr, den);
+            L[e] = xm[e] - d > xlo ? xm[e] - d : xlo;
+            R = xm[e] + d < xhi ? xm[e] + d : xhi;
+        }
+        ul[e] = __logf(L[e]);
+        h[e] = (__logf(R) - ul[e]) * 0.5f;
+    }
+    auto both = [](float v) { return make_float2(v, v); };
+    const float2 h2 = make_float2(h[0], h[1]), nxm = make_float2(-xm[0], -xm[1]);
+    const float2 eh = make_float2(__expf(0.5f * h[0]), __expf(0.5f * h[1]));
+    const float2 ec0 = __fmul2_rn(make_float2(L[0], L[1]), eh), ec1 = __fmul2_rn(ec0, __fmul2_rn(eh, eh));
+    const float2 sl = __fmul2_rn(make_float2(slope[0], slope[1]), both(ks)), nbs = both(-b * ks);
+    const float2 m0 = __fmul2_rn(both(-3.f * ks), __ffma2_rn(both(0.5f), h2, make_float2(ul[0], ul[1])));
+    const float2 m1 = __ffma2_rn(both(-3.f * ks), h2, m0);
+    float2 s0 = both(0.f), s1 = both(0.f);
+    auto node = [&](float2 ec, float2 en, float2 m, float w, float2 s) {
+        const float2 dx = __ffma2_rn(ec, en, nxm);
+        const float2 E = __ffma2_rn(dx, __ffma2_rn(nbs, dx, sl), m);
+        return __ffma2_rn(both(w), make_float2(fn_exp2(E.x), fn_exp2(E.y)), s);
+    };
+#pragma unroll
+    for (int i = 0; i < 10; ++i) {
+        const float2 y = __fmul2_rn(h2, both(0.5f * ks * P.gl10_tf[i]));   // log2 of the node's factor
+        const float2 en = make_float2(fn_exp2(y.x), fn_exp2(y.y));
+        const float2 m3h = __fmul2_rn(both(-3.f), y);
+        s0 = node(ec0, en, __fadd2_rn(m0, m3h), P.gl10_wf[i], s0);
+        s1 = node(ec1, en, __fadd2_rn(m1, m3h), P.gl10_wf[i], s1);
+    }
+    return make_float2(P.dm_lnC_f + phim[0] + __logf(0.5f * h[0] * (s0.x + s1.x)),
+                       P.dm_lnC_f + phim[1] + __logf(0.5f * h[1] * (s0.y + s1.y)));
+}
+
 __device__ __forceinline__ double ln_dist_marg64(const Problem &P, double a, double b)
 {
     return ln_dist_marg<double, 16, 4>(P.gl16_t, P.gl16_w, P.dm_xlo, P.dm_xhi, P.dm_lnC, a, b, 44.0);

@@ -1041,11 +1041,18 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
                         // (every bin exact when the per-bin values are written out)
                         const float thr = lnL_t ? -INFINITY : fmaxf(run_mx, vbest) - 40.f;
 #pragma unroll 1
-                        for (int i = 0; i < jn; ++i) {
-                            const float x = Rd[i * 64];
-                            const float v = dm_bound32(P, x, gqd) >= thr ? ln_dist_marg32(P, x, gqd) : -INFINITY;
-                            Rd[i * 64] = v;
-                            cmx = fmaxf(cmx, v);
+                        for (int i = 0; i < jn; i += 2) {   // (slot jn, when jn is odd, is -infinity)
+                            const float2 x = make_float2(Rd[i * 64], Rd[(i + 1) * 64]);
+                            const bool n0 = dm_bound32(P, x.x, gqd) >= thr;
+                            const bool n1 = i + 1 < jn && dm_bound32(P, x.y, gqd) >= thr;
+                            float2 v = make_float2(-INFINITY, -INFINITY);
+                            if (n0 || n1) {
+                                const float2 r = ln_dist_marg32x2(P, x, gqd);
+                                v = make_float2(n0 ? r.x : -INFINITY, n1 ? r.y : -INFINITY);
+                            }
+                            Rd[i * 64] = v.x;
+                            Rd[(i + 1) * 64] = v.y;
+                            cmx = fmaxf(cmx, fmaxf(v.x, v.y));
                         }
                         if (mine && jn > 0) {
                             const float nm = fmaxf(run_mx, cmx);
