@@ -29,6 +29,7 @@
 
 #include "ile_kernels.h"
 #include "tc_ptx.cuh"
+#include "tile_plan.cuh"
 
 namespace rift {
 
@@ -266,130 +267,82 @@ cudaError_t launch_prep_tt(const double2 *U64, const double2 *V64, int K, int M,
 // four classes by cost, taken in order: the costly ones first, the last ones are small.  A unit
 // is (tile, first, last sample of the tile).
 constexpr int kTcUnitsPerTile = 16;
-constexpr int kTcPlanWarps = 8;
 
 int64_t tc_units_cap(int64_t n_max) { return (n_max + kTcS - 1) / kTcS * kTcUnitsPerTile; }
 
-__global__ void __launch_bounds__(32 * kTcPlanWarps)
-tc_units_kernel(Problem P, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
+static_assert(kTcS == kPlanSamples && kTcCounters == 1 + kPlanClasses, "tiles of the planning code");
+
+__global__ void __launch_bounds__(32 * kPlanWarps)
+tc_units_kernel(PlanProblem P, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
                 const uint32_t *__restrict__ n_dev, int64_t n_theta, unsigned long long *__restrict__ list, int64_t cap,
                 int *__restrict__ counters)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t tile = (int64_t)blockIdx.x * kTcPlanWarps + (threadIdx.x >> 5);
+    __shared__ int cols[kPlanWarps][kMaxDet][kPlanSamples];
+    __shared__ PlanFiles<unsigned long long, kPlanWarps * kTcUnitsPerTile> files;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t tile = (int64_t)blockIdx.x * kPlanWarps + warp;
     const int64_t n_use = n_dev ? min(n, (int64_t)*n_dev) : n;
-    if (tile >= (n_use + kTcS - 1) / kTcS)
-        return;
-    const int K = P.K;
-    const float beta = (float)(P.t_step * P.fs);
-    // steps of a group whose offsets span `sp` columns (see jmax_s in the likelihood kernel)
-    auto steps = [&](int sp) {
-        int jm = beta > 0.f ? (int)((float)(kTcW - 11 - min(sp, kTcSpreadLimit)) / beta) + 1 : kTcMaxBins;
-        jm = max(1, min(jm, kTcMaxBins));
-        return (float)(K * ((P.n_t + jm - 1) / jm));
-    };
-    // quarters of the tile without a sample of the group skip its drains and gathers, which
-    // take about two thirds of a step
-    auto cost = [&](int a, int b, int sp) {
-        return steps(sp) * (0.35f + 0.65f * 0.25f * (float)((b - 1) / 32 - a / 32 + 1));
-    };
-    int i0[kTcS / 32][kMaxDet];
-    unsigned valid[kTcS / 32];
-    int lo[kMaxDet], hi[kMaxDet];
-#pragma unroll
-    for (int k = 0; k < kMaxDet; ++k) {
-        lo[k] = INT_MAX;
-        hi[k] = INT_MIN;
-    }
-#pragma unroll
-    for (int q = 0; q < kTcS / 32; ++q) {
-        const int64_t si = tile * kTcS + 32 * q + lane;
-        const uint32_t g = si < n_use ? perm[si] : 0xffffffffu;
-        const bool ok = (int64_t)g < n_theta;
-        float sa = 0.f, ca = 1.f, sd = 0.f, cd = 1.f;
-        if (ok) {
-            const double *th = theta + 6 * (int64_t)g;
-            sincosf((float)(th[0] - P.gmst), &sa, &ca);
-            sincosf((float)th[1], &sd, &cd);
-        }
-        valid[q] = __ballot_sync(0xffffffffu, ok);
-#pragma unroll
-        for (int k = 0; k < kMaxDet; ++k) {
-            i0[q][k] = 0;
-            if (k < K && ok) {
-                const float u = fmaf((float)P.xfs[k][0], cd * ca, fmaf((float)P.xfs[k][1], cd * sa,
-                                     fmaf((float)P.xfs[k][2], sd, (float)P.ufs0[k])));
-                i0[q][k] = (int)floorf(u);
-                lo[k] = min(lo[k], i0[q][k]);
-                hi[k] = max(hi[k], i0[q][k]);
-            }
-        }
-    }
-    int spread = 0;
-#pragma unroll
-    for (int k = 0; k < kMaxDet; ++k)
-        if (k < K)
-            spread = max(spread, __reduce_max_sync(0xffffffffu, hi[k]) - __reduce_min_sync(0xffffffffu, lo[k]));
-    const float base = steps(0);
-    auto file = [&](int a, int b, float c) {
-        if (lane != 0)
-            return;
-        const int cls = c > 1.75f * base ? 0 : c > 1.35f * base ? 1 : c > 0.7f * base ? 2 : 3;
-        const int64_t at = atomicAdd(counters + 1 + cls, 1);
-        list[((cls == 1 || cls == 2) ? cap : 0) + (cls < 2 ? at : cap - 1 - at)] =
-            ((unsigned long long)tile << 16) | (unsigned)(a << 8) | (unsigned)(b - 1);
-    };
-    if (spread <= kTcSpreadLimit) {
-        file(0, kTcS, cost(0, kTcS, spread));
-        return;
-    }
-    int units = 0, ua = 0, ga = 0;   // units filed, first sample of the open unit and of the open group
-    float uc = 0.f;                  // cost of the open unit's closed groups
-    bool open = false;
-    auto close = [&](int e) {        // close the open group at sample e; close the unit before it when full
-        int sp = 0;
-#pragma unroll
-        for (int k = 0; k < kMaxDet; ++k)
-            if (k < K)
-                sp = max(sp, hi[k] - lo[k]);
-        const float c = cost(ga, e, sp);
-        if (uc > 0.f && uc + c > 2.f * base && units < kTcUnitsPerTile - 1) {
-            file(ua, ga, uc);
-            ++units;
-            ua = ga;
-            uc = 0.f;
-        }
-        uc += c;
-    };
-#pragma unroll
-    for (int q = 0; q < kTcS / 32; ++q)
-        for (int e = 0; e < 32; ++e) {
-            if (!((valid[q] >> e) & 1u))
-                continue;
-            int v[kMaxDet];
-            bool fits = open;
-#pragma unroll
-            for (int k = 0; k < kMaxDet; ++k)
-                if (k < K) {
-                    v[k] = __shfl_sync(0xffffffffu, i0[q][k], e);
-                    fits = fits && max(hi[k], v[k]) - min(lo[k], v[k]) <= kTcSpreadLimit;
+    plan_reset(files);
+    if (tile < (n_use + kTcS - 1) / kTcS) {
+        int (*i0)[kPlanSamples] = cols[warp];
+        int lo, hi;
+        plan_columns(P, theta, perm, tile, n_use, n_theta, i0, lo, hi);
+        // steps of a group whose offsets span `sp` columns (see jmax_s in the likelihood kernel)
+        auto steps = [&](int sp) {
+            int jm = P.beta > 0.f ? (int)((float)(kTcW - 11 - min(sp, kTcSpreadLimit)) / P.beta) + 1 : kTcMaxBins;
+            jm = max(1, min(jm, kTcMaxBins));
+            return (float)(P.K * ((P.n_t + jm - 1) / jm));
+        };
+        // quarters of the tile without a sample of the group skip its drains and gathers, which
+        // take about two thirds of a step
+        auto cost = [&](int a, int b, int sp) {
+            return steps(sp) * (0.35f + 0.65f * 0.25f * (float)((b - 1) / 32 - a / 32 + 1));
+        };
+        const float base = steps(0);
+        auto file = [&](int a, int b, float c) {
+            if (lane == 0)
+                plan_file(files, ((unsigned long long)tile << 16) | (unsigned)(a << 8) | (unsigned)(b - 1),
+                          c > 1.75f * base ? 0 : c > 1.35f * base ? 1 : c > 0.7f * base ? 2 : 3);
+        };
+        // (lane k holds detector k's range)
+        auto spread = [&] { return __reduce_max_sync(0xffffffffu, lane < P.K && lo <= hi ? hi - lo : 0); };
+        const int sp = spread();
+        if (sp <= kTcSpreadLimit) {
+            file(0, kTcS, cost(0, kTcS, sp));
+        } else {
+            int units = 0, ua = 0, ga = 0;   // units filed, first sample of the open unit, of the open group
+            float uc = 0.f;                  // cost of the open unit's closed groups
+            bool open = false;
+            auto close = [&](int e) {        // close the open group at sample e, and the unit before it when full
+                const float c = cost(ga, e, spread());
+                if (uc > 0.f && uc + c > 2.f * base && units < kTcUnitsPerTile - 1) {
+                    file(ua, ga, uc);
+                    ++units;
+                    ua = ga;
+                    uc = 0.f;
                 }
-            if (!fits) {
-                if (open) {
-                    close(32 * q + e);
-                    ga = 32 * q + e;
+                uc += c;
+            };
+#pragma unroll 1
+            for (int e = 0; e < kTcS; ++e) {
+                const int v = lane < P.K ? i0[lane][e] : 0;
+                if (__any_sync(0xffffffffu, v == INT_MIN))
+                    continue;
+                const bool fits =
+                    open && __all_sync(0xffffffffu, lane >= P.K || max(hi, v) - min(lo, v) <= kTcSpreadLimit);
+                if (!fits && open) {
+                    close(e);
+                    ga = e;
                 }
                 open = true;
+                lo = fits ? min(lo, v) : v;
+                hi = fits ? max(hi, v) : v;
             }
-#pragma unroll
-            for (int k = 0; k < kMaxDet; ++k)
-                if (k < K) {
-                    lo[k] = fits ? min(lo[k], v[k]) : v[k];
-                    hi[k] = fits ? max(hi[k], v[k]) : v[k];
-                }
+            close(kTcS);
+            file(ua, kTcS, uc);
         }
-    close(kTcS);
-    file(ua, kTcS, uc);
+    }
+    plan_write(files, list, cap, counters + 1);
 }
 
 // kDM: distance marginalisation (a separate instantiation, so that the plain path keeps
@@ -505,13 +458,10 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
         tc::fence_proxy_async_smem();
         if (tid == 0) {
             // the next unit: classes in order (see tc_units_kernel)
-            int u = abort_s ? INT_MAX : atomicAdd(units.counters, 1), cls = 0;
-            for (; cls < 4 && u >= units.counters[1 + cls]; ++cls)
-                u -= units.counters[1 + cls];
+            const int u = abort_s ? INT_MAX : atomicAdd(units.counters, 1);
+            unsigned long long w;
             tile_s = INT_MAX;
-            if (cls < 4) {
-                const unsigned long long w =
-                    units.list[((cls == 1 || cls == 2) ? units.cap : 0) + (cls < 2 ? u : units.cap - 1 - u)];
+            if (plan_item(units.list, units.cap, units.counters + 1, u, w)) {
                 tile_s = (int)(w >> 16);
                 range_s = (int)(w & 0xffffu);
             }
@@ -1230,8 +1180,8 @@ cudaError_t launch_lnl_tc(const Problem &P, BinTable bt, const double *theta, co
     if (e != cudaSuccess)
         return e;
     const int64_t tiles = (n + kTcS - 1) / kTcS;
-    tc_units_kernel<<<(unsigned)((tiles + kTcPlanWarps - 1) / kTcPlanWarps), 32 * kTcPlanWarps, 0, st>>>(
-        P, theta, perm, n, n_dev, n_theta, units.list, units.cap, units.counters);
+    tc_units_kernel<<<(unsigned)((tiles + kPlanWarps - 1) / kPlanWarps), 32 * kPlanWarps, 0, st>>>(
+        plan_problem(P), theta, perm, n, n_dev, n_theta, units.list, units.cap, units.counters);
     const int grid = (int)std::min<int64_t>(kTcUnitsPerTile * tiles, sms);
     kern<<<grid, kTcThreads, smem, st>>>(P, bt, theta, perm, n, lnL_tmarg, lnL_t, lnpw, lnw, err, units, n_dev,
                                           n_theta, lnl_t_compact, po);
