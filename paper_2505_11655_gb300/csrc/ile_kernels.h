@@ -177,6 +177,9 @@ struct Tc64 {
     unsigned char *scratch;           // coefficient digits of the resident tiles
     unsigned char *records;           // the chunks' sums of a batch whose time bins are split
     int *unit_counter;                // 0 between launches
+    unsigned long long *units;        // [2][units_cap] work units in four classes (tile_plan.cuh)
+    int64_t units_cap;
+    int *unit_counts;                 // [4] units per class
     const long long *pos;             // [n_t] Q positions of the bins relative to the first (2^-48),
                                       // then the exponential's table
     long long u0[kMaxDet];            // Q position of the first bin without delay (2^-48)
@@ -188,6 +191,7 @@ size_t tc64_record_bytes(int64_t n_max, int n_t);
 // Fills pos [n_t + kTc64Table] and u0 [n_det] (host).
 constexpr int kTc64Table = 128;
 void tc64_positions(const rift_ile_config &cfg, long long *pos, long long *u0);
+int64_t tc64_units_cap(int64_t n_max);
 size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms);
 cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half *q_dig, __half *t_dig, int *t_exp,
                              cudaStream_t st);

@@ -54,6 +54,7 @@
 
 #include "ile_kernels.h"
 #include "tc_ptx.cuh"
+#include "tile_plan.cuh"
 
 namespace rift {
 
@@ -77,6 +78,10 @@ constexpr uint64_t kWait = 1000000000ull;
 constexpr int kRecords = 4096;           // (tile, chunk) pairs of a batch whose time bins are split
 constexpr int kSumBits = 52;             // resolution of the log-sum-exp (at most 4000 terms <= 1)
 constexpr size_t kMinSmem = 120 * 1024;  // one block per SM
+constexpr int64_t kPlanFrom = 64;        // tiles from which a batch's units are planned
+constexpr int kUnitsPerTile = 16;
+constexpr float kUnitsPerBlock = 2.2f;
+static_assert(kS == kPlanSamples, "tiles of the planning code");
 static_assert(2 * kAccCols <= 512, "two sets of accumulators in tensor memory");
 static_assert(kS * kMaxDet <= kConsumers, "one (sample, detector) item per consumer thread");
 
@@ -384,6 +389,9 @@ size_t tc64_record_bytes(int64_t n_max, int n_t)
     return (size_t)split_tiles(n_max, n_t) * kS * 16 * ((n_t + kChunk - 1) / kChunk + 1);
 }
 
+// (with records, a tile has at most as many units as chunks)
+int64_t tc64_units_cap(int64_t n_max) { return (n_max + kS - 1) / kS + kRecords; }
+
 size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms)
 {
     const int64_t tiles = (n_max + kS - 1) / kS, blocks = std::min<int64_t>(sms, 16 * tiles);
@@ -432,11 +440,56 @@ __device__ __forceinline__ int64_t device_count(int64_t n, const uint32_t *n_dev
     return c <= skip ? 0 : min(n, (int64_t)c);
 }
 
+// Whether a batch's chunks have records (its time bins may then be split over blocks).
+__host__ __device__ inline bool has_records(int64_t n_tiles, int n_chunks)
+{
+    return n_tiles * n_chunks <= (int64_t)kRecords;
+}
+
+// Units of a batch of kPlanFrom tiles or more: a tile's time is that of the columns its samples'
+// delays span, three and more times the narrowest in thinly sampled parts of the sky, so a tile
+// is cut into parts of its time bins by its width (about kUnitsPerBlock units a block; whole tiles
+// where the batch has no records), and the costly units are taken first.  With every tile in two
+// parts, in the sort's order, the SMs were idle for 28% of a 20,000-sample batch.  One warp per
+// tile.
+__global__ void __launch_bounds__(32 * kPlanWarps)
+units64_kernel(PlanProblem P, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
+               const uint32_t *__restrict__ n_dev, uint32_t skip, int grid, unsigned long long *__restrict__ list,
+               int64_t cap, int *__restrict__ counts)
+{
+    __shared__ int cols[kPlanWarps][kMaxDet][kPlanSamples];
+    __shared__ PlanFiles<unsigned long long, kPlanWarps * kUnitsPerTile> files;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t tile = (int64_t)blockIdx.x * kPlanWarps + warp;
+    const int64_t n_use = device_count(n, n_dev, skip), n_tiles = (n_use + kS - 1) / kS;
+    plan_reset(files);
+    if (tile < n_tiles) {
+        int lo, hi;
+        plan_columns(P, theta, perm, tile, n_use, 0xffffffffll, cols[warp], lo, hi);
+        // batches of a chunk's windows over those of a single sample
+        const int n_chunks = (P.n_t + kChunk - 1) / kChunk;
+        const int span = (int)(P.beta * (float)(kChunk - 1)) + 2;
+        const int own = lane < P.K ? span / kSub + 1 : 0;
+        const int all = lane < P.K ? (span + (lo <= hi ? hi - lo : 0)) / kSub + 1 : 0;
+        const float r = (float)__reduce_add_sync(0xffffffffu, all) / (float)__reduce_add_sync(0xffffffffu, own);
+        const bool split = has_records(n_tiles, n_chunks);
+        const float k = split ? kUnitsPerBlock * (float)grid / (float)n_tiles : 1.f;
+        const int parts = split ? max(1, min(min(n_chunks, kUnitsPerTile), (int)(r * k + 0.5f))) : 1;
+        const float x = r * k / (float)parts;   // about 1 where the batch is split as it wants
+        const int cls = split ? (x > 1.5f ? 0 : x > 1.1f ? 1 : x > 0.8f ? 2 : 3) : (x > 2.4f ? 0 : x > 1.7f ? 1 : x > 1.25f ? 2 : 3);
+        if (lane < parts) {
+            const int c0 = lane * n_chunks / parts, c1 = (lane + 1) * n_chunks / parts;
+            plan_file(files, ((unsigned long long)tile << 16) | (unsigned)(c0 << 8) | (unsigned)c1, cls);
+        }
+    }
+    plan_write(files, list, cap, counts);
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
 lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
                 double *__restrict__ lnL_tmarg, double *__restrict__ lnL_t, const double *__restrict__ lnpw,
                 double *__restrict__ lnw, int *err, int *unit_counter, const uint32_t *__restrict__ n_dev,
-                uint32_t skip)
+                uint32_t skip, int planned)
 {
     extern __shared__ __align__(128) unsigned char sm[];
     const int K = P.K, M = P.M, NT = P.n_t;
@@ -463,14 +516,15 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
     double *ps = reinterpret_cast<double *>(sm + L.ps), *pw = reinterpret_cast<double *>(sm + L.pw);
     double2 *pe = reinterpret_cast<double2 *>(sm + L.pe), *Fs = reinterpret_cast<double2 *>(sm + L.F);
     double2 *Ys = reinterpret_cast<double2 *>(sm + L.Y);
-    __shared__ int unit_s, abort_s;
+    __shared__ int unit_s, tile_s, chunks_s, abort_s;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool producer = warp >= kIssuer;
     const int64_t n_use = device_count(n, n_dev, skip);
     const int64_t n_tiles = (n_use + kS - 1) / kS;
     const int n_chunks = (NT + kChunk - 1) / kChunk, jnom = (NT + n_chunks - 1) / n_chunks;
-    const int parts = parts64(n_tiles, (int)gridDim.x, n_chunks);
+    const int parts = planned ? 1 : parts64(n_tiles, (int)gridDim.x, n_chunks);
+    const bool split = planned ? has_records(n_tiles, n_chunks) : parts > 1;
     const int sq = 55 - exp_above(__longlong_as_double((long long)*X.qmax));
     const uint32_t sub_bytes = (uint32_t)(kSub * kp * 2);           // one digit of a batch's columns
     const size_t ab = a_bytes(kp);
@@ -514,6 +568,18 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             // the first unit by the block's index, the others from the counter
             unit_s = abort_s ? INT_MAX : first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(unit_counter, 1);
             first = false;
+            tile_s = -1;
+            unsigned long long w;
+            if (planned) {
+                if (!abort_s && plan_item(X.units, X.units_cap, X.unit_counts, unit_s, w)) {
+                    tile_s = (int)(w >> 16);
+                    chunks_s = (int)(w & 0xffffu);
+                }
+            } else if ((int64_t)unit_s < n_tiles * parts) {
+                tile_s = unit_s / parts;
+                const int part = unit_s - tile_s * parts;
+                chunks_s = (int)((int64_t)part * n_chunks / parts) << 8 | (int)((int64_t)(part + 1) * n_chunks / parts);
+            }
         }
         if (tid < K) {
             ulo[tid] = LLONG_MAX;
@@ -525,11 +591,10 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             bad[tid] = 0;
         }
         __syncthreads();
-        const int64_t unit = unit_s;
-        if (unit >= n_tiles * parts)
+        const int64_t tile = tile_s;
+        if (tile < 0)
             break;
-        const int64_t tile = unit / parts;
-        const int part = (int)(unit - tile * parts);
+        const int ch0 = chunks_s >> 8, ch1 = chunks_s & 255;
         const int s_of = tid & (kS - 1), grp = tid >> 7;
 
         // ---------------- prologue A: trigonometry in float64, a quarter of it per thread
@@ -668,7 +733,6 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
         tc::fence_proxy_async();
         __syncthreads();
 
-        const int ch0 = (int)((int64_t)part * n_chunks / parts), ch1 = (int)((int64_t)(part + 1) * n_chunks / parts);
         const bool any = ulo[0] != LLONG_MAX;   // a sample with finite delays
         // first column (a multiple of 8) and batches of detector k's window for the bins [j0, j1)
         auto window = [&](int k, int j0, int j1, int &w0, int &nsub) {
@@ -841,6 +905,11 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     int w0, nsub;
                     window(k, j0, j0 + J, w0, nsub);
                     const long long uk = U0[k * kS + gs];
+                    // columns that this warp's samples reach with this thread's share of the bins:
+                    // the other blocks of the window are not looked through
+                    const int wlo = __reduce_min_sync(0xffffffffu, jn > 0 ? (int)((uk + pos[jb]) >> kFrac) : INT_MAX);
+                    const int whi =
+                        __reduce_max_sync(0xffffffffu, jn > 0 ? (int)((uk + pos[jb + jn - 1]) >> kFrac) : INT_MIN);
                     for (int t = 0; t < nsub; t += 2) {
                         tc::named_bar_or(qbar, kConsumers / 4, 0);   // the previous block's gathers are done
                         if (cb == 3 && t > 0)
@@ -852,6 +921,8 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                             break;
                         const int rel = w0 + kSub * t - 1;
                         const unsigned cols = (unsigned)(kSub * min(2, nsub - t));
+                        if (whi - rel < 0 || wlo - rel >= (int)cols)
+                            continue;
 #pragma unroll
                         for (int i = 0; i < kBpt; ++i) {
                             const long long u = uk + pos[min(jb + i, NT - 1)];
@@ -893,7 +964,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     Lse c{Rs[gs], (uint64_t)Rs[kQ * kS + gs]};
                     for (int h = 1; h < kQ; ++h)
                         c = merge64(ds, c, Lse{Rs[h * kS + gs], (uint64_t)Rs[(kQ + h) * kS + gs]}, tbl);
-                    if (parts == 1)
+                    if (!split)
                         run = ch == 0 ? c : merge64(ds, run, c, tbl);
                     else
                         records[((int64_t)ch * n_tiles + tile) * kS + gs] = c;
@@ -903,7 +974,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             if (!failed && gh == 0 && gid[gs] != 0xffffffffu) {
                 const uint32_t gi = gid[gs];
                 int flags = bad[gs];
-                if (parts == 1) {
+                if (!split) {
                     const double r = flags ? __longlong_as_double(0x7ff8000000000000LL)
                                            : lse_value(run, lexp, quad, NT);
                     if (!isfinite(r))
@@ -911,7 +982,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     lnL_tmarg[gi] = r;
                     if (lnw && lnpw)
                         lnw[gi] = r + lnpw[gi];
-                } else if (part == 0) {
+                } else if (ch0 == 0) {
                     records[((int64_t)n_chunks * n_tiles + tile) * kS + gs] =
                         Lse{__double_as_longlong(quad), (uint64_t)(uint32_t)lexp | ((uint64_t)(uint32_t)flags << 32)};
                 }
@@ -923,11 +994,11 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             const uint32_t gi = gid[s_of];
             const double r = __longlong_as_double(0x7ff8000000000000LL);
             atomicOr(err, bad[s_of] | kErrNonFinite);
-            if (parts == 1) {
+            if (!split) {
                 lnL_tmarg[gi] = r;
                 if (lnw && lnpw)
                     lnw[gi] = r;
-            } else if (part == 0) {
+            } else if (ch0 == 0) {
                 records[((int64_t)n_chunks * n_tiles + tile) * kS + s_of] = Lse{0, (uint64_t)kErrNonFinite << 32};
             }
         }
@@ -963,7 +1034,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
 // Merges the chunks' sums of every sample (nothing to do when the bins were not split) and
 // resets the unit counter.
 __global__ void combine64_kernel(const Lse *__restrict__ records, const long long *__restrict__ pos, const uint32_t *__restrict__ perm, int64_t n,
-                                 const uint32_t *__restrict__ n_dev, uint32_t skip, int grid, int n_t, double *__restrict__ lnL_tmarg,
+                                 const uint32_t *__restrict__ n_dev, uint32_t skip, int planned, int grid, int n_t, double *__restrict__ lnL_tmarg,
                                  const double *__restrict__ lnpw, double *__restrict__ lnw, int *err,
                                  int *unit_counter)
 {
@@ -972,7 +1043,7 @@ __global__ void combine64_kernel(const Lse *__restrict__ records, const long lon
     const int64_t n_use = device_count(n, n_dev, skip);
     const int64_t n_tiles = (n_use + kS - 1) / kS;
     const int n_chunks = (n_t + kChunk - 1) / kChunk;
-    if (parts64(n_tiles, grid, n_chunks) == 1)
+    if (planned ? !has_records(n_tiles, n_chunks) : parts64(n_tiles, grid, n_chunks) == 1)
         return;
     __shared__ uint64_t tbl[kTable];
     for (int i = threadIdx.x; i < kTable; i += blockDim.x)
@@ -1016,12 +1087,24 @@ cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta
     const size_t smem = std::max(kMinSmem, layout64(P.K, P.M, P.n_t).end);
     const int64_t tiles = (n + kS - 1) / kS;
     const int grid = (int)std::min<int64_t>(sms, 16 * tiles);
+    // Planned are whole batches (20,011 samples of the largest problem 1409 -> 1328 us a call).  The
+    // time bins of smaller ones are split evenly, and so are those of a device-side list: its
+    // iteration has other kernels beside it or behind it, and more units mean more prologues
+    // (twelve solves as one graph 9.2 -> 9.8 ms when their lists were planned).
+    const int planned = !n_dev && tiles >= kPlanFrom ? 1 : 0;
+    if (planned) {
+        e = cudaMemsetAsync(X.unit_counts, 0, kPlanClasses * sizeof(int), st);
+        if (e != cudaSuccess)
+            return e;
+        units64_kernel<<<(unsigned)((tiles + kPlanWarps - 1) / kPlanWarps), 32 * kPlanWarps, 0, st>>>(
+            plan_problem(P), theta, perm, n, n_dev, skip, grid, X.units, X.units_cap, X.unit_counts);
+    }
     lnl_tc64_kernel<<<grid, kThreads, smem, st>>>(P, X, theta, perm, n, lnL_tmarg, lnL_t, lnpw, lnw, err,
-                                                  X.unit_counter, n_dev, skip);
+                                                  X.unit_counter, n_dev, skip, planned);
     // the split depends on the device count; it never has more tiles than there are records for
     const int64_t most = std::min<int64_t>(tiles, split_tiles(n, P.n_t));
     combine64_kernel<<<(int)std::max<int64_t>(1, most), 128, 0, st>>>(reinterpret_cast<const Lse *>(X.records), X.pos, perm, n,
-                                                                    n_dev, skip, grid, P.n_t, lnL_tmarg, lnpw, lnw, err,
+                                                                    n_dev, skip, planned, grid, P.n_t, lnL_tmarg, lnpw, lnw, err,
                                                                     X.unit_counter);
     return cudaGetLastError();
 }
