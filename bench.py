@@ -63,6 +63,7 @@ TRAFFIC_BY_SOURCE = {
     "02d8362c4117749bf193a68eea6c4ee9c70af5751d9d82631086b1437d6f8777": 5.97e7,
     "a1a0f3fa500f237d67cded3cf3f47eaac17dae8af6c99f541d525a7f85a14ff1": 6.03e7,
     "70258efe81120ca38cdd3f22b5ffc4ac29c4003ba3fdf3b4467adb6ac9f57fc1": 5.97e7,
+    "21b0526213563248a645bad3b51375dfc6c723048d9f563bfd77c6252ca56bd0": 6.78e7,
 }
 
 
@@ -499,7 +500,7 @@ def _setup(local_rank):
 
 
 def _lnl_kernel_name(G, plan):
-    return {G.RIFT_KERNEL_TENSOR: "lnl_tc_kernel", G.RIFT_KERNEL_CUDA_CORE: "lnl_tile_kernel",
+    return {G.RIFT_KERNEL_TENSOR: "lnl_tc_kernel", G.RIFT_KERNEL_CUDA_CORE: "lnl_block_kernel",
             G.RIFT_KERNEL_FP64: "lnl_fp64_kernel"}[plan[0]]
 
 
