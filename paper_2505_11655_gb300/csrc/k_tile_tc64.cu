@@ -23,8 +23,8 @@
 //     node fraction (48 bits), sums over detectors in 64-bit integers;
 //   * the log-sum-exp takes differences to the running maximum as integers and 2^-t from a
 //     128-entry table and a short polynomial in 64-bit fixed point; sums with 2^-52
-//     resolution.  A chunk's bins are summed by four threads relative to their common maximum, and
-//     the chunks' sums merged in order.
+//     resolution.  A chunk's bins are summed by four threads, their sums and the chunks'
+//     merged in a fixed order.
 // The template term is contracted the same way, W_k = Z_k T_k (the real quadratic form of
 // k_tile_tc.cu) and summed against the float64 components.
 //
@@ -497,7 +497,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
     const int kp = L.kp, kcs = kp / 8;
     __half *As = reinterpret_cast<__half *>(sm + L.a);              // [kDig][kS x kp]
     __half *Bs = reinterpret_cast<__half *>(sm + L.b);              // [2][kDig][kSub x kp]
-    long long *Rs = reinterpret_cast<long long *>(sm + L.r);        // [2][kSub][kS] (template term: [kBlk][kS])
+    long long *Rs = reinterpret_cast<long long *>(sm + L.r);        // [1 + kBlk][kS]; row 0 the previous block's last
     long long *pos = reinterpret_cast<long long *>(sm + L.pos);     // [NT] bin offset in Q samples, kFrac fraction bits
     long long *U0 = reinterpret_cast<long long *>(sm + L.u0);       // [K][kS] Q position of the first bin
     double *quads = reinterpret_cast<double *>(sm + L.quad);        // [kQ][kS] template term partials
@@ -820,20 +820,13 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             const int q = warp & 3, cb = warp >> 2, s = 32 * q + lane;   // drain: quarter, 8 columns of 32
             const int gs = s_of, gh = grp;                               // gather: sample, quarter of the bins
             const bool mine = gid[gs] != 0xffffffffu && !bad[gs];
-            // The last column of batch t, for the nodes that straddle two batches: a ring of three rows,
-            // so that a warp that has begun batch t + 1 leaves batch t's (the last row of R and two
-            // tables of the prologue)
-            auto carry = [&](int t) {
-                const int c = t % 3;
-                return c == 0 ? Rs + (size_t)kBlk * kS : reinterpret_cast<long long *>(c == 1 ? mF2 : mY2);
-            };
-            // drain one batch into half `sub` of R
-            auto drain = [&](int sub, long long *last) {
+            // drain one batch into rows 1 + 32 sub.. of R
+            auto drain = [&](int sub) {
                 const uint32_t b = g & 1u;
                 const int ok = tc::mbar_wait(done + b, (g >> 1) & 1u, kWait) ? 1 : 0;
                 ++g;
                 tc::tc_fence_after();
-                long long *out = Rs + (size_t)(kSub * sub + 8 * cb) * kS + s;
+                long long *out = Rs + (size_t)(1 + kSub * sub + 8 * cb) * kS + s;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     uint32_t v[kDig][4];
@@ -844,12 +837,8 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                                      v[o]);
                     tc::tmem_ld_wait();
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const long long x = join_orders(v, i);
-                        out[(4 * h + i) * kS] = x;
-                        if (h == 1 && i == 3 && cb == 3 && last)
-                            last[s] = x;
-                    }
+                    for (int i = 0; i < 4; ++i)
+                        out[(4 * h + i) * kS] = join_orders(v, i);
                 }
                 tc::tc_fence_before();
                 __syncwarp();
@@ -863,7 +852,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             double qacc = 0.0;
             for (int k = 0; k < K && !failed; ++k) {
                 tc::named_bar_or(qbar, kConsumers / 4, 0);   // R free
-                const int ok0 = drain(0, nullptr), ok1 = drain(1, nullptr);
+                const int ok0 = drain(0), ok1 = drain(1);
                 failed = tc::named_bar_or(qbar, kConsumers / 4, !ok0 || !ok1 || abort_s);
                 if (failed)
                     break;
@@ -890,7 +879,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                             const uint32_t hb = w[p][j >> 1] >> (16 * (j & 1));
                             I = I * 256 + (long long)__half2int_rn(__ushort_as_half((unsigned short)hb));
                         }
-                        acc = fma((double)I, (double)Rs[(size_t)nn * kS + gs], acc);
+                        acc = fma((double)I, (double)Rs[(size_t)(1 + nn) * kS + gs], acc);
                     }
                 }
                 qacc += mul_pow2(acc, 56 - 2 * sc - (55 - X.t_exp[k]));
@@ -904,7 +893,6 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             DiffScale ds;
             ds.set(lexp);
             Lse run{LLONG_MIN, 0ull};
-            int nb = 3;   // batches of Q columns drained by this warp (with a start that keeps nb + 2 and nb - 1 alike)
             for (int ch = ch0; ch < ch1 && !failed; ++ch) {
                 const int j0 = ch * jnom, J = min(jnom, NT - j0);
                 const int jq = (J + kQ - 1) / kQ, jb = j0 + gh * jq;
@@ -922,25 +910,26 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     const int wlo = __reduce_min_sync(0xffffffffu, jn > 0 ? (int)((uk + pos[jb]) >> kFrac) : INT_MAX);
                     const int whi =
                         __reduce_max_sync(0xffffffffu, jn > 0 ? (int)((uk + pos[jb + jn - 1]) >> kFrac) : INT_MIN);
-                    // One barrier a batch: the half of R that batch t is drained into was last read by
-                    // the gathers of batch t - 2, which every warp of the quarter finished before the
-                    // barrier of batch t - 1, so a warp drains the next batch while others still gather.
-                    for (int t = 0; t < nsub; ++t, ++nb) {
-                        const int ok = drain(nb & 1, carry(nb));
+                    for (int t = 0; t < nsub; t += 2) {
+                        tc::named_bar_or(qbar, kConsumers / 4, 0);   // the previous block's gathers are done
+                        if (cb == 3 && t > 0)
+                            Rs[s] = Rs[(size_t)kBlk * kS + s];
+                        int ok = drain(0);
+                        if (t + 1 < nsub)
+                            ok &= drain(1);
                         if ((failed = tc::named_bar_or(qbar, kConsumers / 4, !ok || abort_s)))
                             break;
                         const int rel = w0 + kSub * t - 1;
-                        if (whi - rel < 0 || wlo - rel >= kSub)
+                        const unsigned cols = (unsigned)(kSub * min(2, nsub - t));
+                        if (whi - rel < 0 || wlo - rel >= (int)cols)
                             continue;
-                        const long long *half = Rs + (size_t)((nb & 1) * kSub) * kS + gs;
-                        const long long *before = carry(nb + 2) + gs;   // batch nb - 1
 #pragma unroll
                         for (int i = 0; i < kBpt; ++i) {
                             const long long u = uk + pos[min(jb + i, NT - 1)];
                             const int c = (int)(u >> kFrac) - rel;
-                            if (i < jn && (unsigned)c < (unsigned)kSub) {
-                                const long long *r = half + (size_t)c * kS;   // the node's upper column
-                                const long long r0 = *(c ? r - kS : before), dr = (r[0] - r0) * 2;
+                            if (i < jn && (unsigned)c < cols) {
+                                const long long *r = Rs + (size_t)c * kS + gs;
+                                const long long r0 = r[0], dr = (r[kS] - r0) * 2;
                                 const long long f63 = (u << (63 - kFrac)) & 0x7fffffffffffffffLL;
                                 lin[i] += r0 + __mul64hi(dr, f63);
                             }
@@ -961,23 +950,20 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                         if (i < jn)
                             lnL_t[row + i] = __dsub_rn(mul_pow2((double)lin[i], lexp), quad);
                 }
-                // the four threads' maxima, then their terms relative to the chunk's maximum (sums
-                // of the same scale: additions, no exponentials to merge them), where the template
-                // term's partials were (R's halves may be in use by the next chunk)
-                long long *ex = reinterpret_cast<long long *>(quads);
-                ex[gh * kS + gs] = cm;
-                tc::named_bar_or(qbar, kConsumers / 4, 0);
-                cm = max(max(ex[gs], ex[kS + gs]), max(ex[2 * kS + gs], ex[3 * kS + gs]));
-                uint64_t terms = 0ull;
+                Lse part_l{cm, 0ull};
 #pragma unroll
                 for (int i = 0; i < kBpt; ++i)
                     if (i < jn)
-                        terms += term64(ds, (uint64_t)cm - (uint64_t)lin[i], tbl);
+                        part_l.s += term64(ds, (uint64_t)cm - (uint64_t)lin[i], tbl);
+                // the chunk's four parts, where R was; merged by the sample's first thread
                 tc::named_bar_or(qbar, kConsumers / 4, 0);
-                ex[gh * kS + gs] = (long long)terms;
+                Rs[gh * kS + gs] = part_l.m;
+                Rs[(kQ + gh) * kS + gs] = (long long)part_l.s;
                 tc::named_bar_or(qbar, kConsumers / 4, 0);
                 if (gh == 0) {
-                    const Lse c{cm, terms + (uint64_t)ex[kS + gs] + (uint64_t)ex[2 * kS + gs] + (uint64_t)ex[3 * kS + gs]};
+                    Lse c{Rs[gs], (uint64_t)Rs[kQ * kS + gs]};
+                    for (int h = 1; h < kQ; ++h)
+                        c = merge64(ds, c, Lse{Rs[h * kS + gs], (uint64_t)Rs[(kQ + h) * kS + gs]}, tbl);
                     if (!split)
                         run = ch == 0 ? c : merge64(ds, run, c, tbl);
                     else
