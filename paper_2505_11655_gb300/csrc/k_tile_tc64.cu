@@ -23,8 +23,8 @@
 //     node fraction (48 bits), sums over detectors in 64-bit integers;
 //   * the log-sum-exp takes differences to the running maximum as integers and 2^-t from a
 //     128-entry table and a short polynomial in 64-bit fixed point; sums with 2^-52
-//     resolution.  A chunk's bins are summed by four threads, their sums and the chunks'
-//     merged in a fixed order.
+//     resolution.  A chunk's bins are summed by four threads relative to their common maximum, and
+//     the chunks' sums merged in order.
 // The template term is contracted the same way, W_k = Z_k T_k (the real quadratic form of
 // k_tile_tc.cu) and summed against the float64 components.
 //
@@ -950,20 +950,22 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                         if (i < jn)
                             lnL_t[row + i] = __dsub_rn(mul_pow2((double)lin[i], lexp), quad);
                 }
-                Lse part_l{cm, 0ull};
+                // the four threads' maxima, then their terms relative to the chunk's maximum (sums
+                // of the same scale: additions, no exponentials to merge them), where R was
+                tc::named_bar_or(qbar, kConsumers / 4, 0);
+                Rs[gh * kS + gs] = cm;
+                tc::named_bar_or(qbar, kConsumers / 4, 0);
+                cm = max(max(Rs[gs], Rs[kS + gs]), max(Rs[2 * kS + gs], Rs[3 * kS + gs]));
+                uint64_t terms = 0ull;
 #pragma unroll
                 for (int i = 0; i < kBpt; ++i)
                     if (i < jn)
-                        part_l.s += term64(ds, (uint64_t)cm - (uint64_t)lin[i], tbl);
-                // the chunk's four parts, where R was; merged by the sample's first thread
-                tc::named_bar_or(qbar, kConsumers / 4, 0);
-                Rs[gh * kS + gs] = part_l.m;
-                Rs[(kQ + gh) * kS + gs] = (long long)part_l.s;
+                        terms += term64(ds, (uint64_t)cm - (uint64_t)lin[i], tbl);
+                Rs[(kQ + gh) * kS + gs] = (long long)terms;
                 tc::named_bar_or(qbar, kConsumers / 4, 0);
                 if (gh == 0) {
-                    Lse c{Rs[gs], (uint64_t)Rs[kQ * kS + gs]};
-                    for (int h = 1; h < kQ; ++h)
-                        c = merge64(ds, c, Lse{Rs[h * kS + gs], (uint64_t)Rs[(kQ + h) * kS + gs]}, tbl);
+                    const Lse c{cm, terms + (uint64_t)Rs[(kQ + 1) * kS + gs] + (uint64_t)Rs[(kQ + 2) * kS + gs] +
+                                        (uint64_t)Rs[(kQ + 3) * kS + gs]};
                     if (!split)
                         run = ch == 0 ? c : merge64(ds, run, c, tbl);
                     else
