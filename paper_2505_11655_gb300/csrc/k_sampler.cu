@@ -584,7 +584,7 @@ __device__ void block_max(Acc &a)
     }
 }
 
-__device__ void block_sum(Acc &a)   // valid in thread 0
+__device__ void block_sum(Acc &a)   // every thread gets the sums
 {
     __shared__ double ss1[32], ss2[32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -634,7 +634,9 @@ __global__ void __launch_bounds__(kRedThreads) reduce_partial_kernel(const doubl
     block_max(a);
     for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
         const double x = lnw[i];
-        if (!isfinite(x))
+        // (a term below e^-60 of the stripe's largest cannot reach the sums' last bit, however many
+        // of the at most 2^31 samples are such; most samples of a loud event are)
+        if (!isfinite(x) || x - a.mx < -60.0)
             continue;
         const double e = term_exp(x - a.mx, f32);
         a.s1 += e;
@@ -674,28 +676,40 @@ __global__ void __launch_bounds__(kRedThreads) reduce_final_kernel(const double 
         a.s2 += o[2] * f * f;
     }
     block_sum(a);
+    // the record and the pooled one by a warp per float64 chain (every thread has the sums)
+    const double N = (double)n;
+    double *s = stats + 8 * slot;
+    __shared__ double ln_n;
+    double ln_s1 = 0.0;
     if (threadIdx.x == 0) {
-        double N = (double)n;
-        double *s = stats + 8 * slot;
-        double var = a.s2 / (a.s1 * a.s1) - 1.0 / N;
-        s[0] = a.mx + log(a.s1) - log(N);
+        ln_s1 = log(a.s1);
+    } else if (threadIdx.x == 32) {
+        ln_n = log(N);
+    } else if (threadIdx.x == 64) {
+        const double var = a.s2 / (a.s1 * a.s1) - 1.0 / N;
         s[1] = sqrt(var > 0.0 ? var : 0.0);
-        s[2] = a.s1;
-        s[3] = a.s1 * a.s1 / a.s2;
-        s[4] = a.mx;
-        s[5] = a.lmx;
-        s[6] = N;
-        s[7] = 0.0;
-        if (a.bad || !isfinite(s[0]))
-            atomicOr(err, kErrNonFinite);
+    } else if (threadIdx.x == 96) {
         Acc pool = reset ? Acc{-INFINITY, 0.0, 0.0, -INFINITY, 0} : Acc{pooled[0], pooled[1], pooled[2], pooled[4], 0};
-        double pn = reset ? 0.0 : pooled[3];
+        const double pn = reset ? 0.0 : pooled[3];
         pool = acc_merge(pool, a);
         pooled[0] = pool.mx;
         pooled[1] = pool.s1;
         pooled[2] = pool.s2;
         pooled[3] = pn + N;
         pooled[4] = pool.lmx;
+    } else if (threadIdx.x == 128) {
+        s[2] = a.s1;
+        s[3] = a.s1 * a.s1 / a.s2;
+        s[4] = a.mx;
+        s[5] = a.lmx;
+        s[6] = N;
+        s[7] = 0.0;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s[0] = a.mx + ln_s1 - ln_n;
+        if (a.bad || !isfinite(s[0]))
+            atomicOr(err, kErrNonFinite);
     }
 }
 
@@ -795,8 +809,11 @@ __global__ void __launch_bounds__(256) hist_partial_kernel(SamplerDev S, const u
         double x = lnw[i];
         if (!isfinite(x))
             continue;
+        const double t = S.temper * (x - mx);
+        if (t < -64.0)   // below 2^-92: zero in the sums' resolution
+            continue;
         uint64_t lo, hi;
-        to_fixed(term_exp(S.temper * (x - mx), f32), lo, hi);
+        to_fixed(term_exp(t, f32), lo, hi);
         if (!(lo | hi))
             continue;
         uint64_t pk = bins[i];
