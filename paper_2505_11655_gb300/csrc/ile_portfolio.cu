@@ -178,43 +178,22 @@ __global__ void __launch_bounds__(kPfThreads) portfolio_draw_kernel(
     }
 }
 
-// Running (max, sum exp(x - max), sum exp(2 (x - max)), count) of one member's ln w.
+// (max, sum exp(x - max), sum exp(2 (x - max)), count) of each member's ln w, the maxima first and
+// the sums relative to them, so that no merge needs an exponential (a chain on this part's slow
+// float64 pipe: merging such records in trees took 76 + 25 us for 200,000 samples) and a term below
+// e^-60 of the largest, which cannot reach the sums' last bit, none either.
 struct MAcc {
     double mx, s1, s2, cnt;
 };
-
-__device__ __forceinline__ void macc_add(MAcc &a, double x)
-{
-    a.cnt += 1.0;
-    if (!isfinite(x))
-        return;
-    if (x > a.mx) {
-        const double f = a.mx == -INFINITY ? 0.0 : exp(a.mx - x);
-        a.s1 = a.s1 * f + 1.0;
-        a.s2 = a.s2 * f * f + 1.0;
-        a.mx = x;
-    } else {
-        const double e = exp(x - a.mx);
-        a.s1 += e;
-        a.s2 += e * e;
-    }
-}
-
-__device__ __forceinline__ MAcc macc_merge(MAcc a, MAcc b)
-{
-    const double mx = fmax(a.mx, b.mx);
-    if (mx == -INFINITY)
-        return MAcc{mx, 0.0, 0.0, a.cnt + b.cnt};
-    const double fa = a.mx == -INFINITY ? 0.0 : exp(a.mx - mx), fb = b.mx == -INFINITY ? 0.0 : exp(b.mx - mx);
-    return MAcc{mx, a.s1 * fa + b.s1 * fb, a.s2 * fa * fa + b.s2 * fb * fb, a.cnt + b.cnt};
-}
 
 // Pass 1: per block, over a contiguous stripe; partial[blk][member][4].
 __global__ void __launch_bounds__(kPfThreads) member_sums_kernel(const double *__restrict__ lnw,
                                                                  const uint8_t *__restrict__ member, int64_t n,
                                                                  double *__restrict__ partial)
 {
-    __shared__ MAcc sh[kNMembers][kPfThreads];
+    constexpr int kWarps = kPfThreads / 32;
+    __shared__ double sh[3][kNMembers][kWarps], smx[kNMembers][kWarps];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t per = (n + gridDim.x - 1) / gridDim.x;
     const int64_t b0 = (int64_t)blockIdx.x * per, b1 = min(n, b0 + per);
     MAcc a[kNMembers];
@@ -226,49 +205,96 @@ __global__ void __launch_bounds__(kPfThreads) member_sums_kernel(const double *_
         const int mi = member[i];
 #pragma unroll
         for (int m = 0; m < kNMembers; ++m)   // register-resident accumulators: no dynamic index
-            if (mi == m)
-                macc_add(a[m], x);
+            if (mi == m) {
+                a[m].cnt += 1.0;
+                if (isfinite(x))
+                    a[m].mx = fmax(a[m].mx, x);
+            }
     }
+#pragma unroll
+    for (int m = 0; m < kNMembers; ++m) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1)
+            a[m].mx = fmax(a[m].mx, __shfl_xor_sync(0xffffffffu, a[m].mx, o));
+        if (lane == 0)
+            smx[m][w] = a[m].mx;
+    }
+    __syncthreads();
 #pragma unroll
     for (int m = 0; m < kNMembers; ++m)
-        sh[m][threadIdx.x] = a[m];
-    __syncthreads();
-    for (int s = kPfThreads / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
+        for (int v = 0; v < kWarps; ++v)
+            a[m].mx = fmax(a[m].mx, smx[m][v]);
+    for (int64_t i = b0 + threadIdx.x; i < b1; i += blockDim.x) {
+        const double x = lnw[i];
+        const int mi = member[i];
+        const double t = x - (mi == 0 ? a[0].mx : mi == 1 ? a[1].mx : a[2].mx);
+        if (!isfinite(x) || t < -60.0)
+            continue;
+        const double e = exp(t);
 #pragma unroll
-            for (int m = 0; m < kNMembers; ++m)
-                sh[m][threadIdx.x] = macc_merge(sh[m][threadIdx.x], sh[m][threadIdx.x + s]);
-        __syncthreads();
+        for (int m = 0; m < kNMembers; ++m)
+            if (mi == m) {
+                a[m].s1 += e;
+                a[m].s2 += e * e;
+            }
     }
-    if (threadIdx.x < kNMembers) {
-        const MAcc r = sh[threadIdx.x][0];
-        double *o = partial + 4 * kNMembers * blockIdx.x + 4 * threadIdx.x;
-        o[0] = r.mx;
-        o[1] = r.s1;
-        o[2] = r.s2;
-        o[3] = r.cnt;
+#pragma unroll
+    for (int m = 0; m < kNMembers; ++m) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+            a[m].s1 += __shfl_xor_sync(0xffffffffu, a[m].s1, o);
+            a[m].s2 += __shfl_xor_sync(0xffffffffu, a[m].s2, o);
+            a[m].cnt += __shfl_xor_sync(0xffffffffu, a[m].cnt, o);
+        }
+        if (lane == 0) {
+            sh[0][m][w] = a[m].s1;
+            sh[1][m][w] = a[m].s2;
+            sh[2][m][w] = a[m].cnt;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < 3 * kNMembers) {
+        const int m = threadIdx.x / 3, q = threadIdx.x - 3 * m;
+        double v = 0.0;
+        for (int u = 0; u < kWarps; ++u)
+            v += sh[q][m][u];
+        double mx = -INFINITY;
+        for (int u = 0; u < kWarps; ++u)
+            mx = fmax(mx, smx[m][u]);
+        double *o = partial + 4 * kNMembers * blockIdx.x + 4 * m;
+        o[1 + q] = v;
+        if (q == 0)
+            o[0] = mx;
     }
 }
 
-// Pass 2: warp m merges member m's partials into out[m][4]: lane l takes blocks l, l + 32,
-// ... in order, then the lanes' results merge in a fixed tree (deterministic for a given
-// block count; a sequential merge over ~300 blocks is a chain of ~600 float64 exponentials).
+// Pass 2: warp m joins member m's partials into out[m][4]: lane l takes blocks l, l + 32, ...
+// in order, then the lanes' sums join in a fixed tree (deterministic for a given block count).
 __global__ void member_sums_final_kernel(const double *__restrict__ partial, int nb, double *__restrict__ out)
 {
     const int m = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (m >= kNMembers)
         return;
     MAcc a{-INFINITY, 0.0, 0.0, 0.0};
+    for (int b = lane; b < nb; b += 32)
+        a.mx = fmax(a.mx, partial[4 * kNMembers * b + 4 * m]);
+#pragma unroll
+    for (int o = 16; o; o >>= 1)
+        a.mx = fmax(a.mx, __shfl_xor_sync(0xffffffffu, a.mx, o));
     for (int b = lane; b < nb; b += 32) {
         const double *o = partial + 4 * kNMembers * b + 4 * m;
-        a = macc_merge(a, MAcc{o[0], o[1], o[2], o[3]});
+        a.cnt += o[3];
+        if (o[0] == -INFINITY)
+            continue;
+        const double f = exp(o[0] - a.mx);
+        a.s1 += o[1] * f;
+        a.s2 += o[2] * f * f;
     }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const MAcc q{__shfl_down_sync(0xffffffffu, a.mx, o), __shfl_down_sync(0xffffffffu, a.s1, o),
-                     __shfl_down_sync(0xffffffffu, a.s2, o), __shfl_down_sync(0xffffffffu, a.cnt, o)};
-        if (lane < o)
-            a = macc_merge(a, q);
+    for (int o = 16; o; o >>= 1) {
+        a.s1 += __shfl_xor_sync(0xffffffffu, a.s1, o);
+        a.s2 += __shfl_xor_sync(0xffffffffu, a.s2, o);
+        a.cnt += __shfl_xor_sync(0xffffffffu, a.cnt, o);
     }
     if (lane == 0) {
         out[4 * m] = a.mx;
