@@ -157,7 +157,12 @@ lnl_block_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const
         const double sh = trig[s_of], ch = trig[S + s_of], sd = trig[2 * S + s_of], cd = trig[3 * S + s_of];
         // Q-sample position of the first bin, (t_lo + dt_k - q_t0_k) fs
         const double u0 = fma(P.xfs[k][0], cd * ch, fma(P.xfs[k][1], cd * sh, fma(P.xfs[k][2], sd, P.ufs0[k])));
-        const double fl = floor(u0);
+        // (of finite angles: the problem's Q window covers every sky position.  Other samples have
+        // no Q index: they are flagged and take column 0, and no address is formed from them)
+        const bool ok = isfinite(u0);
+        if (!ok)
+            atomicOr(err, kErrRange);
+        const double fl = ok ? floor(u0) : 0.0;
         i0s[k * S + s_of] = (int)fl;
         f0s[k * S + s_of] = (float)(u0 - fl);
         const Cx<float> F = response_f(P.Dten_f[k], (float)(-sh), (float)ch, (float)(-sd * ch), (float)(-sd * sh),

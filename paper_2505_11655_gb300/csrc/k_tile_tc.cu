@@ -537,8 +537,13 @@ lnl_tc_kernel(Problem P, BinTable bt, const double *__restrict__ theta, const ui
             // Q-sample position of the first bin, (t_lo + dt_k - q_t0_k) fs
             const double u0 =
                 fma(P.xfs[k][0], sky[s], fma(P.xfs[k][1], sky[kTcS + s], fma(P.xfs[k][2], sky[2 * kTcS + s], P.ufs0[k])));
-            double fl = floor(u0);
-            int i0 = (int)fl;
+            // (of finite angles: the problem's Q window covers every sky position.  Other samples
+            // have no Q index: they are flagged and take column 0; their terms are NaN)
+            const bool ok = isfinite(u0);
+            if (!ok)
+                atomicOr(err, kErrRange);
+            const double fl = ok ? floor(u0) : 0.0;
+            const int i0 = (int)fl;
             i0s[k * kTcS + s] = i0;
             f0s[k * kTcS + s] = __float2uint_rn((float)(u0 - fl) * 0x1p24f);
             // offset range of the tile at detector k: a warp holds 32 samples of one detector
