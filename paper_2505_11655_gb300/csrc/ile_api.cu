@@ -125,19 +125,27 @@ int wigner_table(int l, int m, double *coef, int8_t *pc, int8_t *ps)
 
 // Fourier coefficients of d(iota) = sum_t coef_t cos(iota/2)^pc_t sin(iota/2)^ps_t, a trigonometric
 // polynomial of degree l in iota (pc_t + ps_t = 2 l), even for even m and odd for odd m (the
-// second index of d^l_{m,2} is even): discrete sums over 4 l points, exact up to rounding.
+// second index of d^l_{m,2} is even).  With z = exp(i iota/2) a term is
+// 4^-l i^-ps (z + 1/z)^pc (z - 1/z)^ps, whose expansion in z has integer coefficients; they are
+// summed over t in double-float64 (as discrete sums of long double functions, emulated on some
+// hosts, the tables of 21 modes took 2.2 ms of every handle's creation).
 void polar_fourier(int l, int m, const double *coef, const int8_t *pc, const int8_t *ps, int nt, double *alpha)
 {
-    const int np = 4 * l;
-    const long double step = 2.0L * 3.14159265358979323846264338327950288L / np;
-    for (int j = 0; j < np; ++j) {
-        const long double c = std::cos(0.5L * j * step), s = std::sin(0.5L * j * step);
-        long double d = 0.0L;
-        for (int t = 0; t < nt; ++t)
-            d += (long double)coef[t] * std::pow(c, (int)pc[t]) * std::pow(s, (int)ps[t]);
-        for (int u = 0; u <= l; ++u)
-            alpha[u] += (double)(d * ((m & 1) ? std::sin(u * j * step) : std::cos(u * j * step)) * (u ? 2.0L : 1.0L) / np);
+    double hi[kMaxL + 1] = {}, lo[kMaxL + 1] = {};
+    for (int t = 0; t < nt; ++t) {
+        int w[2 * kMaxL + 1] = {1};   // of z^(2 l - 2 n)
+        for (int f = 0; f < 2 * l; ++f)
+            for (int n = f + 1; n > 0; --n)
+                w[n] += f < pc[t] ? w[n - 1] : -w[n - 1];
+        for (int u = 0; u <= l; ++u) {   // exp(i u iota) = z^(2 u)
+            const double c = ((ps[t] >> 1) & 1) ? -w[l - u] : w[l - u];
+            const double p = c * coef[t], v = hi[u] + p, r = v - hi[u];
+            lo[u] += std::fma(c, coef[t], -p) + ((hi[u] - (v - r)) + (p - r));
+            hi[u] = v;
+        }
     }
+    for (int u = 0; u <= l; ++u)
+        alpha[u] = std::ldexp(hi[u] + lo[u], (u ? 1 : 0) - 2 * l);
 }
 
 // Gauss-Legendre nodes and weights on [-1, 1]: Newton's method on P_n from the
