@@ -48,6 +48,7 @@
 //
 // All waits are bounded (1 s by the global timer), as in k_tile_tc.cu.
 #include <algorithm>
+#include <array>
 #include <climits>
 #include <cmath>
 #include <cuda_fp16.h>
@@ -398,15 +399,29 @@ size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms)
     return (size_t)blocks * K * a_bytes((2 * M + 15) / 16 * 16);
 }
 
+// 2^-(i/128) in units 2^-63 (constants: filled once)
+static const long long *exp2_table()
+{
+    static const std::array<long long, kTable> table = [] {
+        std::array<long long, kTable> t{};
+        for (int i = 0; i < kTable; ++i)
+            t[i] = (long long)(uint64_t)std::ldexp(std::exp2(-(long double)i / kTable), 63);
+        return t;
+    }();
+    return table.data();
+}
+
 void tc64_positions(const rift_ile_config &cfg, long long *pos, long long *u0)
 {
-    for (int j = 0; j < cfg.n_t; ++j) {
-        const long double t =
-            cfg.n_t > 1 ? j * ((long double)cfg.t_hi_s - (long double)cfg.t_lo_s) / (cfg.n_t - 1) : 0.0L;
-        pos[j] = std::llround(std::ldexp(t * (long double)cfg.fs_hz, kFrac));
-    }
-    for (int i = 0; i < kTable; ++i)
-        pos[cfg.n_t + i] = (long long)(uint64_t)std::ldexp(std::exp2(-(long double)i / kTable), 63);
+    // the step with 32 bits behind a position's last (long double is emulated on some hosts: three
+    // operations a bin, with the table above, were 0.3 ms of every handle's creation)
+    __extension__ typedef __int128 wide;
+    constexpr int kGuard = 32;
+    const long double range = (long double)cfg.t_hi_s - (long double)cfg.t_lo_s;
+    const wide step = cfg.n_t > 1 ? (wide)std::ldexp(range * (long double)cfg.fs_hz / (cfg.n_t - 1), kFrac + kGuard) : 0;
+    for (int j = 0; j < cfg.n_t; ++j)
+        pos[j] = (long long)((j * step + ((wide)1 << (kGuard - 1))) >> kGuard);
+    std::copy_n(exp2_table(), kTable, pos + cfg.n_t);
     for (int k = 0; k < cfg.n_det; ++k)
         u0[k] = std::llround(
             std::ldexp(((long double)cfg.t_lo_s - (long double)cfg.q_t0_s[k]) * (long double)cfg.fs_hz, kFrac));
