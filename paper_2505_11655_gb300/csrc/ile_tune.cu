@@ -31,6 +31,10 @@ namespace {
 constexpr int64_t kTuneMinBatch = 4096;   // smaller batches take the untuned default
 constexpr uint32_t kAdaptedAfter = 2;      // iterations after which a sampler counts as adapted
 constexpr int64_t kAdaptedMinBatch = 1 << 19;   // smaller batches keep their first plan
+// Part of a class's name in a kept file: a plan timed on other kernels, or whose numbers meant
+// another sort key, is no plan of these.  Raised with every change of the candidates or of what
+// they run (1: 64-sample CUDA-core tiles, sky keys on the (ra, sin dec) rectangle, unnamed).
+constexpr int kPlanVersion = 2;
 
 struct TuneCache {
     std::mutex mu;
@@ -90,6 +94,7 @@ std::string class_key(const rift_ile_t *h, int64_t n)
     s << "K" << h->prob.K << "_kp" << kp << "_nt" << h->prob.n_t << "_nq" << h->prob.n_q << "_n4^" << nb;
     if (h->prob.dist_marg)   // the distance-marginalised instance is a kernel of its own
         s << "_dm";
+    s << "_v" << kPlanVersion;
     return s.str();
 }
 
