@@ -394,9 +394,10 @@ int lnl_float64(rift_ile_t *h, const double *theta, int64_t n, bool keyed, doubl
         CK(launch_sort(h->grid, h->key, n, h->sort_scratch, h->perm, h->stream, &k));
         k += keyed ? 0 : 1;
     }
+    int l = 0;
     CK(launch_lnl_tc64(h->prob, h->x64, theta, sort ? h->perm : nullptr, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err,
-                       h->stream));
-    h->launches += k + 2;
+                       h->stream, nullptr, 0, &l));
+    h->launches += k + l;
     return RIFT_OK;
 }
 

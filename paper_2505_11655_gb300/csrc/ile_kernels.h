@@ -196,10 +196,11 @@ size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms);
 cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half *q_dig, __half *t_dig, int *t_exp,
                              cudaStream_t st);
 // perm lists the samples (min(n, *n_dev) of them when a device count is given, none when that is
-// at most `skip`; null: in order); outputs at the sample's index.
+// at most `skip`; null: in order); outputs at the sample's index.  *launched: kernels enqueued.
 cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta, const uint32_t *perm, int64_t n,
                             double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
-                            cudaStream_t st, const uint32_t *n_dev = nullptr, uint32_t skip = 0);
+                            cudaStream_t st, const uint32_t *n_dev = nullptr, uint32_t skip = 0,
+                            int *launched = nullptr);
 cudaError_t prepare_tc64_kernels();
 
 // Precision mode RIFT_MIXED: indices of the samples with key[i] >= stats[slot].max - margin

@@ -1091,7 +1091,7 @@ __global__ void combine64_kernel(const Lse *__restrict__ records, const long lon
 
 cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta, const uint32_t *perm, int64_t n,
                             double *lnL_tmarg, double *lnL_t, const double *lnpw, double *lnw, int *err,
-                            cudaStream_t st, const uint32_t *n_dev, uint32_t skip)
+                            cudaStream_t st, const uint32_t *n_dev, uint32_t skip, int *launched)
 {
     if (n <= 0)
         return cudaSuccess;
@@ -1123,6 +1123,8 @@ cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta
     combine64_kernel<<<(int)std::max<int64_t>(1, most), 128, 0, st>>>(reinterpret_cast<const Lse *>(X.records), X.pos, perm, n,
                                                                     n_dev, skip, planned, grid, P.n_t, lnL_tmarg, lnpw, lnw, err,
                                                                     X.unit_counter);
+    if (launched)
+        *launched = 2 + planned;
     return cudaGetLastError();
 }
 
