@@ -936,7 +936,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                             break;
                         const int rel = w0 + kSub * t - 1;
                         const unsigned cols = (unsigned)(kSub * min(2, nsub - t));
-                        if (whi - rel < 0 || wlo - rel >= (int)cols)
+                        if (whi < rel || wlo >= rel + (int)cols)   // (also a warp without bins)
                             continue;
 #pragma unroll
                         for (int i = 0; i < kBpt; ++i) {
@@ -960,6 +960,9 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                         cm = max(cm, lin[i]);
                 if (lnL_t) {
                     const int64_t row = (int64_t)gid[gs] * NT + jb;
+                    if (gid[gs] != 0xffffffffu && !mine)   // a flagged sample has no values
+                        for (int i = 0; i < jq && jb + i < j0 + J; ++i)
+                            lnL_t[row + i] = __longlong_as_double(0x7ff8000000000000LL);
 #pragma unroll
                     for (int i = 0; i < kBpt; ++i)
                         if (i < jn)
@@ -1011,6 +1014,9 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             const uint32_t gi = gid[s_of];
             const double r = __longlong_as_double(0x7ff8000000000000LL);
             atomicOr(err, bad[s_of] | kErrNonFinite);
+            if (lnL_t)
+                for (int j = ch0 * jnom; j < min(NT, ch1 * jnom); ++j)
+                    lnL_t[(int64_t)gi * NT + j] = r;
             if (!split) {
                 lnL_tmarg[gi] = r;
                 if (lnw && lnpw)
