@@ -375,6 +375,17 @@ constexpr float kFixThreshold = 600.f;
 // and launches break even there).
 constexpr int64_t kTc64Unsorted = 512;
 
+// Whether the tensor-core kernel in chunks of the handle's batch size beats the plain kernel on
+// more samples than that: a chunk costs about 90 us + 2e-3 us x (detectors x modes x bins), a sample
+// of the plain kernel 0.1 us + 2e-5 us x the same.  Measured (draws of 2 detectors, 2 modes, 401 bins
+// and of 3, 21, 1001; us by chunks | plain): batch size 64 84 a chunk | 0.14 a draw and 150 | 1.35, 512
+// 99 | 0.14 and 229 | 1.35; 20,000 draws of the small problem on a handle for 64 samples 26318 | 2821.
+bool pays_in_chunks(const rift_ile_t *h)
+{
+    const double w = (double)h->prob.K * h->prob.M * h->prob.n_t;
+    return (double)h->cap * (0.1 + 2e-5 * w) >= 90.0 + 2e-3 * w;
+}
+
 int lnl_float64(rift_ile_t *h, const double *theta, int64_t n, bool keyed, double *lnL_tmarg, double *lnL_t,
                 const double *lnpw, double *lnw)
 {
@@ -1362,7 +1373,8 @@ int rift_ile_fair_draws(rift_ile_t *h, int64_t n_draws, uint64_t seed, int mem, 
         return RIFT_ESTATE;
     const int nt = h->prob.n_t;
     int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_draws, (int64_t)(16 << 20) / nt));
-    if (h->tc64_on)
+    const bool plain = !h->tc64_on || (chunk > h->cap && !pays_in_chunks(h));
+    if (!plain)
         chunk = std::min(chunk, h->cap);   // the sort's buffers hold cap samples
     std::vector<void *> tmp;
     auto grab = [&](size_t bytes) -> void * {
@@ -1398,7 +1410,12 @@ int rift_ile_fair_draws(rift_ile_t *h, int64_t n_draws, uint64_t seed, int mem, 
         // time bins from each drawn sample's per-bin ln L, in float64 (the draws are few)
         for (int64_t c0 = 0; c0 < n_draws; c0 += chunk) {
             const int64_t m = std::min(chunk, n_draws - c0);
-            RK(lnl_float64(h, th + 6 * c0, m, false, lt, bins, nullptr, nullptr));
+            if (plain) {
+                CK(launch_lnl_fp64(h->prob, th + 6 * c0, m, lt, bins, nullptr, nullptr, h->err, h->stream));
+                h->launches += 1;
+            } else {
+                RK(lnl_float64(h, th + 6 * c0, m, false, lt, bins, nullptr, nullptr));
+            }
             CK(launch_fair_time(bins, m, nt, Ut + c0, h->prob.t_lo, h->prob.t_step, jj + c0, tt + c0, h->stream));
             h->launches += 1;
         }

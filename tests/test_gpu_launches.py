@@ -44,3 +44,20 @@ def test_counts(G, mode, n):
             a = G.rift_ile_kernel_launches(h.h)
             k = seen(f)
             assert G.rift_ile_kernel_launches(h.h) - a == k
+
+
+@pytest.mark.parametrize("modes,cap", [(2, 64), (21, 32)])
+def test_many_draws_from_a_small_handle(G, modes, cap):
+    """Draws beyond a small handle's batch size are not evaluated in chunks of it, a sort and a
+    tensor-core launch each; the draws are those of a large handle."""
+    import numpy as np
+    p = S.make_problem(("H1", "L1"), modes, 4096.0, n_t=201, snr=15.0, seed=S.config_seed(6, 132))
+    out = []
+    for size in (cap, 6000):
+        with G.ILE(p, precision=G.RIFT_FP64, max_samples=size, seed=4) as h:
+            h.marginalize(cap)
+            a = G.rift_ile_kernel_launches(h.h)
+            out.append(h.fair_draws(5000, seed=9))
+            assert G.rift_ile_kernel_launches(h.h) - a <= 24
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
