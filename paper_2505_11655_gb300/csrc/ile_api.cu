@@ -290,28 +290,14 @@ int sync_and_err(rift_ile_t *h, int *flags_out)
 
 bool use_fp32(const rift_ile_t *h) { return h->cfg.precision != RIFT_FP64; }
 
-// Without a tuned plan: tensor-core tiles pay off from the batch size at which they overtake the
-// CUDA-core kernel (which takes any spread of delays at the same cost): 10,000 samples with one
-// detector, 16,000 with more, and with three detectors, whose sort key is the sky position, once
-// a tile of the sorted batch spans about one window of 64 columns (256 samples per patch of that
-// size on the delays' surface).  Measured (us, CUDA cores | tensor cores): 2 detectors, 9 modes,
-// 16384 Hz, 10,000 samples 272 | 347, 30,000 457 | 333; 3 detectors, 21 modes, 16384 Hz, 20,000
-// samples 639 | 761, 30,000 847 | 793; 3 detectors, 9 modes, 4096 Hz, 10,000 samples 256 | 330,
-// 20,000 331 | 303; 1 detector, 2 modes, 10,000 samples 182 | 181.
-int64_t tc_min_batch(const rift_ile_t *h)
-{
-    const Problem &P = h->prob;
-    if (P.K == 1)
-        return 10000;
-    double span = 0.0;
-    for (int k = 0; P.K >= 3 && k < P.K; ++k) {
-        double r2 = 0.0;
-        for (int i = 0; i < 3; ++i)
-            r2 += P.xpos[k][i] * P.xpos[k][i];
-        span = std::max(span, 2.0 * std::sqrt(r2) * P.fs / 64.0);
-    }
-    return (int64_t)std::min(1e6, std::max(16000.0, 256.0 * span * span));
-}
+// Without a tuned plan: tensor-core tiles from this batch size.  They are faster from 10,000 to
+// 30,000 samples up (99,999 samples, us, CUDA cores | tensor cores: 2 detectors, 9 modes, 16384 Hz
+// 1067 | 471; 3, 21 2164 | 808; 2, 2, 4096 Hz 523 | 310), but their operands are float16 pairs (22
+// bits): below the line a batch keeps the float32 products of the CUDA-core kernel.  20,000 samples,
+// rms error of ln L, CUDA cores | tensor cores: 2 detectors, 9 modes, SNR 20 2.2e-5 | 2.3e-5, SNR 40
+// 3.0e-5 | 3.6e-5, SNR 150 5.9e-5 | 1.8e-4; 1 detector, 12 modes, SNR 40 4.0e-5 | 5.5e-5, SNR 150
+// 1.2e-4 | 6.0e-4.
+constexpr int64_t kTcMinBatch = 100000;
 
 bool use_tc(const rift_ile_t *h, int64_t n)
 {
@@ -319,7 +305,7 @@ bool use_tc(const rift_ile_t *h, int64_t n)
         return false;
     if (h->tc_mode == 1)
         return true;
-    return h->plan.tc >= 0 ? h->plan.tc == 1 : n >= tc_min_batch(h);
+    return h->plan.tc >= 0 ? h->plan.tc == 1 : n >= kTcMinBatch;
 }
 
 // Below this many samples the CUDA-core kernel takes them in index order: their windows'
