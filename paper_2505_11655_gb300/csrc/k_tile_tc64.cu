@@ -26,7 +26,9 @@
 //     resolution.  A chunk's bins are summed by four threads relative to their common maximum, and
 //     the chunks' sums merged in order.
 // The template term is contracted the same way, W_k = Z_k T_k (the real quadratic form of
-// k_tile_tc.cu) and summed against the float64 components.
+// k_tile_tc.cu), with one order more (it is the whole of a faint sample's value, and what the orders
+// beyond 6 leave out does not average away in a quadratic form), and summed against the components
+// in 128-bit integers.
 //
 // Tiles are 128 samples in the order of the sky sort.  A tile's window on the Q grid is as
 // wide as its samples' delays need (no sub-groups: a chunk of 64 time bins walks the
@@ -41,8 +43,10 @@
 // Measured (3 detectors, 21 modes, 16384 Hz, 1001 bins, 20011 prior samples): 20.3 ms for the
 // plain float64 kernel (70% of the float64 issue rate), 1.35 ms here; 100,000 samples 98.5 ->
 // 4.3 ms; 64 samples of the smallest problem (2 detectors, 2 modes) 109 -> 107 us.  Against
-// 80-bit arithmetic its per-bin values are closer than the plain kernel's (rms 2.7e-13
-// against 4.1e-13 here).  What bounds it now is instruction issue (46% of the slots: the
+// 80-bit arithmetic (8 problems at 3 SNRs, 1000 prior samples each, relative norms) its per-bin values
+// are closer than the plain kernel's (0.45 to 0.85 of its error), ln L is as close (geometric mean of
+// the ratios 0.94; the template term alone 4.0e-16 to 5.9e-16 in both: the geometry's roundings).
+// With orders to 6 and float64 sums the template term had up to 6.6e-16.  What bounds it now is instruction issue (46% of the slots: the
 // joins of the accumulators, the gathers' 64-bit arithmetic) and the tail of uneven tiles; the
 // tensor pipe is 26% busy, the float64 pipe 11%.
 //
@@ -52,6 +56,7 @@
 #include <climits>
 #include <cmath>
 #include <cuda_fp16.h>
+#include <type_traits>
 
 #include "ile_kernels.h"
 #include "tc_ptx.cuh"
@@ -71,7 +76,8 @@ constexpr int kIssuer = kConsumers / 32, kStager = kIssuer + 1;
 constexpr int kQ = kConsumers / kS;      // threads per sample
 constexpr int kBpt = 16;                 // time bins per thread and chunk
 constexpr int kChunk = kQ * kBpt;
-constexpr int kAccCols = kDig * kSub;    // tensor-memory columns of one set of accumulators
+constexpr int kOrders = kDig + 1;        // (the last of the template term only)
+constexpr int kAccCols = kOrders * kSub; // tensor-memory columns of one set of accumulators
 constexpr int kTable = kTc64Table;       // entries 2^-(i/128) of the exponential
 constexpr int kFrac = 48;                // fraction bits of a Q position
 constexpr int kPows = kMaxPow + 1;
@@ -87,7 +93,7 @@ static_assert(2 * kAccCols <= 512, "two sets of accumulators in tensor memory");
 static_assert(kS * kMaxDet <= kConsumers, "one (sample, detector) item per consumer thread");
 
 struct Layout64 {
-    size_t a, b, r, pos, u0, quad, sc, gid, bad, tbl, m2, lo, bar, tptr, end;
+    size_t a, b, r, pos, u0, sc, gid, bad, tbl, m2, lo, bar, tptr, end;
     size_t nv, e5, ps, pw, pe, F, Y, pend;   // prologue tables, aliased on a, b, r
     int kp;
 };
@@ -114,7 +120,6 @@ __host__ __device__ inline Layout64 layout64(int K, int M, int n_t)
     o = p > o ? al64(p) : o;
     L.pos = o;  o = al64(o + (size_t)n_t * 8, 16);
     L.u0 = o;   o = al64(o + (size_t)K * kS * 8, 16);
-    L.quad = o; o = al64(o + (size_t)kQ * kS * 8, 16);
     L.sc = o;   o = al64(o + (size_t)kS * 4, 16);
     L.gid = o;  o = al64(o + (size_t)kS * 4, 16);
     L.bad = o;  o = al64(o + (size_t)kS * 4, 16);
@@ -302,6 +307,8 @@ struct DiffScale {
     }
 };
 
+__extension__ typedef __int128 wide128;
+
 // Log-sum-exp over bins: sum of exp(lin - max) in units 2^-kSumBits, max as an integer.
 struct Lse {
     long long m;
@@ -334,14 +341,43 @@ __device__ __forceinline__ Lse merge64(const DiffScale &ds, Lse a, Lse b, const 
     return a;
 }
 
-__device__ __forceinline__ double lse_value(Lse v, int lexp, double quad, int n_t)
+// A double and what it lacks.
+struct Two {
+    double hi, lo;
+};
+
+__device__ __forceinline__ Two two_sum(double a, double b)
+{
+    const double s = __dadd_rn(a, b), r = __dsub_rn(s, a);
+    return {s, __dadd_rn(__dsub_rn(a, __dsub_rn(s, r)), __dsub_rn(b, r))};
+}
+
+// (v has fewer than 2^62)
+__device__ __forceinline__ Two two_of(long long v)
+{
+    const double h = (double)v;
+    return {h, (double)(v - (long long)h)};
+}
+
+// max 2^lexp - quad + ln(sum) - ln(n_t) with one rounding of its large terms
+__device__ __forceinline__ double lse_value(Lse v, int lexp, double quad, float quad_lo, int n_t)
 {
     const double sum = (double)v.s * (1.0 / (double)(1ull << kSumBits));
-    return __dsub_rn(mul_pow2((double)v.m, lexp), quad) + __dsub_rn(log(sum), log((double)n_t));
+    const Two m = two_of(v.m), d = two_sum(mul_pow2(m.hi, lexp), -quad);
+    const double rest = __dadd_rn(d.lo, __dsub_rn(mul_pow2(m.lo, lexp), (double)quad_lo));
+    return __dadd_rn(d.hi, __dadd_rn(rest, __dsub_rn(log(sum), log((double)n_t))));
+}
+
+// What the combination needs of a sample beside its chunks' sums and its template term: the scale
+// (|lexp| < 4400), the error flags and what the template term lacks.
+__device__ __forceinline__ uint64_t pack_info(int lexp, int flags, float quad_lo)
+{
+    return (uint64_t)(uint16_t)(int16_t)lexp | ((uint64_t)(uint16_t)flags << 16) |
+           ((uint64_t)__float_as_uint(quad_lo) << 32);
 }
 
 // one accumulator set joined to X (see the head of the file)
-__device__ __forceinline__ long long join_orders(const uint32_t (&v)[kDig][4], int i)
+template <int kN> __device__ __forceinline__ long long join_orders(const uint32_t (&v)[kN][4], int i)
 {
     constexpr float kMagic = 12582912.f;   // 1.5 2^23: float bits 0x4B400000 + integer
     constexpr uint64_t kB = 0x4B400000ull;
@@ -352,7 +388,10 @@ __device__ __forceinline__ long long join_orders(const uint32_t (&v)[kDig][4], i
     const uint32_t b3 = __float_as_uint(__uint_as_float(v[3][i]) + kMagic);
     const uint32_t b4 = __float_as_uint(__uint_as_float(v[4][i]) + kMagic);
     const uint32_t b5 = __float_as_uint(__uint_as_float(v[5][i]) + kMagic);
-    const uint32_t b6 = __float_as_uint(fmaf(__uint_as_float(v[6][i]), 0x1p-8f, kMagic));
+    float last = __uint_as_float(v[6][i]);
+    if (kN > kDig)
+        last = fmaf(__uint_as_float(v[kN - 1][i]), 0x1p-8f, last);
+    const uint32_t b6 = __float_as_uint(fmaf(last, 0x1p-8f, kMagic));
     uint64_t x = (uint64_t)b5 + b6 - kBias;
     x += (uint64_t)b4 * 256u;
     x += (uint64_t)b3 * 65536u;
@@ -515,7 +554,6 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
     long long *Rs = reinterpret_cast<long long *>(sm + L.r);        // [1 + kBlk][kS]; row 0 the previous block's last
     long long *pos = reinterpret_cast<long long *>(sm + L.pos);     // [NT] bin offset in Q samples, kFrac fraction bits
     long long *U0 = reinterpret_cast<long long *>(sm + L.u0);       // [K][kS] Q position of the first bin
-    double *quads = reinterpret_cast<double *>(sm + L.quad);        // [kQ][kS] template term partials
     int *scs = reinterpret_cast<int *>(sm + L.sc);                  // [kS] c = I 2^-sc
     uint32_t *gid = reinterpret_cast<uint32_t *>(sm + L.gid);
     int *bad = reinterpret_cast<int *>(sm + L.bad);                 // [kS] error flags of the sample
@@ -645,14 +683,26 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     pp *= sh;
                 }
             } else {
-                double sp, cp;
-                sincos(valid ? th[3] : 0.0, &sp, &cp);
-                double er = 1.0, ei = 0.0;   // exp(-i j phi)
-                for (int j = 0; j <= kMaxL; ++j) {
-                    pe[j * kS + s_of] = make_double2(er, ei);
-                    const double t = er * cp + ei * sp;
-                    ei = ei * cp - er * sp;
-                    er = t;
+                // exp(-i j phi): the first two from the functions (2 phi is exact), the others from
+                // the one two below, brought back to modulus one (the products' roundings add up in
+                // the modulus, and twice that in the template term)
+                const double phi = valid ? th[3] : 0.0;
+                double2 e[2];
+#pragma unroll 1
+                for (int j = 1; j <= 2; ++j) {
+                    double sp, cp;
+                    sincos(j * phi, &sp, &cp);
+                    pe[j * kS + s_of] = make_double2(cp, -sp);
+                }
+                pe[s_of] = make_double2(1.0, 0.0);
+                e[1] = pe[kS + s_of];
+                const double2 two = e[0] = pe[2 * kS + s_of];
+#pragma unroll
+                for (int j = 3; j <= kMaxL; ++j) {
+                    const double2 x = e[j & 1];
+                    const double t = x.x * two.x - x.y * two.y, u = x.x * two.y + x.y * two.x;
+                    const double over = 0.5 * fma(t, t, fma(u, u, -1.0));
+                    pe[j * kS + s_of] = e[j & 1] = make_double2(fma(-over, t, t), fma(-over, u, u));
                 }
             }
         }
@@ -758,7 +808,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
         int failed = 0;
         if (warp == kIssuer) {
             if (lane == 0 && any) {
-                auto batch = [&]() {
+                auto batch = [&](bool wide) {   // wide: orders 0..7, else 0..6
                     const uint32_t b = g & 1u, u = g >> 1;
                     if (!tc::mbar_wait(full + b, u & 1u, kWait) ||
                         (u > 0 && !tc::mbar_wait(empty + b, (u - 1u) & 1u, kWait)))
@@ -768,10 +818,16 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     for (int kk = 0; kk < kp / 16; ++kk) {
                         const uint64_t bd = desc(B, 256u * (uint32_t)kk);
 #pragma unroll
-                        for (int i = 0; i < kDig; ++i)
-                            tc::mma_f16_ss(tmem + b * kAccCols + (uint32_t)(i * kSub),
-                                           desc(As + (size_t)i * kS * kp, 256u * (uint32_t)kk), bd,
-                                           tc::idesc_f16_f32(kS, (uint32_t)((kDig - i) * kSub)), (kk | i) != 0);
+                        for (int i = 0; i < kDig; ++i) {
+                            const uint64_t ad = desc(As + (size_t)i * kS * kp, 256u * (uint32_t)kk);
+                            if (wide && i == 1)   // the first of order 7's products, by itself: it starts the sum
+                                tc::mma_f16_ss(tmem + b * kAccCols + (uint32_t)(kDig * kSub), ad,
+                                               desc(B + (size_t)(kDig - 1) * kSub * kp, 256u * (uint32_t)kk),
+                                               tc::idesc_f16_f32(kS, kSub), kk != 0);
+                            const int digits = kDig - i + (wide && i > 1 ? 1 : 0);
+                            tc::mma_f16_ss(tmem + b * kAccCols + (uint32_t)(i * kSub), ad, bd,
+                                           tc::idesc_f16_f32(kS, (uint32_t)(digits * kSub)), (kk | i) != 0);
+                        }
                     }
                     tc::mma_commit(done + b);
                     ++g;
@@ -779,7 +835,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                 };
                 auto digits = [&]() { return tc::mbar_wait(fullA, (ga++) & 1u, kWait); };
                 for (int k = 0; k < K && !failed; ++k)
-                    failed = !digits() || !batch() || !batch();
+                    failed = !digits() || !batch(true) || !batch(true);
                 for (int ch = ch0; ch < ch1 && !failed; ++ch)
                     for (int k = 0; k < K && !failed; ++k) {
                         int w0, nsub;
@@ -787,7 +843,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                         if (K > 1)
                             failed = !digits();
                         for (int t = 0; t < nsub && !failed; ++t)
-                            failed = !batch();
+                            failed = !batch(false);
                     }
             }
             __syncwarp();
@@ -835,8 +891,9 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             const int q = warp & 3, cb = warp >> 2, s = 32 * q + lane;   // drain: quarter, 8 columns of 32
             const int gs = s_of, gh = grp;                               // gather: sample, quarter of the bins
             const bool mine = gid[gs] != 0xffffffffu && !bad[gs];
-            // drain one batch into rows 1 + 32 sub.. of R
-            auto drain = [&](int sub) {
+            // drain one batch of kN orders into rows 1 + 32 sub.. of R
+            auto drain = [&](int sub, auto orders) {
+                constexpr int kN = decltype(orders)::value;
                 const uint32_t b = g & 1u;
                 const int ok = tc::mbar_wait(done + b, (g >> 1) & 1u, kWait) ? 1 : 0;
                 ++g;
@@ -844,9 +901,9 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                 long long *out = Rs + (size_t)(1 + kSub * sub + 8 * cb) * kS + s;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
-                    uint32_t v[kDig][4];
+                    uint32_t v[kN][4];
 #pragma unroll
-                    for (int o = 0; o < kDig; ++o)
+                    for (int o = 0; o < kN; ++o)
                         tc::tmem_ld4(tmem + ((uint32_t)(32 * q) << 16) + b * kAccCols +
                                          (uint32_t)(o * kSub + 8 * cb + 4 * h),
                                      v[o]);
@@ -864,14 +921,18 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             const int sc = scs[gs];
 
             // ---- template term: W = Z T, quad = kappa sum_k sum_n z_n W_n
-            double qacc = 0.0;
+            wide128 qacc = 0;
+            int et = X.t_exp[0];
+            for (int k = 1; k < K; ++k)
+                et = max(et, X.t_exp[k]);
             for (int k = 0; k < K && !failed; ++k) {
                 tc::named_bar_or(qbar, kConsumers / 4, 0);   // R free
-                const int ok0 = drain(0), ok1 = drain(1);
+                const std::integral_constant<int, kOrders> all{};
+                const int ok0 = drain(0, all), ok1 = drain(1, all);
                 failed = tc::named_bar_or(qbar, kConsumers / 4, !ok0 || !ok1 || abort_s);
                 if (failed)
                     break;
-                double acc = 0.0;
+                wide128 acc = 0;   // below 2^120
                 const __half *zs = scratch + ((size_t)k * kDig * kS + (size_t)(gs >> 3) * 8) * kp + (gs & 7) * 8;
                 for (int kc = gh; kc < kcs; kc += kQ) {
                     uint32_t w[kDig][4];
@@ -894,15 +955,33 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                             const uint32_t hb = w[p][j >> 1] >> (16 * (j & 1));
                             I = I * 256 + (long long)__half2int_rn(__ushort_as_half((unsigned short)hb));
                         }
-                        acc = fma((double)I, (double)Rs[(size_t)(1 + nn) * kS + gs], acc);
+                        acc += (wide128)I * Rs[(size_t)(1 + nn) * kS + gs];
                     }
                 }
-                qacc += mul_pow2(acc, 56 - 2 * sc - (55 - X.t_exp[k]));
+                qacc += acc >> min(et - X.t_exp[k], 127);   // (a unit of W is 2^55 of these)
             }
-            quads[gh * kS + gs] = qacc;
-            // the four partials of a sample belong to the warps of its quarter (q == gs / 32)
+            // the four partials of a sample belong to the warps of its quarter (q == gs / 32); they
+            // meet in rows of R behind the last component's
+            long long *const qs = Rs + (size_t)(kBlk - 2 * kQ) * kS + gs;
+            qs[2 * gh * kS] = (long long)qacc;
+            qs[(2 * gh + 1) * kS] = (long long)(qacc >> 64);
             failed = tc::named_bar_or(qbar, kConsumers / 4, failed);
-            const double quad = P.kappa * ((quads[gs] + quads[kS + gs]) + (quads[2 * kS + gs] + quads[3 * kS + gs]));
+            double quad = 0.0;
+            float quad_lo = 0.f;
+            if (gh == 0 || lnL_t) {
+                qacc = 0;
+#pragma unroll
+                for (int h = 0; h < kQ; ++h)
+                    qacc += (wide128)qs[(2 * h + 1) * kS] << 64 | (uint64_t)qs[2 * h * kS];
+                // the 62 leading bits as two doubles
+                const uint64_t mag = (uint64_t)((qacc < 0 ? -qacc : qacc) >> 64);
+                const int sh = mag ? __clzll((long long)mag) - 2 : 62;
+                const Two v = two_of((long long)((qacc << sh) >> 64));
+                const int e = 64 - sh + 56 - 2 * sc - (55 - et);
+                const double lo = P.kappa * mul_pow2(v.lo, e);
+                quad = P.kappa * mul_pow2(v.hi, e);
+                quad_lo = fabs(lo) < 1e30 ? (float)lo : 0.f;
+            }
 
             const int lexp = 56 - sc - sq;   // lin = X 2^lexp
             DiffScale ds;
@@ -929,9 +1008,10 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                         tc::named_bar_or(qbar, kConsumers / 4, 0);   // the previous block's gathers are done
                         if (cb == 3 && t > 0)
                             Rs[s] = Rs[(size_t)kBlk * kS + s];
-                        int ok = drain(0);
+                        const std::integral_constant<int, kDig> most{};
+                        int ok = drain(0, most);
                         if (t + 1 < nsub)
-                            ok &= drain(1);
+                            ok &= drain(1, most);
                         if ((failed = tc::named_bar_or(qbar, kConsumers / 4, !ok || abort_s)))
                             break;
                         const int rel = w0 + kSub * t - 1;
@@ -996,7 +1076,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                 int flags = bad[gs];
                 if (!split) {
                     const double r = flags ? __longlong_as_double(0x7ff8000000000000LL)
-                                           : lse_value(run, lexp, quad, NT);
+                                           : lse_value(run, lexp, quad, quad_lo, NT);
                     if (!isfinite(r))
                         flags |= kErrNonFinite;
                     lnL_tmarg[gi] = r;
@@ -1004,7 +1084,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                         lnw[gi] = r + lnpw[gi];
                 } else if (ch0 == 0) {
                     records[((int64_t)n_chunks * n_tiles + tile) * kS + gs] =
-                        Lse{__double_as_longlong(quad), (uint64_t)(uint32_t)lexp | ((uint64_t)(uint32_t)flags << 32)};
+                        Lse{__double_as_longlong(quad), pack_info(lexp, flags, quad_lo)};
                 }
                 if (flags)
                     atomicOr(err, flags);
@@ -1022,7 +1102,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                 if (lnw && lnpw)
                     lnw[gi] = r;
             } else if (ch0 == 0) {
-                records[((int64_t)n_chunks * n_tiles + tile) * kS + s_of] = Lse{0, (uint64_t)kErrNonFinite << 32};
+                records[((int64_t)n_chunks * n_tiles + tile) * kS + s_of] = Lse{0, pack_info(0, kErrNonFinite, 0.f)};
             }
         }
         failed = __syncthreads_or(failed || abort_s);
@@ -1074,16 +1154,16 @@ __global__ void combine64_kernel(const Lse *__restrict__ records, const long lon
     __syncthreads();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_use; i += (int64_t)gridDim.x * blockDim.x) {
         const Lse info = records[(int64_t)n_chunks * n_tiles * kS + i];
-        const int lexp = (int)(uint32_t)info.s;
+        const int lexp = (int)(int16_t)info.s, flags = (int)(uint16_t)(info.s >> 16);
         const uint32_t g = perm ? perm[i] : (uint32_t)i;
         double r = __longlong_as_double(0x7ff8000000000000LL);
-        if ((info.s >> 32) == 0) {
+        if (flags == 0) {
             DiffScale ds;
             ds.set(lexp);
             Lse run = records[i];
             for (int c = 1; c < n_chunks; ++c)
                 run = merge64(ds, run, records[(int64_t)c * n_tiles * kS + i], tbl);
-            r = lse_value(run, lexp, __longlong_as_double(info.m), n_t);
+            r = lse_value(run, lexp, __longlong_as_double(info.m), __uint_as_float((uint32_t)(info.s >> 32)), n_t);
         }
         if (!isfinite(r))
             atomicOr(err, kErrNonFinite);
