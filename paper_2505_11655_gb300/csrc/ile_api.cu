@@ -290,6 +290,8 @@ int sync_and_err(rift_ile_t *h, int *flags_out)
 
 bool use_fp32(const rift_ile_t *h) { return h->cfg.precision != RIFT_FP64; }
 
+bool use_tc64(const rift_ile_t *h) { return h->tc64_on && !h->plain64; }
+
 // Without a tuned plan: tensor-core tiles from this batch size.  They are faster from 10,000 to
 // 30,000 samples up (99,999 samples, us, CUDA cores | tensor cores: 2 detectors, 9 modes, 16384 Hz
 // 1067 | 471; 3, 21 2164 | 808; 2, 2, 4096 Hz 523 | 310), but their operands are float16 pairs (22
@@ -375,7 +377,7 @@ bool pays_in_chunks(const rift_ile_t *h)
 int lnl_float64(rift_ile_t *h, const double *theta, int64_t n, bool keyed, double *lnL_tmarg, double *lnL_t,
                 const double *lnpw, double *lnw)
 {
-    if (!h->tc64_on) {
+    if (!use_tc64(h)) {
         CK(launch_lnl_fp64(h->prob, theta, n, lnL_tmarg, lnL_t, lnpw, lnw, h->err, h->stream));
         h->launches += 1;
         return RIFT_OK;
@@ -409,7 +411,7 @@ int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmar
     CK(launch_reduce(key, lnL_tmarg, n, h->red_partial, h->stats, kScratchSlot, h->pooled_scratch, 1, h->err,
                      h->stream));
     CK(launch_select(key, sorts_batch(h, n) ? h->perm : nullptr, n, h->stats, kScratchSlot, kMixedMargin, h->sel_idx, h->sel_count, h->stream));
-    if (h->tc64_on) {
+    if (use_tc64(h)) {
         CK(launch_refine_few(h->prob, theta, h->sel_idx, h->sel_count, kRefineFew, lnL_tmarg, lnpw, lnw, h->err,
                              h->stream));
         CK(launch_lnl_tc64(h->prob, h->x64, theta, h->sel_idx, n, lnL_tmarg, nullptr, lnpw, lnw, h->err,
@@ -842,7 +844,7 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
         int *unit_counter = nullptr;
         long long *pos = nullptr;
         unsigned long long *units = nullptr;
-        if ((rc = dalloc(h, &h->qmax64, (size_t)2)) || (rc = dalloc(h, &h->q_dig, tc64_q_halves(K, M, P.tc_groups))) ||
+        if ((rc = dalloc(h, &h->qmax64, tc64_scale_words(K, M))) || (rc = dalloc(h, &h->q_dig, tc64_q_halves(K, M, P.tc_groups))) ||
             (rc = dalloc(h, &h->t_dig, tc64_t_halves(K, M))) || (rc = dalloc(h, &h->t_exp64, (size_t)kMaxDet)) ||
             (rc = dalloc(h, &scratch, tc64_scratch_bytes(K, M, N, sms))) ||
             (rc = dalloc(h, &records, tc64_record_bytes(N, cfg->n_t))) || (rc = dalloc(h, &pos, (size_t)cfg->n_t + kTc64Table)) ||
@@ -961,7 +963,7 @@ int64_t rift_ile_footprint(const rift_ile_config *cfg)
         K * 2 * groups * kp * 8 * 2, 5 * kRedBlocks * 8, 152 * 12 * B * 8, 8 * (RIFT_MAX_ITER + 1) * 8, 3 * 8 * 8,
         N * 4, 16, 6 * B * 8, 6 * (B + 1) * 8, 6 * B * 8, 16, (int64_t)kSelectWords * 4,
         cfg->precision == RIFT_MIXED && !digits ? std::min<int64_t>(N, kRefineRows) * nt * 8 : 0,
-        digits ? 2 * (int64_t)(tc64_q_halves(K, M, groups) + tc64_t_halves(K, M)) + 7 * 16 + 8 * (nt + kTc64Table) +
+        digits ? 2 * (int64_t)(tc64_q_halves(K, M, groups) + tc64_t_halves(K, M)) + 8 * (int64_t)tc64_scale_words(K, M) + 7 * 16 + 8 * (nt + kTc64Table) +
                      (int64_t)(16 * tc64_units_cap(N) + tc64_scratch_bytes(K, M, N, 152) + tc64_record_bytes(N, cfg->n_t))
                : 0,
         // large-term correction: per-sample side outputs and list, double-float tables of the
@@ -1132,14 +1134,16 @@ int install_overlaps(rift_ile_t *h)
         h->launches += 3;
     }
     if (h->tc64_on) {
-        CK(launch_prep_tc64(h->prob, h->qmax64, h->q_dig, h->t_dig, h->t_exp64, h->stream));
+        CK(launch_prep_tc64(h->prob, h->qmax64, h->q_dig, h->t_dig, h->t_exp64, h->err, h->stream));
         h->launches += 3;
     }
     if (h->fix_on) {
         CK(launch_fix_prep(h->prob, h->fix, h->stream));
         h->launches += 2;
     }
-    int rc = sync_and_err(h);
+    int flags = 0;
+    int rc = sync_and_err(h, &flags);
+    h->plain64 = (flags & kNoteUneven) != 0;
     h->have_overlaps = (rc == RIFT_OK);
     return rc;
 }
@@ -1359,7 +1363,7 @@ int rift_ile_fair_draws(rift_ile_t *h, int64_t n_draws, uint64_t seed, int mem, 
         return RIFT_ESTATE;
     const int nt = h->prob.n_t;
     int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(n_draws, (int64_t)(16 << 20) / nt));
-    const bool plain = !h->tc64_on || (chunk > h->cap && !pays_in_chunks(h));
+    const bool plain = !use_tc64(h) || (chunk > h->cap && !pays_in_chunks(h));
     if (!plain)
         chunk = std::min(chunk, h->cap);   // the sort's buffers hold cap samples
     std::vector<void *> tmp;

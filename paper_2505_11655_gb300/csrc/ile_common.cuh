@@ -25,6 +25,7 @@ constexpr int kMaxPow = 2 * kMaxL + 2;   // largest power of cos(iota/2), sin(io
 
 // Error flags raised by kernels (OR-ed into a device word).
 constexpr int kErrRange = 1;
+constexpr int kNoteUneven = 256;   // in the error word of an overlaps' installation: no error (k_tile_tc64.cu)
 constexpr int kErrNonFinite = 2;
 constexpr int kErrTimeout = 4;
 

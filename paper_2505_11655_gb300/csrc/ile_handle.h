@@ -17,7 +17,11 @@ struct LaunchPlan {
     int tc = -1;         // 1 tensor-core tiles, 0 CUDA-core tiles, -1 not chosen yet
     int per_cell = 4;    // samples per Hilbert sky cell
     int delay3 = 0;      // three or more detectors: 1 sorts by a Morton key of three delays
-    bool operator==(const LaunchPlan &o) const { return tc == o.tc && per_cell == o.per_cell && delay3 == o.delay3; }
+    int plain64 = 0;     // rift_ile::plain64 (what a captured sequence was recorded with)
+    bool operator==(const LaunchPlan &o) const
+    {
+        return tc == o.tc && per_cell == o.per_cell && delay3 == o.delay3 && plain64 == o.plain64;
+    }
     bool operator!=(const LaunchPlan &o) const { return !(*this == o); }
 };
 
@@ -72,6 +76,7 @@ struct rift_ile {
     float fix_thr = 0.f;
     // float64-accurate tensor-core likelihood (RIFT_FP64 batches, RIFT_MIXED re-evaluation)
     bool tc64_on = false;
+    bool plain64 = false;   // the overlaps are too uneven for its fixed point
     rift::Tc64 x64{};
     unsigned long long *qmax64 = nullptr;
     __half *q_dig = nullptr, *t_dig = nullptr;

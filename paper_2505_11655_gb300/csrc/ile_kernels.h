@@ -171,7 +171,7 @@ cudaError_t launch_prep_tc(const double2 *Q64, int K, int M, int n_q, int groups
 // Float64-accurate likelihood on the tensor cores (k_tile_tc64.cu): digits of Q and of the
 // template matrices, and the kernel's scratch.
 struct Tc64 {
-    const unsigned long long *qmax;   // bits of max|Q|
+    const unsigned long long *qmax;   // bits of the largest |Re Q|, |Im Q| that a bin can reach
     const __half *q_dig, *t_dig;
     const int *t_exp;
     unsigned char *scratch;           // coefficient digits of the resident tiles
@@ -193,8 +193,10 @@ constexpr int kTc64Table = 128;
 void tc64_positions(const rift_ile_config &cfg, long long *pos, long long *u0);
 int64_t tc64_units_cap(int64_t n_max);
 size_t tc64_scratch_bytes(int K, int M, int64_t n_max, int sms);
+size_t tc64_scale_words(int K, int M);   // of qmax: the scale, then (largest, mean square) of every (detector, mode)
+// *err gets kNoteUneven where the overlaps' sizes are too different for one scale.
 cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half *q_dig, __half *t_dig, int *t_exp,
-                             cudaStream_t st);
+                             int *err, cudaStream_t st);
 // perm lists the samples (min(n, *n_dev) of them when a device count is given, none when that is
 // at most `skip`; null: in order); outputs at the sample's index.  *launched: kernels enqueued.
 cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta, const uint32_t *perm, int64_t n,

@@ -178,6 +178,7 @@ int choose_plan_tuned(rift_ile_t *h, int64_t n, bool measure_allowed);
 int choose_plan(rift_ile_t *h, int64_t n, bool measure_allowed)
 {
     const int rc = choose_plan_tuned(h, n, measure_allowed);
+    h->plan.plain64 = h->plain64 ? 1 : 0;
     apply_sort_override(h);
     return rc;
 }

@@ -4,8 +4,9 @@
 // The float64 pipe of this part does about two operations a clock and SM, so the plain
 // float64 kernel (k_lnl.cu) is bound by it: 6 operations a mode, bin and detector.  Here
 // the mode sum, the interpolation and the log-sum-exp over the time bins run in fixed point
-// instead, exactly or to at least float64's resolution, and the float64 pipe is left with
-// the per-sample geometry:
+// instead, exactly or to float64's resolution of the largest |c| times the largest |Q|, and the
+// float64 pipe is left with the per-sample geometry (overlaps that are too uneven for one scale
+// take the plain kernel: uneven64 below):
 //   * the coefficients c_k,lm of a sample (one power-of-two scale over its detectors and
 //     modes) and Q (one scale) are rounded to 55-bit integers, each cut into kDig = 7
 //     balanced base-256 digits d_0..d_6 (|d| <= 128, exact in float16);
@@ -193,23 +194,112 @@ __device__ __forceinline__ uint32_t digit_pair(uint64_t x, uint64_t y, int part)
     return r;
 }
 
-__global__ void max64_kernel(const double2 *__restrict__ Q, int64_t count, unsigned long long *__restrict__ out)
+// Q columns that some sample's bins reach, per detector (the Q window may be wider; what lies in
+// the rest of it is no scale of anything).
+struct Reach {
+    int lo[kMaxDet], hi[kMaxDet];
+    double inv[kMaxDet];   // 1 / columns
+};
+
+Reach reach_of(const Problem &P)
 {
+    Reach r{};
+    for (int k = 0; k < P.K; ++k) {
+        double d2 = 0.0;
+        for (int i = 0; i < 3; ++i)
+            d2 += P.xfs[k][i] * P.xfs[k][i];
+        const double d = std::sqrt(d2), last = P.ufs0[k] + (P.n_t - 1) * P.t_step * P.fs;
+        r.lo[k] = (int)std::max(0.0, std::floor(P.ufs0[k] - d) - 1.0);
+        r.hi[k] = (int)std::min((double)(P.n_q - 1), std::floor(last + d) + 2.0);
+        r.inv[k] = 1.0 / (r.hi[k] - r.lo[k] + 1);
+    }
+    return r;
+}
+
+// One block per (detector, mode): the largest component and the mean square modulus over the
+// reachable columns; the largest of all to out[0].
+__global__ void __launch_bounds__(256) scale64_kernel(const double2 *__restrict__ Q, int M, int n_q, Reach reach,
+                                                      unsigned long long *__restrict__ out, double2 *__restrict__ sizes)
+{
+    __shared__ unsigned long long ms[8];
+    __shared__ double ss[8];
+    const int k = blockIdx.x / M, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const double2 *row = Q + (size_t)blockIdx.x * n_q;
     unsigned long long m = 0ull;   // non-negative doubles order as integers
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < count; e += (int64_t)gridDim.x * blockDim.x) {
-        const double2 q = Q[e];
+    double s = 0.0;
+    for (int c = reach.lo[k] + threadIdx.x; c <= reach.hi[k]; c += blockDim.x) {
+        const double2 q = row[c];
         m = max(m, (unsigned long long)__double_as_longlong(fabs(q.x)));
         m = max(m, (unsigned long long)__double_as_longlong(fabs(q.y)));
+        s = fma(q.x, q.x, fma(q.y, q.y, s));
     }
 #pragma unroll
-    for (int o = 16; o; o >>= 1)
+    for (int o = 16; o; o >>= 1) {
         m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m)
-        atomicMax(out, m);
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    if (lane == 0) {
+        ms[warp] = m;
+        ss[warp] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < 8; ++w) {
+            m = max(m, ms[w]);
+            s += ss[w];
+        }
+        sizes[blockIdx.x] = make_double2(__longlong_as_double((long long)m), s * reach.inv[k]);
+        if (m)
+            atomicMax(out, m);
+    }
+}
+
+// Whether one scale serves: the largest component is at most kUneven times the rms of every
+// detector's strongest mode, and of the strongest mode with m = 2 and with m = -2 (alone in a
+// face-on or face-off sample).  An error in fixed point is 8e-17 of the largest |c| times the
+// largest |Q|, whichever detectors and modes a sample's value is made of; the plain kernel's bins
+// carry the rounding of their positions, 2.4e-14 of the local term at 16384 Hz, 300 times as much.
+// (Of the synthetic problems at SNRs of 8 to 150 the most uneven has 33.)  Zero rows say nothing.
+constexpr double kUneven = 256.0;
+
+// by a warp (non-negative doubles as integers: comparisons of doubles take the slow float64 pipe)
+__device__ bool uneven64(const Problem &P, const double2 *sizes)
+{
+    using Bits = unsigned long long;
+    const int lane = threadIdx.x & 31;
+    Bits top = 0, det[kMaxDet] = {}, pol[2] = {};
+    for (int e = lane; e < P.K * P.M; e += 32) {
+        const int k = e / P.M, s = P.mode_m[e - k * P.M];
+        const Bits largest = (Bits)__double_as_longlong(sizes[e].x), square = (Bits)__double_as_longlong(sizes[e].y);
+        top = max(top, largest);
+#pragma unroll
+        for (int i = 0; i < kMaxDet; ++i)
+            det[i] = k == i ? max(det[i], square) : det[i];
+        pol[0] = s == 2 ? max(pol[0], square) : pol[0];
+        pol[1] = s == -2 ? max(pol[1], square) : pol[1];
+    }
+    auto most = [](Bits v) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1)
+            v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+        return v;
+    };
+    Bits least = ~0ull;
+    auto take = [&](Bits v) {
+        v = most(v);
+        least = v ? min(least, v) : least;
+    };
+#pragma unroll
+    for (int i = 0; i < kMaxDet; ++i)
+        take(det[i]);
+    take(pol[0]);
+    take(pol[1]);
+    const double t = __longlong_as_double((long long)most(top));
+    return least != ~0ull && !(t * t <= kUneven * kUneven * __longlong_as_double((long long)least));
 }
 
 // Q digits: [K][kDig][groups][kp/8][8 columns][8 components]
-__global__ void digits_q_kernel(const double2 *__restrict__ Q, int K, int M, int n_q, int groups, int kp,
+__global__ void digits_q_kernel(const double2 *__restrict__ Q, int K, int M, int n_q, int groups, int kp, Reach reach,
                                 const unsigned long long *__restrict__ qmax, __half *__restrict__ out)
 {
     const int sq = 55 - exp_above(__longlong_as_double((long long)*qmax));
@@ -221,7 +311,7 @@ __global__ void digits_q_kernel(const double2 *__restrict__ Q, int K, int M, int
         const int g = (int)(w / (kp * 8)), rem = (int)(w - (int64_t)g * kp * 8);
         const int kc = rem / 64, row = (rem / 8) % 8, m = (8 * kc + rem % 8) / 2, c = 8 * g + row;
         uint64_t x = digit_bytes(0), y = x;
-        if (c < n_q && m < M) {
+        if (c >= reach.lo[k] && c <= reach.hi[k] && m < M) {
             const double2 q = Q[((int64_t)k * M + m) * n_q + c];
             x = digit_bytes(__double2ll_rn(ldexp(q.x, sq)));
             y = digit_bytes(__double2ll_rn(ldexp(q.y, sq)));
@@ -241,15 +331,17 @@ __device__ __forceinline__ double template_entry(const double2 *U, const double2
 }
 
 // Template digits: [K][kDig][kBlk/8 groups][kp/8][8 columns of T][8 components]; exps[k]
-// such that |T_k| < 2^exps[k].  One block per detector.
-__global__ void digits_t_kernel(const double2 *__restrict__ U64, const double2 *__restrict__ V64, int M, int kp,
-                                __half *__restrict__ out, int *__restrict__ exps)
+// such that |T_k| < 2^exps[k].  One block per detector (the last one looks at the overlaps' sizes too).
+__global__ void digits_t_kernel(Problem P, int kp, const double2 *__restrict__ sizes, __half *__restrict__ out,
+                                int *__restrict__ exps, int *err)
 {
     __shared__ unsigned long long mx;
-    const int k = blockIdx.x, R2 = 2 * M;
-    const double2 *U = U64 + (size_t)k * M * M, *V = V64 + (size_t)k * M * M;
+    const int k = blockIdx.x, M = P.M, R2 = 2 * M;
+    const double2 *U = P.U64 + (size_t)k * M * M, *V = P.V64 + (size_t)k * M * M;
     if (threadIdx.x == 0)
         mx = 0ull;
+    if (k == P.K - 1 && threadIdx.x >= blockDim.x - 32 && uneven64(P, sizes) && (threadIdx.x & 31) == 0)
+        atomicOr(err, kNoteUneven);
     __syncthreads();
     for (int e = threadIdx.x; e < R2 * R2; e += blockDim.x)
         atomicMax(&mx, (unsigned long long)__double_as_longlong(fabs(template_entry(U, V, M, e / R2, e % R2))));
@@ -466,19 +558,22 @@ void tc64_positions(const rift_ile_config &cfg, long long *pos, long long *u0)
             std::ldexp(((long double)cfg.t_lo_s - (long double)cfg.q_t0_s[k]) * (long double)cfg.fs_hz, kFrac));
 }
 
+size_t tc64_scale_words(int K, int M) { return 2 + 2 * (size_t)K * M; }
+
 cudaError_t launch_prep_tc64(const Problem &P, unsigned long long *qmax, __half *q_dig, __half *t_dig, int *t_exp,
-                             cudaStream_t st)
+                             int *err, cudaStream_t st)
 {
     const int kp = (2 * P.M + 15) / 16 * 16;
     cudaError_t e = cudaMemsetAsync(qmax, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess)
         return e;
-    const int64_t cnt = (int64_t)P.K * P.M * P.n_q;
-    max64_kernel<<<(int)std::min<int64_t>((cnt + 255) / 256, 512), 256, 0, st>>>(P.Q64, cnt, qmax);
+    const Reach reach = reach_of(P);
+    double2 *sizes = reinterpret_cast<double2 *>(qmax + 2);
+    scale64_kernel<<<P.K * P.M, 256, 0, st>>>(P.Q64, P.M, P.n_q, reach, qmax, sizes);
     const int64_t tot = (int64_t)P.K * P.tc_groups * kp * 4;
-    digits_q_kernel<<<(int)std::min<int64_t>((tot + 255) / 256, 2048), 256, 0, st>>>(P.Q64, P.K, P.M, P.n_q,
-                                                                                    P.tc_groups, kp, qmax, q_dig);
-    digits_t_kernel<<<P.K, 512, 0, st>>>(P.U64, P.V64, P.M, kp, t_dig, t_exp);
+    digits_q_kernel<<<(int)std::min<int64_t>((tot + 255) / 256, 2048), 256, 0, st>>>(
+        P.Q64, P.K, P.M, P.n_q, P.tc_groups, kp, reach, qmax, q_dig);
+    digits_t_kernel<<<P.K, 512, 0, st>>>(P, kp, sizes, t_dig, t_exp, err);
     return cudaGetLastError();
 }
 
