@@ -848,16 +848,16 @@ int rift_ile_create(const rift_ile_config *cfg, void *cuda_stream, rift_ile_t **
             (rc = dalloc(h, &h->t_dig, tc64_t_halves(K, M))) || (rc = dalloc(h, &h->t_exp64, (size_t)kMaxDet)) ||
             (rc = dalloc(h, &scratch, tc64_scratch_bytes(K, M, N, sms))) ||
             (rc = dalloc(h, &records, tc64_record_bytes(N, cfg->n_t))) || (rc = dalloc(h, &pos, (size_t)cfg->n_t + kTc64Table)) ||
-            (rc = dalloc(h, &unit_counter, (size_t)8)) ||
+            (rc = dalloc(h, &unit_counter, (size_t)8 + sms)) ||
             (rc = dalloc(h, &units, (size_t)2 * tc64_units_cap(N)))) {
             release(h);
             return rc;
         }
-        h->x64 = Tc64{h->qmax64, h->q_dig, h->t_dig, h->t_exp64, scratch, records, unit_counter, units,
+        h->x64 = Tc64{h->qmax64, h->q_dig, h->t_dig, h->t_exp64, scratch, records, unit_counter, unit_counter + 8, units,
                       tc64_units_cap(N), unit_counter + 4, pos, {}};
         std::vector<long long> host_pos(cfg->n_t + kTc64Table);
         tc64_positions(h->cfg, host_pos.data(), h->x64.u0);
-        if (cudaMemsetAsync(unit_counter, 0, sizeof(int), h->stream) ||
+        if (cudaMemsetAsync(unit_counter, 0, sizeof(int) * (8 + sms), h->stream) ||
             cudaMemcpyAsync(pos, host_pos.data(), sizeof(long long) * host_pos.size(), cudaMemcpyHostToDevice, h->stream) ||
             cudaStreamSynchronize(h->stream)) {
             cudaGetLastError();
@@ -963,7 +963,7 @@ int64_t rift_ile_footprint(const rift_ile_config *cfg)
         K * 2 * groups * kp * 8 * 2, 5 * kRedBlocks * 8, 152 * 12 * B * 8, 8 * (RIFT_MAX_ITER + 1) * 8, 3 * 8 * 8,
         N * 4, 16, 6 * B * 8, 6 * (B + 1) * 8, 6 * B * 8, 16, (int64_t)kSelectWords * 4,
         cfg->precision == RIFT_MIXED && !digits ? std::min<int64_t>(N, kRefineRows) * nt * 8 : 0,
-        digits ? 2 * (int64_t)(tc64_q_halves(K, M, groups) + tc64_t_halves(K, M)) + 8 * (int64_t)tc64_scale_words(K, M) + 7 * 16 + 8 * (nt + kTc64Table) +
+        digits ? 2 * (int64_t)(tc64_q_halves(K, M, groups) + tc64_t_halves(K, M)) + 8 * (int64_t)tc64_scale_words(K, M) + 8 * 16 + 152 * 4 + 8 * (nt + kTc64Table) +
                      (int64_t)(16 * tc64_units_cap(N) + tc64_scratch_bytes(K, M, N, 152) + tc64_record_bytes(N, cfg->n_t))
                : 0,
         // large-term correction: per-sample side outputs and list, double-float tables of the

@@ -177,6 +177,7 @@ struct Tc64 {
     unsigned char *scratch;           // coefficient digits of the resident tiles
     unsigned char *records;           // the chunks' sums of a batch whose time bins are split
     int *unit_counter;                // 0 between launches
+    int *arrived;                     // [multiprocessors] units of a tile that are done; 0 between launches
     unsigned long long *units;        // [2][units_cap] work units in four classes (tile_plan.cuh)
     int64_t units_cap;
     int *unit_counts;                 // [4] units per class

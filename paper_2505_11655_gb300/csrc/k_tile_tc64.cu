@@ -155,6 +155,25 @@ __host__ __device__ inline int parts64(int64_t tiles, int grid, int n_chunks)
     return best;
 }
 
+// Samples per tile and parts of a batch whose units are not planned.  While every tile of a quarter of
+// the lanes and every chunk of bins has a block of its own, the tiles are that small: a block's
+// prologue is bound by the float64 pipe and takes a quarter of the time (us a call: 512 samples of 1
+// detector, 1 mode, 101 bins 101 -> 90, 64 of 3, 21, 1001 276 -> 262; the plain kernel takes 77 and
+// 757).
+struct Cut64 {
+    int samples, parts;
+    int64_t tiles;
+};
+
+__host__ __device__ inline Cut64 cut64(int64_t n, int grid, int n_chunks)
+{
+    const int64_t small = (n + 31) / 32, tiles = (n + kS - 1) / kS;
+    const int most = n_chunks < 16 ? n_chunks : 16;
+    if (small * most <= grid)
+        return {32, most, small};
+    return {kS, parts64(tiles, grid, n_chunks), tiles};
+}
+
 // ---------------------------------------------------------------- digits
 
 // Position of the leading bit: |x| < 2^e for every x with |x| <= m (0 for m = 0).
@@ -634,11 +653,39 @@ units64_kernel(PlanProblem P, const double *__restrict__ theta, const uint32_t *
     plan_write(files, list, cap, counts);
 }
 
+// The value of sample i (index g) from its chunks' sums; `padded` samples a chunk.
+__device__ __forceinline__ void merge_sample(const Lse *records, int64_t padded, int64_t i, int n_chunks, int n_t,
+                                             const uint64_t *tbl, uint32_t g, double *__restrict__ lnL_tmarg,
+                                             const double *__restrict__ lnpw, double *__restrict__ lnw, int *err)
+{
+    // (other blocks' writes: not through this SM's first-level cache)
+    auto load = [&](int64_t at) {
+        const longlong2 v = __ldcg(reinterpret_cast<const longlong2 *>(records + at));
+        return Lse{v.x, (uint64_t)v.y};
+    };
+    const Lse info = load(n_chunks * padded + i);
+    const int lexp = (int)(int16_t)info.s, flags = (int)(uint16_t)(info.s >> 16);
+    double r = __longlong_as_double(0x7ff8000000000000LL);
+    if (flags == 0) {
+        DiffScale ds;
+        ds.set(lexp);
+        Lse run = load(i);
+        for (int c = 1; c < n_chunks; ++c)
+            run = merge64(ds, run, load(c * padded + i), tbl);
+        r = lse_value(run, lexp, __longlong_as_double(info.m), __uint_as_float((uint32_t)(info.s >> 32)), n_t);
+    }
+    if (!isfinite(r))
+        atomicOr(err, kErrNonFinite);
+    lnL_tmarg[g] = r;
+    if (lnw && lnpw)
+        lnw[g] = r + lnpw[g];
+}
+
 __global__ void __launch_bounds__(kThreads, 1)
 lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint32_t *__restrict__ perm, int64_t n,
                 double *__restrict__ lnL_tmarg, double *__restrict__ lnL_t, const double *__restrict__ lnpw,
                 double *__restrict__ lnw, int *err, int *unit_counter, const uint32_t *__restrict__ n_dev,
-                uint32_t skip, int planned)
+                uint32_t skip, int planned, int fused)
 {
     extern __shared__ __align__(128) unsigned char sm[];
     const int K = P.K, M = P.M, NT = P.n_t;
@@ -664,14 +711,15 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
     double *ps = reinterpret_cast<double *>(sm + L.ps), *pw = reinterpret_cast<double *>(sm + L.pw);
     double2 *pe = reinterpret_cast<double2 *>(sm + L.pe), *Fs = reinterpret_cast<double2 *>(sm + L.F);
     double2 *Ys = reinterpret_cast<double2 *>(sm + L.Y);
-    __shared__ int unit_s, tile_s, chunks_s, abort_s;
+    __shared__ int unit_s, tile_s, chunks_s, abort_s, last_s;
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool producer = warp >= kIssuer;
     const int64_t n_use = device_count(n, n_dev, skip);
-    const int64_t n_tiles = (n_use + kS - 1) / kS;
     const int n_chunks = (NT + kChunk - 1) / kChunk, jnom = (NT + n_chunks - 1) / n_chunks;
-    const int parts = planned ? 1 : parts64(n_tiles, (int)gridDim.x, n_chunks);
+    const Cut64 cut = planned ? Cut64{kS, 1, (n_use + kS - 1) / kS} : cut64(n_use, (int)gridDim.x, n_chunks);
+    const int64_t n_tiles = cut.tiles;
+    const int parts = cut.parts;
     const bool split = planned ? has_records(n_tiles, n_chunks) : parts > 1;
     const int sq = 55 - exp_above(__longlong_as_double((long long)*X.qmax));
     const uint32_t sub_bytes = (uint32_t)(kSub * kp * 2);           // one digit of a batch's columns
@@ -714,7 +762,11 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
         tc::fence_proxy_async_smem();
         if (tid == 0) {
             // the first unit by the block's index, the others from the counter
-            unit_s = abort_s ? INT_MAX : first ? (int)blockIdx.x : (int)gridDim.x + atomicAdd(unit_counter, 1);
+            // (no others where a launch merges for itself)
+            unit_s = abort_s ? INT_MAX
+                     : first ? (int)blockIdx.x
+                     : fused ? INT_MAX
+                             : (int)gridDim.x + atomicAdd(unit_counter, 1);
             first = false;
             tile_s = -1;
             unsigned long long w;
@@ -747,12 +799,15 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
 
         // ---------------- prologue A: trigonometry in float64, a quarter of it per thread
         if (!producer) {
-            const int64_t si = tile * kS + s_of;
-            const uint32_t gi = si >= n_use ? 0xffffffffu : perm ? perm[si] : (uint32_t)si;
+            const int64_t si = tile * cut.samples + s_of;
+            const uint32_t gi = s_of >= cut.samples || si >= n_use ? 0xffffffffu : perm ? perm[si] : (uint32_t)si;
             const double *th = theta + 6 * (int64_t)gi;
             const bool valid = gi != 0xffffffffu;
-            if (grp == 0) {
+            if (grp == 0)
                 gid[s_of] = gi;
+            if (!__any_sync(0xffffffffu, valid)) {
+                // a lane quarter without samples: its rows of every table are left as they are
+            } else if (grp == 0) {
                 const Sky sk = sky_of(valid ? th[0] : 0.0, valid ? th[1] : 0.0, P.gmst);
                 nv[s_of] = sk.cd * sk.ch;
                 nv[kS + s_of] = sk.cd * sk.sh;
@@ -802,8 +857,9 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             }
         }
         __syncthreads();
+        const bool live = !producer && __any_sync(0xffffffffu, gid[s_of] != 0xffffffffu);
         // ---------------- B: delays, x F_k, harmonics, and the largest |F|^2 and |Y|^2
-        if (!producer) {
+        if (live) {
             if (tid < kS * K) {
                 const int k = grp;
                 const double n0 = nv[s_of], n1 = nv[kS + s_of], n2 = nv[2 * kS + s_of];
@@ -846,7 +902,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
         }
         __syncthreads();
         // ---------------- C: the sample's scale and the digits of its coefficients
-        if (!producer) {
+        if (live) {
             const double f2 = __longlong_as_double((long long)mF2[s_of]), y2 = __longlong_as_double((long long)mY2[s_of]);
             int ef = 0, ey = 0;
             const bool zero = !(f2 > 0.0) || !(y2 > 0.0) || !isfinite(f2) || !isfinite(y2);
@@ -982,6 +1038,25 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     }
             }
             __syncwarp();
+        } else if (any && !live) {
+            // the four warps of a lane quarter without samples: its accumulators stay where they are
+            auto pass = [&]() {
+                const uint32_t b = g & 1u;
+                const bool ok = tc::mbar_wait(done + b, (g >> 1) & 1u, kWait);
+                ++g;
+                __syncwarp();
+                tc::mbar_arrive_if(empty + b, lane == 0);
+                return ok;
+            };
+            for (int k = 0; k < K && !failed; ++k)
+                failed = !pass() || !pass();
+            for (int ch = ch0; ch < ch1 && !failed; ++ch)
+                for (int k = 0; k < K && !failed; ++k) {
+                    int w0, nsub;
+                    window(k, ch * jnom, min(NT, (ch + 1) * jnom), w0, nsub);
+                    for (int t = 0; t < nsub && !failed; ++t)
+                        failed = !pass();
+                }
         } else if (any) {
             const int q = warp & 3, cb = warp >> 2, s = 32 * q + lane;   // drain: quarter, 8 columns of 32
             const int gs = s_of, gh = grp;                               // gather: sample, quarter of the bins
@@ -1162,7 +1237,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     if (!split)
                         run = ch == 0 ? c : merge64(ds, run, c, tbl);
                     else
-                        records[((int64_t)ch * n_tiles + tile) * kS + gs] = c;
+                        records[((int64_t)ch * n_tiles + tile) * cut.samples + gs] = c;
                 }
             }
             // the sample's value (or what the combination needs), by its first thread
@@ -1178,7 +1253,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                     if (lnw && lnpw)
                         lnw[gi] = r + lnpw[gi];
                 } else if (ch0 == 0) {
-                    records[((int64_t)n_chunks * n_tiles + tile) * kS + gs] =
+                    records[((int64_t)n_chunks * n_tiles + tile) * cut.samples + gs] =
                         Lse{__double_as_longlong(quad), pack_info(lexp, flags, quad_lo)};
                 }
                 if (flags)
@@ -1197,10 +1272,17 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
                 if (lnw && lnpw)
                     lnw[gi] = r;
             } else if (ch0 == 0) {
-                records[((int64_t)n_chunks * n_tiles + tile) * kS + s_of] = Lse{0, pack_info(0, kErrNonFinite, 0.f)};
+                records[((int64_t)n_chunks * n_tiles + tile) * cut.samples + s_of] = Lse{0, pack_info(0, kErrNonFinite, 0.f)};
             }
         }
+        if (fused && split)
+            __threadfence();   // this thread's records, before its block's arrival
         failed = __syncthreads_or(failed || abort_s);
+        if (fused && split && tid == 0) {   // (every unit arrives, a failed one too: the counts end at zero)
+            last_s = atomicAdd(X.arrived + tile, 1) == parts - 1;
+            if (last_s)
+                X.arrived[tile] = 0;
+        }
         if (failed) {
             if (tid == 0) {
                 atomicOr(err, kErrTimeout);
@@ -1208,6 +1290,14 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
             }
             __syncthreads();
             continue;
+        }
+        if (fused && split) {
+            __syncthreads();
+            if (last_s && !producer && grp == 0 && gid[s_of] != 0xffffffffu) {
+                __threadfence();
+                merge_sample(records, n_tiles * cut.samples, tile * cut.samples + s_of, n_chunks, NT, tbl, gid[s_of],
+                             lnL_tmarg, lnpw, lnw, err);
+            }
         }
     }
     // leave: no copy of this block still landing (after a failure the issuer may not have
@@ -1230,7 +1320,7 @@ lnl_tc64_kernel(Problem P, Tc64 X, const double *__restrict__ theta, const uint3
 }
 
 // Merges the chunks' sums of every sample (nothing to do when the bins were not split) and
-// resets the unit counter.
+// resets the unit counter, after a launch that does not merge for itself.
 __global__ void combine64_kernel(const Lse *__restrict__ records, const long long *__restrict__ pos, const uint32_t *__restrict__ perm, int64_t n,
                                  const uint32_t *__restrict__ n_dev, uint32_t skip, int planned, int grid, int n_t, double *__restrict__ lnL_tmarg,
                                  const double *__restrict__ lnpw, double *__restrict__ lnw, int *err,
@@ -1239,32 +1329,17 @@ __global__ void combine64_kernel(const Lse *__restrict__ records, const long lon
     if (blockIdx.x == 0 && threadIdx.x == 0)
         *unit_counter = 0;   // for the next launch
     const int64_t n_use = device_count(n, n_dev, skip);
-    const int64_t n_tiles = (n_use + kS - 1) / kS;
     const int n_chunks = (n_t + kChunk - 1) / kChunk;
-    if (planned ? !has_records(n_tiles, n_chunks) : parts64(n_tiles, grid, n_chunks) == 1)
+    const Cut64 cut = planned ? Cut64{kS, 1, (n_use + kS - 1) / kS} : cut64(n_use, grid, n_chunks);
+    if (planned ? !has_records(cut.tiles, n_chunks) : cut.parts == 1)
         return;
+    const int64_t padded = cut.tiles * cut.samples;
     __shared__ uint64_t tbl[kTable];
     for (int i = threadIdx.x; i < kTable; i += blockDim.x)
         tbl[i] = (uint64_t)pos[n_t + i];
     __syncthreads();
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_use; i += (int64_t)gridDim.x * blockDim.x) {
-        const Lse info = records[(int64_t)n_chunks * n_tiles * kS + i];
-        const int lexp = (int)(int16_t)info.s, flags = (int)(uint16_t)(info.s >> 16);
-        const uint32_t g = perm ? perm[i] : (uint32_t)i;
-        double r = __longlong_as_double(0x7ff8000000000000LL);
-        if (flags == 0) {
-            DiffScale ds;
-            ds.set(lexp);
-            Lse run = records[i];
-            for (int c = 1; c < n_chunks; ++c)
-                run = merge64(ds, run, records[(int64_t)c * n_tiles * kS + i], tbl);
-            r = lse_value(run, lexp, __longlong_as_double(info.m), __uint_as_float((uint32_t)(info.s >> 32)), n_t);
-        }
-        if (!isfinite(r))
-            atomicOr(err, kErrNonFinite);
-        lnL_tmarg[g] = r;
-        if (lnw && lnpw)
-            lnw[g] = r + lnpw[g];
+        merge_sample(records, padded, i, n_chunks, n_t, tbl, perm ? perm[i] : (uint32_t)i, lnL_tmarg, lnpw, lnw, err);
     }
 }
 
@@ -1297,15 +1372,22 @@ cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta
         units64_kernel<<<(unsigned)((tiles + kPlanWarps - 1) / kPlanWarps), 32 * kPlanWarps, 0, st>>>(
             plan_problem(P), theta, perm, n, n_dev, skip, grid, X.units, X.units_cap, X.unit_counts);
     }
+    // a block per unit: the last of a tile's units merges its chunks' sums, and no kernel follows
+    // (5 to 14 us of a call of 1 to 2000 samples: 512 of 2 detectors, 2 modes, 401 bins 118 -> 109,
+    // the plain kernel 116)
+    const Cut64 cut = cut64(n, grid, (P.n_t + kChunk - 1) / kChunk);
+    const int fused = !n_dev && !planned && cut.tiles * cut.parts <= grid ? 1 : 0;
     lnl_tc64_kernel<<<grid, kThreads, smem, st>>>(P, X, theta, perm, n, lnL_tmarg, lnL_t, lnpw, lnw, err,
-                                                  X.unit_counter, n_dev, skip, planned);
+                                                  X.unit_counter, n_dev, skip, planned, fused);
+    if (launched)
+        *launched = 2 + planned - fused;
+    if (fused)
+        return cudaGetLastError();
     // the split depends on the device count; it never has more tiles than there are records for
     const int64_t most = std::min<int64_t>(tiles, split_tiles(n, P.n_t));
     combine64_kernel<<<(int)std::max<int64_t>(1, most), 128, 0, st>>>(reinterpret_cast<const Lse *>(X.records), X.pos, perm, n,
                                                                     n_dev, skip, planned, grid, P.n_t, lnL_tmarg, lnpw, lnw, err,
                                                                     X.unit_counter);
-    if (launched)
-        *launched = 2 + planned;
     return cudaGetLastError();
 }
 
