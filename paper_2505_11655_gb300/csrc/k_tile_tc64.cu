@@ -86,7 +86,8 @@ constexpr uint64_t kWait = 1000000000ull;
 constexpr int kRecords = 4096;           // (tile, chunk) pairs of a batch whose time bins are split
 constexpr int kSumBits = 52;             // resolution of the log-sum-exp (at most 4000 terms <= 1)
 constexpr size_t kMinSmem = 120 * 1024;  // one block per SM
-constexpr int64_t kPlanFrom = 64;        // tiles from which a batch's units are planned
+constexpr int64_t kPlanFrom = 128;       // tiles from which a batch's units are planned,
+constexpr double kPlanSpan = 12.0 * kSub;   // where the delays span this many columns
 constexpr int kUnitsPerTile = 16;
 constexpr float kUnitsPerBlock = 2.2f;
 static_assert(kS == kPlanSamples, "tiles of the planning code");
@@ -1360,11 +1361,21 @@ cudaError_t launch_lnl_tc64(const Problem &P, const Tc64 &X, const double *theta
     const size_t smem = std::max(kMinSmem, layout64(P.K, P.M, P.n_t).end);
     const int64_t tiles = (n + kS - 1) / kS;
     const int grid = (int)std::min<int64_t>(sms, 16 * tiles);
-    // Planned are whole batches (20,011 samples of the largest problem 1409 -> 1328 us a call).  The
-    // time bins of smaller ones are split evenly, and so are those of a device-side list: its
-    // iteration has other kernels beside it or behind it, and more units mean more prologues
-    // (twelve solves as one graph 9.2 -> 9.8 ms when their lists were planned).
-    const int planned = !n_dev && tiles >= kPlanFrom ? 1 : 0;
+    // Planned are whole batches whose tiles' widths differ by more than the plan costs: two detectors
+    // or more (one detector's sort key is its delay) whose delays span many batches of columns.
+    // 16384 Hz, 20,011 samples: 3 detectors, 21 modes 1.06 times the speed of an even split, 2, 9
+    // 1.12; 40,000 1.04 and 1.01; 12,000 0.92 and 0.94.  4096 Hz or one detector, 20,011 samples 0.98
+    // to 0.99, 8200 0.72 to 0.85.  The time bins of the others are split evenly, and so are those of a
+    // device-side list: its iteration has other kernels beside it or behind it, and more units mean
+    // more prologues (twelve solves as one graph 9.2 -> 9.8 ms when their lists were planned).
+    double span = 0.0;
+    for (int k = 0; k < P.K; ++k) {
+        double r2 = 0.0;
+        for (int i = 0; i < 3; ++i)
+            r2 += P.xfs[k][i] * P.xfs[k][i];
+        span = std::max(span, 2.0 * std::sqrt(r2));
+    }
+    const int planned = !n_dev && tiles >= kPlanFrom && P.K > 1 && span >= kPlanSpan ? 1 : 0;
     if (planned) {
         e = cudaMemsetAsync(X.unit_counts, 0, kPlanClasses * sizeof(int), st);
         if (e != cudaSuccess)

@@ -45,3 +45,18 @@ def test_small_batches(G, dets, modes, n_t):
     with G.ILE(p, precision=G.RIFT_FP64, max_samples=97) as s:
         for c in (1, 33, 97):
             assert np.array_equal(s.eval(th[:c]), full[:c])
+
+
+@pytest.mark.parametrize("n_t,n", [(1001, 20011), (65, 17000), (401, 90001)])
+def test_planned_batches(G, n_t, n):
+    """Large batches of wide delays, whose units are planned by the tiles' widths: split time grids
+    and whole tiles (too many for the split's records)."""
+    p = S.make_problem(("H1", "L1", "V1"), 4, 16384.0, n_t=n_t, snr=20.0, seed=S.config_seed(6, 190))
+    th = S.prior_samples(n, 191)
+    with G.ILE(p, precision=G.RIFT_FP64, max_samples=n) as s:
+        full = s.eval(th)
+        a = G.rift_ile_kernel_launches(s.h)
+        assert np.array_equal(s.eval(th), full)
+        assert G.rift_ile_kernel_launches(s.h) - a == 10   # keys, two passes of three, plan, likelihood, merge
+        pick = np.random.default_rng(0).choice(n, 600, replace=False)
+        assert np.array_equal(s.eval(th[pick]), full[pick])
