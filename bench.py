@@ -64,6 +64,7 @@ TRAFFIC_BY_SOURCE = {
     "a1a0f3fa500f237d67cded3cf3f47eaac17dae8af6c99f541d525a7f85a14ff1": 6.03e7,
     "70258efe81120ca38cdd3f22b5ffc4ac29c4003ba3fdf3b4467adb6ac9f57fc1": 5.97e7,
     "21b0526213563248a645bad3b51375dfc6c723048d9f563bfd77c6252ca56bd0": 6.78e7,
+    "018981b7599231227db8509dbff72b0a4c69212c2e3c0c09721eb2dc3ad00804": 6.79e7,
 }
 
 

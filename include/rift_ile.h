@@ -57,7 +57,7 @@ extern "C" {
 #define RIFT_QUAD_QUARTER 0 /* kappa = 1/4, as printed in Eq. (def:lnL:Decomposed) */
 #define RIFT_QUAD_HALF 1    /* kappa = 1/2 (equivalent to QUARTER with U, V doubled)  */
 
-#define RIFT_FP64 0  /* every step in float64: the plain reference GPU path               */
+#define RIFT_FP64 0  /* float64, or fixed point of its resolution: the reference precision */
 #define RIFT_FP32 1  /* float32 bulk arithmetic; float64 delays, log-sum-exp and sums; the  */
                      /* samples with large data and template terms corrected in           */
                      /* double-float, so every ln L is within 1e-3 of the float64 value   */

@@ -42,14 +42,14 @@
 // not depend on the batch, the tile or the split.
 //
 // Measured (3 detectors, 21 modes, 16384 Hz, 1001 bins, 20011 prior samples): 20.3 ms for the
-// plain float64 kernel (70% of the float64 issue rate), 1.35 ms here; 100,000 samples 98.5 ->
-// 4.3 ms; 64 samples of the smallest problem (2 detectors, 2 modes) 109 -> 107 us.  Against
+// plain float64 kernel (70% of the float64 issue rate), 1.25 to 1.29 ms here; 100,000 samples 98.5
+// -> 4.0 ms; 64 samples of 2 detectors, 2 modes, 401 bins 116 -> 99 us.  Against
 // 80-bit arithmetic (8 problems at 3 SNRs, 1000 prior samples each, relative norms) its per-bin values
-// are closer than the plain kernel's (0.45 to 0.85 of its error), ln L is as close (geometric mean of
-// the ratios 0.94; the template term alone 4.0e-16 to 5.9e-16 in both: the geometry's roundings).
-// With orders to 6 and float64 sums the template term had up to 6.6e-16.  What bounds it now is instruction issue (46% of the slots: the
-// joins of the accumulators, the gathers' 64-bit arithmetic) and the tail of uneven tiles; the
-// tensor pipe is 26% busy, the float64 pipe 11%.
+// are closer than the plain kernel's (0.45 to 0.83 of its error), ln L is as close (geometric mean of
+// the ratios 0.94; the template term alone 3.7e-16 to 5.9e-16 in both: the geometry's roundings).
+// With orders to 6 and float64 sums the template term had up to 6.6e-16.  What bounds it now is
+// instruction issue (43% of the slots: the joins of the accumulators, the gathers' 64-bit
+// arithmetic) and the quarters' barriers; the tensor pipe is 26% busy, the float64 pipe 13%.
 //
 // All waits are bounded (1 s by the global timer), as in k_tile_tc.cu.
 #include <algorithm>
