@@ -20,7 +20,7 @@
 // neighbours in the sort: unsorted or thinly spread samples cost the union of their windows
 // (at most 1.4 times one window at 16384 Hz).  Tiles of 64 samples over 256-column windows, which
 // this replaces, needed compact tiles: a call with 256 samples of 3 detectors, 21 modes, 1001 bins at
-// 16384 Hz took 2.2 ms, now 0.30 ms; 10,000 of 2 detectors and 9 modes 0.63 ms, now 0.27 ms.
+// 16384 Hz took 2.2 ms, now 0.16 ms; 10,000 of 2 detectors and 9 modes 0.62 ms, now 0.22 ms.
 // Eight samples a block, two blocks per SM: with sixteen, Q is read half as often, but the
 // prologue's latency has one other block less to hide behind (5-8% slower).
 #include <algorithm>
